@@ -50,6 +50,10 @@ layernorm_kernel(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __res
     const int wr = warp / WPR, wp = warp % WPR;           // row of the CTA's group, part of the row
     const int nvec = D >> 3;                              // 16-byte vectors per row
     const float inv_d = 1.f / static_cast<float>(D);
+    // (launched with programmatic stream serialization: nothing in device memory is touched before the previous kernel
+    // of the stream has finished)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     int it = 0;
     for (long long row0 = static_cast<long long>(blockIdx.x) * RPB; row0 < M; row0 += static_cast<long long>(gridDim.x) * RPB, it ^= 1) {
         const long long row = row0 + wr;
@@ -129,9 +133,18 @@ int launch_ln_nv(const void* X, const void* R, const void* gamma, const void* be
     const long long cap = static_cast<long long>(device_sm_count()) * 8;      // 8 CTAs of 256 threads per SM
     const int grid = static_cast<int>(blocks_needed < cap ? blocks_needed : cap);
     auto bf = [](const void* p) { return static_cast<const __nv_bfloat16*>(p); };
-    if (R) layernorm_kernel<NV, WPR, true><<<grid, LN_WARPS * 32, 0, st>>>(bf(X), bf(R), bf(gamma), bf(beta), static_cast<__nv_bfloat16*>(Y), M, D, eps);
-    else   layernorm_kernel<NV, WPR, false><<<grid, LN_WARPS * 32, 0, st>>>(bf(X), nullptr, bf(gamma), bf(beta), static_cast<__nv_bfloat16*>(Y), M, D, eps);
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(LN_WARPS * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = R ? cudaLaunchKernelEx(&cfg, layernorm_kernel<NV, WPR, true>, bf(X), bf(R), bf(gamma), bf(beta), static_cast<__nv_bfloat16*>(Y), M, D, eps)
+                            : cudaLaunchKernelEx(&cfg, layernorm_kernel<NV, WPR, false>, bf(X), bf(nullptr), bf(gamma), bf(beta), static_cast<__nv_bfloat16*>(Y), M, D, eps);
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
 }  // namespace

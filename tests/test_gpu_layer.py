@@ -161,6 +161,31 @@ def test_fully_connected(api, shape):
     assert np.mean(g == oracle.bf16_bits_to_f64(oracle.round_to_bf16_bits(ref))) > 0.98
 
 
+# one size for every tile that launch_gemm chooses, ragged in M, contraction lengths that no split divides evenly
+TILE_SHAPES = [(131, 1024, 256), (1, 576, 512), (500, 320, 1024), (500, 1088, 1024), (601, 256, 768), (2100, 64, 1024),
+               (300, 512, 4096), (1300, 192, 2048), (3000, 1024, 1024), (2600, 256, 2304), (4100, 128, 2560)]
+
+
+@pytest.mark.parametrize("shape", TILE_SHAPES)
+def test_fully_connected_tiles(api, shape):
+    """fp32 sums of K products of order 1 / sqrt(K): the stored bf16 is the rounded oracle value except next to a rounding
+    boundary; two launches (split contractions included) give the same bits."""
+    M, K, Nout = shape
+    rng = np.random.default_rng(M + K)
+    X = rand_bits(rng, (M, K)); W = rand_bits(rng, (Nout, K), sigma=K ** -0.5)
+    Xt, Wt = bf16_tensor(X), bf16_tensor(W)
+    Y = torch.full((M, Nout), 5.0, device="cuda", dtype=torch.bfloat16); Y2 = Y.clone()
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    api.flat_fc_fwd(Xt, Wt, Y, status=status)
+    api.flat_fc_fwd(Xt, Wt, Y2, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(Y, Y2)
+    ref = oracle.fully_connected(X, W)
+    g = bf16_to_f64(Y)
+    assert np.abs(g - ref).max() <= np.abs(ref).max() * 2.0 ** -7
+    assert np.mean(g == oracle.bf16_bits_to_f64(oracle.round_to_bf16_bits(ref))) > 0.98
+
+
 def test_layer_and_packed_calls_in_a_cuda_graph_on_two_streams(api):
     """The widened entry points also only enqueue work: a layer call and a packed variable-length call are
     captured on two streams of one graph (they run concurrently) and the replays reproduce the direct launches
