@@ -1,4 +1,8 @@
-"""ctypes binding of libflat_attn.so: argument marshalling only, same names as include/flat_attn.h.
+"""Binding of libflat_attn.so: argument marshalling only, same names as include/flat_attn.h.
+
+Calls on the device go through the extension module `_binding` (csrc/binding.cpp), which reads plain arguments in
+native code; what it hands back (-1: an argument that is not plain) takes the long way through ctypes, whose checks say
+what is wrong with it.
 
 Importing this module loads the CUDA library and raises if it is missing -- there is no
 CPU fallback.  Tensor arguments are torch tensors (device memory and streams are all
@@ -7,6 +11,7 @@ PyTorch is used for); every computation happens inside the library's kernels.
 from __future__ import annotations
 
 import ctypes
+import glob
 import os
 
 import torch
@@ -20,6 +25,11 @@ if not os.path.exists(LIB_PATH):
         "`__graft_entry__.build()`); there is no fallback path")
 
 _lib = ctypes.CDLL(LIB_PATH)
+
+if not glob.glob(os.path.join(_HERE, "_binding*.so")):
+    raise ImportError("the extension module _binding is not built (run `python -m paper_2107_06419_b200.build`)")
+
+from . import _binding  # noqa: E402  (after the library that it calls)
 
 FLAT_OK = 0
 FLAT_DTYPE_BF16, FLAT_DTYPE_F32 = 0, 1
@@ -229,6 +239,11 @@ def _check(rc: int):
 
 def flat_attn_fwd(Q, K, V, O, scale, stream=None):
     """Fused attention, bf16 CUDA tensors Q,O [B,H,Nq,d] and K,V [B,H,Nk,d]; writes O in place."""
+    rc = _binding.fwd(Q, K, V, O, scale, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return O
     p = _params(Q, K, V, O, scale, None, None, FLAT_VARIANT_AUTO)
     if p.dtype != FLAT_DTYPE_BF16:
         raise TypeError("flat_attn_fwd takes bfloat16 tensors; use flat_attn_fwd_ex for float32")
@@ -244,6 +259,11 @@ def flat_attn_fwd_ex(Q, K, V, O, scale, k_valid_len=None, status=None, variant=F
     (bfloat16 or float32) is added to the scaled logits before the softmax (-inf switches a pair off);
     `block_mask` (uint8 [B or 1, H or 1, ceil(Nq/128), ceil(Nk/128)]) prunes 128 x 128 blocks of the logit
     matrix (0 = the block takes no part)."""
+    rc = _binding.fwd_ex(Q, K, V, O, scale, k_valid_len, status, variant, stream, causal, lse, bias, block_mask)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return O
     p = _params(Q, K, V, O, scale, k_valid_len, status, variant, causal=causal, lse=lse, bias=bias,
                 block_mask=block_mask)
     _check(_lib.flat_attn_fwd_ex(ctypes.byref(p), _stream_ptr(stream)))
@@ -278,6 +298,11 @@ def flat_attn_bwd_ex(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, k_valid_len=
                      stream=None):
     """Backward pass: writes dQ [B,H,Nq,d], dK, dV [B,H,Nk,d] (bf16 CUDA tensors) from Q, K, V, the
     forward's O and lse [B,H,Nq] (float32), and dO; `delta` [B,H,Nq] float32 is scratch."""
+    rc = _binding.bwd_ex(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, k_valid_len, status, causal, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return dQ, dK, dV
     p = _bwd_params(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, k_valid_len, status, causal)
     _check(_lib.flat_attn_bwd_ex(ctypes.byref(p), _stream_ptr(stream)))
     return dQ, dK, dV
@@ -285,10 +310,7 @@ def flat_attn_bwd_ex(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, k_valid_len=
 
 def flat_attn_bwd(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, stream=None):
     """flat_attn_bwd_ex without masks and without a status word."""
-    p = _bwd_params(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, None, None, False)
-    _check(_lib.flat_attn_bwd(p.Q, p.K, p.V, p.O, p.dO, p.lse, p.dQ, p.dK, p.dV, p.delta, p.B, p.H, p.Nq, p.Nk, p.d,
-                              p.scale, _stream_ptr(stream)))
-    return dQ, dK, dV
+    return flat_attn_bwd_ex(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, stream=stream)
 
 
 def flat_attn_naive_fwd(Q, K, V, O, L, A, scale, stream=None):
@@ -372,6 +394,11 @@ def flat_out_proj_fwd(O, Wo, Y, status=None, stream=None):
 def flat_attn_layer_fwd(X, Wqkv, Wo, Y, Q, K, V, O, scale, causal=False, status=None, stream=None):
     """A self-attention layer: Q/K/V projection, fused attention, Output projection.  Q, K, V, O
     [B,H,N,d] are caller-owned buffers for the intermediates."""
+    rc = _binding.layer_fwd(X, Wqkv, Wo, Y, Q, K, V, O, scale, causal, status, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return Y
     B, H, N, d = Q.shape
     Dm = X.shape[2]
     _bf16_cuda("X", X, (B, N, Dm)); _bf16_cuda("Wqkv", Wqkv, (3 * H * d, Dm)); _bf16_cuda("Wo", Wo, (Dm, H * d))
@@ -386,6 +413,11 @@ def flat_attn_layer_fwd(X, Wqkv, Wo, Y, Q, K, V, O, scale, causal=False, status=
 
 def flat_fc_fwd(X, W, Y, status=None, stream=None):
     """Fully connected operator: X [..., K], W [Nout, K] -> Y [..., Nout] (bf16, no bias)."""
+    rc = _binding.fc_fwd(X, W, Y, status, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return Y
     K, Nout = X.shape[-1], W.shape[0]
     M = X.numel() // K
     _bf16_cuda("X", X, X.shape); _bf16_cuda("W", W, (Nout, K)); _bf16_cuda("Y", Y, tuple(X.shape[:-1]) + (Nout,))
@@ -395,6 +427,11 @@ def flat_fc_fwd(X, W, Y, status=None, stream=None):
 
 def flat_layernorm_fwd(X, gamma, beta, Y, eps=1e-5, residual=None, stream=None):
     """Y = gamma * layer_norm(X + residual) + beta over the last axis (bf16 CUDA tensors; gamma, beta [D])."""
+    rc = _binding.layernorm_fwd(X, gamma, beta, Y, eps, residual, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return Y
     D = X.shape[-1]
     M = X.numel() // D
     _bf16_cuda("X", X, X.shape); _bf16_cuda("Y", Y, X.shape); _bf16_cuda("gamma", gamma, (D,)); _bf16_cuda("beta", beta, (D,))
@@ -409,6 +446,11 @@ def flat_attn_varlen_fwd(Q, K, V, O, cu_seqlens_q, cu_seqlens_k, max_seqlen_q, s
                          stream=None):
     """Fused attention over a packed batch: Q, O [total_q, H, d], K, V [total_k, H, d] (bf16 CUDA);
     cu_seqlens_q / _k int32 CUDA tensors of num_seqs + 1 offsets."""
+    rc = _binding.varlen_fwd(Q, K, V, O, cu_seqlens_q, cu_seqlens_k, max_seqlen_q, scale, causal, status, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return O
     total_q, H, d = Q.shape
     total_k = K.shape[0]
     _bf16_cuda("Q", Q, (total_q, H, d)); _bf16_cuda("O", O, (total_q, H, d))

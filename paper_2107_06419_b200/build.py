@@ -1,10 +1,11 @@
-"""Compile libflat_attn.so for sm_100a with nvcc (in-tree, next to this file)."""
+"""Compile libflat_attn.so for sm_100a with nvcc, and the extension module _binding that calls it (in-tree, next to this file)."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -20,17 +21,21 @@ def nvcc_path() -> str:
     raise RuntimeError("nvcc not found: libflat_attn.so cannot be built")
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB):
+BINDING = os.path.join(HERE, "_binding.so")
+
+
+def _older(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS]
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not is_stale():
-        return LIB
+def is_stale() -> bool:
+    return _older(LIB, [os.path.join(CSRC, s) for s in SOURCES + HEADERS])
+
+
+def build_library(verbose: bool = False) -> None:
     tmp = LIB + ".%d.tmp" % os.getpid()
     cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
            "-shared", "-Xcompiler", "-fPIC", "-cudart", "static", "--threads", "0"]
@@ -39,6 +44,27 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd += [os.path.join(CSRC, s) for s in SOURCES] + ["-o", tmp]
     subprocess.check_call(cmd)
     os.replace(tmp, LIB)
+
+
+def build_binding() -> None:
+    """The extension module next to the library, which it is linked against (found through its own folder)."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include"), sysconfig.get_paths()["include"]]
+    tmp = BINDING + ".%d.tmp" % os.getpid()
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC"] + ["-I" + d for d in include]
+                          + [os.path.join(CSRC, "binding.cpp"), "-o", tmp, "-L" + os.path.join(root, "lib"), "-lc10",
+                             "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L" + HERE, "-l:libflat_attn.so",
+                             "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, BINDING)
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    if force or is_stale():
+        build_library(verbose)
+    if force or _older(BINDING, [os.path.join(CSRC, "binding.cpp"), os.path.join(HERE, "..", "include", "flat_attn.h")]):
+        build_binding()
     return LIB
 
 
