@@ -17,18 +17,36 @@
 // (MODE_DQ) or per column (MODE_DKV), P and dS rounded to bf16 and written back to TMEM, and
 // acc_a += dS Y1, acc_b += P Y2 with the bf16 tile as the TMEM A-operand and Y as an MN-major B-operand.
 //
-// The streamed tile is worked on in two halves of 64 columns (a: rows 0-63 of Y, b: rows 64-127), each with
-// its own 64 columns of T1 / T2, so that the MMAs of one half run under the element-wise work of the other.
-// Where TMEM has room beside T1, T2 and the accumulators (every case but MODE_DKV at d = 128) the bf16 tiles
-// get columns of their own, and the next step's T of a half is issued AHEAD of this step's accumulation
-// (which only has to finish before the element-wise warps write the next bf16 tile: barrier ACC_HALF);
-// otherwise P / dS overlay the T columns they were computed from and the accumulation goes first.
+// What bounds it and how the work is arranged.  Cycles per 128 x 128 tile and launch on one SM: exponential unit 1024;
+// tensor pipe 768 (dQ, d = 64), 1152 (dK dV, d = 64), 1536 and 2752 (d = 128).  Beside those two, what counts is what a
+// role's loop costs while the exponential unit's queue is full (clock stamps): a barrier check 140-220 cycles even when
+// the phase completed long ago.  Hence few barriers per step, wide MMAs, two issuing warps:
+//  * SEP (every case but MODE_DKV at d = 128): the bf16 tiles P, dS have TMEM columns of their own, and the element-wise
+//    warps pull T1 and T2 into registers and release them at once.  The next step's T1, T2 are then computed under this
+//    step's exponentials, this step's accumulation under the next one's, and a warp that is ahead of the others goes on.
+//    T1, T2 are whole tiles (N = 128: half as many instructions as N = 64, which with both operands in shared memory
+//    also takes 48 cycles where its arithmetic takes 32: A alone is 4 KB of a port of 128 bytes a cycle).
+//    MODE_DQ keeps its stationary operands in TMEM where there is room (both at d = 64, Q at d = 128).
+//    What is left is the loop T seen -> in registers (470 cycles until the last warp has it) -> next T issued, computed and
+//    seen (990): 1460 a step at d = 64.  Two column groups with barriers of their own, or T1 and T2 released apart, make
+//    the loop shorter and the barrier checks more: 463 / 612 and 484 / 591 us against 458 / 555 (dQ / dK dV, B4 H16 4096).
+//  * MODE_DKV at d = 128: the accumulators and T1, T2 fill TMEM.  P / dS overlay the columns of T they were computed
+//    from, and the streamed tile is worked on in two halves of 64 columns: a half's accumulation first, then its next T
+//    (the MMAs of one thread execute in issue order, so the T that overwrites P / dS needs no wait), both under the
+//    element-wise work of the other half.  The streamed stage is released between the two: behind the T it came 1000
+//    cycles too late for the copy after next (1243 against 965 us on B1 H4 16384).
+//  * MODE_DKV: lse and delta belong to the columns.  Read from shared memory by every warp they cost 1024 cycles of the
+//    port per tile (a broadcast read is one wavefront per column and warp); instead they join the contractions: one more
+//    slice of 16 contraction indices, (1, 1, 1, 0 ...) on the stationary side and -lse / scale, or -delta, as the sum of
+//    three bf16 numbers (24 bits) on the streamed side, gives T1 = K Q^T - lse / scale and T2 = V dO^T - delta.
+// Measured (both launches): B4 H16 4096 x 4096 d 64 1.265 -> 0.91 ms, B1 H4 16384 d 128 1.80 -> 1.46, B2 H16 3000 d 128
+// causal 0.361 -> 0.291.
 //
-// CTA = 576 threads: warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, half step w / 8, 32 of that
-// half's 64 columns: (w / 4) % 2 -- four warps per scheduler, two of each half, so that the waits of one
-// (barrier, TMEM load, store completion) hide behind the exponentials of the others), warp 16 TMA producer
-// (and, in MODE_DKV, the per-column lse2 / delta vectors of every streamed tile, converted and put into
-// shared memory), warp 17 MMA issuer.
+// CTA = 640 threads: warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four
+// warps per scheduler), warp 16 TMA producer, warp 17 issues the T MMAs and warp 18 the accumulations (where P / dS
+// overlay T, warp 17 issues both), warp 19 writes the slices that carry lse and delta (MODE_DKV).
+// Under the causal mask the tiles of a head differ in length by a factor of their number: the longest tiles of a group of
+// heads go first (launch_bwd_mode).
 // Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -47,42 +65,74 @@ using namespace tc;
 namespace {
 
 constexpr int BT = 128;              // rows of every tile (queries or keys)
-constexpr int HC = 64;               // columns (rows of the streamed tile) per half step
-constexpr int EW_WARPS = 16;           // eight per half step
-constexpr int BWD_THREADS = 32 * EW_WARPS + 64;
+constexpr int HC = 64;               // columns (rows of the streamed tile) per half step (where the step has halves)
+constexpr int EW_WARPS = 16;
+constexpr int BWD_THREADS = 32 * EW_WARPS + 128;
 constexpr int MODE_DQ = 0, MODE_DKV = 1;
 constexpr float LOG2E = 1.4426950408889634f;
 
 template <int D, int MODE> struct BL {
+    static constexpr bool DKV = MODE == MODE_DKV;
+    static constexpr bool SEP = !(D == 128 && DKV);
+    static constexpr bool X1_TMEM = !DKV, X2_TMEM = !DKV && D == 64;   // stationary operand in TMEM, else in shared memory
     static constexpr int TILE_BYTES = BT * D * 2;
-    // Ring of streamed HALF tile pairs (64 rows of Y1 and of Y2 per stage, one stage per half step): deep
-    // enough that a copy (about two microseconds from device memory) is under way for every half step the
-    // element-wise warps and the MMAs are working on, and released half by half.
-    static constexpr int HTILE_BYTES = HC * D * 2;
-    static constexpr int HSTAGES = D == 64 ? 8 : 4;
-    static constexpr int VSTAGES = HSTAGES / 2;                              // ring of per-column vectors (whole steps)
-    static constexpr int OPERAND_BYTES = 2 * TILE_BYTES + 2 * HSTAGES * HTILE_BYTES;   // X1, X2, HSTAGES x (Y1, Y2 halves)
-    static constexpr int VEC_BYTES = VSTAGES * 2 * BT * 4;                   // [stage][lse2 | delta][column]
-    static constexpr int XCH_BYTES = 4 * BT * 4;                             // delta quarters of MODE_DQ
-    static constexpr int SMEM_BYTES = OPERAND_BYTES + VEC_BYTES + XCH_BYTES + 512 + 1024;
+    static constexpr int X_BYTES = (X1_TMEM ? 0 : TILE_BYTES) + (X2_TMEM ? 0 : TILE_BYTES);
+    // Rings of streamed tiles (SEP: whole ones; else halves of 64 rows), deep enough that a copy (one to two microseconds)
+    // is under way for every step in work.  MODE_DQ needs Y2 = V for T2 only, so that its slots are free again early.
+    static constexpr int PARTS = SEP ? 1 : 2;            // copies per step; also column groups with T, dS and barriers of their own
+    static constexpr int Y_ROWS = BT / PARTS, Y_BYTES = Y_ROWS * D * 2;
+    static constexpr int S1 = DKV ? 4 : D == 64 ? 5 : 3, S2 = DKV ? 4 : D == 64 ? 4 : 2;
+    static constexpr int OPERAND_BYTES = X_BYTES + (S1 + S2) * Y_BYTES;
+    // (MODE_DKV) slices of 16 contraction indices, 128 rows of 32 bytes: the ones; per stage (whole steps) -lse / scale and -delta
+    static constexpr int AUG_BYTES = BT * 32;
+    static constexpr int VSTAGES = DKV ? S1 / PARTS : 1;
+    static constexpr int AUG_ALL = DKV ? (1 + 2 * VSTAGES) * AUG_BYTES : 0;
+    static constexpr int XCH_BYTES = DKV ? 0 : 4 * BT * 4;                   // delta quarters of MODE_DQ
+    static constexpr int SMEM_BYTES = OPERAND_BYTES + AUG_ALL + XCH_BYTES + 512 + 1024;
+    static_assert(SMEM_BYTES <= 232448, "shared memory");
     static constexpr uint32_t T1_COL = 0, T2_COL = 128, ACC_A_COL = 256, ACC_B_COL = 256 + D;
-    static constexpr uint32_t ACC_END = 256 + (MODE == MODE_DKV ? 2 : 1) * D;
-    static constexpr bool SEP = ACC_END + 128 <= 512;                        // room for the bf16 tiles beside T1 / T2
-    static constexpr uint32_t DS_COL = ACC_END, P_COL = ACC_END + 64;        // (SEP) 32 columns per half each
+    static constexpr uint32_t ACC_END = 256 + (DKV ? 2 : 1) * D;
+    // (SEP) bf16 tiles: dS 64 columns, P 64 (MODE_DKV) or the stationary operands (MODE_DQ)
+    static constexpr uint32_t P_COL = ACC_END + 64, X1_COL = ACC_END + 64, X2_COL = X1_COL + D / 2;
     static constexpr uint32_t TMEM_COLS = 512;
-    // columns of the bf16 dS / P tile that element-wise warp-half h (0 / 1) writes in half step `half`,
-    // and of contraction slice k (16 indices, k = 0..3) of that half step
-    __host__ __device__ static constexpr uint32_t ds_store(int half, int h) { return SEP ? DS_COL + half * 32 + h * 16 : T2_COL + half * HC + h * 32; }
-    __host__ __device__ static constexpr uint32_t p_store(int half, int h) { return SEP ? P_COL + half * 32 + h * 16 : T1_COL + half * HC + h * 32; }
-    __host__ __device__ static constexpr uint32_t ds_slice(int half, int k) { return ds_store(half, k / 2) + (k % 2) * 8; }
-    __host__ __device__ static constexpr uint32_t p_slice(int half, int k) { return p_store(half, k / 2) + (k % 2) * 8; }
-    // barriers.  T_FULL / PD_FULL / ACC_HALF [half]: the half's T1, T2 are computed / its dS (and P) are
-    // written / the MMAs that read them have completed -- once per step each; VEC_FULL [stage]: the step's
-    // lse2 / delta vectors are in shared memory (MODE_DKV)
-    static constexpr int BAR_X_FULL = 0, BAR_Y_FULL = 1, BAR_Y_EMPTY = 1 + HSTAGES, BAR_T_FULL = 1 + 2 * HSTAGES,
-                         BAR_PD_FULL = BAR_T_FULL + 2, BAR_ACC_HALF = BAR_PD_FULL + 2, BAR_VEC_FULL = BAR_ACC_HALF + 2,
-                         BAR_ACC_DONE = BAR_VEC_FULL + VSTAGES, NUM_BARS = BAR_ACC_DONE + 1;
+    static_assert(!SEP || (DKV ? P_COL + 64 : X1_COL + D / 2 + (X2_TMEM ? D / 2 : 0)) <= TMEM_COLS, "tensor memory");
+    // columns of the bf16 dS / P tile that warp group g (32 of the step's columns each, 0..3) writes, and of contraction
+    // slice k (16 indices, k = 0..7); without SEP each lies over the logits it came from
+    __host__ __device__ static constexpr uint32_t ds_store(int g) { return SEP ? ACC_END + g * 16 : T2_COL + g * 32; }
+    __host__ __device__ static constexpr uint32_t p_store(int g) { return SEP ? P_COL + g * 16 : T1_COL + g * 32; }
+    __host__ __device__ static constexpr uint32_t ds_slice(int k) { return ds_store(k / 2) + (k % 2) * 8; }
+    __host__ __device__ static constexpr uint32_t p_slice(int k) { return p_store(k / 2) + (k % 2) * 8; }
+    // barriers.  X_FULL: stationary tiles in shared memory; X_TMEM: in TMEM (one arrival per element-wise warp);
+    // Y_FULL [S1]: the copy's Y1 and Y2 have landed (and, MODE_DKV, warp 19 has written the step's slices);
+    // Y1_EMPTY [S1], Y2_EMPTY [S2] (MODE_DQ): read; ACC_STEP (SEP): the MMAs that read dS, P have completed; ACC_DONE:
+    // everything accumulated; per column group: T_FULL: T1, T2 computed; PD_FULL: dS (and P) written; T_FREE (SEP): T1, T2
+    // taken into registers.  Without SEP warp 18 arrives on PD_FULL, too, once the half's next copy has landed, so that the
+    // issuing warp has one barrier to look at.
+    static constexpr int BAR_X_FULL = 0, BAR_X_TMEM = 1, BAR_Y_FULL = 2, BAR_Y1_EMPTY = BAR_Y_FULL + S1,
+                         BAR_Y2_EMPTY = BAR_Y1_EMPTY + S1, BAR_ACC_STEP = BAR_Y2_EMPTY + S2, BAR_ACC_DONE = BAR_ACC_STEP + 1,
+                         BAR_T_FULL = BAR_ACC_DONE + 1, BAR_T_FREE = BAR_T_FULL + PARTS, BAR_PD_FULL = BAR_T_FREE + 1,
+                         NUM_BARS = BAR_PD_FULL + PARTS;
+    static constexpr int PD_ARRIVALS = SEP ? EW_WARPS : EW_WARPS / 2 + 1;
+    static_assert(NUM_BARS * 8 + 8 <= 512, "barriers");
 };
+
+// Shared-memory descriptor of a slice tile: K-major rows of 32 bytes, 32-byte swizzle, eight rows 256 bytes apart.
+__device__ __forceinline__ uint64_t aug_desc(uint32_t smem_addr) {
+    return static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (static_cast<uint64_t>(256 >> 4) << 32) | (1ull << 46) | (6ull << 61);
+}
+// Row r of a slice tile: x as the sum of three bf16 numbers, the other thirteen elements zero (the second 16 bytes of a row
+// are written once, by the clearing pass).  The swizzle exchanges the two halves of a row where bit 2 of r is set.
+__device__ __forceinline__ void aug_store(uint8_t* tile, int r, float x) {
+    const float hi = __bfloat162float(__float2bfloat16_rn(x)), rest = x - hi, mid = __bfloat162float(__float2bfloat16_rn(rest));
+    *reinterpret_cast<uint4*>(tile + r * 32 + ((r >> 2) & 1) * 16) = make_uint4(pack_bf16x2(hi, mid), pack_bf16x2(rest - mid, 0.f), 0u, 0u);
+}
+
+// What the logits are multiplied by in the exponent (base 2).  Not below 1e-30: -lse / scale must be a number, and whatever
+// 1e-30 times a logit is, it is nothing beside the exponent.
+__device__ __forceinline__ float exponent_factor(float scale) {
+    const float c = scale * LOG2E;
+    return fabsf(c) >= 1e-30f ? c : 1e-30f;
+}
 
 __device__ __forceinline__ void ew_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
@@ -91,26 +141,60 @@ template <int D, int MODE>
 __global__ void __launch_bounds__(BWD_THREADS, 1)
 bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ CUtensorMap tmX2,
               const __grid_constant__ CUtensorMap tmY1, const __grid_constant__ CUtensorMap tmY2,
-              const __nv_bfloat16* __restrict__ dOg, const __nv_bfloat16* __restrict__ Og,
+              const __nv_bfloat16* __restrict__ X1g, const __nv_bfloat16* __restrict__ X2g, const __nv_bfloat16* __restrict__ Og,
               const float* __restrict__ lse, float* __restrict__ delta,
               __nv_bfloat16* __restrict__ outA, __nv_bfloat16* __restrict__ outB,
-              int H, int Nq, int Nk, float scale, const int32_t* __restrict__ valid_len, int coff, int32_t* status) {
+              int BH, int H, int Nq, int Nk, float scale, const int32_t* __restrict__ valid_len, int coff, int group, int32_t* status) {
     using LY = BL<D, MODE>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* X1s = base;
-    uint8_t* X2s = X1s + LY::TILE_BYTES;
-    uint8_t* Ys = X2s + LY::TILE_BYTES;                  // half stage s: Y1 rows at 2 s, Y2 rows at 2 s + 1 (half tiles)
-    float* vec = reinterpret_cast<float*>(base + LY::OPERAND_BYTES);
-    float* xch = vec + LY::VSTAGES * 2 * BT;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(xch + 4 * BT);
+    uint8_t* X2s = X1s + (LY::X1_TMEM ? 0 : LY::TILE_BYTES);
+    uint8_t* Y1s = base + LY::X_BYTES;                   // rings of streamed tiles
+    uint8_t* Y2s = Y1s + LY::S1 * LY::Y_BYTES;
+    uint8_t* aug = base + LY::OPERAND_BYTES;             // (MODE_DKV) ones, then per stage -lse / scale and -delta
+    float* xch = reinterpret_cast<float*>(base + LY::OPERAND_BYTES + LY::AUG_ALL);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + LY::OPERAND_BYTES + LY::AUG_ALL + LY::XCH_BYTES);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int bh = blockIdx.y;
-    const int x0 = blockIdx.x * BT;                      // first row of the stationary tile (query or key)
     const int NX = MODE == MODE_DQ ? Nq : Nk;            // rows of the stationary tensors
+    // CTA -> (head, tile): `group` heads at a time, their tiles side by side, the longest first under the causal mask
+    // (the last query tiles, the first key tiles)
+    const int tiles = (NX + BT - 1) / BT;
+    const int per = group * tiles, first_head = static_cast<int>(blockIdx.x) / per * group;
+    const int heads = BH - first_head < group ? BH - first_head : group;
+    const int at = static_cast<int>(blockIdx.x) % per, bh = first_head + at % heads;
+    const int tile = (MODE == MODE_DQ && coff < (1 << 29)) ? tiles - 1 - at / heads : at / heads;
+    const int x0 = tile * BT;                            // first row of the stationary tile (query or key)
+
+    if (threadIdx.x == EW_WARPS * 32) {
+        for (int i = 0; i < LY::NUM_BARS; ++i) {
+            const bool y_full = i >= LY::BAR_Y_FULL && i < LY::BAR_Y1_EMPTY;
+            mbar_init(&bars[i], i == LY::BAR_X_TMEM || i == LY::BAR_T_FREE ? EW_WARPS : i >= LY::BAR_PD_FULL ? LY::PD_ARRIVALS
+                                : y_full && LY::DKV ? 2 : 1);
+        }
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) { tmem_alloc(tmem_slot, LY::TMEM_COLS); tmem_relinquish(); }
+    if (LY::DKV) {                                       // clear the slice tiles and write the ones
+        for (int i = threadIdx.x; i < LY::AUG_ALL / 16; i += BWD_THREADS) {
+            const int r = i >> 1;                        // (row of the first tile)
+            const bool ones = i < LY::AUG_BYTES / 16 && (i & 1) == ((r >> 2) & 1);
+            reinterpret_cast<uint4*>(aug)[i] = ones ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async_smem();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    // (launched with programmatic stream serialization: nothing in device memory is touched before the previous kernel of
+    // the stream -- the forward pass, or the dQ launch that writes delta -- has finished)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
     int nkeys = Nk;                                      // keys of this batch that take part at all
     if (valid_len) { nkeys = valid_len[bh / H]; nkeys = nkeys < 0 ? 0 : (nkeys > Nk ? Nk : nkeys); }
     // Range of streamed tiles [y_begin, y_end) that hold at least one visible (query, key) pair.
@@ -126,191 +210,252 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         if (first > 0) y_begin = static_cast<int>(first / BT < y_end ? first / BT : y_end);
     }
     const int nsteps = y_end - y_begin;
-
-    if (threadIdx.x == EW_WARPS * 32) {
-        for (int i = 0; i < LY::NUM_BARS; ++i) mbar_init(&bars[i], (i >= LY::BAR_PD_FULL && i < LY::BAR_ACC_HALF) ? EW_WARPS / 2 : 1);
-        *abort_flag = 0;
-        fence_mbar_init();
-    }
-    if (warp == 0) { tmem_alloc(tmem_slot, LY::TMEM_COLS); tmem_relinquish(); }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
     auto wait_warp = [&](int bar, uint32_t parity, int code) {
-        return __all_sync(0xffffffffu, bounded_wait(&bars[bar], parity, abort_flag, status, code));
+        return __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * bar, parity, abort_s, status, code));
     };
+    const int ncopies = LY::PARTS * nsteps;              // copies of the rings: step j, or half g & 1 of step g >> 1
 
     if (warp == EW_WARPS) {
-        // ------------------------------------------------------------ TMA producer (+ column vectors)
-        // The whole warp walks the loop; lane 0 issues the copies.  MODE_DKV: the 32 lanes also fetch
-        // the streamed tile's lse and delta (4 columns each), turn lse into base-2 units (+inf switches a
-        // column off: a query without keys, or past the end) and put both into the step's buffer.
+        // ------------------------------------------------------------ TMA producer (lane 0 issues the copies)
         if (nsteps > 0) {
             if (lane == 0) {
                 prefetch_tensormap(&tmX1); prefetch_tensormap(&tmX2); prefetch_tensormap(&tmY1); prefetch_tensormap(&tmY2);
-                mbar_arrive_expect_tx(&bars[LY::BAR_X_FULL], 2 * LY::TILE_BYTES);
-#pragma unroll
-                for (int c = 0; c < D / 64; ++c) {
-                    tma_load_3d(X1s + c * BT * 128, &tmX1, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
-                    tma_load_3d(X2s + c * BT * 128, &tmX2, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
-                }
-            }
-            int issued = 0;
-            bool ok = true;
-            for (int g = 0; g < 2 * nsteps && ok; ++g) {     // half steps: g = 2 j + half
-                const int s = g % LY::HSTAGES, j = g >> 1, half = g & 1;
-                ok = wait_warp(LY::BAR_Y_EMPTY + s, ((g / LY::HSTAGES) & 1) ^ 1, 0x500 + s);
-                if (!ok) break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(&bars[LY::BAR_Y_FULL + s], 2 * LY::HTILE_BYTES);
+                if (LY::X_BYTES > 0) {
+                    mbar_arrive_expect_tx(&bars[LY::BAR_X_FULL], LY::X_BYTES);
 #pragma unroll
                     for (int c = 0; c < D / 64; ++c) {
-                        tma_load_3d(Ys + (2 * s) * LY::HTILE_BYTES + c * HC * 128, &tmY1, &bars[LY::BAR_Y_FULL + s], c * 64,
-                                    (y_begin + j) * BT + half * HC, bh);
-                        tma_load_3d(Ys + (2 * s + 1) * LY::HTILE_BYTES + c * HC * 128, &tmY2, &bars[LY::BAR_Y_FULL + s], c * 64,
-                                    (y_begin + j) * BT + half * HC, bh);
+                        if (!LY::X1_TMEM) tma_load_3d(X1s + c * BT * 128, &tmX1, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
+                        if (!LY::X2_TMEM) tma_load_3d(X2s + c * BT * 128, &tmX2, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
+                    }
+                }
+            }
+            bool ok = true;
+            int issued = 0;
+            for (int g = 0; g < ncopies && ok; ++g) {
+                const int s1 = g % LY::S1, s2 = g % LY::S2, y = y_begin * BT + g * LY::Y_ROWS;
+                ok = wait_warp(LY::BAR_Y1_EMPTY + s1, ((g / LY::S1) & 1) ^ 1, 0x500);
+                if (!LY::DKV && ok) ok = wait_warp(LY::BAR_Y2_EMPTY + s2, ((g / LY::S2) & 1) ^ 1, 0x501);
+                if (!ok) break;
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(&bars[LY::BAR_Y_FULL + s1], 2 * LY::Y_BYTES);
+#pragma unroll
+                    for (int c = 0; c < D / 64; ++c) {
+                        tma_load_3d(Y1s + s1 * LY::Y_BYTES + c * LY::Y_ROWS * 128, &tmY1, &bars[LY::BAR_Y_FULL + s1], c * 64, y, bh);
+                        tma_load_3d(Y2s + s2 * LY::Y_BYTES + c * LY::Y_ROWS * 128, &tmY2, &bars[LY::BAR_Y_FULL + s1], c * 64, y, bh);
                     }
                 }
                 issued = g + 1;
-                if (MODE == MODE_DKV && half == 1) {
-                    // The step's vectors go into ring slot j % VSTAGES, last read in step j - VSTAGES.  The
-                    // stage just granted (the SECOND half's) was released behind the second half of that
-                    // step, i.e. after all of its element-wise work.
-                    float l2[4], dl[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int i = (y_begin + j) * BT + lane * 4 + e;
-                        l2[e] = INFINITY; dl[e] = 0.f;
-                        if (i < Nq) {
-                            const float l = lse[static_cast<int64_t>(bh) * Nq + i];
-                            l2[e] = l == -INFINITY ? INFINITY : l * LOG2E;
-                            dl[e] = delta[static_cast<int64_t>(bh) * Nq + i];
-                        }
-                    }
-                    float* vb = vec + (j % LY::VSTAGES) * 2 * BT + lane * 4;
-                    *reinterpret_cast<float4*>(vb) = make_float4(l2[0], l2[1], l2[2], l2[3]);
-                    *reinterpret_cast<float4*>(vb + BT) = make_float4(dl[0], dl[1], dl[2], dl[3]);
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&bars[LY::BAR_VEC_FULL + j % LY::VSTAGES]);
-                }
             }
             if (!ok && lane == 0) {
-                drain_wait(&bars[LY::BAR_X_FULL], 0);
-                for (int g = issued > LY::HSTAGES ? issued - LY::HSTAGES : 0; g < issued; ++g)
-                    drain_wait(&bars[LY::BAR_Y_FULL + g % LY::HSTAGES], (g / LY::HSTAGES) & 1);
+                if (LY::X_BYTES > 0) drain_wait(&bars[LY::BAR_X_FULL], 0);
+                for (int g = issued > LY::S1 ? issued - LY::S1 : 0; g < issued; ++g)
+                    drain_wait(&bars[LY::BAR_Y_FULL + g % LY::S1], (g / LY::S1) & 1);
             }
         }
-    } else if (warp == EW_WARPS + 1) {
-        // ------------------------------------------------------------ MMA issuer
-        //   T(j, half):   T1 = X1 Y1[half]^T and T2 = X2 Y2[half]^T into the half's 64 columns of T1 / T2;
-        //   ACC(j, half): once the element-wise warps have written the half's dS (and P):
-        //                 acc_a += dS Y1[half] (and acc_b += P Y2[half]).
-        // Issue order per half, behind PD_FULL(j, half):  T(j+1, half) then ACC(j, half) where the bf16
-        // tiles have columns of their own; ACC(j, half) then T(j+1, half) where they overlay T1 / T2 (the
-        // MMAs of one thread execute in issue order, so the T that overwrites them needs no wait).
+    } else if (LY::DKV && warp == EW_WARPS + 3) {
+        // ------------------------------------------------------------ the slices that carry lse and delta (MODE_DKV)
+        // Four queries per lane and step, fetched a step ahead.  A query that is switched off (no visible key, or past the
+        // end) gets a first term so large that 2^(c T1) is 0 whatever its logits are.
+        const float ce = exponent_factor(scale), inv = -LOG2E / ce, off = copysignf(3e38f, -ce);
+        float l[4], dl[4];
+        auto fetch = [&](int j) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = (y_begin + j) * BT + e * 32 + lane;
+                l[e] = i < Nq ? lse[static_cast<int64_t>(bh) * Nq + i] : -INFINITY;
+                dl[e] = i < Nq ? delta[static_cast<int64_t>(bh) * Nq + i] : 0.f;
+            }
+        };
+        if (nsteps > 0) fetch(0);
+        bool ok = true;
+        for (int j = 0; j < nsteps && ok; ++j) {
+            const int v = j % LY::VSTAGES, g = LY::PARTS * j + LY::PARTS - 1;   // the step's (last) copy
+            float x[4], y[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                x[e] = l[e] == -INFINITY ? off : l[e] * inv;
+                x[e] = x[e] > 3e38f ? 3e38f : x[e] < -3e38f ? -3e38f : x[e];
+                y[e] = -dl[e];
+            }
+            if (j + 1 < nsteps) fetch(j + 1);
+            // (slot v was last read by the T MMAs of step j - VSTAGES; that step has released the stage of this step's
+            // (last) copy behind its accumulation, i.e. after them)
+            ok = wait_warp(LY::BAR_Y1_EMPTY + g % LY::S1, ((g / LY::S1) & 1) ^ 1, 0x502);
+            if (!ok) break;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                aug_store(aug + (1 + 2 * v) * LY::AUG_BYTES, e * 32 + lane, x[e]);
+                aug_store(aug + (2 + 2 * v) * LY::AUG_BYTES, e * 32 + lane, y[e]);
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&bars[LY::BAR_Y_FULL + g % LY::S1]);
+                if (LY::PARTS == 2) mbar_arrive(&bars[LY::BAR_Y_FULL + (g - 1) % LY::S1]);
+            }
+        }
+    } else if (warp == EW_WARPS + 1 || warp == EW_WARPS + 2) {
+        // ------------------------------------------------------------ MMA issuers
+        //   T(j):   T1 = X1 Y1^T and T2 = X2 Y2^T (+ the slices);   ACC(j): acc_a += dS Y1 (and acc_b += P Y2).
+        // SEP: warp 17 issues T(j+1) as soon as T(j) is in registers, warp 18 ACC(j) as soon as dS (and P) are written.
+        // Otherwise warp 17 issues, per half, ACC(j) and behind it T(j+1).
         // The whole warp walks the loop (uniform control flow) and one elected lane issues: the MMA and
         // commit instructions take their operands from uniform registers, which the compiler can only
         // use when it knows that a single thread runs the code.
         if (nsteps > 0) {
-            constexpr uint32_t IDESC_T = make_idesc_bf16(BT, HC, 0, 0);
-            constexpr uint32_t IDESC_ACC = make_idesc_bf16(BT, D, 0, 1);
-            bool ok = wait_warp(LY::BAR_X_FULL, 0, 0x510);
+            constexpr int YR = LY::Y_ROWS;
+            constexpr uint32_t IDESC_T = make_idesc_bf16(BT, YR, 0, 0), IDESC_ACC = make_idesc_bf16(BT, D, 0, 1);
+            constexpr uint64_t Y16 = LY::Y_BYTES >> 4, AUG16 = LY::AUG_BYTES >> 4;           // descriptor units of 16 bytes
+            bool ok = true;
             // descriptors of the first feature slice of each operand (the others are constant offsets away)
             const uint64_t x1d = make_smem_desc_sw128(smem_u32(X1s), 16, 1024);            // K-major
             const uint64_t x2d = make_smem_desc_sw128(smem_u32(X2s), 16, 1024);
-            const uint64_t ykd = make_smem_desc_sw128(smem_u32(Ys), 16, 1024);             // Y1 half of stage 0, K-major
-            const uint64_t ymd = make_smem_desc_sw128(smem_u32(Ys), HC * 128, 1024);       // Y1 half of stage 0, MN-major
-            constexpr uint64_t HTILE16 = LY::HTILE_BYTES >> 4;                              // descriptor units of 16 bytes
+            const uint64_t y1k = make_smem_desc_sw128(smem_u32(Y1s), 16, 1024), y2k = make_smem_desc_sw128(smem_u32(Y2s), 16, 1024);
+            const uint64_t y1m = make_smem_desc_sw128(smem_u32(Y1s), YR * 128, 1024);      // MN-major
+            const uint64_t y2m = make_smem_desc_sw128(smem_u32(Y2s), YR * 128, 1024);
+            const uint64_t augd = aug_desc(smem_u32(aug));
             // Consecutive MMAs into ONE accumulator wait for each other, so the slices of independent
-            // products are issued in turn: T1 and T2 of a half, and the accumulations acc_a and acc_b.
-            auto issue_t = [&](int j, int half) {
-                // (feature slice k of a K-major operand: panel k / 4 of 64 features, 32 bytes per slice; a panel
-                // is 128 rows of 128 bytes for the stationary tiles, 64 rows for the streamed half tiles)
-                const uint64_t y1 = ykd + static_cast<uint64_t>(2 * ((2 * j + half) % LY::HSTAGES)) * HTILE16;
-                const uint64_t y2 = y1 + HTILE16;
+            // products are issued in turn: T1 and T2, and the accumulations acc_a and acc_b.
+            // (feature slice k of a K-major operand: panel k / 4 of 64 features, 32 bytes per slice; a panel
+            // is 128 rows of 128 bytes for the stationary tiles, YR rows for the streamed ones)
+            // g: the copy; half: its column group (0 where a copy is a whole step)
+            auto issue_t = [&](int g, int half) {
+                const uint64_t y1 = y1k + static_cast<uint64_t>(g % LY::S1) * Y16, y2 = y2k + static_cast<uint64_t>(g % LY::S2) * Y16;
+                const uint32_t t1 = tmem + LY::T1_COL + half * HC, t2 = tmem + LY::T2_COL + half * HC;
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k) {
                     const uint64_t xoff = static_cast<uint64_t>(((k / 4) * (BT * 128) + (k % 4) * 32) >> 4);
-                    const uint64_t yoff = static_cast<uint64_t>(((k / 4) * (HC * 128) + (k % 4) * 32) >> 4);
-                    mma_ss(tmem + LY::T1_COL + half * HC, x1d + xoff, y1 + yoff, IDESC_T, k > 0);
-                    mma_ss(tmem + LY::T2_COL + half * HC, x2d + xoff, y2 + yoff, IDESC_T, k > 0);
+                    const uint64_t yoff = static_cast<uint64_t>(((k / 4) * (YR * 128) + (k % 4) * 32) >> 4);
+                    if (LY::X1_TMEM) mma_ts(t1, tmem + LY::X1_COL + k * 8, y1 + yoff, IDESC_T, k > 0);
+                    else             mma_ss(t1, x1d + xoff, y1 + yoff, IDESC_T, k > 0);
+                    if (LY::X2_TMEM) mma_ts(t2, tmem + LY::X2_COL + k * 8, y2 + yoff, IDESC_T, k > 0);
+                    else             mma_ss(t2, x2d + xoff, y2 + yoff, IDESC_T, k > 0);
+                }
+                if (LY::DKV) {
+                    const uint64_t av = augd + static_cast<uint64_t>(1 + 2 * ((g / LY::PARTS) % LY::VSTAGES)) * AUG16 + static_cast<uint64_t>((half * HC * 32) >> 4);
+                    mma_ss(t1, augd, av, IDESC_T, 1);
+                    mma_ss(t2, augd, av + AUG16, IDESC_T, 1);
                 }
                 tc_commit(&bars[LY::BAR_T_FULL + half]);
+                if (!LY::DKV) tc_commit(&bars[LY::BAR_Y2_EMPTY + g % LY::S2]);
             };
-            auto issue_acc = [&](int j, int half) {
-                const uint64_t y1 = ymd + static_cast<uint64_t>(2 * ((2 * j + half) % LY::HSTAGES)) * HTILE16;
-                const uint64_t y2 = y1 + HTILE16;
-                const uint32_t acc = (j > 0 || half > 0) ? 1u : 0u;
+            auto issue_acc = [&](int g, int half) {
+                const uint64_t y1 = y1m + static_cast<uint64_t>(g % LY::S1) * Y16, y2 = y2m + static_cast<uint64_t>(g % LY::S2) * Y16;
 #pragma unroll
-                for (int k = 0; k < HC / 16; ++k) {
-                    mma_ts(tmem + LY::ACC_A_COL, tmem + (half == 0 ? LY::ds_slice(0, k) : LY::ds_slice(1, k)),
-                           y1 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, k > 0 ? 1u : acc);
-                    if (MODE == MODE_DKV)
-                        mma_ts(tmem + LY::ACC_B_COL, tmem + (half == 0 ? LY::p_slice(0, k) : LY::p_slice(1, k)),
-                               y2 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, k > 0 ? 1u : acc);
+                for (int k = 0; k < YR / 16; ++k) {
+                    mma_ts(tmem + LY::ACC_A_COL, tmem + (half == 0 ? LY::ds_slice(k) : LY::ds_slice(4 + k)),
+                           y1 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, (g > 0 || k > 0));
+                    if (LY::DKV)
+                        mma_ts(tmem + LY::ACC_B_COL, tmem + (half == 0 ? LY::p_slice(k) : LY::p_slice(4 + k)),
+                               y2 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, (g > 0 || k > 0));
                 }
-                if (LY::SEP) tc_commit(&bars[LY::BAR_ACC_HALF + half]);
+                if (LY::SEP) tc_commit(&bars[LY::BAR_ACC_STEP]);
+                tc_commit(&bars[LY::BAR_Y1_EMPTY + g % LY::S1]);
+                if (g == ncopies - 1) tc_commit(&bars[LY::BAR_ACC_DONE]);
             };
-            auto y_full = [&](int g, int code) {         // the copy of half step g has landed
-                return wait_warp(LY::BAR_Y_FULL + g % LY::HSTAGES, (g / LY::HSTAGES) & 1, code);
-            };
-            if (ok) ok = y_full(0, 0x520) && y_full(1, 0x520);
-            if (ok) {
-                tc_fence_after();
-                if (elect_one()) { issue_t(0, 0); issue_t(0, 1); }
-                __syncwarp();
+            auto y_full = [&](int g, int code) { return wait_warp(LY::BAR_Y_FULL + g % LY::S1, (g / LY::S1) & 1, code); };
+            if (warp == EW_WARPS + 1) {
+                if (LY::X_BYTES > 0) ok = wait_warp(LY::BAR_X_FULL, 0, 0x510);
+                if (ok && LY::X1_TMEM) ok = wait_warp(LY::BAR_X_TMEM, 0, 0x511);
             }
-            for (int j = 0; j < nsteps && ok; ++j) {
-                const bool more = j + 1 < nsteps;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    // (the next half step's copy landed long ago: its barrier is checked before the wait for the
-                    // element-wise warps, not behind it, where the check would sit in the chain of the half)
-                    if (more) ok = y_full(2 * (j + 1) + half, 0x521);
-                    if (ok) ok = wait_warp(LY::BAR_PD_FULL + half, j & 1, 0x530 + half);
+            if (LY::SEP && warp == EW_WARPS + 1) {
+                for (int j = 0; j < nsteps && ok; ++j) {
+                    ok = y_full(j, 0x520);
+                    if (ok && j > 0) ok = wait_warp(LY::BAR_T_FREE, (j - 1) & 1, 0x522);
                     if (!ok) break;
                     tc_fence_after();
-                    if (elect_one()) {
-                        if (LY::SEP && more) issue_t(j + 1, half);
-                        issue_acc(j, half);
-                        if (!LY::SEP && more) issue_t(j + 1, half);
-                        tc_commit(&bars[LY::BAR_Y_EMPTY + (2 * j + half) % LY::HSTAGES]);
-                        if (half == 1 && !more) tc_commit(&bars[LY::BAR_ACC_DONE]);
-                    }
+                    if (elect_one()) issue_t(j, 0);
                     __syncwarp();
+                }
+            } else if (LY::SEP) {
+                for (int j = 0; j < nsteps && ok; ++j) {
+                    ok = y_full(j, 0x523);
+                    if (ok) ok = wait_warp(LY::BAR_PD_FULL, j & 1, 0x530);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) issue_acc(j, 0);
+                    __syncwarp();
+                }
+            } else if (warp == EW_WARPS + 1) {
+                ok = ok && y_full(0, 0x520) && y_full(1, 0x520);
+                if (ok) {
+                    tc_fence_after();
+                    if (elect_one()) { issue_t(0, 0); issue_t(1, 1); }
+                    __syncwarp();
+                }
+                for (int j = 0; j < nsteps && ok; ++j) {
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const int g = 2 * j + half;
+                        ok = wait_warp(LY::BAR_PD_FULL + half, j & 1, 0x531);
+                        if (!ok) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            issue_acc(g, half);
+                            if (g + 2 < ncopies) issue_t(g + 2, half);
+                        }
+                        __syncwarp();
+                    }
+                }
+            } else {
+                // (the half's next copy: looked at here, so that the issuing warp does not have to; not before the half's
+                // previous phase is over, which this arrival does not belong to)
+                for (int g = 0; g < ncopies && ok; ++g) {
+                    if (g + 2 < ncopies) ok = y_full(g + 2, 0x521);
+                    if (ok && g >= 2) ok = wait_warp(LY::BAR_PD_FULL + (g & 1), ((g >> 1) - 1) & 1, 0x532);
+                    if (ok && lane == 0) mbar_arrive(&bars[LY::BAR_PD_FULL + (g & 1)]);
                 }
             }
         }
-    } else {
+    } else if (warp < EW_WARPS) {
         // ------------------------------------------------------------ element-wise + epilogue (warps 0-15)
-        const int q = warp & 3, h = (warp >> 2) & 1, half = warp >> 3, part = warp >> 2;
+        const int q = warp & 3, part = warp >> 2;        // lane quarter, 32 of the step's columns
         const int r = q * 32 + lane;                     // lane of the TMEM = row of the stationary tile
         const int xr = x0 + r;                           // that row's index (query in MODE_DQ, key in MODE_DKV)
         const uint32_t tl = tmem + (static_cast<uint32_t>(q * 32) << 16);
-        const float c2 = scale * LOG2E;
+        const float c2 = exponent_factor(scale);
         bool ok = true;
-        // Per-lane terms (MODE_DQ): lse of the row in base-2 units (+inf switches a row off: no key, or
-        // past the end) and delta = sum_t dO O, each of the row's four warps summing a quarter of the features.
+        // MODE_DQ: the row's quarter (this warp's part of the features) of the stationary operands that live in TMEM (rows
+        // past the end are zeros); lse of the row in base-2 units (+inf switches a row off: no key, or past the end) and
+        // delta = sum_t dO O, each of the row's four warps summing a quarter of the features.
         float lse2_r = INFINITY, delta_r = 0.f;
-        if (MODE == MODE_DQ) {
+        if (!LY::DKV) {
             float sum = 0.f;
-            if (xr < Nq) {
-                const uint4* a = reinterpret_cast<const uint4*>(dOg + (static_cast<int64_t>(bh) * Nq + xr) * D + part * (D / 4));
-                const uint4* b = reinterpret_cast<const uint4*>(Og + (static_cast<int64_t>(bh) * Nq + xr) * D + part * (D / 4));
+            uint32_t w1[D / 8], w2[D / 8];               // packed pairs of Q and dO
+#pragma unroll
+            for (int i = 0; i < D / 8; ++i) w1[i] = w2[i] = 0u;
+            if (xr < NX) {
+                const int64_t at_row = (static_cast<int64_t>(bh) * NX + xr) * D + part * (D / 4);
+                const uint4* a = reinterpret_cast<const uint4*>(X1g + at_row);
+                const uint4* b = reinterpret_cast<const uint4*>(X2g + at_row);
+                const uint4* c = reinterpret_cast<const uint4*>(Og + at_row);
 #pragma unroll
                 for (int v = 0; v < D / 32; ++v) {
-                    const uint4 av = a[v], bv = b[v];
-                    const uint32_t aw[4] = {av.x, av.y, av.z, av.w}, bw[4] = {bv.x, bv.y, bv.z, bv.w};
+                    const uint4 av = a[v], bv = b[v], cv = c[v];
+                    const uint32_t cw[4] = {cv.x, cv.y, cv.z, cv.w};
+                    w1[4 * v] = av.x; w1[4 * v + 1] = av.y; w1[4 * v + 2] = av.z; w1[4 * v + 3] = av.w;
+                    w2[4 * v] = bv.x; w2[4 * v + 1] = bv.y; w2[4 * v + 2] = bv.z; w2[4 * v + 3] = bv.w;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        sum = fmaf(__uint_as_float(aw[e] << 16), __uint_as_float(bw[e] << 16), sum);
-                        sum = fmaf(__uint_as_float(aw[e] & 0xffff0000u), __uint_as_float(bw[e] & 0xffff0000u), sum);
+                        sum = fmaf(__uint_as_float(w2[4 * v + e] << 16), __uint_as_float(cw[e] << 16), sum);
+                        sum = fmaf(__uint_as_float(w2[4 * v + e] & 0xffff0000u), __uint_as_float(cw[e] & 0xffff0000u), sum);
                     }
                 }
                 const float l = lse[static_cast<int64_t>(bh) * Nq + xr];
                 lse2_r = l == -INFINITY ? INFINITY : l * LOG2E;
             }
+            // (D / 2 columns hold a row; a quarter is D / 8)
+            if constexpr (D == 64) {
+                tmem_st_x8(tl + LY::X1_COL + part * 8, w1);
+                tmem_st_x8(tl + LY::X2_COL + part * 8, w2);
+            } else {
+                tmem_st_x16(tl + LY::X1_COL + part * 16, w1);
+            }
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars[LY::BAR_X_TMEM]);
             xch[part * BT + r] = sum;
             ew_sync();
             delta_r = (xch[r] + xch[BT + r]) + (xch[2 * BT + r] + xch[3 * BT + r]);
@@ -320,83 +465,80 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         const long long rlim = static_cast<long long>(xr) + 1 + coff;
         const int nrow = rlim < nkeys ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : nkeys;
         const bool key_live = xr < nkeys;
-        const uint64_t c22 = pack2(c2, c2);
-        const int cq = half * HC + h * 32;               // this warp's 32 columns of every step
-        const uint32_t ds_addr = tl + (half == 0 ? LY::ds_store(0, 0) : LY::ds_store(1, 0)) + h * (LY::ds_store(0, 1) - LY::ds_store(0, 0));
-        const uint32_t p_addr = tl + (half == 0 ? LY::p_store(0, 0) : LY::p_store(1, 0)) + h * (LY::p_store(0, 1) - LY::p_store(0, 0));
+        const uint64_t c22 = pack2(c2, c2), nl2 = pack2(-lse2_r, -lse2_r), dl2 = pack2(delta_r, delta_r);
+        const int cq = part * 32;                        // this warp's 32 columns of every step
+        const int cgroup = LY::PARTS == 2 ? part >> 1 : 0;
+        const uint32_t ds_addr = tl + LY::ds_store(0) + part * (LY::ds_store(1) - LY::ds_store(0));
+        const uint32_t p_addr = tl + LY::p_store(0) + part * (LY::p_store(1) - LY::p_store(0));
         for (int j = 0; j < nsteps && ok; ++j) {
-            if (MODE == MODE_DKV) ok = wait_warp(LY::BAR_VEC_FULL + j % LY::VSTAGES, static_cast<uint32_t>(j / LY::VSTAGES) & 1u, 0x548);
-            if (ok) ok = wait_warp(LY::BAR_T_FULL + half, j & 1, 0x540 + half);
+            ok = wait_warp(LY::BAR_T_FULL + cgroup, j & 1, 0x540 + cgroup);
             if (!ok) break;
             tc_fence_after();
+            uint32_t t1[32], t2[32];
+            tmem_ld_x32(tl + LY::T1_COL + cq, t1);
+            tmem_ld_x32(tl + LY::T2_COL + cq, t2);
             const int y0 = (y_begin + j) * BT + cq;      // index of the first of the columns (key or query)
             // all 32 x 32 (row, column) pairs of this warp visible?  (then no per-element selection)
             const bool fast = __all_sync(0xffffffffu, MODE == MODE_DQ ? y0 + 32 <= nrow
                                                                       : key_live && static_cast<long long>(y0) + coff >= xr);
-            const float* lv = vec + (j % LY::VSTAGES) * 2 * BT + cq;
+            // (own columns for the bf16 tiles: the MMAs that read the previous step's must be done before they are
+            // overwritten.  They mostly are by now; the check here costs nothing, its result is wanted after the exponentials)
+            bool acc_done = true;
+            if (LY::SEP && j > 0) acc_done = mbar_test_wait_s(bars_s + 8 * LY::BAR_ACC_STEP, (j - 1) & 1);
+            tc_wait_ld();
+            if (LY::SEP) {                               // T1, T2 may be overwritten by the next step's
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_s(bars_s + 8 * LY::BAR_T_FREE);
+            }
             uint32_t pk[16], dk[16];
-            // two loads of 16 columns each from T1 and T2 (few registers live at a time)
+            // MODE_DQ:  p = 2^(c T1 - lse2), ds = p (T2 - delta);  MODE_DKV: p = 2^(c T1), ds = p T2 (lse and delta are in T1
+            // and T2).  On packed pairs: two results per issue slot.
+            if (fast) {
 #pragma unroll
-            for (int sub = 0; sub < 2; ++sub) {
-                uint32_t t1[16], t2[16];
-                tmem_ld_x16(tl + LY::T1_COL + cq + sub * 16, t1);
-                tmem_ld_x16(tl + LY::T2_COL + cq + sub * 16, t2);
-                tc_wait_ld();
-                // p = 2^(c T1 - lse2), ds = p (T2 - delta), on packed pairs (two results per issue slot)
-                if (fast) {
+                for (int i = 0; i < 32; i += 2) {
+                    const uint64_t s2 = pack2(__uint_as_float(t1[i]), __uint_as_float(t1[i + 1]));
+                    float a0, a1;
+                    unpack2(LY::DKV ? mul2(s2, c22) : fma2(s2, c22, nl2), a0, a1);
+                    t1[i] = __float_as_uint(ex2_approx(a0)); t1[i + 1] = __float_as_uint(ex2_approx(a1));
+                }
 #pragma unroll
-                    for (int i = 0; i < 16; i += 4) {
-                        uint64_t nl[2], dl[2];           // -lse2 and delta of columns i..i+1, i+2..i+3
-                        if (MODE == MODE_DQ) {
-                            nl[0] = nl[1] = pack2(-lse2_r, -lse2_r);
-                            dl[0] = dl[1] = pack2(delta_r, delta_r);
-                        } else {
-                            const float4 a4 = *reinterpret_cast<const float4*>(lv + sub * 16 + i);
-                            const float4 b4 = *reinterpret_cast<const float4*>(lv + BT + sub * 16 + i);
-                            nl[0] = pack2(-a4.x, -a4.y); nl[1] = pack2(-a4.z, -a4.w);
-                            dl[0] = pack2(b4.x, b4.y); dl[1] = pack2(b4.z, b4.w);
-                        }
+                for (int i = 0; i < 32; i += 2) {
+                    const uint64_t g2 = pack2(__uint_as_float(t2[i]), __uint_as_float(t2[i + 1]));
+                    const float p0 = __uint_as_float(t1[i]), p1 = __uint_as_float(t1[i + 1]);
+                    float d0, d1;
+                    unpack2(mul2(pack2(p0, p1), LY::DKV ? g2 : sub2(g2, dl2)), d0, d1);
+                    if (LY::DKV) pk[i / 2] = pack_bf16x2(p0, p1);
+                    dk[i / 2] = pack_bf16x2(d0, d1);
+                }
+            } else {
 #pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int x = i + 2 * e;
-                            float a0, a1;
-                            unpack2(fma2(pack2(__uint_as_float(t1[x]), __uint_as_float(t1[x + 1])), c22, nl[e]), a0, a1);
-                            const float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
-                            float d0, d1;
-                            unpack2(mul2(pack2(p0, p1), sub2(pack2(__uint_as_float(t2[x]), __uint_as_float(t2[x + 1])), dl[e])), d0, d1);
-                            if (MODE == MODE_DKV) pk[sub * 8 + x / 2] = pack_bf16x2(p0, p1);
-                            dk[sub * 8 + x / 2] = pack_bf16x2(d0, d1);
-                        }
+                for (int i = 0; i < 32; i += 2) {
+                    float p[2], ds[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int col = y0 + i + e;
+                        const bool live = MODE == MODE_DQ ? col < nrow : key_live && static_cast<long long>(col) + coff >= xr;
+                        p[e] = live ? ex2_approx(fmaf(__uint_as_float(t1[i + e]), c2, LY::DKV ? 0.f : -lse2_r)) : 0.f;
+                        ds[e] = p[e] * (__uint_as_float(t2[i + e]) - (LY::DKV ? 0.f : delta_r));
                     }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        float p[2], ds[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int col = y0 + sub * 16 + i + e;
-                            const float lse2 = MODE == MODE_DQ ? lse2_r : lv[sub * 16 + i + e];
-                            const float dl = MODE == MODE_DQ ? delta_r : lv[BT + sub * 16 + i + e];
-                            const bool live = MODE == MODE_DQ ? col < nrow : key_live && static_cast<long long>(col) + coff >= xr;
-                            p[e] = live ? ex2_approx(fmaf(__uint_as_float(t1[i + e]), c2, -lse2)) : 0.f;
-                            ds[e] = p[e] * (__uint_as_float(t2[i + e]) - dl);
-                        }
-                        pk[sub * 8 + i / 2] = pack_bf16x2(p[0], p[1]);
-                        dk[sub * 8 + i / 2] = pack_bf16x2(ds[0], ds[1]);
-                    }
+                    if (LY::DKV) pk[i / 2] = pack_bf16x2(p[0], p[1]);
+                    dk[i / 2] = pack_bf16x2(ds[0], ds[1]);
                 }
             }
-            // (own columns for the bf16 tiles: the MMAs that read the previous step's must be done)
-            if (LY::SEP && j > 0) {
-                ok = wait_warp(LY::BAR_ACC_HALF + half, static_cast<uint32_t>(j - 1) & 1u, 0x542 + half);
-                if (!ok) break;
+            if (LY::SEP) {
+                if (!__all_sync(0xffffffffu, acc_done)) {
+                    ok = wait_warp(LY::BAR_ACC_STEP, static_cast<uint32_t>(j - 1) & 1u, 0x542);
+                    if (!ok) break;
+                }
+                tc_fence_after();
             }
-            if (MODE == MODE_DKV) tmem_st_x16(p_addr, pk);
+            if (LY::DKV) tmem_st_x16(p_addr, pk);
             tmem_st_x16(ds_addr, dk);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars[LY::BAR_PD_FULL + half]);
+            if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::BAR_PD_FULL + cgroup));
         }
         if (ok && nsteps > 0) ok = __all_sync(0xffffffffu, bounded_wait(&bars[LY::BAR_ACC_DONE], 0, abort_flag, status, 0x550));
         if (ok) {
@@ -438,36 +580,48 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     if (warp == 0) tmem_dealloc(tmem, LY::TMEM_COLS);
 }
 
+template <int D, int MODE>
+int launch_bwd_mode(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t st) {
+    using LY = BL<D, MODE>;
+    if (!ensure_dynamic_smem<bwd_tc_kernel<D, MODE>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+    const int BH = p.B * p.H, tiles = ((MODE == MODE_DQ ? p.Nq : p.Nk) + BT - 1) / BT;
+    if (static_cast<int64_t>(tiles) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
+    // Without the causal mask the tiles of a head run side by side and share its streamed tensors in L2.  With it, the
+    // tiles of as many heads as fit L2 together (48 MB of streamed tensors) are dealt longest first: what is left at the
+    // end are the short ones.
+    const int64_t streamed = static_cast<int64_t>(MODE == MODE_DQ ? p.Nk : p.Nq) * D * 4;
+    const int64_t fit = (48ll << 20) / streamed;
+    const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(tiles) * BH);
+    cfg.blockDim = dim3(BWD_THREADS);
+    cfg.dynamicSmemBytes = LY::SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto bf = [](const void* x) { return static_cast<const __nv_bfloat16*>(x); };
+    const cudaError_t e = cudaLaunchKernelEx(
+        &cfg, bwd_tc_kernel<D, MODE>, m[0], m[1], m[2], m[3], bf(MODE == MODE_DQ ? p.Q : p.K), bf(MODE == MODE_DQ ? p.dO : p.V), bf(p.O),
+        p.lse, p.delta, static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? p.dQ : p.dK),
+        static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? nullptr : p.dV), BH, p.H, p.Nq, p.Nk, p.scale, p.k_valid_len,
+        p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status);
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
 template <int D>
 int launch_bwd_d(const BwdProblem& p, cudaStream_t st) {
-    // every tensor is stationary (boxes of 128 rows) in one launch and streamed (boxes of 64 rows) in the other
-    CUtensorMap tmQ, tmK, tmV, tmdO, tmQh, tmKh, tmVh, tmdOh;
+    // stationary tiles are boxes of 128 rows; streamed ones too, or boxes of 64 rows (the dK dV launch at d = 128)
+    constexpr int YR = BL<D, MODE_DKV>::Y_ROWS;
+    CUtensorMap tmK, tmV, tmdO, tmQs, tmdOs;
     const int BH = p.B * p.H;
-    if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BT) || !make_map(&tmK, p.K, BH, p.Nk, D, BT) ||
-        !make_map(&tmV, p.V, BH, p.Nk, D, BT) || !make_map(&tmdO, p.dO, BH, p.Nq, D, BT) ||
-        !make_map(&tmQh, p.Q, BH, p.Nq, D, HC) || !make_map(&tmKh, p.K, BH, p.Nk, D, HC) ||
-        !make_map(&tmVh, p.V, BH, p.Nk, D, HC) || !make_map(&tmdOh, p.dO, BH, p.Nq, D, HC))
+    if (!make_map(&tmK, p.K, BH, p.Nk, D, BT) || !make_map(&tmV, p.V, BH, p.Nk, D, BT) || !make_map(&tmdO, p.dO, BH, p.Nq, D, BT) ||
+        !make_map(&tmQs, p.Q, BH, p.Nq, D, YR) || !make_map(&tmdOs, p.dO, BH, p.Nq, D, YR))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<bwd_tc_kernel<D, MODE_DQ>>(BL<D, MODE_DQ>::SMEM_BYTES)) return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<bwd_tc_kernel<D, MODE_DKV>>(BL<D, MODE_DKV>::SMEM_BYTES)) return FLAT_ERR_CUDA;
-    const int coff = p.causal ? p.Nk - p.Nq : (1 << 30);
-    const __nv_bfloat16* dO = static_cast<const __nv_bfloat16*>(p.dO);
-    const __nv_bfloat16* O = static_cast<const __nv_bfloat16*>(p.O);
-    {
-        dim3 grid((p.Nq + BT - 1) / BT, BH);
-        bwd_tc_kernel<D, MODE_DQ><<<grid, BWD_THREADS, BL<D, MODE_DQ>::SMEM_BYTES, st>>>(
-            tmQ, tmdO, tmKh, tmVh, dO, O, p.lse, p.delta, static_cast<__nv_bfloat16*>(p.dQ), nullptr, p.H, p.Nq, p.Nk,
-            p.scale, p.k_valid_len, coff, p.status);
-        if (cudaGetLastError() != cudaSuccess) return FLAT_ERR_CUDA;
-    }
-    {
-        dim3 grid((p.Nk + BT - 1) / BT, BH);
-        bwd_tc_kernel<D, MODE_DKV><<<grid, BWD_THREADS, BL<D, MODE_DKV>::SMEM_BYTES, st>>>(
-            tmK, tmV, tmQh, tmdOh, dO, O, p.lse, p.delta, static_cast<__nv_bfloat16*>(p.dK),
-            static_cast<__nv_bfloat16*>(p.dV), p.H, p.Nq, p.Nk, p.scale, p.k_valid_len, coff, p.status);
-        if (cudaGetLastError() != cudaSuccess) return FLAT_ERR_CUDA;
-    }
-    return FLAT_OK;
+    const int rc = launch_bwd_mode<D, MODE_DQ>(p, {tmdO, tmdO, tmK, tmV}, st);   // (tmX1: Q goes straight to TMEM, not by TMA)
+    return rc != FLAT_OK ? rc : launch_bwd_mode<D, MODE_DKV>(p, {tmK, tmV, tmQs, tmdOs}, st);
 }
 
 }  // namespace
