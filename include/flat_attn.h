@@ -99,8 +99,10 @@ enum {
     FLAT_VARIANT_TC2_SPLIT16 = 15, /* TC2_SPLIT2 over a cluster of sixteen CTAs (more than the portable cluster size:
                                   taken only where the device can hold such a cluster): bf16, d = 128       */
     FLAT_VARIANT_TC2_HALVES_SPLIT16 = 16, /* TC2_HALVES over a cluster of sixteen CTAs: bf16, d = 64               */
-    FLAT_VARIANT_SMALL = 17    /* small heads on the tensor cores, each weight as the sum of two bf16 numbers: bf16,
+    FLAT_VARIANT_SMALL = 17,   /* small heads on the tensor cores, each weight as the sum of two bf16 numbers: bf16,
                                   d in {16,32}, no bias, no pruning map (what AUTO picks there)  */
+    FLAT_VARIANT_DECODE = 18   /* at most sixteen queries per head, bound by the stream of keys and values: bf16,
+                                  d in {64,128}, no bias, no pruning map (what AUTO picks there)  */
 };
 
 typedef struct flat_attn_params {
@@ -127,7 +129,7 @@ typedef struct flat_attn_params {
                                   path only: lse[b,h,i] = log sum_j exp(scale * q_i . k_j) over the
                                   keys that row i sees (natural logarithm; -inf for a row without
                                   any).  It is what flat_attn_bwd needs from the forward pass.
-                                  Written by the SIMT, SMALL, TC2, TC2_SINGLE and TC3 kernels (AUTO picks
+                                  Written by the SIMT, SMALL, DECODE, TC2, TC2_SINGLE and TC3 kernels (AUTO picks
                                   among these when it is set); FLAT_ERR_UNSUPPORTED for the others.
                                   The paper has no counterpart (it stops at inference).           */
     const void* bias;          /* optional device tensor added to the SCALED logits before the

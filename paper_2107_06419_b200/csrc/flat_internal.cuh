@@ -77,6 +77,8 @@ int launch_fused_tc3(const Problem& p, cudaStream_t st);
 extern thread_local int g_last_schedule;
 bool tf32_applies(const Problem& p);               // fp32, d = 64, no bias, no pruning map
 int launch_fused_tf32(const Problem& p, cudaStream_t st);     // fp32 tensors through split tf32 products
+bool decode_applies(const Problem& p);             // bf16, d in {64, 128}, at most 16 queries, no bias, no pruning map
+int launch_fused_decode(const Problem& p, cudaStream_t st);
 bool small_applies(const Problem& p);              // bf16, d in {16, 32}, no bias, no pruning map
 int launch_fused_small(const Problem& p, cudaStream_t st);
 bool rgran_applies(const Problem& p);              // bf16, d = 64, Nk <= 512
@@ -119,6 +121,38 @@ inline bool ensure_dynamic_smem(size_t bytes) {
         return false;
     if (bit) done.fetch_or(bit, std::memory_order_release);
     return true;
+}
+
+// Clusters of sixteen CTAs are more than the portable cluster size: the kernel must opt in, and the device must be
+// able to hold such a cluster at all (sixteen free SMs in one GPC).  Asked once per kernel and device; returns the
+// number of such clusters the device holds at a time (0: none, or the query failed).
+template <auto kern>                                     // (one set of flags per kernel, not per kernel type)
+inline int clusters_of_sixteen(int threads, int bytes) {
+    static std::atomic<uint64_t> asked{0};
+    static std::atomic<int> resident[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    const uint64_t bit = 1ull << dev;
+    if (!(asked.load(std::memory_order_acquire) & bit)) {
+        int n = 0;
+        bool good = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        if (good) {
+            cudaLaunchConfig_t q = {};
+            q.gridDim = dim3(16, 1);
+            q.blockDim = dim3(threads);
+            q.dynamicSmemBytes = bytes;
+            cudaLaunchAttribute a[1];
+            a[0].id = cudaLaunchAttributeClusterDimension;
+            a[0].val.clusterDim.x = 16; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
+            q.attrs = a;
+            q.numAttrs = 1;
+            good = cudaOccupancyMaxActiveClusters(&n, kern, &q) == cudaSuccess && n >= 1;
+        }
+        if (!good) { cudaGetLastError(); n = 0; }
+        resident[dev].store(n, std::memory_order_release);
+        asked.fetch_or(bit, std::memory_order_release);
+    }
+    return resident[dev].load(std::memory_order_acquire);
 }
 
 // Number of SMs of the current device (cached per host thread); 148 if the query fails.

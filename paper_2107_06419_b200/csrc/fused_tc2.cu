@@ -29,8 +29,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include <type_traits>
 
 #include "flat_internal.cuh"
@@ -824,38 +822,6 @@ bool make_bias_map(CUtensorMap* m, const Problem& p) {
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p.bias), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Clusters of sixteen CTAs are more than the portable cluster size: the kernel must opt in, and the device must be
-// able to hold such a cluster at all (sixteen free SMs in one GPC).  Asked once per kernel and device; returns the
-// number of such clusters the device holds at a time (0: none, or the query failed).
-template <auto kern>                                     // (one set of flags per kernel, not per kernel type)
-int clusters_of_sixteen(int threads, int bytes) {
-    static std::atomic<uint64_t> asked{0};
-    static std::atomic<int> resident[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    const uint64_t bit = 1ull << dev;
-    if (!(asked.load(std::memory_order_acquire) & bit)) {
-        int n = 0;
-        bool good = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-        if (good) {
-            cudaLaunchConfig_t q = {};
-            q.gridDim = dim3(16, 1);
-            q.blockDim = dim3(threads);
-            q.dynamicSmemBytes = bytes;
-            cudaLaunchAttribute a[1];
-            a[0].id = cudaLaunchAttributeClusterDimension;
-            a[0].val.clusterDim.x = 16; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
-            q.attrs = a;
-            q.numAttrs = 1;
-            good = cudaOccupancyMaxActiveClusters(&n, kern, &q) == cudaSuccess && n >= 1;
-        }
-        if (!good) { cudaGetLastError(); n = 0; }
-        resident[dev].store(n, std::memory_order_release);
-        asked.fetch_or(bit, std::memory_order_release);
-    }
-    return resident[dev].load(std::memory_order_acquire);
 }
 
 template <int D, int NT>
