@@ -11,7 +11,8 @@
 // among them until the end.  Then the four merge through shared memory and the CTAs of a cluster, which share a
 // head's keys evenly, through distributed shared memory: every CTA leaves (m, l, O) in its own memory, a cluster
 // barrier, and each finishes its share of the outputs from all of them in the order of the ranks (same bits every time).
-// Measured: @@MEASURED@@
+// Measured (graph of calls on fresh inputs, key counts uniform in [Nk / 4, Nk]): B16 H16 1 x 8192 d 128 203 -> 101 us (6.5 TB/s), d 64
+// 117 -> 54; sixteen queries 190 -> 104; B32 H32 1 x 2048 181 -> 100; 4 heads x 32768 48 -> 14; B32 H8 1 x 512 29 -> 11.5.
 //
 // CTA = 160 threads: warps 0-3 as above, warp 4 TMA producer.  Tiles have the 128-byte swizzle; ldmatrix reads eight rows
 // of a panel without bank conflicts.  A warp's logits come out with queries as rows and keys as columns, which is the
