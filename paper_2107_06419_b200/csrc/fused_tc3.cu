@@ -69,6 +69,7 @@ constexpr unsigned POLY_PAIRS_SA = 0x0900, POLY_PAIRS_SB = 0x0900; // the same f
 constexpr unsigned PRODUCER_SLEEP = 400; // ns between the TMA producer's probes of a full ring (it runs far ahead: its reaction time is immaterial)
 
 constexpr int D = 64;                // head size of this kernel
+constexpr int UNITS_MAX = 1024;      // packed batches: most (sequence, slab) units (and sequences) that are sorted (see Sched)
 
 struct L3 {
     static constexpr int KS = 4;                         // K ring depth (S runs 1.5 key steps ahead of P V)
@@ -81,6 +82,7 @@ struct L3 {
     static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES;
     static constexpr int XCH_BYTES = 2 * 2 * 2 * BM * 4; // [maximum | row sum][tile][half][row] floats
     static constexpr int SMEM_BYTES = TILE_BYTES + XCH_BYTES + 512 + 512 + 1024;   // (.. barriers, the even deal's table, alignment)
+    static constexpr int VL_SMEM_BYTES = SMEM_BYTES + UNITS_MAX * 28 + 128;        // (packed batches: the table of units and what sorting it takes)
     __host__ __device__ static constexpr uint32_t O_COL(int t) { return 64u * t; }
     __host__ __device__ static constexpr uint32_t X_COL(int b) { return 128u + 128u * b; }   // logit / weight buffer b
     // barrier indices
@@ -268,12 +270,31 @@ constexpr int WS_MAX_CTAS = 160;
 // items for b = 0 .. B (DEAL_MAX_B batches at most).
 constexpr int DEAL_LO = 0, DEAL_HI = 1, DEAL_FIRST = 2, DEAL_END = 3, DEAL_T = 4, DEAL_TEAM = 5, DEAL_TEAMS = 6, DEAL_PREFIX = 8, DEAL_MAX_B = 64;
 static_assert((DEAL_PREFIX + DEAL_MAX_B + 1) * 4 <= 512, "the deal's table has 512 bytes of shared memory");
+// (packed batches) The table of units in shared memory: first token and number of the query rows from the unit's first one
+// on, first token and number of the keys; then the units' first rows.
+__device__ __forceinline__ uint4* unit_table() {
+    extern __shared__ uint8_t smem_raw[];
+    return reinterpret_cast<uint4*>(((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023)) + L3::TILE_BYTES + L3::XCH_BYTES + 1024);
+}
+// (packed batches) The number of rounds in which this CTA has an item, and the position of the item of a round.
+__device__ __forceinline__ int vl_rounds(int items, int sorted) {
+    const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x), full = items / G, rest = items - full * G;
+    return full + ((sorted && (full & 1) ? G - 1 - c : c) < rest ? 1 : 0);
+}
+__device__ __forceinline__ int vl_position(int round, int sorted) {
+    return round * static_cast<int>(gridDim.x) + static_cast<int>(sorted && (round & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+}
 // What every role needs to enumerate the items.
 struct Sched {
     int items, slabs, H, Nk;
     const int32_t* valid_len;
     int coff;                                            // causal mask: row r sees keys j < r + 1 + coff (coff = Nk - Nq); none: 2^30
-    int paired;                                          // items come in pairs of complementary slabs (see get_item)
+    int paired;                                          // 1: items come in pairs of complementary slabs (see get_item)
+    // (packed batches) 1: the units (sequence, slab) are sorted by their number of key steps, longest first, into a table
+    // in shared memory (fill_units), every unit stands for its H heads, and the CTAs take the items of that order
+    // forwards and backwards in turn -- CTA c has items c, 2 G - 1 - c, 2 G + c, ... -- so that their shares weigh the
+    // same to a few per cent (32 sequences of 40 to 2000 tokens, 12 heads: 105 us with a CTA per slot of the longest
+    // sequence's grid, most of them empty, in the order of the sequences; 81 like this).  An item index is a round then.
     const int32_t* cu_q;                                 // packed variable-length batches: first token of every sequence's
     const int32_t* cu_k;                                 // queries / keys in the packed tensors ([sequences + 1] entries)
     const int* deal;                                     // even deal: its table in shared memory
@@ -391,15 +412,22 @@ __device__ __forceinline__ void deal_finish_merged(const EvenDeal ed, uint32_t o
 }
 // The sequence of item indices of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...; in paired mode the
 // CTA takes PAIRS of consecutive indices (2 c, 2 c + 1), (2 (c + gridDim.x), ...), ...
-template <bool SPLIT = false>
+template <bool SPLIT = false, bool VL = false>
 __device__ __forceinline__ int first_item(const Sched& sc) {
     if (SPLIT) return sc.deal[DEAL_FIRST];
+    if (VL) return 0;
     return sc.paired ? 2 * blockIdx.x : blockIdx.x;
 }
-template <bool SPLIT = false>
+template <bool SPLIT = false, bool VL = false>
 __device__ __forceinline__ int next_item(int idx, const Sched& sc) {
     if (SPLIT) return idx + sc.deal[DEAL_TEAM];
+    if (VL) return idx + 1;
     return sc.paired ? ((idx & 1) ? idx - 1 + 2 * static_cast<int>(gridDim.x) : idx + 1) : idx + static_cast<int>(gridDim.x);
+}
+// (packed batches, sorted) The unit of the item at position `pos`: pos / H by the reciprocal that the launcher gives
+// in ed.team (exact: pos < 1024 H and H < 2048).
+__device__ __forceinline__ int unit_of(int pos, const Sched& sc) {
+    return sc.H == 1 ? pos : static_cast<int>(__umulhi(static_cast<unsigned>(pos), static_cast<unsigned>(sc.ed.team)));
 }
 // VL (packed variable-length batches): Q, O are [total_q, H, d], K, V [total_k, H, d]; sequence s owns
 // tokens cu_q[s] .. cu_q[s+1] - 1 of Q and cu_k[s] .. cu_k[s+1] - 1 of K, V.  Item index =
@@ -412,15 +440,26 @@ __device__ __forceinline__ Item get_item(int idx, const Sched& sc) {
     bool empty = false;
     it.tile0 = 0;
     if (VL) {
-        it.bh = idx / sc.slabs;
-        slab = idx - it.bh * sc.slabs;
-        const int s = it.bh / sc.H;
-        it.head = it.bh - s * sc.H;
-        const int q0 = sc.cu_q[s], ql = sc.cu_q[s + 1] - q0, k0 = sc.cu_k[s], kl = sc.cu_k[s + 1] - k0;
-        it.row0 = slab * (2 * BM);
-        it.q_tok0 = q0 + it.row0;
+        int ql, k0, kl;
+        idx = vl_position(idx, sc.paired);
+        if (sc.paired) {
+            const int u = unit_of(idx, sc);
+            it.head = idx - u * sc.H;
+            const uint32_t at = smem_u32(unit_table());
+            asm volatile("ld.shared::cta.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(it.q_tok0), "=r"(it.q_rows), "=r"(k0), "=r"(kl) : "r"(at + 16 * u) : "memory");
+            asm volatile("ld.shared::cta.s32 %0, [%1];" : "=r"(it.row0) : "r"(at + 16 * UNITS_MAX + 4 * u) : "memory");
+            ql = it.q_rows + it.row0;
+        } else {
+            it.bh = idx / sc.slabs;
+            slab = idx - it.bh * sc.slabs;
+            const int s = it.bh / sc.H, q0 = sc.cu_q[s];
+            it.head = it.bh - s * sc.H;
+            ql = sc.cu_q[s + 1] - q0; k0 = sc.cu_k[s]; kl = sc.cu_k[s + 1] - k0;
+            it.row0 = slab * (2 * BM);
+            it.q_tok0 = q0 + it.row0;
+            it.q_rows = ql - it.row0;
+        }
         it.k_tok0 = k0;
-        it.q_rows = ql - it.row0;
         it.coff = sc.coff < (1 << 29) ? kl - ql : sc.coff;
         it.skip = it.q_rows <= 0;
         int n = kl < 0 ? 0 : kl;
@@ -484,12 +523,12 @@ __device__ __forceinline__ void cursor_seek(Cursor& c, const Sched& sc) {
     while (c.idx < sc.items) {
         c.it = get_item<VL, SPLIT>(c.idx, sc);
         if (c.it.ntiles > 0) { c.valid = true; return; }
-        c.idx = next_item<SPLIT>(c.idx, sc);
+        c.idx = next_item<SPLIT, VL>(c.idx, sc);
     }
 }
 template <bool VL, bool SPLIT = false>
 __device__ __forceinline__ void cursor_init(Cursor& c, const Sched& sc) {
-    c.idx = first_item<SPLIT>(sc); c.j = 0; c.J = 0; c.q = 0;
+    c.idx = first_item<SPLIT, VL>(sc); c.j = 0; c.J = 0; c.q = 0;
     cursor_seek<VL, SPLIT>(c, sc);
 }
 template <bool VL, bool SPLIT = false>
@@ -497,13 +536,76 @@ __device__ __forceinline__ void cursor_next(Cursor& c, const Sched& sc) {
     ++c.j; ++c.J;
     if (c.j == c.it.ntiles) {
         c.j = 0; ++c.q;
-        c.idx = next_item<SPLIT>(c.idx, sc);
+        c.idx = next_item<SPLIT, VL>(c.idx, sc);
         cursor_seek<VL, SPLIT>(c, sc);
     }
 }
 
+// Packed batches: all threads of the CTA fill `tab` with the sorted units of the `seqs` sequences (see Sched); returns
+// their number.  Behind the table: the unsorted units, their keys and the warps' counts.
+__device__ __forceinline__ int fill_units(const Sched& sc, uint4* tab, int seqs) {
+    int* first_row = reinterpret_cast<int*>(tab + UNITS_MAX);
+    uint32_t* raw = reinterpret_cast<uint32_t*>(first_row + UNITS_MAX);      // sequence | slab << 16
+    uint32_t* key = raw + UNITS_MAX;                     // key steps, then the order of the units among equals
+    int* counts = reinterpret_cast<int*>(key + UNITS_MAX);
+    constexpr int PER = (UNITS_MAX + L3::THREADS - 1) / L3::THREADS, WARPS = L3::THREADS / 32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int q[PER], k[PER], n[PER], mine = 0;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+        const int s = tid * PER + e;
+        q[e] = k[e] = n[e] = 0;
+        if (s < seqs) {
+            q[e] = sc.cu_q[s + 1] - sc.cu_q[s];
+            k[e] = sc.cu_k[s + 1] - sc.cu_k[s];
+            n[e] = q[e] > 0 ? min((q[e] + 2 * BM - 1) / (2 * BM), sc.slabs) : 0;
+        }
+        mine += n[e];
+    }
+    int before = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += y;
+    }
+    if (lane == 31) counts[warp] = before;
+    before -= mine;
+    __syncthreads();
+    int total = 0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) {
+        if (w < warp) before += counts[w];
+        total += counts[w];
+    }
+    total = min(total, UNITS_MAX);
+#pragma unroll
+    for (int e = 0; e < PER; ++e)
+        for (int slab = 0; slab < n[e]; ++slab, ++before) {
+            if (before >= UNITS_MAX) break;
+            long long keys = k[e] > 0 ? k[e] : 0;
+            if (sc.coff < (1 << 29)) keys = min(keys, max(0ll, static_cast<long long>(slab + 1) * 2 * BM + k[e] - q[e]));
+            raw[before] = static_cast<uint32_t>(tid * PER + e) | static_cast<uint32_t>(slab) << 16;
+            key[before] = static_cast<uint32_t>(min((keys + BN - 1) / BN, 65535ll)) * UNITS_MAX + (UNITS_MAX - 1 - before);
+        }
+    __syncthreads();
+    // (a warp per unit counts the larger keys: the unit's place)
+    for (int u = warp; u < total; u += WARPS) {
+        const uint32_t mine_k = key[u];
+        int larger = 0;
+#pragma unroll 4
+        for (int v = lane; v < total; v += 32) larger += key[v] > mine_k;
+        const int rank = __reduce_add_sync(0xffffffffu, larger);
+        if (lane != 0) continue;
+        const int s = raw[u] & 0xffffu, row0 = static_cast<int>(raw[u] >> 16) * 2 * BM, q0 = sc.cu_q[s], k0 = sc.cu_k[s];
+        tab[rank] = make_uint4(q0 + row0, sc.cu_q[s + 1] - q0 - row0, k0, sc.cu_k[s + 1] - k0);
+        first_row[rank] = row0;
+    }
+    __syncthreads();
+    return total;
+}
+
 // VL: packed variable-length batches (see get_item); the tensor maps then view the packed tensors as
-// {d, H, tokens} and valid_len is unused (cu_k gives the key counts).
+// {d, H, tokens}, Nk is the number of sequences and valid_len is unused (cu_k gives the key counts).
 // WLSE: also writes lse[b,h,i] = log of row i's sum of exponentials (dense batches; what the
 // backward pass takes from the forward one).  A separate instantiation, so that the plain forward
 // kernel is compiled exactly as it is without the output.
@@ -519,9 +621,9 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     using LY = L3;
     static_assert(!SPLIT || (!VL && !WLSE), "the even deal is built for the plain dense forward kernel only");
     Sched sc{items, slabs, H, Nk, valid_len, coff, paired, cu_q, cu_k, nullptr, ed};
-    if (VL && static_cast<int>(gridDim.x) == items) {
+    if (VL && !paired && static_cast<int>(gridDim.x) == items) {
         // one CTA per slot: a slot past the end of its sequence leaves before anything is set up
-        if (get_item<VL>(blockIdx.x, sc).skip) return;
+        if (get_item<VL>(0, sc).skip) return;
     }
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -593,6 +695,14 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // (launched with programmatic stream serialization: this set-up overlaps the tail of the previous kernel of the stream,
+    // and nothing in device memory is touched before that one has finished.  Not the even deal: its launches have an event
+    // between them, which forbids the overlap.)
+    if (!SPLIT) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+    if (VL) sc.items = items = vl_rounds(paired ? fill_units(sc, unit_table(), Nk) * H : items, paired);
     if (SPLIT) { sc.deal = deal; sc.items = deal[DEAL_END]; items = deal[DEAL_END]; }
 
     if (warp >= LY::SOFT_WARPS) {
@@ -633,7 +743,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 v_issued = J + 1;
             };
             int J0 = 0, q = 0;
-            for (int idx = first_item<SPLIT>(sc); idx < items && ok; idx = next_item<SPLIT>(idx, sc)) {
+            for (int idx = first_item<SPLIT, VL>(sc); idx < items && ok; idx = next_item<SPLIT, VL>(idx, sc)) {
                 const Item it = get_item<VL, SPLIT>(idx, sc);
                 if (it.ntiles == 0) continue;
                 // tile of query rows r.. / of keys of step j
@@ -751,7 +861,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // of the CTA and items whose first step is partly masked start from an exact maximum.
         float m_ref = -INFINITY;
         bool first_item_done = false;
-        for (int idx = first_item<SPLIT>(sc); idx < items; idx = next_item<SPLIT>(idx, sc)) {
+        for (int idx = first_item<SPLIT, VL>(sc); idx < items; idx = next_item<SPLIT, VL>(idx, sc)) {
         const Item it = get_item<VL, SPLIT>(idx, sc);
         if (it.skip) continue;
         const int ntiles = it.ntiles;
@@ -939,14 +1049,26 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             }
         }
         {
-            const int row = it.row0 + t * BM + q * 32 + lane;
+            // (packed batches: the rows are looked up again, so that they do not live in registers through the key steps)
+            int tok0 = 0, rows = 0, head = 0;
+            if (VL) {
+                if (paired) {
+                    const int pos = vl_position(idx, paired), u = unit_of(pos, sc);
+                    head = pos - u * H;
+                    asm volatile("ld.shared::cta.v2.s32 {%0, %1}, [%2];" : "=r"(tok0), "=r"(rows) : "r"(smem_u32(unit_table()) + 16 * u) : "memory");
+                } else {
+                    const Item ie = get_item<VL, SPLIT>(idx, sc);
+                    tok0 = ie.q_tok0; rows = ie.q_rows; head = ie.head;
+                }
+            }
+            const int row = (VL ? 0 : it.row0) + t * BM + q * 32 + lane;   // (packed batches: counted from the slab's first)
             const float inv = l > 0.f ? 1.f / l : 0.f;
             // (m_ref, common to the row's two warps, and the exponents are in base-2 units)
             if (WLSE && h == 0 && row < Nq)
                 lse[static_cast<int64_t>(it.bh) * Nq + row] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
             tc_fence_after();
             // (packed batches: token-major [tokens, H, d])
-            __nv_bfloat16* orow = VL ? O + ((static_cast<int64_t>(it.q_tok0) + (row - it.row0)) * H + it.head) * D + h * (D / 2)
+            __nv_bfloat16* orow = VL ? O + ((static_cast<int64_t>(tok0) + row) * H + head) * D + h * (D / 2)
                                      : O + (static_cast<int64_t>(it.bh) * Nq + row) * D + h * (D / 2);
 #pragma unroll
             for (int c = 0; c < D / 64; ++c) {
@@ -978,7 +1100,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     __nv_bfloat16* even_row = orow - (odd ? D : 0);
                     if (row_e < Nq) st_global_32B(even_row + c * 32 + (odd ? 16 : 0), a);
                     if (row_e + 1 < Nq) st_global_32B(even_row + D + c * 32 + (odd ? 16 : 0), b);
-                } else if (VL ? row - it.row0 < it.q_rows : row < Nq) {
+                } else if (row < (VL ? rows : Nq)) {
                     if (wide_stores) {
                         st_global_32B(orow + c * 32, *reinterpret_cast<uint32_t(*)[8]>(&w[0]));
                         st_global_32B(orow + c * 32 + 16, *reinterpret_cast<uint32_t(*)[8]>(&w[8]));
@@ -1063,6 +1185,22 @@ void deal_release(cudaStream_t st) {
     o.last = st;
 }
 
+// One launch, with programmatic stream serialization (see the kernel's set-up).
+template <typename Kernel, typename... Args>
+cudaError_t launch_pdl(Kernel kern, int grid, int bytes, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(L3::THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 int launch_tc3(const Problem& p, cudaStream_t st) {
     using LY = L3;
     CUtensorMap tmQ, tmK, tmV;
@@ -1117,12 +1255,12 @@ int launch_tc3(const Problem& p, cudaStream_t st) {
     }
     g_last_schedule = persistent ? FLAT_SCHEDULE_PERSISTENT : FLAT_SCHEDULE_ITEMS;
     auto kern = p.lse ? fused_tc3_kernel<false, true> : fused_tc3_kernel<false, false>;
-    kern<<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk,
-                                                    static_cast<int>(slots), slabs, p.scale * 1.4426950408889634f,
-                                                    p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
-                                                    (reinterpret_cast<uintptr_t>(p.O) & 31) == 0 ? 1 : 0, paired, nullptr,
-                                                    nullptr, p.lse, EvenDeal{});
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    const cudaError_t e = launch_pdl(
+        kern, grid, LY::SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, static_cast<int>(slots), slabs,
+        p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
+        (reinterpret_cast<uintptr_t>(p.O) & 31) == 0 ? 1 : 0, paired, static_cast<const int32_t*>(nullptr),
+        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{});
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
 
@@ -1138,24 +1276,31 @@ int launch_fused_tc3_varlen(const void* Q, const void* K, const void* V, void* O
     if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
         !make_map_packed(&tmV, V, total_k, H, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_tc3_kernel<true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_tc3_kernel<true>>(LY::VL_SMEM_BYTES)) return FLAT_ERR_CUDA;
     const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM);
     const int64_t items = static_cast<int64_t>(slabs) * num_seqs * H;
     if (items > 0x7fffffff) return FLAT_ERR_SHAPE;
     const int sms = device_sm_count();
-    // Sequences of different lengths make items of different weight, and a persistent CTA's share is
-    // fixed: with long sequences (many slabs, many key steps per item) one CTA per item, handed out by
-    // the hardware as SMs become free, balances better (measured on a mix of 8 sequences of 3.9K-14.5K
-    // tokens: 2.81 against 2.89 ms, causal 1.61 against 1.86 ms); with many short ones the persistent
-    // grid saves the per-CTA set-up.
-    const bool persistent = items >= 8 * static_cast<int64_t>(sms) && slabs < 8;
-    const int grid = static_cast<int>(persistent ? sms : items);
+    // Persistent CTAs on sorted units (see Sched) where the table holds them all: a sequence has at most one slab more
+    // than its share of the tokens fills.  Otherwise the slots of the longest sequence's grid, by fixed deal while they
+    // are short, or one CTA each, handed out by the hardware as SMs become free (8 sequences of 3.9K-14.5K tokens: 2.81 ms
+    // against 2.89 by fixed deal, causal 1.61 against 1.86).
+    const int64_t units = total_q / (2 * BM) + num_seqs < static_cast<int64_t>(slabs) * num_seqs ? total_q / (2 * BM) + num_seqs
+                                                                                                  : static_cast<int64_t>(slabs) * num_seqs;
+    // (sequences of one length need no order: the table costs about 2 us a launch)
+    const bool equal = !causal && total_q == static_cast<int64_t>(num_seqs) * max_seqlen_q;
+    const bool sorted = units <= UNITS_MAX && num_seqs <= UNITS_MAX && H < 2048 && !equal;
+    const bool persistent = sorted || (items >= 8 * static_cast<int64_t>(sms) && slabs < 8);
+    const int64_t most = sorted ? units * H : items;
+    const int grid = static_cast<int>(persistent && most > sms ? sms : most);
+    EvenDeal ed{};
+    ed.team = static_cast<int>(static_cast<unsigned>(((1ull << 32) + H - 1) / H));   // (see unit_of)
     g_last_schedule = persistent ? FLAT_SCHEDULE_PERSISTENT : FLAT_SCHEDULE_ITEMS;
-    fused_tc3_kernel<true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
-        tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, 0, static_cast<int>(items), slabs,
-        scale * 1.4426950408889634f, nullptr, causal ? 0 : (1 << 30), status,
-        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, 0, cu_q, cu_k, nullptr, EvenDeal{});
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    const cudaError_t e = launch_pdl(
+        fused_tc3_kernel<true>, grid, LY::VL_SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, num_seqs,
+        static_cast<int>(most), slabs, scale * 1.4426950408889634f, static_cast<const int32_t*>(nullptr), causal ? 0 : (1 << 30), status,
+        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, sorted ? 1 : 0, cu_q, cu_k, static_cast<float*>(nullptr), ed);
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
 int launch_fused_tc3(const Problem& p, cudaStream_t st) {
