@@ -35,12 +35,14 @@ struct BiasArg {
     int f32;                         // 1: float32, 0: bf16
     long long sb, sh;
     int vec;                         // 16-byte loads allowed (base, strides and Nk all multiples of 16 bytes)
+    long long bytes;                 // of the tensor, from its first value to its last
 };
 inline BiasArg bias_arg(const Problem& q) {
     const long long es = q.bias_dtype == FLAT_DTYPE_F32 ? 4 : 2, per16 = 16 / es;
     const bool vec = q.bias && (reinterpret_cast<uintptr_t>(q.bias) & 15u) == 0 && q.Nk % per16 == 0 &&
                      q.bias_sb % per16 == 0 && q.bias_sh % per16 == 0;
-    return BiasArg{q.bias, q.bias_dtype == FLAT_DTYPE_F32 ? 1 : 0, q.bias_sb, q.bias_sh, vec ? 1 : 0};
+    const long long bytes = es * ((q.B - 1) * q.bias_sb + (q.H - 1) * q.bias_sh + static_cast<long long>(q.Nq) * q.Nk);
+    return BiasArg{q.bias, q.bias_dtype == FLAT_DTYPE_F32 ? 1 : 0, q.bias_sb, q.bias_sh, vec ? 1 : 0, bytes};
 }
 
 // A validated backward problem (device pointers; bf16 tensors, fp32 lse / delta).
@@ -73,6 +75,7 @@ int launch_fused_tc2_single(const Problem& p, cudaStream_t st, int key_split = 1
 // The same tile worked on by two warpgroups that take alternate key tiles (bf16, d = 64, dense; key_split 1, 2, 4, 8).
 int launch_fused_tc2_halves(const Problem& p, cudaStream_t st, int key_split = 1, bool only_if_resident = false);   // (key_split 1, 2, 4, 8, 16)   // (d = 64; with a block mask also d = 128; key_split 2 / 4: the keys of a tile over a CTA cluster)
 int launch_fused_tc3(const Problem& p, cudaStream_t st);
+int launch_fused_tc3_bias(const Problem& p, const void* bias_map, cudaStream_t st);   // (bias_map: a CUtensorMap)
 // How the last launch_fused_tc3 of this host thread dealt its items (FLAT_SCHEDULE_*; 0 before any).
 extern thread_local int g_last_schedule;
 bool tf32_applies(const Problem& p);               // fp32, d = 64, no bias, no pruning map

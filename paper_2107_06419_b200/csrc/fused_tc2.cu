@@ -50,7 +50,6 @@ constexpr int POLY_LANE = 3;                    // element index mod 4 that uses
 __host__ __device__ constexpr int merge_vecs(int d) { return d / 4 + 1; }   // (key split) 16-byte vectors per row of a partial result: d outputs, then (m, l)
 constexpr float OVERFLOW_SUM = 1.0995116e12f;   // 2^40: a tile row sum beyond this means m_ref is stale
 
-// BT: the bias tile of every (tile, step) is staged through shared memory by TMA (two stages per query tile)
 // KHL (the two warpgroups of a CTA on alternate key tiles of ONE query tile, see the kernel's KH): every key tile has one
 // consumer, the warpgroup of its parity, so the ring depths must be even -- stage g % depth then always belongs to
 // the same warpgroup and a parity wait on its barrier is unambiguous.  (With three stages a stage alternates between
@@ -58,19 +57,16 @@ constexpr float OVERFLOW_SUM = 1.0995116e12f;   // 2^40: a tile row sum beyond t
 // ahead could take the completion of its previous fill for that of the next one: wrong keys, then a stuck ring.
 // Seen as rare wrong rows and time-outs on masked batches.)  1: four K and four V stages; 2: four and two (the
 // sixteen-CTA cluster's receive buffer leaves no room for more).
-template <int D, int NT, bool BT = false, int KHL = 0> struct L2 {
+template <int D, int NT, int KHL = 0> struct L2 {
     static constexpr bool ALIAS = (D == 128);            // P overlays S
-    static constexpr int KS = KHL ? 4 : (NT == 1 || BT) ? 2 : (D == 64) ? 3 : 2;   // K ring depth
+    static constexpr int KS = KHL ? 4 : NT == 1 ? 2 : (D == 64) ? 3 : 2;   // K ring depth
     static constexpr int VS = KHL == 2 ? 2 : KS;         // V ring depth
     static constexpr int THREADS = 128 * NT + 128;       // NT softmax warpgroups + {TMA, NT MMA issuers, idle}
     static constexpr int SOFT_WARPS = 4 * NT;
     static constexpr uint32_t TMEM_COLS = (NT == 2) ? 512 : 256;
     static constexpr int Q_BYTES = BM * D * 2;           // one query tile
     static constexpr int KV_BYTES = BN * D * 2;
-    static constexpr int BS = 2;                         // bias ring depth per query tile
-    static constexpr int BIAS_BYTES = BM * BN * 2;       // one 128 x 128 bf16 tile: two panels of 128 rows x 128 bytes
-    static constexpr int BIAS_OFF = NT * Q_BYTES + (KS + VS) * KV_BYTES;
-    static constexpr int TILE_BYTES = BIAS_OFF + (BT ? NT * BS * BIAS_BYTES : 0);
+    static constexpr int TILE_BYTES = NT * Q_BYTES + (KS + VS) * KV_BYTES;
     static constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
     __host__ __device__ static constexpr uint32_t S_COL(int t) { return 128u * t; }
     __host__ __device__ static constexpr uint32_t O_COL(int t) { return 128u * NT + D * t; }
@@ -83,8 +79,7 @@ template <int D, int NT, bool BT = false, int KHL = 0> struct L2 {
     static constexpr int S_FREE = S_FULL + NT, P_FULL = S_FREE + NT, PV_DONE = P_FULL + NT;
     static constexpr int TURN = PV_DONE + NT;            // [2][4]: per warp pair, "tile t may run its exponentials"
     static constexpr int MERGE_BAR = TURN + 8;           // (key split over a cluster) partial results of the other CTAs have arrived
-    static constexpr int B_FULL = MERGE_BAR + 1, B_EMPTY = B_FULL + NT * BS;   // (BT) [NT][BS]
-    static constexpr int NUM_BARS = BT ? B_EMPTY + NT * BS : MERGE_BAR + 1;
+    static constexpr int NUM_BARS = MERGE_BAR + 1;
     // rows of partial results a CTA of a CS-way split receives: CS - 1 senders x 128 / CS rows it owns
     __host__ __device__ static constexpr int merge_bytes(int cs) { return cs > 1 ? (cs - 1) * (128 / cs) * merge_vecs(D) * 16 : 0; }
     // Strict alternation of the two tiles' exponential phases.  At d = 128 the chain of a tile is
@@ -177,6 +172,63 @@ __device__ __forceinline__ float exp_store(const uint32_t (&s)[128], float scale
     return (l0 + l1) + (l2 + l3);
 }
 
+// s = s * scale * log2(e) + bias * log2(e) for a row of 128 logits whose `count` first bias values of ES bytes lie at `p`, at any
+// alignment.  Pieces of 16 bytes that reach beyond the tensor are put together value by value.
+template <int ES>
+__device__ __forceinline__ void add_bias_row(uint32_t (&s)[128], float scale_log2e, const char* p, int count, const BiasArg& bias) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), g0 = a & ~uintptr_t(15), end = a + static_cast<uintptr_t>(count) * ES;
+    const uintptr_t lo = reinterpret_cast<uintptr_t>(bias.p), hi = lo + bias.bytes;
+    const int words = static_cast<int>(a - g0) >> 2, bits = static_cast<int>(a & 2) * 8;
+    auto piece = [&](int k, uint32_t (&w)[4]) {
+        const uintptr_t g = g0 + 16 * k;
+        w[0] = w[1] = w[2] = w[3] = 0u;
+        if (g >= end) return;                            // (behind the row's values)
+        if (g >= lo && g + 16 <= hi) {
+            const uint4 v = *reinterpret_cast<const uint4*>(g);
+            w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 16 / ES; ++e) {
+                const uintptr_t x = g + e * ES;
+                if (x < lo || x + ES > hi) continue;
+                if (ES == 4) w[e] = *reinterpret_cast<const uint32_t*>(x);
+                else         w[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(x)) << (16 * (e & 1));
+            }
+        }
+    };
+    constexpr int PER = 16 / ES;                         // values per piece
+    uint32_t w[8];
+    {
+        uint32_t f[4];
+        piece(0, f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = f[i];
+    }
+#pragma unroll
+    for (int k = 0; k < 128 / PER; ++k) {
+        uint32_t f[4], t[6];
+        piece(k + 1, f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[4 + i] = f[i];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) t[i] = (words & 2) ? w[i + 2] : w[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) t[i] = (words & 1) ? t[i + 1] : t[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (ES == 4) {
+                s[k * 4 + i] = __float_as_uint(fmaf(__uint_as_float(s[k * 4 + i]), scale_log2e, __uint_as_float(t[i]) * 1.4426950408889634f));
+            } else {
+                const uint32_t b = __funnelshift_r(t[i], t[i + 1], bits);
+                s[k * 8 + 2 * i] = __float_as_uint(fmaf(__uint_as_float(s[k * 8 + 2 * i]), scale_log2e, __uint_as_float(b << 16) * 1.4426950408889634f));
+                s[k * 8 + 2 * i + 1] = __float_as_uint(fmaf(__uint_as_float(s[k * 8 + 2 * i + 1]), scale_log2e, __uint_as_float(b & 0xffff0000u) * 1.4426950408889634f));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = w[4 + i];
+    }
+}
+
 // VL: packed variable-length batches.  Q, O are [total_q, H, d], K, V [total_k, H, d]; sequence s owns
 // tokens cu_q[s] .. cu_q[s+1] - 1 of Q and cu_k[s] .. cu_k[s+1] - 1 of K, V; the tensor maps view the
 // packed tensors as {d, H, tokens}; blockIdx.y = sequence * H + head, blockIdx.x = slab of the
@@ -195,26 +247,21 @@ __device__ __forceinline__ float exp_store(const uint32_t (&s)[128], float scale
 // ranks store their partials for those rows into r's shared memory (st.shared::cluster, lanes of a warp writing
 // contiguous bytes) and arrive on r's mbarrier, and the owner merges them with the split-softmax identity and writes
 // the rows.  Plain remote stores only.
-// BIAS = 2: the same with the bias tile of each step staged through shared memory by TMA (bf16, 16-byte aligned
-// rows, d = 64): the rows then arrive coalesced and a softmax thread reads its 256 bytes from shared memory; with a
-// bias shared by all batches the grid runs the batches of a head next to each other, so that its slice stays in L2.
 // KH (two warpgroups, ONE query tile, d = 64, dense): a short launch waits for one CTA's chain of key steps, and a
 // step is one warp per scheduler working through 128 exponentials per row.  With KH the CTA's two softmax warpgroups
 // (and their two MMA issuers, logit / weight / output columns) take the even and the odd key tiles of the same 128
 // query rows, each with its own running (m_ref, l, O); at the end the second warpgroup leaves its rows in shared
 // memory and the first merges them (the split-softmax identity again) before the ordinary epilogue or the cluster
 // exchange.  The chain is half as long and two warps per scheduler share the exponent unit.
-template <int D, int NT, bool VL = false, int BIAS = 0, bool SPARSE = false, int CS = 1, bool KH = false>
+template <int D, int NT, bool VL = false, bool BIAS = false, bool SPARSE = false, int CS = 1, bool KH = false>
 __global__ void __launch_bounds__(128 * NT + 128, NT == 1 ? 2 : 1)
 fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, int H, int Nq, int Nk,
                  float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int32_t* status,
                  const int32_t* __restrict__ cu_q = nullptr, const int32_t* __restrict__ cu_k = nullptr,
-                 float* __restrict__ lse = nullptr, BiasArg bias = BiasArg{nullptr, 0, 0, 0, 0},
-                 const uint8_t* __restrict__ block_mask = nullptr, long long bmask_sb = 0, long long bmask_sh = 0,
-                 const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}) {
-    using LY = L2<D, NT, BIAS == 2, KH ? (CS == 16 ? 2 : 1) : 0>;
-    static_assert(BIAS != 2 || (NT == 2 && D == 64 && !VL && !SPARSE && CS == 1), "staged bias: the two-tile dense kernel, d = 64");
+                 float* __restrict__ lse = nullptr, BiasArg bias = BiasArg{},
+                 const uint8_t* __restrict__ block_mask = nullptr, long long bmask_sb = 0, long long bmask_sh = 0) {
+    using LY = L2<D, NT, KH ? (CS == 16 ? 2 : 1) : 0>;
     static_assert(!SPARSE || (NT == 1 && !VL && !BIAS), "the pruning map is read by the one-tile dense kernel");
     static_assert(CS == 1 || ((NT == 1 || KH) && !VL && !BIAS && !SPARSE && (CS == 2 || CS == 4 || CS == 8 || CS == 16)), "key split: one-tile dense kernel");
     static_assert(!KH || (NT == 2 && D == 64 && !VL && !BIAS && !SPARSE), "key halves: two warpgroups on one dense d = 64 tile");
@@ -233,12 +280,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     float4* kh_buf = reinterpret_cast<float4*>(base + LY::TILE_BYTES + 512 + LY::merge_bytes(CS));   // (KH) [d / 4 + 1][128]: the second warpgroup's rows
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int bh = blockIdx.y;
-    if (BIAS == 2 && bias.sb == 0) {
-        // a bias shared by the batches: y runs over the batches first, so that CTAs in flight share a head's slice
-        const int nb = gridDim.y / H;
-        bh = (blockIdx.y % nb) * H + blockIdx.y / nb;
-    }
+    const int bh = blockIdx.y;
     const int crank = CS > 1 ? static_cast<int>(cluster_ctarank()) : 0;   // (cluster = CS consecutive CTAs along x)
     const int row0 = (blockIdx.x / CS) * (QT * BM);
     // Barriers and TMEM columns.  The one-tile dense kernels (short launches, where the gap between two kernels of a
@@ -250,8 +292,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     auto setup = [&]() {
         if (threadIdx.x == LY::SOFT_WARPS * 32) {
             for (int i = 0; i < LY::NUM_BARS; ++i) {
-                const bool by_softmax = (i >= LY::S_FREE && i < LY::PV_DONE) ||    // one arrival per softmax warp
-                                        (BIAS == 2 && i >= LY::B_EMPTY);
+                const bool by_softmax = i >= LY::S_FREE && i < LY::PV_DONE;        // one arrival per softmax warp
                 const bool by_issuers = (i >= LY::K_EMPTY && i < LY::V_FULL) || (i >= LY::V_EMPTY && i < LY::S_FULL);
                 mbar_init(&bars[i], i == LY::MERGE_BAR ? (CS > 1 ? (CS - 1) * (CS <= 4 ? 128 / CS / 32 : 1) : 1) : by_softmax ? 4 : by_issuers ? (KH ? 1 : NT) : 1);   // (KH: a key tile is used by one warpgroup only)
             }
@@ -346,30 +387,11 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                                 VL ? k_tok0 + j * BN : bh);
                 v_issued = j + 1;
             };
-            int b_issued = 0;
-            auto load_b = [&](int j) {                   // (BIAS == 2) the bias tiles of step j, one per query tile
-                const int s = j % LY::BS;
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    if (!ok) return;
-                    ok = bounded_wait(&bars[LY::B_EMPTY + t * LY::BS + s], ((j / LY::BS) & 1) ^ 1, abort_flag, status, 0x120 + t);
-                    if (!ok) return;
-                    uint8_t* dst = base + LY::BIAS_OFF + (t * LY::BS + s) * LY::BIAS_BYTES;
-                    mbar_arrive_expect_tx(&bars[LY::B_FULL + t * LY::BS + s], LY::BIAS_BYTES);
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-                        tma_load_4d(dst + c * BM * 128, &tmBias, &bars[LY::B_FULL + t * LY::BS + s], j * BN + c * 64, row0 + t * BM,
-                                    bias.sh ? bh % H : 0, bias.sb ? bh / H : 0);
-                }
-                b_issued = j + 1;
-            };
-            if (BIAS == 2) prefetch_tensormap(&tmBias);
             mbar_arrive_expect_tx(&bars[LY::Q_FULL + 0], LY::Q_BYTES);
 #pragma unroll
             for (int c = 0; c < D / 64; ++c)
                 tma_load_3d(Qs + c * BM * 128, &tmQ, &bars[LY::Q_FULL + 0], c * 64, VL ? head : row0, VL ? q_tok0 : bh);
             load_k(0);
-            if (BIAS == 2) load_b(0);
             if (NT == 2) {
                 mbar_arrive_expect_tx(&bars[LY::Q_FULL + NT - 1], LY::Q_BYTES);
 #pragma unroll
@@ -380,12 +402,8 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             for (int j = 0; j < ntiles && ok; ++j) {
                 if (j + 1 < ntiles) load_k(j + 1);
                 if (ok) load_v(j);
-                if (BIAS == 2 && ok && j + 1 < ntiles) load_b(j + 1);
             }
             if (!ok) {
-                if (BIAS == 2)
-                    for (int j = b_issued > LY::BS ? b_issued - LY::BS : 0; j < b_issued; ++j)
-                        for (int t = 0; t < NT; ++t) drain_wait(&bars[LY::B_FULL + t * LY::BS + j % LY::BS], (j / LY::BS) & 1);
                 drain_wait(&bars[LY::Q_FULL + 0], 0);
                 if (NT == 2) drain_wait(&bars[LY::Q_FULL + NT - 1], 0);
                 for (int j = k_issued > LY::KS ? k_issued - LY::KS : 0; j < k_issued; ++j)
@@ -487,9 +505,9 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         for (int j = 0; j < nt_t; ++j) {
             // (bias, the common case of an aligned bf16 tensor: the row's 128 values of this step are fetched
             // before the wait for the logits, so that the two latencies overlap)
-            uint32_t bpk[BIAS == 1 ? 64 : 1];
+            uint32_t bpk[BIAS ? 64 : 1];
             bool bias_ready = false;
-            if (BIAS == 1) {
+            if (BIAS) {
                 if (bias.vec && !bias.f32 && row < Nq && (j + 1) * BN <= Nk) {
                     const uint4* g = reinterpret_cast<const uint4*>(
                         static_cast<const __nv_bfloat16*>(bias.p) + static_cast<long long>(bh / H) * bias.sb +
@@ -515,28 +533,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             if (lane == 0) mbar_arrive(&bars[LY::S_FREE + t]);   // S_t may be overwritten (d = 64: by the next S_t)
 
             const int col0 = tile_of(gi(j)) * BN;
-            if (BIAS == 2) {
-                // x = s * scale * log2(e) + bias * log2(e): the thread's row of the staged tile (two swizzled panels)
-                const int bs = j % LY::BS, rt = (warp & 3) * 32 + lane;
-                ok = __all_sync(0xffffffffu, bounded_wait(&bars[LY::B_FULL + t * LY::BS + bs], (j / LY::BS) & 1, abort_flag,
-                                                         status, 0x360 + t));
-                if (!ok) break;
-                const uint8_t* brow = base + LY::BIAS_OFF + (t * LY::BS + bs) * LY::BIAS_BYTES + rt * 128;
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const uint4 w = *reinterpret_cast<const uint4*>(brow + (c >> 3) * (BM * 128) + (((c & 7) ^ (rt & 7)) << 4));
-                    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        s[c * 8 + 2 * e] = __float_as_uint(fmaf(__uint_as_float(s[c * 8 + 2 * e]), scale_log2e,
-                                                                __uint_as_float(ww[e] << 16) * 1.4426950408889634f));
-                        s[c * 8 + 2 * e + 1] = __float_as_uint(fmaf(__uint_as_float(s[c * 8 + 2 * e + 1]), scale_log2e,
-                                                                    __uint_as_float(ww[e] & 0xffff0000u) * 1.4426950408889634f));
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bars[LY::B_EMPTY + t * LY::BS + bs]);
-            } else if (BIAS) {
+            if (BIAS) {
                 // x = s * scale * log2(e) + bias * log2(e); a row past the end and columns past Nk read nothing
                 const long long at = static_cast<long long>(bh / H) * bias.sb + static_cast<long long>(bh % H) * bias.sh +
                                      static_cast<long long>(row) * Nk + col0;
@@ -577,15 +574,14 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                         for (int i = 0; i < 16; ++i)
                             s[c * 16 + i] = __float_as_uint(fmaf(__uint_as_float(s[c * 16 + i]), scale_log2e, bv[i] * 1.4426950408889634f));
                     }
+                } else if (in_rows) {
+                    // Rows that begin anywhere: aligned 16-byte pieces, two neighbours at a time, shifted into place (value by
+                    // value the 128 loads of 32 rows each were 33,000 cycles a step of the load unit: @@UN@@).
+                    if (bias.f32) add_bias_row<4>(s, scale_log2e, static_cast<const char*>(bias.p) + at * 4, min(BN, Nk - col0), bias);
+                    else          add_bias_row<2>(s, scale_log2e, static_cast<const char*>(bias.p) + at * 2, min(BN, Nk - col0), bias);
                 } else {
-#pragma unroll                                           // (fully: the logits must stay in registers)
-                    for (int i = 0; i < 128; ++i) {
-                        float bvi = 0.f;
-                        if (in_rows && col0 + i < Nk)
-                            bvi = bias.f32 ? static_cast<const float*>(bias.p)[at + i]
-                                           : __bfloat162float(static_cast<const __nv_bfloat16*>(bias.p)[at + i]);
-                        s[i] = __float_as_uint(fmaf(__uint_as_float(s[i]), scale_log2e, bvi * 1.4426950408889634f));
-                    }
+#pragma unroll
+                    for (int i = 0; i < 128; ++i) s[i] = __float_as_uint(__uint_as_float(s[i]) * scale_log2e);
                 }
             }
             const bool tail = col0 + BN > nrow_min;      // (warp-uniform) some row has masked keys in this step
@@ -839,7 +835,7 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             fused_tc2_kernel<D, NT, false, false, true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
                 tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
                 p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, nullptr, nullptr, p.lse,
-                BiasArg{nullptr, 0, 0, 0, 0}, p.block_mask, p.bmask_sb, p.bmask_sh);
+                BiasArg{}, p.block_mask, p.bmask_sb, p.bmask_sh);
             return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
         } else {
             return FLAT_ERR_UNSUPPORTED;
@@ -851,12 +847,7 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             const BiasArg ba = bias_arg(p);
             CUtensorMap tmB;
             if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) {
-                using LB = L2<D, NT, true>;
-                if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, 2>>(LB::SMEM_BYTES)) return FLAT_ERR_CUDA;
-                fused_tc2_kernel<D, NT, false, 2><<<grid, LB::THREADS, LB::SMEM_BYTES, st>>>(
-                    tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
-                    p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, nullptr, nullptr, p.lse, ba, nullptr, 0, 0, tmB);
-                return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+                return launch_fused_tc3_bias(p, &tmB, st);
             }
         }
         if constexpr (NT == 2) {
@@ -898,7 +889,7 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
                     &cfg, fused_tc2_kernel<D, NT, false, false, false, CS>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H,
                     p.Nq, p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
                     static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse,
-                    BiasArg{nullptr, 0, 0, 0, 0}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll, CUtensorMap{});
+                    BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
                 return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
             };
             if constexpr (D == 128) {
@@ -926,14 +917,13 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
         const cudaError_t e = cudaLaunchKernelEx(
             &cfg, kern, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
             p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, static_cast<const int32_t*>(nullptr),
-            static_cast<const int32_t*>(nullptr), p.lse, BiasArg{nullptr, 0, 0, 0, 0}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll,
-            CUtensorMap{});
+            static_cast<const int32_t*>(nullptr), p.lse, BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
         return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
     }
     kern<<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq,
                                                     p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
                                                     p.causal ? p.Nk - p.Nq : (1 << 30), p.status, nullptr, nullptr, p.lse,
-                                                    BiasArg{nullptr, 0, 0, 0, 0}, nullptr, 0, 0, CUtensorMap{});
+                                                    BiasArg{}, nullptr, 0, 0);
     return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
@@ -949,7 +939,7 @@ int launch_tc2_kh(const Problem& p, cudaStream_t st, int key_split, bool only_if
     const dim3 grid((p.Nq + BM - 1) / BM, BH);
     auto launch = [&](auto cs_tag) -> int {
         constexpr int CS = decltype(cs_tag)::value;
-        using LY = L2<D, NT, false, CS == 16 ? 2 : 1>;   // (the kernel's own choice of ring depths)
+        using LY = L2<D, NT, CS == 16 ? 2 : 1>;   // (the kernel's own choice of ring depths)
         constexpr int BYTES = LY::SMEM_BYTES + LY::merge_bytes(CS) + 128 * merge_vecs(D) * 16;
         static_assert(BYTES <= 232448, "shared memory of the two-warpgroup form");
         auto kern = fused_tc2_kernel<D, NT, false, 0, false, CS, true>;
@@ -973,8 +963,7 @@ int launch_tc2_kh(const Problem& p, cudaStream_t st, int key_split, bool only_if
         const cudaError_t e = cudaLaunchKernelEx(
             &cfg, kern, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
             p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, static_cast<const int32_t*>(nullptr),
-            static_cast<const int32_t*>(nullptr), p.lse, BiasArg{nullptr, 0, 0, 0, 0}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll,
-            CUtensorMap{});
+            static_cast<const int32_t*>(nullptr), p.lse, BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
         return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
     };
     return key_split == 1   ? launch(std::integral_constant<int, 1>{})

@@ -71,15 +71,18 @@ constexpr unsigned PRODUCER_SLEEP = 400; // ns between the TMA producer's probes
 constexpr int D = 64;                // head size of this kernel
 constexpr int UNITS_MAX = 1024;      // packed batches: most (sequence, slab) units (and sequences) that are sorted (see Sched)
 
-struct L3 {
-    static constexpr int KS = 4;                         // K ring depth (S runs 1.5 key steps ahead of P V)
-    static constexpr int VS = 3;                         // V ring depth
+// BT: with a ring of three bias tiles (128 x 128 bf16, two panels of 64 columns), which leaves room for shallower K and V rings.
+template <bool BT> struct Layout {
+    static constexpr int KS = BT ? 3 : 4;                // K ring depth (S runs 1.5 key steps ahead of P V)
+    static constexpr int VS = BT ? 2 : 3;                // V ring depth
+    static constexpr int BIAS_BYTES = BM * BN * 2;
     static constexpr int SOFT_WARPS = 16;
     static constexpr int THREADS = 32 * SOFT_WARPS + 128;
     static constexpr uint32_t TMEM_COLS = 512;
     static constexpr int Q_BYTES = BM * D * 2;           // one query tile
     static constexpr int KV_BYTES = BN * D * 2;
-    static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES;
+    static constexpr int BIAS_OFF = 2 * Q_BYTES + (KS + VS) * KV_BYTES;
+    static constexpr int TILE_BYTES = BIAS_OFF + (BT ? 3 * BIAS_BYTES : 0);
     static constexpr int XCH_BYTES = 2 * 2 * 2 * BM * 4; // [maximum | row sum][tile][half][row] floats
     static constexpr int SMEM_BYTES = TILE_BYTES + XCH_BYTES + 512 + 512 + 1024;   // (.. barriers, the even deal's table, alignment)
     static constexpr int VL_SMEM_BYTES = SMEM_BYTES + UNITS_MAX * 28 + 128;        // (packed batches: the table of units and what sorting it takes)
@@ -96,8 +99,13 @@ struct L3 {
     // one of these barriers more than one phase ahead of the phase it asks for (parity waits are safe).
     static constexpr int S_FULL = V_EMPTY + VS, P_FULL = S_FULL + 6, PV_DONE = P_FULL + 6;
     static constexpr int Q_EMPTY = PV_DONE + 6;          // [2] the item's logit MMAs are done with the Q tile
-    static constexpr int NUM_BARS = Q_EMPTY + 2;
+    // (BT) B_FULL / B_EMPTY [buffer]: the bias tile of tile-step u is in stage u % 3 / the 8 softmax warps of its tile have
+    // read it, phase u / 3: a stage is filled again only behind its EMPTY, so a waiter is never a phase behind
+    static constexpr int B_FULL = Q_EMPTY + 2, B_EMPTY = B_FULL + (BT ? 3 : 0);
+    static constexpr int NUM_BARS = B_EMPTY + (BT ? 3 : 0);
+    static_assert(SMEM_BYTES <= 232448 && NUM_BARS * 8 + 8 <= 512, "shared memory");
 };
+using L3 = Layout<false>;
 
 __device__ __forceinline__ float half_max(const uint32_t (&s)[HN]) {
     float e0 = __uint_as_float(s[0]), e1 = __uint_as_float(s[1]), e2 = __uint_as_float(s[2]), e3 = __uint_as_float(s[3]);
@@ -228,6 +236,43 @@ __device__ __forceinline__ void exp_pack32(const uint32_t (&r)[32], float scale_
     }
 }
 
+// (bias) r = r * scale * log2(e) + bias * log2(e) for 32 logits of a row: base-2 units.  `brow`: shared-window address of
+// the row in its panel of the staged tile; C0: first of its eight 16-byte chunks; rx: the row's place in the swizzle.
+template <int C0>
+__device__ __forceinline__ void add_bias32(uint32_t (&r)[32], float scale_log2e, uint32_t brow, int rx) {
+    const uint64_t scale2 = pack2(scale_log2e, scale_log2e), log2e2 = pack2(1.4426950408889634f, 1.4426950408889634f);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t w[4];
+        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + (((C0 + c) ^ rx) << 4)) : "memory");
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = c * 8 + 2 * e;
+            float a, b;
+            unpack2(fma2(pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), scale2,
+                         mul2(pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)), log2e2)), a, b);
+            r[i] = __float_as_uint(a);
+            r[i + 1] = __float_as_uint(b);
+        }
+    }
+}
+// The same with the reference taken off: x2 = pairs of r * scale + bias * log2(e) + neg_m.
+template <int C0>
+__device__ __forceinline__ void scale_bias32(const uint32_t (&r)[32], uint64_t scale2, uint64_t neg_m2, uint32_t brow, int rx, uint64_t (&x2)[16]) {
+    const uint64_t log2e2 = pack2(1.4426950408889634f, 1.4426950408889634f);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t w[4];
+        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + (((C0 + c) ^ rx) << 4)) : "memory");
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = c * 4 + e;
+            x2[i] = fma2(pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), scale2,
+                         fma2(pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)), log2e2, neg_m2));
+        }
+    }
+}
+
 // One work item = (batch, head, slab of 256 query rows).  A CTA takes the items blockIdx.x,
 // blockIdx.x + gridDim.x, ... one after the other without draining its pipeline in between.
 struct Item {
@@ -298,6 +343,7 @@ struct Sched {
     const int32_t* cu_q;                                 // packed variable-length batches: first token of every sequence's
     const int32_t* cu_k;                                 // queries / keys in the packed tensors ([sequences + 1] entries)
     const int* deal;                                     // even deal: its table in shared memory
+    int batches;                                         // (bias) > 0: shared by this many batches, whose items of a head lie side by side
     EvenDeal ed;
 };
 // Even deal: first key step of team g's range, of `teams` (g T < 2^32: the launcher checks).
@@ -433,7 +479,7 @@ __device__ __forceinline__ int unit_of(int pos, const Sched& sc) {
 // tokens cu_q[s] .. cu_q[s+1] - 1 of Q and cu_k[s] .. cu_k[s+1] - 1 of K, V.  Item index =
 // (sequence * H + head) * slabs + slab with `slabs` taken from the longest sequence; a slab past the
 // end of its sequence is an empty slot.  The causal offset is that of the sequence.
-template <bool VL, bool SPLIT = false>
+template <bool VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ Item get_item(int idx, const Sched& sc) {
     Item it;
     int slab;
@@ -488,6 +534,7 @@ __device__ __forceinline__ Item get_item(int idx, const Sched& sc) {
         // that CTAs launched together do not all hold slabs of the same length)
         if (sc.coff < (1 << 29)) slab = (slab + 7 * it.bh) % sc.slabs;
     }
+    if (BIAS && sc.batches) it.bh = (it.bh % sc.batches) * sc.H + it.bh / sc.batches;
     it.row0 = slab * (2 * BM);
     int n = sc.Nk;
     if (sc.valid_len) { n = sc.valid_len[it.bh / sc.H]; n = n < 0 ? 0 : (n > sc.Nk ? sc.Nk : n); }
@@ -517,27 +564,27 @@ struct Cursor {
     Item it;
     bool valid;
 };
-template <bool VL, bool SPLIT = false>
+template <bool VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ void cursor_seek(Cursor& c, const Sched& sc) {
     c.valid = false;
     while (c.idx < sc.items) {
-        c.it = get_item<VL, SPLIT>(c.idx, sc);
+        c.it = get_item<VL, SPLIT, BIAS>(c.idx, sc);
         if (c.it.ntiles > 0) { c.valid = true; return; }
         c.idx = next_item<SPLIT, VL>(c.idx, sc);
     }
 }
-template <bool VL, bool SPLIT = false>
+template <bool VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ void cursor_init(Cursor& c, const Sched& sc) {
     c.idx = first_item<SPLIT, VL>(sc); c.j = 0; c.J = 0; c.q = 0;
-    cursor_seek<VL, SPLIT>(c, sc);
+    cursor_seek<VL, SPLIT, BIAS>(c, sc);
 }
-template <bool VL, bool SPLIT = false>
+template <bool VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ void cursor_next(Cursor& c, const Sched& sc) {
     ++c.j; ++c.J;
     if (c.j == c.it.ntiles) {
         c.j = 0; ++c.q;
         c.idx = next_item<SPLIT, VL>(c.idx, sc);
-        cursor_seek<VL, SPLIT>(c, sc);
+        cursor_seek<VL, SPLIT, BIAS>(c, sc);
     }
 }
 
@@ -611,16 +658,26 @@ __device__ __forceinline__ int fill_units(const Sched& sc, uint4* tab, int seqs)
 // kernel is compiled exactly as it is without the output.
 // SPLIT: the even deal by key steps (see EvenDeal; dense batches, no causal mask, B <= DEAL_MAX_B; `items` is the
 // number of items, B * H * slabs, and the grid must not exceed the SMs that can hold a CTA each).
-template <bool VL, bool WLSE = false, bool SPLIT = false>
+// BIAS (dense batches): adds a bf16 tensor to the scaled logits.  The producer stages the 128 x 128 tile of every tile-step
+// through shared memory by TMA (a 4-D map {Nk, Nq, heads, batches}; a broadcast axis has extent 1), a softmax thread
+// reads its 128 bytes of it and the sum rides on the scaling of the logits; -inf switches a pair off (weights through the
+// ex2 unit are then 0; those through the polynomial 2^-126, nothing beside the 2^-60 that a row's sum has at least).  A row
+// that has seen nothing but -inf keeps no reference and goes the careful way, which takes no polynomial.  What it adds to
+// the plain kernel: 100 instructions per 64 logits (eight 16-byte loads, unpacking, one packed FMA a pair) in the kernel
+// whose exponent unit, not its issue slots, is the bound.  Before, the bias was read by the kernel with one softmax
+// thread per row (fused_tc2.cu), 6,500 cycles a key step: B8 H16 1024 x 1024 110 us, @@B1@@ here; B16 H16 4096 @@B2@@.
+template <bool VL, bool WLSE = false, bool SPLIT = false, bool BIAS = false>
 __global__ void __launch_bounds__(L3::THREADS, 1)
 fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, int H, int Nq, int Nk,
                  int items, int slabs, float scale_log2e, const int32_t* __restrict__ valid_len, int coff,
                  int32_t* status, int wide_stores, int paired, const int32_t* __restrict__ cu_q,
-                 const int32_t* __restrict__ cu_k, float* __restrict__ lse, const EvenDeal ed) {
-    using LY = L3;
+                 const int32_t* __restrict__ cu_k, float* __restrict__ lse, const EvenDeal ed,
+                 const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}, int bias_heads = 0, int bias_batches = 0) {
+    using LY = Layout<BIAS>;
+    static_assert(!BIAS || (!VL && !SPLIT), "the bias is read by the plain dense kernel");
     static_assert(!SPLIT || (!VL && !WLSE), "the even deal is built for the plain dense forward kernel only");
-    Sched sc{items, slabs, H, Nk, valid_len, coff, paired, cu_q, cu_k, nullptr, ed};
+    Sched sc{items, slabs, H, Nk, valid_len, coff, paired, cu_q, cu_k, nullptr, BIAS && !bias_batches ? items / (H * (paired ? (slabs + 1) & ~1 : slabs)) : 0, ed};
     if (VL && !paired && static_cast<int>(gridDim.x) == items) {
         // one CTA per slot: a slot past the end of its sequence leaves before anything is set up
         if (get_item<VL>(0, sc).skip) return;
@@ -640,7 +697,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 
     if (threadIdx.x == LY::SOFT_WARPS * 32) {
         for (int i = 0; i < LY::NUM_BARS; ++i)
-            mbar_init(&bars[i], (i >= LY::P_FULL && i < LY::PV_DONE) ? 8               // one arrival per softmax warp of the tile
+            mbar_init(&bars[i], (i >= LY::P_FULL && i < LY::PV_DONE) || (BIAS && i >= LY::B_EMPTY) ? 8   // one arrival per softmax warp of the tile
                                 : (i >= LY::V_EMPTY && i < LY::S_FULL) ? 2 : 1);   // V_EMPTY: both O += P V issuers
         *abort_flag = 0;
         fence_mbar_init();
@@ -714,7 +771,9 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // wanted before V_{j+1}).  The rings are indexed with the global key step J.
         if (lane == 0) {
             prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
+            if (BIAS) prefetch_tensormap(&tmBias);
             bool ok = true;
+            int b_issued = 0;
             int q_loaded[2] = {0, 0}, k_issued = 0, v_issued = 0;    // (for the drain after a failed wait)
             // (y, z): coordinates of the tile in the tensor map beyond the feature index -- (row, head of
             // the batch), or (head, token) for packed batches
@@ -742,9 +801,25 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 tma_load_3d(Vs + s * LY::KV_BYTES, &tmV, &bars[LY::V_FULL + s], 0, y, z);
                 v_issued = J + 1;
             };
+            // the bias tiles of both tile-steps of key step j (global: J)
+            auto load_b = [&](const Item& it, int J, int j) {
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int g = 2 * J + t, s = g % 3;
+                    if (ok) ok = bounded_wait_s<PRODUCER_SLEEP>(bars_s + 8 * (LY::B_EMPTY + s), ((g / 3) & 1) ^ 1, abort_s, status, 0x130 + t);
+                    if (!ok) return;
+                    uint8_t* dst = base + LY::BIAS_OFF + s * LY::BIAS_BYTES;
+                    mbar_arrive_expect_tx(&bars[LY::B_FULL + s], LY::BIAS_BYTES);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+                        tma_load_4d(dst + c * BM * 128, &tmBias, &bars[LY::B_FULL + s], j * BN + c * 64, it.row0 + t * BM,
+                                    bias_heads ? it.bh % H : 0, bias_batches ? it.bh / H : 0);
+                    b_issued = g + 1;
+                }
+            };
             int J0 = 0, q = 0;
             for (int idx = first_item<SPLIT, VL>(sc); idx < items && ok; idx = next_item<SPLIT, VL>(idx, sc)) {
-                const Item it = get_item<VL, SPLIT>(idx, sc);
+                const Item it = get_item<VL, SPLIT, BIAS>(idx, sc);
                 if (it.ntiles == 0) continue;
                 // tile of query rows r.. / of keys of step j
                 auto qy = [&](int r) { return VL ? it.head : r; };
@@ -754,15 +829,19 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 load_q(0, q, qy(it.row0), qz(it.row0));
                 if (ok) load_k(J0, ky(0), kz(0));
                 if (ok) load_q(1, q, qy(it.row0 + BM), qz(it.row0 + BM));
+                if (BIAS && ok) load_b(it, J0, 0);
                 if (ok && it.ntiles > 1) load_k(J0 + 1, ky(1), kz(1));
                 for (int j = 0; j < it.ntiles && ok; ++j) {
                     load_v(J0 + j, ky(j), kz(j));
+                    if (BIAS && ok && j + 1 < it.ntiles) load_b(it, J0 + j + 1, j + 1);
                     if (ok && j + 2 < it.ntiles) load_k(J0 + j + 2, ky(j + 2), kz(j + 2));
                 }
                 J0 += it.ntiles;
                 ++q;
             }
             if (!ok) {
+                if (BIAS)
+                    for (int g = b_issued > 3 ? b_issued - 3 : 0; g < b_issued; ++g) drain_wait(&bars[LY::B_FULL + g % 3], (g / 3) & 1);
                 for (int t = 0; t < 2; ++t)
                     if (q_loaded[t] > 0) drain_wait(&bars[LY::Q_FULL + t], (q_loaded[t] - 1) & 1);
                 for (int J = k_issued > LY::KS ? k_issued - LY::KS : 0; J < k_issued; ++J)
@@ -787,7 +866,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             if (ok) tc_fence_after();
         };
         Cursor c;
-        cursor_init<VL, SPLIT>(c, sc);
+        cursor_init<VL, SPLIT, BIAS>(c, sc);
         if (warp == LY::SOFT_WARPS + 3) {
             const uint64_t q_desc = make_smem_desc_sw128(smem_u32(Qs), 16, 1024);
             const uint64_t k_desc = make_smem_desc_sw128(smem_u32(Ks), 16, 1024);
@@ -814,7 +893,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     }
                     __syncwarp();
                 }
-                cursor_next<VL, SPLIT>(c, sc);
+                cursor_next<VL, SPLIT, BIAS>(c, sc);
             }
         } else {
             const int t = warp - LY::SOFT_WARPS - 1;
@@ -835,7 +914,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     tc_commit(&bars[LY::V_EMPTY + vs]);
                 }
                 __syncwarp();
-                cursor_next<VL, SPLIT>(c, sc);
+                cursor_next<VL, SPLIT, BIAS>(c, sc);
             }
         }
       }
@@ -851,7 +930,12 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // maxima (its partner's is BM floats away: flip bit 9; the row sums sit 4 * BM floats further)
         const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
         const uint32_t xm_own = smem_u32(xch + ((t * 2 + h) * BM + q * 32 + lane));
-        const bool neg_scale = scale_log2e < 0.f;
+        const bool neg_scale = !BIAS && scale_log2e < 0.f;
+        // (bias) the thread's row in stage 0's panel of this key half; logits are scaled as they meet the bias, so the routines
+        // below go on with scale 1
+        const uint32_t brow0 = smem_u32(base + LY::BIAS_OFF) + h * (BM * 128) + (q * 32 + lane) * 128;
+        const int rx = lane & 7;
+        const float sc1 = BIAS ? 1.f : scale_log2e;
         bool ok = true;
         int b = t;                                       // buffer of tile-step g = 2 J + t: g % 3
         int g = t;                                       // this tile's next tile-step (J: key steps of all items so far)
@@ -862,7 +946,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         float m_ref = -INFINITY;
         bool first_item_done = false;
         for (int idx = first_item<SPLIT, VL>(sc); idx < items; idx = next_item<SPLIT, VL>(idx, sc)) {
-        const Item it = get_item<VL, SPLIT>(idx, sc);
+        const Item it = get_item<VL, SPLIT, BIAS>(idx, sc);
         if (it.skip) continue;
         const int ntiles = it.ntiles;
         // keys this thread's row sees (all the item's keys unless the causal mask cuts the row short);
@@ -883,8 +967,10 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             // partner (reading TMEM that may not be ready is harmless, nothing is stored), so that the
             // two always pass the same sequence of named barriers and leave together.
             ok = bounded_wait_s(bars_s + 8 * (LY::S_FULL + t * 3 + b), xph, abort_s, status, 0x300 + t);
+            if (BIAS && ok) ok = bounded_wait_s(bars_s + 8 * (LY::B_FULL + b), static_cast<uint32_t>(g / 3) & 1u, abort_s, status, 0x340 + t);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
+            const uint32_t brow = brow0 + (BIAS ? b * LY::BIAS_BYTES : 0);
             const int col0 = j * BN + h * HN;
             const bool tail = col0 + HN > nrow_min;      // (warp-uniform) some row has masked keys in this step
             const int nvalid = nrow > col0 ? (nrow - col0 < HN ? nrow - col0 : HN) : 0;   // per row
@@ -903,21 +989,25 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 tmem_ld_x32(s_addr, r);
                 tc_wait_ld();
                 if (tail) {
-                    exp_pack32<true, false>(r, scale_log2e, -m_ref, nvalid, ls, pk[0]);
+                    if (BIAS) add_bias32<0>(r, scale_log2e, brow, rx);
+                    exp_pack32<true, false>(r, sc1, -m_ref, nvalid, ls, pk[0]);
                     tmem_ld_x32(s_addr + 32, r);
                     tc_wait_ld();
-                    exp_pack32<true, false>(r, scale_log2e, -m_ref, nvalid - 32, ls, pk[1]);
+                    if (BIAS) add_bias32<4>(r, scale_log2e, brow, rx);
+                    exp_pack32<true, false>(r, sc1, -m_ref, nvalid - 32, ls, pk[1]);
                     lt = (ls[0] + ls[1]) + (ls[2] + ls[3]);
                 } else {
                     const uint64_t scale2 = pack2(scale_log2e, scale_log2e), neg_m2 = pack2(-m_ref, -m_ref);
                     uint64_t l2[2] = {0ull, 0ull};
                     uint64_t x2[16];
                     float xmax = 0.f;
-                    scale32(r, scale2, neg_m2, x2);
+                    if (BIAS) scale_bias32<0>(r, scale2, neg_m2, brow, rx, x2);
+                    else      scale32(r, scale2, neg_m2, x2);
                     tmem_ld_x32(s_addr + 32, r);         // the second 32 logits arrive during the first 32 exponentials
                     exp_pack_x2<USE_POLY, SPLIT ? POLY_PAIRS_SA : POLY_PAIRS_A>(x2, l2, xmax, pk[0]);
                     tc_wait_ld();
-                    scale32(r, scale2, neg_m2, x2);
+                    if (BIAS) scale_bias32<4>(r, scale2, neg_m2, brow, rx, x2);
+                    else      scale32(r, scale2, neg_m2, x2);
                     exp_pack_x2<USE_POLY, SPLIT ? POLY_PAIRS_SB : POLY_PAIRS_B>(x2, l2, xmax, pk[1]);
                     float a, b2, c, d2;
                     unpack2(l2[0], a, b2);
@@ -939,12 +1029,16 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     tmem_ld_x32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
                     tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
                     tc_wait_ld();
+                    if (BIAS) {
+                        add_bias32<0>(*reinterpret_cast<uint32_t(*)[32]>(&s[0]), scale_log2e, brow, rx);
+                        add_bias32<4>(*reinterpret_cast<uint32_t(*)[32]>(&s[32]), scale_log2e, brow, rx);
+                    }
                     if (tail) {
                         const uint32_t excl = __float_as_uint(neg_scale ? INFINITY : -INFINITY);
 #pragma unroll
                         for (int i = 0; i < HN; ++i) if (i >= nvalid) s[i] = excl;
                     }
-                    if (nvalid > 0) mx = (neg_scale ? half_min(s) : half_max(s)) * scale_log2e;
+                    if (nvalid > 0) mx = (neg_scale ? half_min(s) : half_max(s)) * sc1;
                 }
                 st_shared_f32(xm_own, mx);
                 pair_sync(pair_id);
@@ -980,13 +1074,15 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 // the logits are read again, 32 at a time; with the fresh maximum every argument is <= 0,
                 // so the ordinary routine (polynomial lanes included) applies unless part of the half is masked
                 ls[0] = ls[1] = ls[2] = ls[3] = 0.f;
-                if (tail) {
+                if (tail || BIAS) {
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t r[32];
                         tmem_ld_x32(s_addr + c * 32, r);
                         tc_wait_ld();
-                        exp_pack32<true, false>(r, scale_log2e, -m_ref, nvalid - c * 32, ls, pk[c]);
+                        if (BIAS) { if (c == 0) add_bias32<0>(r, scale_log2e, brow, rx); else add_bias32<4>(r, scale_log2e, brow, rx); }
+                        // (every pair so far switched off by the bias: 0 stands in for the reference, the weights are 2^-inf)
+                        exp_pack32<true, false>(r, sc1, BIAS && m_ref == -INFINITY ? 0.f : -m_ref, nvalid - c * 32, ls, pk[c]);
                     }
                 } else {
                     const uint64_t scale2 = pack2(scale_log2e, scale_log2e), neg_m2 = pack2(-m_ref, -m_ref);
@@ -1011,6 +1107,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             // careful path waits for anything)
             if (careful && pair_any(pair_id, !ok)) ok = false;
             if (!ok) break;
+            if (BIAS && lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + b));   // (behind the vote, which both warps' reads precede)
             tmem_st_x16(s_addr, pk[0]);
             tmem_st_x16(s_addr + 16, pk[1]);
             l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
@@ -1259,7 +1356,7 @@ int launch_tc3(const Problem& p, cudaStream_t st) {
         kern, grid, LY::SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, static_cast<int>(slots), slabs,
         p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
         (reinterpret_cast<uintptr_t>(p.O) & 31) == 0 ? 1 : 0, paired, static_cast<const int32_t*>(nullptr),
-        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{});
+        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{}, CUtensorMap{}, 0, 0);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
@@ -1299,7 +1396,32 @@ int launch_fused_tc3_varlen(const void* Q, const void* K, const void* V, void* O
     const cudaError_t e = launch_pdl(
         fused_tc3_kernel<true>, grid, LY::VL_SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, num_seqs,
         static_cast<int>(most), slabs, scale * 1.4426950408889634f, static_cast<const int32_t*>(nullptr), causal ? 0 : (1 << 30), status,
-        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, sorted ? 1 : 0, cu_q, cu_k, static_cast<float*>(nullptr), ed);
+        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, sorted ? 1 : 0, cu_q, cu_k, static_cast<float*>(nullptr), ed, CUtensorMap{}, 0, 0);
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
+// The same kernel with a bf16 bias, whose tensor map ({Nk, Nq, heads, batches}, boxes of 64 x 128) the caller has made.
+int launch_fused_tc3_bias(const Problem& p, const void* bias_map, cudaStream_t st) {
+    using LY = Layout<true>;
+    CUtensorMap tmQ, tmK, tmV;
+    const int BH = p.B * p.H;
+    if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map(&tmK, p.K, BH, p.Nk, D, BN) || !make_map(&tmV, p.V, BH, p.Nk, D, BN))
+        return FLAT_ERR_CUDA;
+    if (!(p.lse ? ensure_dynamic_smem<fused_tc3_kernel<false, true, false, true>>(LY::SMEM_BYTES)
+                : ensure_dynamic_smem<fused_tc3_kernel<false, false, false, true>>(LY::SMEM_BYTES)))
+        return FLAT_ERR_CUDA;
+    const int slabs = (p.Nq + 2 * BM - 1) / (2 * BM), sms = device_sm_count();
+    const int64_t items = static_cast<int64_t>(slabs) * BH;
+    const bool persistent = items >= (p.k_valid_len ? 8 : 2) * static_cast<int64_t>(sms);      // (as launch_tc3)
+    const int paired = persistent && p.causal ? 1 : 0;
+    const int64_t slots = paired ? static_cast<int64_t>((slabs + 1) & ~1) * BH : items;
+    if (slots > 0x7fffffff) return FLAT_ERR_SHAPE;
+    const cudaError_t e = launch_pdl(
+        p.lse ? fused_tc3_kernel<false, true, false, true> : fused_tc3_kernel<false, false, false, true>,
+        static_cast<int>(persistent ? sms : items), LY::SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk,
+        static_cast<int>(slots), slabs, p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
+        (reinterpret_cast<uintptr_t>(p.O) & 31) == 0 ? 1 : 0, paired, static_cast<const int32_t*>(nullptr),
+        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{}, *static_cast<const CUtensorMap*>(bias_map), p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
