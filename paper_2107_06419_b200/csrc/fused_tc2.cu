@@ -172,14 +172,13 @@ __device__ __forceinline__ float exp_store(const uint32_t (&s)[128], float scale
     return (l0 + l1) + (l2 + l3);
 }
 
-// s = s * scale * log2(e) + bias * log2(e) for a row of 128 logits whose `count` first bias values of ES bytes lie at `p`, at any
+// s = s * scale * log2(e) + bias * log2(e) for a row of 128 logits whose `count` first bf16 bias values lie at `p`, at any
 // alignment.  Pieces of 16 bytes that reach beyond the tensor are put together value by value.
-template <int ES>
 __device__ __forceinline__ void add_bias_row(uint32_t (&s)[128], float scale_log2e, const char* p, int count, const BiasArg& bias) {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p), g0 = a & ~uintptr_t(15), end = a + static_cast<uintptr_t>(count) * ES;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), g0 = a & ~uintptr_t(15), end = a + static_cast<uintptr_t>(count) * 2;
     const uintptr_t lo = reinterpret_cast<uintptr_t>(bias.p), hi = lo + bias.bytes;
     const int words = static_cast<int>(a - g0) >> 2, bits = static_cast<int>(a & 2) * 8;
-    auto piece = [&](int k, uint32_t (&w)[4]) {
+    auto piece = [&](int k, uint32_t* w) {
         const uintptr_t g = g0 + 16 * k;
         w[0] = w[1] = w[2] = w[3] = 0u;
         if (g >= end) return;                            // (behind the row's values)
@@ -188,41 +187,27 @@ __device__ __forceinline__ void add_bias_row(uint32_t (&s)[128], float scale_log
             w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
         } else {
 #pragma unroll
-            for (int e = 0; e < 16 / ES; ++e) {
-                const uintptr_t x = g + e * ES;
-                if (x < lo || x + ES > hi) continue;
-                if (ES == 4) w[e] = *reinterpret_cast<const uint32_t*>(x);
-                else         w[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(x)) << (16 * (e & 1));
+            for (int e = 0; e < 8; ++e) {
+                const uintptr_t x = g + e * 2;
+                if (x >= lo && x + 2 <= hi) w[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(x)) << (16 * (e & 1));
             }
         }
     };
-    constexpr int PER = 16 / ES;                         // values per piece
     uint32_t w[8];
-    {
-        uint32_t f[4];
-        piece(0, f);
+    piece(0, w);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = f[i];
-    }
-#pragma unroll
-    for (int k = 0; k < 128 / PER; ++k) {
-        uint32_t f[4], t[6];
-        piece(k + 1, f);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[4 + i] = f[i];
+    for (int k = 0; k < 16; ++k) {
+        uint32_t t[6];
+        piece(k + 1, w + 4);
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = (words & 2) ? w[i + 2] : w[i];
 #pragma unroll
         for (int i = 0; i < 5; ++i) t[i] = (words & 1) ? t[i + 1] : t[i];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            if (ES == 4) {
-                s[k * 4 + i] = __float_as_uint(fmaf(__uint_as_float(s[k * 4 + i]), scale_log2e, __uint_as_float(t[i]) * 1.4426950408889634f));
-            } else {
-                const uint32_t b = __funnelshift_r(t[i], t[i + 1], bits);
-                s[k * 8 + 2 * i] = __float_as_uint(fmaf(__uint_as_float(s[k * 8 + 2 * i]), scale_log2e, __uint_as_float(b << 16) * 1.4426950408889634f));
-                s[k * 8 + 2 * i + 1] = __float_as_uint(fmaf(__uint_as_float(s[k * 8 + 2 * i + 1]), scale_log2e, __uint_as_float(b & 0xffff0000u) * 1.4426950408889634f));
-            }
+            const uint32_t b = __funnelshift_r(t[i], t[i + 1], bits);
+            s[k * 8 + 2 * i] = __float_as_uint(fmaf(__uint_as_float(s[k * 8 + 2 * i]), scale_log2e, __uint_as_float(b << 16) * 1.4426950408889634f));
+            s[k * 8 + 2 * i + 1] = __float_as_uint(fmaf(__uint_as_float(s[k * 8 + 2 * i + 1]), scale_log2e, __uint_as_float(b & 0xffff0000u) * 1.4426950408889634f));
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) w[i] = w[4 + i];
@@ -575,10 +560,18 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                             s[c * 16 + i] = __float_as_uint(fmaf(__uint_as_float(s[c * 16 + i]), scale_log2e, bv[i] * 1.4426950408889634f));
                     }
                 } else if (in_rows) {
-                    // Rows that begin anywhere: aligned 16-byte pieces, two neighbours at a time, shifted into place (value by
-                    // value the 128 loads of 32 rows each were 33,000 cycles a step of the load unit: @@UN@@).
-                    if (bias.f32) add_bias_row<4>(s, scale_log2e, static_cast<const char*>(bias.p) + at * 4, min(BN, Nk - col0), bias);
-                    else          add_bias_row<2>(s, scale_log2e, static_cast<const char*>(bias.p) + at * 2, min(BN, Nk - col0), bias);
+                    // Rows that begin anywhere.  bf16: aligned 16-byte pieces, two neighbours at a time, shifted into place
+                    // (B8 H16 1001 x 1001: 257 us, 346 value by value; d = 128 334 and 416; staged word by word by one warp 657); fp32: value
+                    // by value (487 us against 576).
+                    const int count = Nk - col0 < BN ? Nk - col0 : BN;
+                    if (bias.f32) {
+#pragma unroll                                           // (fully: the logits must stay in registers)
+                        for (int i = 0; i < 128; ++i)
+                            s[i] = __float_as_uint(fmaf(__uint_as_float(s[i]), scale_log2e,
+                                                        (i < count ? static_cast<const float*>(bias.p)[at + i] : 0.f) * 1.4426950408889634f));
+                    } else {
+                        add_bias_row(s, scale_log2e, static_cast<const char*>(bias.p) + at * 2, count, bias);
+                    }
                 } else {
 #pragma unroll
                     for (int i = 0; i < 128; ++i) s[i] = __float_as_uint(__uint_as_float(s[i]) * scale_log2e);
@@ -843,12 +836,10 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
     }
     if (p.bias) {
         if constexpr (NT == 2 && D == 64) {
-            // bf16 bias with 16-byte aligned rows: tiles staged through shared memory by TMA
+            // bf16 bias with 16-byte aligned rows: the half-row kernel, tiles staged through shared memory by TMA
             const BiasArg ba = bias_arg(p);
             CUtensorMap tmB;
-            if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) {
-                return launch_fused_tc3_bias(p, &tmB, st);
-            }
+            if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) return launch_fused_tc3_bias(p, &tmB, st);
         }
         if constexpr (NT == 2) {
             if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
