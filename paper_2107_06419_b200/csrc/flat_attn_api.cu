@@ -115,13 +115,9 @@ int run_fused(const flat::Problem& q, int variant, cudaStream_t st) {
                 v = ((2 * ctas2 >= sms && q.Nk > 1024) || (ctas2 >= 2 * sms && !q.k_valid_len && slabs_fill))
                         ? FLAT_VARIANT_TC3 : FLAT_VARIANT_TC2_SINGLE;
             }
-            // d = 128: the two-tile kernel (lazy reference maximum, polynomial exp2, packed arithmetic)
-            // is ahead of its single-tile predecessor even when it leaves SMs empty (B2 H8 2048 keys:
-            // 0.037 against 0.096 ms); only tiny problems (256 keys or fewer, less than one CTA per SM)
-            // are at par or a few per cent better on the 128-row CTAs.
-            else           v = (ctas2 >= sms || q.Nk > 256) ? FLAT_VARIANT_TC2 : FLAT_VARIANT_TC;
-            // (the single-tile predecessor kernel has no causal mask and does not write lse)
-            if ((q.causal || q.lse) && v == FLAT_VARIANT_TC) v = FLAT_VARIANT_TC2;
+            // d = 128: the two-tile kernel, even when it leaves SMs empty (B2 H8 2048 keys: 0.037 against 0.096 ms
+            // on its single-tile predecessor, B16 H8 256 keys: 18.4 against 26.6 us, B8 H8 128 keys: the same).
+            else           v = FLAT_VARIANT_TC2;
             // (the bias is read by the two-tile kernel with one thread per row)
             if (q.bias) v = FLAT_VARIANT_TC2;
             // (pruned attention runs on the one-tile kernel: a CTA walks the list of its query tile's kept key tiles)
@@ -450,7 +446,7 @@ int flat_attn_varlen_fwd(const void* Q, const void* K, const void* V, void* O, c
     if ((reinterpret_cast<uintptr_t>(cu_seqlens_q) & 3u) || (reinterpret_cast<uintptr_t>(cu_seqlens_k) & 3u) ||
         (status && (reinterpret_cast<uintptr_t>(status) & 3u)))
         return FLAT_ERR_ALIGN;
-    const int r = (d == 64 ? flat::launch_fused_tc3_varlen : flat::launch_fused_tc2_varlen)(
+    const int r = (d == 64 ? flat::launch_fused_tc3_varlen : flat::launch_fused_d128_varlen)(
         Q, K, V, O, cu_seqlens_q, cu_seqlens_k, num_seqs, H, total_q, total_k, max_seqlen_q, scale, causal,
         status_or_library_word(status),
         static_cast<cudaStream_t>(stream));

@@ -68,6 +68,7 @@ int check_params(const flat_attn_params_t* p);
 int launch_fused_simt(const Problem& p, cudaStream_t st);
 int launch_naive(const Problem& p, void* L, void* A, cudaStream_t st);
 int launch_fused_tc(const Problem& p, cudaStream_t st);
+int launch_fused_d128(const Problem& p, cudaStream_t st);    // (bf16, d = 128, no bias, no pruning map)
 int launch_fused_tc2(const Problem& p, cudaStream_t st);      // (also the tensor-core kernel for calls with a bias)
 // (only_if_resident: sixteen-CTA clusters only when all clusters of the launch can run at the same time; else
 // FLAT_ERR_UNSUPPORTED)
@@ -86,8 +87,8 @@ bool small_applies(const Problem& p);              // bf16, d in {16, 32}, no bi
 int launch_fused_small(const Problem& p, cudaStream_t st);
 bool rgran_applies(const Problem& p);              // bf16, d = 64, Nk <= 512
 int launch_fused_rgran(const Problem& p, cudaStream_t st);
-// Packed variable-length batches (bf16; fused_tc3: d = 64, fused_tc2: d = 128): Q, O [total_q, H, d], K, V [total_k, H, d].
-int launch_fused_tc2_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q,
+// Packed variable-length batches (bf16; fused_tc3: d = 64, fused_d128: d = 128): Q, O [total_q, H, d], K, V [total_k, H, d].
+int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q,
                             const int32_t* cu_k, int num_seqs, int H, int64_t total_q, int64_t total_k,
                             int max_seqlen_q, float scale, int causal, int32_t* status, cudaStream_t st);
 int launch_fused_tc3_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q,

@@ -1,0 +1,421 @@
+// Fused Logit-Softmax-Attend for d = 128 (bf16 in, fp32 accumulate, bf16 out): two query tiles of 128 rows per CTA, keys in
+// steps of 64 with the logits of the step after next computed ahead.
+//
+// Paper mapping (Section 5, 5.1, 5.2): shared outer loops = (batch, head) and a slab of 256 query rows (R-granularity);
+// Logit and Attend interleaved over the key steps with the streaming softmax between them (a reference maximum and a
+// running sum replace the paper's full-row slice on chip; same function).
+//
+// What bounds it: the tensor pipe.  The two outputs take 256 of TMEM's 512 columns, so there is room for 256 columns of
+// logits.  With one 128-key tile per query tile in them (fused_tc2_kernel), the weights have to overlay the logits and a
+// tile's chain runs in series -- softmax, O += P V, next logits, 3,800 cycles of which the pipe works 2 x 1024 for both
+// tiles.  With steps of 64 keys every query tile has TWO logit buffers: S(j + 1) is there when softmax(j) is done, and
+// O += P(j) V and S(j + 2), which takes P(j)'s columns, have a whole softmax step to run in.  The price is that a
+// logit MMA of N = 64 with both operands in shared memory takes 48 cycles where its arithmetic takes 32 (A alone is 4 KB of
+// a port of 128 bytes a cycle): 1280 cycles of the pipe per 64 keys of both tiles, against 1024.
+// Measured, against fused_tc2_kernel on the same GPU (us): B4 H16 4096^2 460 -> 428, causal 347 -> 256; H8 64K causal 7,780 ->
+// 6,380 (1,380 TFLOP/s; a cuBLAS GEMM of 8192^3 reaches 1,650 in a burst, 1,395 sustained); B2 H16 3000 causal 120 -> 97; B32
+// H16 512^2 110 -> 106.  The causal gain is also the order: the longest slabs first, so that short ones are left at the end.
+//
+// CTA = 384 threads: warps 0-3 / 4-7 softmax of tile A / B (thread = row = TMEM lane), warp 8 TMA producer, warps 9 / 10 MMA
+// issuers of tile A / B (one elected lane), warp 11 idle (it completes the warpgroup for the register hand-over).
+// TMEM columns: S(t, b) 128 t + 64 b (b = step parity), P over the first 32 of them, O_t 256 + 128 t.
+// The softmax takes no row maximum after the first step: any reference gives the exact softmax, and a step whose row sum
+// passes 2^40 is redone with a fresh maximum.  One exponential in four goes through a polynomial on the FMA pipe.
+// VL: packed batches (Q, O [total_q, H, d], K, V [total_k, H, d]), a CTA per (sequence, head, slab of the longest sequence).
+// Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "flat_internal.cuh"
+#include "ptx_sm100.cuh"
+#include "tc_common.cuh"
+
+namespace flat {
+
+using namespace ptx;
+using namespace tc;
+
+namespace {
+
+constexpr int D = 128;
+constexpr int BM = 128;              // rows per query tile (two tiles per CTA)
+constexpr int BN = 64;               // keys per step
+constexpr int KS = 5, VS = 5;        // ring depths
+constexpr int THREADS = 384;
+constexpr int POLY_LANE = 3;         // element index mod 4 that takes the polynomial (none: B4 H16 4096 keys 450 us against 428)
+constexpr float OVERFLOW_SUM = 1.0995116e12f;   // 2^40
+
+constexpr int Q_BYTES = BM * D * 2, KV_BYTES = BN * D * 2;
+constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES;
+constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
+static_assert(SMEM_BYTES <= 232448, "shared memory");
+__host__ __device__ constexpr uint32_t S_COL(int t, int b) { return 128u * t + 64u * b; }
+__host__ __device__ constexpr uint32_t O_COL(int t) { return 256u + 128u * t; }
+// barriers: S_FULL / P_FULL / PV_DONE [tile][step parity], each once every second step.  (One PV_DONE a tile is not enough: a warp
+// ahead of the others of its tile has its last logits when O += P V of the third last step is done, and would take that one's
+// parity for the last one's.)
+constexpr int Q_FULL = 0, K_FULL = 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS,
+              P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, NUM_BARS = PV_DONE + 4;
+
+// p_i = 2^(s_i * scale + neg_m) of 64 logits; bf16(p) to 32 TMEM columns at `p_addr`; returns the fp32 sum of the unrounded p.
+// TAIL: only the first `nvalid` take part.
+template <bool TAIL>
+__device__ __forceinline__ float exp_store(const uint32_t (&s)[BN], float scale_log2e, float neg_m, uint32_t p_addr, int nvalid) {
+    uint64_t sum0 = 0ull, sum1 = 0ull;
+    const uint64_t scale2 = pack2(scale_log2e, scale_log2e), neg_m2 = pack2(neg_m, neg_m);
+#pragma unroll
+    for (int c = 0; c < BN / 32; ++c) {
+        uint32_t pk[16];
+        float p[32];
+#pragma unroll
+        for (int i = 0; i < 32; i += 2)
+            unpack2(fma2(pack2(__uint_as_float(s[c * 32 + i]), __uint_as_float(s[c * 32 + i + 1])), scale2, neg_m2), p[i], p[i + 1]);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            p[i] = !TAIL && (i & 3) == POLY_LANE ? ex2_poly(p[i]) : ex2_approx(p[i]);
+            if (TAIL && c * 32 + i >= nvalid) p[i] = 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+            sum0 = add2(sum0, pack2(p[i], p[i + 1]));
+            sum1 = add2(sum1, pack2(p[i + 2], p[i + 3]));
+            pk[i / 2] = pack_bf16x2(p[i], p[i + 1]);
+            pk[i / 2 + 1] = pack_bf16x2(p[i + 2], p[i + 3]);
+        }
+        tmem_st_x16(p_addr + c * 16, pk);
+    }
+    float a, b, cc, d;
+    unpack2(sum0, a, b);
+    unpack2(sum1, cc, d);
+    return (a + b) + (cc + d);
+}
+
+__device__ __forceinline__ float row_extreme(const uint32_t (&s)[BN], bool smallest) {
+    float e0 = __uint_as_float(s[0]), e1 = __uint_as_float(s[1]);
+#pragma unroll
+    for (int i = 2; i < BN; i += 2) {
+        e0 = smallest ? fminf(e0, __uint_as_float(s[i])) : fmaxf(e0, __uint_as_float(s[i]));
+        e1 = smallest ? fminf(e1, __uint_as_float(s[i + 1])) : fmaxf(e1, __uint_as_float(s[i + 1]));
+    }
+    return smallest ? fminf(e0, e1) : fmaxf(e0, e1);
+}
+
+template <bool VL>
+__global__ void __launch_bounds__(THREADS, 1)
+fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                  __nv_bfloat16* __restrict__ O, int BH, int H, int Nq, int Nk, float scale_log2e, const int32_t* __restrict__ valid_len,
+                  int coff, int group, int32_t* status, const int32_t* __restrict__ cu_q, const int32_t* __restrict__ cu_k,
+                  float* __restrict__ lse) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* Qs = base;
+    uint8_t* Ks = Qs + 2 * Q_BYTES;
+    uint8_t* Vs = Ks + KS * KV_BYTES;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + TILE_BYTES);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    int bh, row0, n = Nk;
+    int head = 0, q_tok0 = 0, k_tok0 = 0, q_rows = 0;    // (packed batches only)
+    if (VL) {
+        // the slabs of a sequence side by side; under the causal mask the last slabs (the longest) of all sequences first
+        bh = group ? blockIdx.x : blockIdx.y;
+        row0 = static_cast<int>(group ? gridDim.y - 1 - blockIdx.y : blockIdx.x) * (2 * BM);
+        const int s = bh / H;
+        head = bh - s * H;
+        const int q0 = cu_q[s], ql = cu_q[s + 1] - q0, k0 = cu_k[s], kl = cu_k[s + 1] - k0;
+        if (row0 >= ql) return;                          // (the whole CTA: nothing is set up yet)
+        q_tok0 = q0 + row0; k_tok0 = k0; q_rows = ql - row0;
+        n = kl < 0 ? 0 : kl;
+        if (coff < (1 << 29)) coff = kl - ql;
+    } else {
+        // `group` heads at a time, their slabs side by side, the longest first under the causal mask
+        const int slabs = (Nq + 2 * BM - 1) / (2 * BM), per = group * slabs, first = static_cast<int>(blockIdx.x) / per * group;
+        const int heads = BH - first < group ? BH - first : group, at = static_cast<int>(blockIdx.x) % per;
+        bh = first + at % heads;
+        row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * (2 * BM);
+    }
+
+    if (threadIdx.x == 256) {
+        for (int i = 0; i < NUM_BARS; ++i)
+            mbar_init(&bars[i], i >= P_FULL && i < PV_DONE ? 4 : (i >= K_EMPTY && i < V_FULL) || (i >= V_EMPTY && i < S_FULL) ? 2 : 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    // (launched with programmatic stream serialization, packed batches aside: this set-up overlaps the tail of the previous
+    // kernel of the stream, and nothing in device memory is touched before that one has finished)
+    if (!VL) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
+    }
+    const uint32_t tmem = *tmem_slot;
+    {
+        // Causal mask (coff = Nk - Nq; 2^30 = none): row r sees keys j < r + 1 + coff, so the last row bounds the CTA's keys
+        const long long lim = static_cast<long long>(row0) + 2 * BM + coff;
+        if (lim < n) n = lim < 0 ? 0 : static_cast<int>(lim);
+    }
+    const int nsteps = (n + BN - 1) / BN;
+    const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
+
+    if (warp >= 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (warp == 8) {
+            // ------------------------------------------------------------ TMA producer
+            if (lane == 0 && nsteps > 0) {
+                prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
+                bool ok = true;
+                int k_issued = 0, v_issued = 0;
+                auto load_q = [&](int t) {
+                    mbar_arrive_expect_tx(&bars[Q_FULL + t], Q_BYTES);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+                        tma_load_3d(Qs + t * Q_BYTES + c * BM * 128, &tmQ, &bars[Q_FULL + t], c * 64, VL ? head : row0 + t * BM, VL ? q_tok0 + t * BM : bh);
+                };
+                auto load_k = [&](int j) {
+                    const int s = j % KS;
+                    ok = bounded_wait_s(bars_s + 8 * (K_EMPTY + s), ((j / KS) & 1) ^ 1, abort_s, status, 0xa00 + s);
+                    if (!ok) return;
+                    mbar_arrive_expect_tx(&bars[K_FULL + s], KV_BYTES);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+                        tma_load_3d(Ks + s * KV_BYTES + c * BN * 128, &tmK, &bars[K_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
+                    k_issued = j + 1;
+                };
+                auto load_v = [&](int j) {
+                    const int s = j % VS;
+                    ok = bounded_wait_s(bars_s + 8 * (V_EMPTY + s), ((j / VS) & 1) ^ 1, abort_s, status, 0xa10 + s);
+                    if (!ok) return;
+                    mbar_arrive_expect_tx(&bars[V_FULL + s], KV_BYTES);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+                        tma_load_3d(Vs + s * KV_BYTES + c * BN * 128, &tmV, &bars[V_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
+                    v_issued = j + 1;
+                };
+                load_q(0);
+                load_k(0);
+                load_q(1);
+                if (nsteps > 1) load_k(1);
+                for (int j = 0; j < nsteps && ok; ++j) {
+                    load_v(j);
+                    if (ok && j + 2 < nsteps) load_k(j + 2);
+                }
+                if (!ok) {
+                    drain_wait(&bars[Q_FULL], 0);
+                    drain_wait(&bars[Q_FULL + 1], 0);
+                    for (int j = k_issued > KS ? k_issued - KS : 0; j < k_issued; ++j) drain_wait(&bars[K_FULL + j % KS], (j / KS) & 1);
+                    for (int j = v_issued > VS ? v_issued - VS : 0; j < v_issued; ++j) drain_wait(&bars[V_FULL + j % VS], (j / VS) & 1);
+                }
+            }
+        } else if (warp <= 10) {
+            // ------------------------------------------------------------ MMA issuer of tile t (whole warp walks, one lane issues)
+            const int t = warp - 9;
+            if (nsteps > 0) {
+                constexpr uint32_t IDESC_S = make_idesc_bf16(BM, BN, 0, 0), IDESC_PV = make_idesc_bf16(BM, D, 0, 1);
+                const uint64_t q_desc = make_smem_desc_sw128(smem_u32(Qs) + t * Q_BYTES, 16, 1024);
+                const uint64_t k_desc = make_smem_desc_sw128(smem_u32(Ks), 16, 1024);
+                const uint64_t v_desc = make_smem_desc_sw128(smem_u32(Vs), BN * 128, 1024);
+                bool ok = true;
+                auto wait = [&](int bar, uint32_t parity, int code) {
+                    if (ok) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * bar, parity, abort_s, status, code));
+                };
+                auto issue_s = [&](int j) {              // S_t(j) = Q_t K_j^T, then release the K stage
+                    const uint64_t kd = k_desc + static_cast<uint64_t>(((j % KS) * KV_BYTES) >> 4);
+#pragma unroll
+                    for (int k = 0; k < D / 16; ++k)
+                        mma_ss(tmem + S_COL(t, j & 1), q_desc + static_cast<uint64_t>(((k / 4) * (BM * 128) + (k % 4) * 32) >> 4),
+                               kd + static_cast<uint64_t>(((k / 4) * (BN * 128) + (k % 4) * 32) >> 4), IDESC_S, k > 0);
+                    tc_commit(&bars[S_FULL + 2 * t + (j & 1)]);
+                    tc_commit(&bars[K_EMPTY + j % KS]);
+                };
+                auto issue_pv = [&](int j) {             // O_t += P_t(j) V_j, then release the V stage
+                    const uint64_t vd = v_desc + static_cast<uint64_t>(((j % VS) * KV_BYTES) >> 4);
+#pragma unroll
+                    for (int k = 0; k < BN / 16; ++k)
+                        mma_ts(tmem + O_COL(t), tmem + S_COL(t, j & 1) + k * 8, vd + static_cast<uint64_t>((k * 2048) >> 4), IDESC_PV, (j > 0 || k > 0));
+                    tc_commit(&bars[PV_DONE + 2 * t + (j & 1)]);
+                    tc_commit(&bars[V_EMPTY + j % VS]);
+                };
+                wait(Q_FULL + t, 0, 0xa20);
+                for (int j = 0; j < 2 && j < nsteps; ++j) {
+                    wait(K_FULL + j, 0, 0xa21);
+                    tc_fence_after();
+                    if (ok && elect_one()) issue_s(j);
+                    __syncwarp();
+                }
+                for (int j = 0; j < nsteps && ok; ++j) {
+                    const bool more = j + 2 < nsteps;
+                    wait(V_FULL + j % VS, (j / VS) & 1, 0xa22);
+                    if (more) wait(K_FULL + (j + 2) % KS, ((j + 2) / KS) & 1, 0xa23);
+                    wait(P_FULL + 2 * t + (j & 1), (j >> 1) & 1, 0xa24);
+                    if (!ok) break;
+                    tc_fence_after();
+                    // (S(j + 2) overwrites P(j): it goes behind the MMAs that read it)
+                    if (elect_one()) { issue_pv(j); if (more) issue_s(j + 2); }
+                    __syncwarp();
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ softmax + epilogue (warps 0-7)
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        const int t = warp >> 2;
+        const int row = row0 + t * BM + (warp & 3) * 32 + lane;
+        const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const uint32_t my_bars = bars_s + 8 * (S_FULL + 2 * t);       // S_FULL of the tile; P_FULL and PV_DONE 32 and 64 bytes on
+        const bool neg_scale = scale_log2e < 0.f;
+        float m_ref = -INFINITY, l = 0.f;
+        bool ok = true;
+        const long long rlim = static_cast<long long>(row) + 1 + coff;
+        const int nrow = rlim < n ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : n;
+        const int nrow_min = __shfl_sync(0xffffffffu, nrow, 0);
+        for (int j = 0; j < nsteps; ++j) {
+            const uint32_t s_addr = tl + S_COL(t, j & 1);
+            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 8 * (j & 1), (j >> 1) & 1, abort_s, status, 0xa30 + t));
+            if (!ok) break;
+            tc_fence_after();
+            uint32_t s[BN];
+            tmem_ld_x32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+            tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+            tc_wait_ld();
+            const int col0 = j * BN;
+            const bool tail = col0 + BN > nrow_min;      // (warp-uniform) some row has masked keys in this step
+            const int nvalid = nrow > col0 ? (nrow - col0 < BN ? nrow - col0 : BN) : 0;
+            if (tail) {
+                const uint32_t excl = __float_as_uint(neg_scale ? INFINITY : -INFINITY);
+#pragma unroll
+                for (int i = 0; i < BN; ++i) if (i >= nvalid) s[i] = excl;
+            }
+            bool careful = j == 0 || tail;
+            float lt = 0.f;
+            if (!careful) {
+                lt = exp_store<false>(s, scale_log2e, -m_ref, s_addr, BN);
+                careful = __any_sync(0xffffffffu, !(lt <= OVERFLOW_SUM));
+                if (careful) {           // (the weights went over the first half of the logits only: 32 registers less to keep)
+                    tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+                    tc_wait_ld();
+                }
+            }
+            if (careful) {
+                const float mx = nvalid > 0 ? row_extreme(s, neg_scale) * scale_log2e : -INFINITY;
+                if (__any_sync(0xffffffffu, mx > m_ref + RESCALE_THRESHOLD)) {
+                    const float m_new = fmaxf(m_ref, mx);
+                    const float alpha = m_new == -INFINITY ? 1.f : ex2_approx(m_ref - m_new);   // 0 on the row's first keys
+                    l *= alpha;
+                    if (j > 0) {
+                        ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((j - 1) & 1), ((j - 1) >> 1) & 1, abort_s, status, 0xa32 + t));
+                        if (!ok) break;
+                        tc_fence_after();
+#pragma unroll 1                          // (rare; unrolled, its registers made the common path spill: 428 -> 482 us)
+                        for (int c = 0; c < D / 16; ++c) {
+                            uint32_t r[16];
+                            tmem_ld_x16(tl + O_COL(t) + c * 16, r);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+                            tmem_st_x16(tl + O_COL(t) + c * 16, r);
+                        }
+                    }
+                    m_ref = m_new;
+                }
+                lt = exp_store<true>(s, scale_log2e, m_ref == -INFINITY ? 0.f : -m_ref, s_addr, nvalid);
+            }
+            l += lt;
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_s(my_bars + 32 + 8 * (j & 1));
+        }
+        if (ok && nsteps > 0)
+            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((nsteps - 1) & 1), ((nsteps - 1) >> 1) & 1, abort_s, status, 0xa34 + t));
+        if (ok) {
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            if (!VL && lse && row < Nq)
+                lse[static_cast<int64_t>(bh) * Nq + row] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
+            tc_fence_after();
+            __nv_bfloat16* orow = VL ? O + ((static_cast<int64_t>(q_tok0) + (row - row0)) * H + head) * D
+                                     : O + (static_cast<int64_t>(bh) * Nq + row) * D;
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t r[32];
+                if (nsteps > 0) {
+                    tmem_ld_x32(tl + O_COL(t) + c * 32, r);
+                    tc_wait_ld();
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) r[i] = 0u;      // no valid key: O = 0
+                }
+                if (VL ? row - row0 < q_rows : row < Nq) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        uint4 w;
+                        w.x = pack_bf16x2(__uint_as_float(r[8 * v + 0]) * inv, __uint_as_float(r[8 * v + 1]) * inv);
+                        w.y = pack_bf16x2(__uint_as_float(r[8 * v + 2]) * inv, __uint_as_float(r[8 * v + 3]) * inv);
+                        w.z = pack_bf16x2(__uint_as_float(r[8 * v + 4]) * inv, __uint_as_float(r[8 * v + 5]) * inv);
+                        w.w = pack_bf16x2(__uint_as_float(r[8 * v + 6]) * inv, __uint_as_float(r[8 * v + 7]) * inv);
+                        *reinterpret_cast<uint4*>(orow + c * 32 + v * 8) = w;
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+}  // namespace
+
+int launch_fused_d128(const Problem& p, cudaStream_t st) {
+    if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || p.bias || p.block_mask) return FLAT_ERR_UNSUPPORTED;
+    CUtensorMap tmQ, tmK, tmV;
+    const int BH = p.B * p.H, slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
+    if (static_cast<int64_t>(slabs) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
+    if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map(&tmK, p.K, BH, p.Nk, D, BN) || !make_map(&tmV, p.V, BH, p.Nk, D, BN))
+        return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<false>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
+    // without the causal mask the slabs of a head run side by side and share K and V in L2; with it, those of as many heads as
+    // fit L2 together (48 MB of K and V) go longest first: what is left at the end are the short ones
+    const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 4);
+    const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(slabs) * BH);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
+                                             p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status,
+                                             static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse);
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
+int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q, const int32_t* cu_k, int num_seqs,
+                             int H, int64_t total_q, int64_t total_k, int max_seqlen_q, float scale, int causal, int32_t* status,
+                             cudaStream_t st) {
+    if (static_cast<int64_t>(num_seqs) * H > 65535) return FLAT_ERR_SHAPE;      // (grid y)
+    CUtensorMap tmQ, tmK, tmV;
+    if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
+        !make_map_packed(&tmV, V, total_k, H, D, BN))
+        return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<true>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
+    const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535;
+    const dim3 grid(group ? num_seqs * H : slabs, group ? slabs : num_seqs * H);
+    fused_d128_kernel<true><<<grid, THREADS, SMEM_BYTES, st>>>(
+        tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), num_seqs * H, H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
+        causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr);
+    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
+}  // namespace flat

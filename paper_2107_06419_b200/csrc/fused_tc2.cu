@@ -214,11 +214,6 @@ __device__ __forceinline__ void add_bias_row(uint32_t (&s)[128], float scale_log
     }
 }
 
-// VL: packed variable-length batches.  Q, O are [total_q, H, d], K, V [total_k, H, d]; sequence s owns
-// tokens cu_q[s] .. cu_q[s+1] - 1 of Q and cu_k[s] .. cu_k[s+1] - 1 of K, V; the tensor maps view the
-// packed tensors as {d, H, tokens}; blockIdx.y = sequence * H + head, blockIdx.x = slab of the
-// sequence's rows (a CTA past the end of its sequence leaves at once); the causal offset is that of
-// the sequence; valid_len is unused.
 // BIAS: a separate instantiation that adds a bias tensor to the scaled logits (dense batches): the softmax
 // thread fetches its row's 128 values of the step straight from device memory -- a bf16 bias adds
 // 2 B H Nq Nk bytes of traffic, four times |Q|+|K|+|V|+|O| on a 4096 x 4096, d = 64 problem.
@@ -238,18 +233,17 @@ __device__ __forceinline__ void add_bias_row(uint32_t (&s)[128], float scale_log
 // query rows, each with its own running (m_ref, l, O); at the end the second warpgroup leaves its rows in shared
 // memory and the first merges them (the split-softmax identity again) before the ordinary epilogue or the cluster
 // exchange.  The chain is half as long and two warps per scheduler share the exponent unit.
-template <int D, int NT, bool VL = false, bool BIAS = false, bool SPARSE = false, int CS = 1, bool KH = false>
+template <int D, int NT, bool BIAS = false, bool SPARSE = false, int CS = 1, bool KH = false>
 __global__ void __launch_bounds__(128 * NT + 128, NT == 1 ? 2 : 1)
 fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, int H, int Nq, int Nk,
                  float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int32_t* status,
-                 const int32_t* __restrict__ cu_q = nullptr, const int32_t* __restrict__ cu_k = nullptr,
-                 float* __restrict__ lse = nullptr, BiasArg bias = BiasArg{},
+                                  float* __restrict__ lse = nullptr, BiasArg bias = BiasArg{},
                  const uint8_t* __restrict__ block_mask = nullptr, long long bmask_sb = 0, long long bmask_sh = 0) {
     using LY = L2<D, NT, KH ? (CS == 16 ? 2 : 1) : 0>;
-    static_assert(!SPARSE || (NT == 1 && !VL && !BIAS), "the pruning map is read by the one-tile dense kernel");
-    static_assert(CS == 1 || ((NT == 1 || KH) && !VL && !BIAS && !SPARSE && (CS == 2 || CS == 4 || CS == 8 || CS == 16)), "key split: one-tile dense kernel");
-    static_assert(!KH || (NT == 2 && D == 64 && !VL && !BIAS && !SPARSE), "key halves: two warpgroups on one dense d = 64 tile");
+    static_assert(!SPARSE || (NT == 1 && !BIAS), "the pruning map is read by the one-tile dense kernel");
+    static_assert(CS == 1 || ((NT == 1 || KH) && !BIAS && !SPARSE && (CS == 2 || CS == 4 || CS == 8 || CS == 16)), "key split: one-tile dense kernel");
+    static_assert(!KH || (NT == 2 && D == 64 && !BIAS && !SPARSE), "key halves: two warpgroups on one dense d = 64 tile");
     constexpr int QT = KH ? 1 : NT;                      // query tiles of the CTA
     __shared__ uint16_t tile_list[SPARSE ? 1024 : 1];    // the kept key tiles of this query tile, ascending
     __shared__ int tile_count;
@@ -273,7 +267,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     // start its own set-up (griddepcontrol.launch_dependents) and wait for the previous one to finish
     // (griddepcontrol.wait) before the first access to device memory: launched with programmatic stream
     // serialization, consecutive kernels overlap one's tail with the other's prologue.
-    constexpr bool PDL = ((NT == 1 || KH) && !VL && !SPARSE && !BIAS);
+    constexpr bool PDL = ((NT == 1 || KH) && !SPARSE && !BIAS);
     auto setup = [&]() {
         if (threadIdx.x == LY::SOFT_WARPS * 32) {
             for (int i = 0; i < LY::NUM_BARS; ++i) {
@@ -295,16 +289,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     int n = Nk;
-    int head = 0, q_tok0 = 0, k_tok0 = 0, q_rows = 0;    // (packed batches only)
-    if (VL) {
-        const int s = bh / H;
-        head = bh - s * H;
-        const int q0 = cu_q[s], ql = cu_q[s + 1] - q0, k0 = cu_k[s], kl = cu_k[s + 1] - k0;
-        if (row0 >= ql) return;                          // (the whole CTA: nothing is set up yet)
-        q_tok0 = q0 + row0; k_tok0 = k0; q_rows = ql - row0;
-        n = kl < 0 ? 0 : kl;
-        if (coff < (1 << 29)) coff = kl - ql;
-    } else if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
+    if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
     {
         // Causal mask (coff = Nk - Nq; 2^30 = none): row r sees keys j < r + 1 + coff, so the CTA's
         // last row bounds the keys of all its rows.
@@ -357,8 +342,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 mbar_arrive_expect_tx(&bars[LY::K_FULL + s], LY::KV_BYTES);
 #pragma unroll
                 for (int c = 0; c < D / 64; ++c)
-                    tma_load_3d(Ks + s * LY::KV_BYTES + c * BN * 128, &tmK, &bars[LY::K_FULL + s], c * 64, VL ? head : tile_of(j) * BN,
-                                VL ? k_tok0 + j * BN : bh);
+                    tma_load_3d(Ks + s * LY::KV_BYTES + c * BN * 128, &tmK, &bars[LY::K_FULL + s], c * 64, tile_of(j) * BN, bh);
                 k_issued = j + 1;
             };
             auto load_v = [&](int j) {
@@ -368,21 +352,20 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 mbar_arrive_expect_tx(&bars[LY::V_FULL + s], LY::KV_BYTES);
 #pragma unroll
                 for (int c = 0; c < D / 64; ++c)
-                    tma_load_3d(Vs + s * LY::KV_BYTES + c * BN * 128, &tmV, &bars[LY::V_FULL + s], c * 64, VL ? head : tile_of(j) * BN,
-                                VL ? k_tok0 + j * BN : bh);
+                    tma_load_3d(Vs + s * LY::KV_BYTES + c * BN * 128, &tmV, &bars[LY::V_FULL + s], c * 64, tile_of(j) * BN, bh);
                 v_issued = j + 1;
             };
             mbar_arrive_expect_tx(&bars[LY::Q_FULL + 0], LY::Q_BYTES);
 #pragma unroll
             for (int c = 0; c < D / 64; ++c)
-                tma_load_3d(Qs + c * BM * 128, &tmQ, &bars[LY::Q_FULL + 0], c * 64, VL ? head : row0, VL ? q_tok0 : bh);
+                tma_load_3d(Qs + c * BM * 128, &tmQ, &bars[LY::Q_FULL + 0], c * 64, row0, bh);
             load_k(0);
             if (NT == 2) {
                 mbar_arrive_expect_tx(&bars[LY::Q_FULL + NT - 1], LY::Q_BYTES);
 #pragma unroll
                 for (int c = 0; c < D / 64; ++c)
                     tma_load_3d(Qs + (NT - 1) * LY::Q_BYTES + c * BM * 128, &tmQ, &bars[LY::Q_FULL + NT - 1], c * 64,
-                                VL ? head : row0 + (KH ? 0 : BM), VL ? q_tok0 + BM : bh);   // (KH: the same rows again)
+                                row0 + (KH ? 0 : BM), bh);   // (KH: the same rows again)
             }
             for (int j = 0; j < ntiles && ok; ++j) {
                 if (j + 1 < ntiles) load_k(j + 1);
@@ -761,11 +744,10 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         if (ok) {
             const float inv = l > 0.f ? 1.f / l : 0.f;
             // (dense batches only) log of the row's sum of exponentials; m_ref and the exponents are in base-2 units
-            if (!VL && lse && row < Nq)
+            if (lse && row < Nq)
                 lse[static_cast<int64_t>(bh) * Nq + row] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
             tc_fence_after();
-            __nv_bfloat16* orow = VL ? O + ((static_cast<int64_t>(q_tok0) + (row - row0)) * H + head) * D
-                                     : O + (static_cast<int64_t>(bh) * Nq + row) * D;
+            __nv_bfloat16* orow = O + (static_cast<int64_t>(bh) * Nq + row) * D;
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t r[32];
@@ -776,7 +758,7 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
                     for (int i = 0; i < 32; ++i) r[i] = 0u;      // no valid key: O = 0
                 }
-                if (VL ? row - row0 < q_rows : row < Nq) {
+                if (row < Nq) {
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
                         uint4 w;
@@ -824,10 +806,10 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
     dim3 grid((p.Nq + NT * BM - 1) / (NT * BM), BH);
     if (p.block_mask) {
         if constexpr (NT == 1) {
-            if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, false, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
-            fused_tc2_kernel<D, NT, false, false, true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
+            if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+            fused_tc2_kernel<D, NT, false, true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
                 tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
-                p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, nullptr, nullptr, p.lse,
+                p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse,
                 BiasArg{}, p.block_mask, p.bmask_sb, p.bmask_sh);
             return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
         } else {
@@ -842,10 +824,10 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) return launch_fused_tc3_bias(p, &tmB, st);
         }
         if constexpr (NT == 2) {
-            if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
-            fused_tc2_kernel<D, NT, false, true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
+            if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+            fused_tc2_kernel<D, NT, true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
                 tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
-                p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, nullptr, nullptr, p.lse, bias_arg(p));
+                p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse, bias_arg(p));
             return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
         } else {
             return FLAT_ERR_UNSUPPORTED;
@@ -857,11 +839,11 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             auto launch = [&](auto cs_tag) -> int {
                 constexpr int CS = decltype(cs_tag)::value;
                 constexpr int BYTES = LY::SMEM_BYTES + LY::merge_bytes(CS);
-                if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, false, false, CS>>(BYTES)) return FLAT_ERR_CUDA;
+                if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, false, CS>>(BYTES)) return FLAT_ERR_CUDA;
                 if constexpr (CS > 8) {
                     // (the dispatcher only wants them when all clusters of the launch run at once: 8 clusters of sixteen
                     // one-per-SM CTAs took 80 us where clusters of eight take 41)
-                    const int fit = clusters_of_sixteen<fused_tc2_kernel<D, NT, false, false, false, CS>>(LY::THREADS, BYTES);
+                    const int fit = clusters_of_sixteen<fused_tc2_kernel<D, NT, false, false, CS>>(LY::THREADS, BYTES);
                     if (fit < 1 || (only_if_resident && static_cast<int64_t>(grid.x) * grid.y > fit)) return FLAT_ERR_UNSUPPORTED;
                 }
                 cudaLaunchConfig_t cfg = {};
@@ -877,9 +859,9 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
                 cfg.attrs = attr;
                 cfg.numAttrs = 2;
                 const cudaError_t e = cudaLaunchKernelEx(
-                    &cfg, fused_tc2_kernel<D, NT, false, false, false, CS>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H,
+                    &cfg, fused_tc2_kernel<D, NT, false, false, CS>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H,
                     p.Nq, p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
-                    static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse,
+                    p.lse,
                     BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
                 return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
             };
@@ -891,9 +873,9 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
         }
     }
     if (key_split != 1) return FLAT_ERR_UNSUPPORTED;
-    auto kern = fused_tc2_kernel<D, NT>;
-    if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
     if constexpr (NT == 1) {
+        auto kern = fused_tc2_kernel<D, NT>;
+        if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
         // short launches: the kernel may start while its predecessor in the stream drains (see its prologue)
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = grid;
@@ -907,15 +889,17 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
         cfg.numAttrs = 1;
         const cudaError_t e = cudaLaunchKernelEx(
             &cfg, kern, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
-            p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, static_cast<const int32_t*>(nullptr),
-            static_cast<const int32_t*>(nullptr), p.lse, BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
+            p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse, BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
         return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    } else if constexpr (D == 64) {
+        if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+        fused_tc2_kernel<D, NT><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
+            tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
+            p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse);
+        return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    } else {
+        return launch_fused_d128(p, st);                 // (two tiles, d = 128, no bias: a kernel of its own, fused_d128.cu)
     }
-    kern<<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq,
-                                                    p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
-                                                    p.causal ? p.Nk - p.Nq : (1 << 30), p.status, nullptr, nullptr, p.lse,
-                                                    BiasArg{}, nullptr, 0, 0);
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
 // Key halves (see the kernel's KH): d = 64, dense, one 128-row tile per CTA worked on by two warpgroups, optionally
@@ -933,10 +917,10 @@ int launch_tc2_kh(const Problem& p, cudaStream_t st, int key_split, bool only_if
         using LY = L2<D, NT, CS == 16 ? 2 : 1>;   // (the kernel's own choice of ring depths)
         constexpr int BYTES = LY::SMEM_BYTES + LY::merge_bytes(CS) + 128 * merge_vecs(D) * 16;
         static_assert(BYTES <= 232448, "shared memory of the two-warpgroup form");
-        auto kern = fused_tc2_kernel<D, NT, false, 0, false, CS, true>;
-        if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, 0, false, CS, true>>(BYTES)) return FLAT_ERR_CUDA;
+        auto kern = fused_tc2_kernel<D, NT, false, false, CS, true>;
+        if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, false, false, CS, true>>(BYTES)) return FLAT_ERR_CUDA;
         if constexpr (CS > 8) {
-            const int fit = clusters_of_sixteen<fused_tc2_kernel<D, NT, false, 0, false, CS, true>>(LY::THREADS, BYTES);
+            const int fit = clusters_of_sixteen<fused_tc2_kernel<D, NT, false, false, CS, true>>(LY::THREADS, BYTES);
             if (fit < 1 || (only_if_resident && static_cast<int64_t>(grid.x) * grid.y > fit)) return FLAT_ERR_UNSUPPORTED;
         }
         cudaLaunchConfig_t cfg = {};
@@ -953,8 +937,7 @@ int launch_tc2_kh(const Problem& p, cudaStream_t st, int key_split, bool only_if
         cfg.numAttrs = CS > 1 ? 2 : 1;
         const cudaError_t e = cudaLaunchKernelEx(
             &cfg, kern, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f,
-            p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, static_cast<const int32_t*>(nullptr),
-            static_cast<const int32_t*>(nullptr), p.lse, BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
+            p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse, BiasArg{}, static_cast<const uint8_t*>(nullptr), 0ll, 0ll);
         return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
     };
     return key_split == 1   ? launch(std::integral_constant<int, 1>{})
@@ -966,24 +949,6 @@ int launch_tc2_kh(const Problem& p, cudaStream_t st, int key_split, bool only_if
 
 }  // namespace
 
-
-int launch_fused_tc2_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q,
-                            const int32_t* cu_k, int num_seqs, int H, int64_t total_q, int64_t total_k,
-                            int max_seqlen_q, float scale, int causal, int32_t* status, cudaStream_t st) {
-    constexpr int D = 128, NT = 2;
-    using LY = L2<D, NT>;
-    if (static_cast<int64_t>(num_seqs) * H > 65535) return FLAT_ERR_SHAPE;      // (grid y)
-    CUtensorMap tmQ, tmK, tmV;
-    if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
-        !make_map_packed(&tmV, V, total_k, H, D, BN))
-        return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
-    dim3 grid((max_seqlen_q + NT * BM - 1) / (NT * BM), num_seqs * H);
-    fused_tc2_kernel<D, NT, true><<<grid, LY::THREADS, LY::SMEM_BYTES, st>>>(
-        tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
-        causal ? 0 : (1 << 30), status, cu_q, cu_k);
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
-}
 
 namespace {
 
