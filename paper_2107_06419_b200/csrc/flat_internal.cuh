@@ -68,7 +68,7 @@ int check_params(const flat_attn_params_t* p);
 int launch_fused_simt(const Problem& p, cudaStream_t st);
 int launch_naive(const Problem& p, void* L, void* A, cudaStream_t st);
 int launch_fused_tc(const Problem& p, cudaStream_t st);
-int launch_fused_d128(const Problem& p, cudaStream_t st);    // (bf16, d = 128, no bias, no pruning map)
+int launch_fused_d128(const Problem& p, const void* bias_map, cudaStream_t st);    // (bf16, d = 128, no pruning map; with a bias its tensor map: {Nk, Nq, heads, batches}, boxes of 64 x 128)
 int launch_fused_tc2(const Problem& p, cudaStream_t st);      // (also the tensor-core kernel for calls with a bias)
 // (only_if_resident: sixteen-CTA clusters only when all clusters of the launch can run at the same time; else
 // FLAT_ERR_UNSUPPORTED)

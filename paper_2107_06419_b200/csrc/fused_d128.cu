@@ -42,22 +42,26 @@ namespace {
 constexpr int D = 128;
 constexpr int BM = 128;              // rows per query tile (two tiles per CTA)
 constexpr int BN = 64;               // keys per step
-constexpr int KS = 5, VS = 5;        // ring depths
 constexpr int THREADS = 384;
 constexpr int POLY_LANE = 3;         // element index mod 4 that takes the polynomial (none: B4 H16 4096 keys 450 us against 428)
 constexpr float OVERFLOW_SUM = 1.0995116e12f;   // 2^40
 
 constexpr int Q_BYTES = BM * D * 2, KV_BYTES = BN * D * 2;
-constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES;
-constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
-static_assert(SMEM_BYTES <= 232448, "shared memory");
+constexpr int BIAS_BYTES = BM * BN * 2;   // a bias tile: 128 rows of 64 values
 __host__ __device__ constexpr uint32_t S_COL(int t, int b) { return 128u * t + 64u * b; }
 __host__ __device__ constexpr uint32_t O_COL(int t) { return 256u + 128u * t; }
-// barriers: S_FULL / P_FULL / PV_DONE [tile][step parity], each once every second step.  (One PV_DONE a tile is not enough: a warp
-// ahead of the others of its tile has its last logits when O += P V of the third last step is done, and would take that one's
-// parity for the last one's.)
-constexpr int Q_FULL = 0, K_FULL = 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS,
-              P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, NUM_BARS = PV_DONE + 4;
+// Ring depths and barriers.  BT: with two bias tiles per query tile, which take the room of two K and two V stages.
+// S_FULL / P_FULL / PV_DONE [tile][step parity], each once every second step.  (One PV_DONE a tile is not enough: a warp ahead of
+// the others of its tile has its last logits when O += P V of the third last step is done, and would take that one's parity for
+// the last one's.)  B_FULL / B_EMPTY [step parity][tile]: the bias tile / the four softmax warps of the tile have read it.
+template <bool BT> struct Layout {
+    static constexpr int KS = BT ? 3 : 5, VS = KS;
+    static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES + (BT ? 4 * BIAS_BYTES : 0);
+    static constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
+    static constexpr int Q_FULL = 0, K_FULL = 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS,
+                         P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, B_FULL = PV_DONE + 4, B_EMPTY = B_FULL + 4, NUM_BARS = B_EMPTY + 4;
+    static_assert(SMEM_BYTES <= 232448 && NUM_BARS * 8 + 8 <= 512, "shared memory");
+};
 
 // p_i = 2^(s_i * scale + neg_m) of 64 logits; bf16(p) to 32 TMEM columns at `p_addr`; returns the fp32 sum of the unrounded p.
 // TAIL: only the first `nvalid` take part.
@@ -92,6 +96,26 @@ __device__ __forceinline__ float exp_store(const uint32_t (&s)[BN], float scale_
     return (a + b) + (cc + d);
 }
 
+// s = s * scale * log2(e) + bias * log2(e), base-2 units; `brow`: shared-window address of the thread's 128-byte row of the bias
+// tile, rx: the row's place in the swizzle.
+__device__ __forceinline__ void add_bias(uint32_t (&s)[BN], float scale_log2e, uint32_t brow, int rx) {
+    const uint64_t scale2 = pack2(scale_log2e, scale_log2e), log2e2 = pack2(1.4426950408889634f, 1.4426950408889634f);
+#pragma unroll
+    for (int c = 0; c < BN / 8; ++c) {
+        uint32_t w[4];
+        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + ((c ^ rx) << 4)) : "memory");
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = c * 8 + 2 * e;
+            float a, b;
+            unpack2(fma2(pack2(__uint_as_float(s[i]), __uint_as_float(s[i + 1])), scale2,
+                         mul2(pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)), log2e2)), a, b);
+            s[i] = __float_as_uint(a);
+            s[i + 1] = __float_as_uint(b);
+        }
+    }
+}
+
 __device__ __forceinline__ float row_extreme(const uint32_t (&s)[BN], bool smallest) {
     float e0 = __uint_as_float(s[0]), e1 = __uint_as_float(s[1]);
 #pragma unroll
@@ -102,19 +126,24 @@ __device__ __forceinline__ float row_extreme(const uint32_t (&s)[BN], bool small
     return smallest ? fminf(e0, e1) : fmaxf(e0, e1);
 }
 
-template <bool VL>
+// BIAS: the bias tiles (bf16, rows on 16-byte boundaries) come through TMA, one per query tile and step, two ahead.
+template <bool VL, bool BIAS>
 __global__ void __launch_bounds__(THREADS, 1)
 fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                   __nv_bfloat16* __restrict__ O, int BH, int H, int Nq, int Nk, float scale_log2e, const int32_t* __restrict__ valid_len,
                   int coff, int group, int32_t* status, const int32_t* __restrict__ cu_q, const int32_t* __restrict__ cu_k,
-                  float* __restrict__ lse) {
+                  float* __restrict__ lse, const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}, int bias_heads = 0,
+                  int bias_batches = 0) {
+    using LY = Layout<BIAS>;
+    constexpr int KS = LY::KS, VS = LY::VS;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* Qs = base;
     uint8_t* Ks = Qs + 2 * Q_BYTES;
     uint8_t* Vs = Ks + KS * KV_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + TILE_BYTES);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
+    uint8_t* Bs = Vs + VS * KV_BYTES;                    // (bias) [step parity][tile]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + LY::TILE_BYTES);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -140,8 +169,9 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     }
 
     if (threadIdx.x == 256) {
-        for (int i = 0; i < NUM_BARS; ++i)
-            mbar_init(&bars[i], i >= P_FULL && i < PV_DONE ? 4 : (i >= K_EMPTY && i < V_FULL) || (i >= V_EMPTY && i < S_FULL) ? 2 : 1);
+        for (int i = 0; i < LY::NUM_BARS; ++i)
+            mbar_init(&bars[i], (i >= LY::P_FULL && i < LY::PV_DONE) || i >= LY::B_EMPTY ? 4
+                                : (i >= LY::K_EMPTY && i < LY::V_FULL) || (i >= LY::V_EMPTY && i < LY::S_FULL) ? 2 : 1);
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -166,52 +196,68 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
 
     if (warp >= 8) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         if (warp == 8) {
             // ------------------------------------------------------------ TMA producer
             if (lane == 0 && nsteps > 0) {
                 prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
                 bool ok = true;
-                int k_issued = 0, v_issued = 0;
+                int k_issued = 0, v_issued = 0, b_issued = 0;
                 auto load_q = [&](int t) {
-                    mbar_arrive_expect_tx(&bars[Q_FULL + t], Q_BYTES);
+                    mbar_arrive_expect_tx(&bars[LY::Q_FULL + t], Q_BYTES);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
-                        tma_load_3d(Qs + t * Q_BYTES + c * BM * 128, &tmQ, &bars[Q_FULL + t], c * 64, VL ? head : row0 + t * BM, VL ? q_tok0 + t * BM : bh);
+                        tma_load_3d(Qs + t * Q_BYTES + c * BM * 128, &tmQ, &bars[LY::Q_FULL + t], c * 64, VL ? head : row0 + t * BM, VL ? q_tok0 + t * BM : bh);
                 };
                 auto load_k = [&](int j) {
                     const int s = j % KS;
-                    ok = bounded_wait_s(bars_s + 8 * (K_EMPTY + s), ((j / KS) & 1) ^ 1, abort_s, status, 0xa00 + s);
+                    ok = bounded_wait_s(bars_s + 8 * (LY::K_EMPTY + s), ((j / KS) & 1) ^ 1, abort_s, status, 0xa00 + s);
                     if (!ok) return;
-                    mbar_arrive_expect_tx(&bars[K_FULL + s], KV_BYTES);
+                    mbar_arrive_expect_tx(&bars[LY::K_FULL + s], KV_BYTES);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
-                        tma_load_3d(Ks + s * KV_BYTES + c * BN * 128, &tmK, &bars[K_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
+                        tma_load_3d(Ks + s * KV_BYTES + c * BN * 128, &tmK, &bars[LY::K_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
                     k_issued = j + 1;
                 };
                 auto load_v = [&](int j) {
                     const int s = j % VS;
-                    ok = bounded_wait_s(bars_s + 8 * (V_EMPTY + s), ((j / VS) & 1) ^ 1, abort_s, status, 0xa10 + s);
+                    ok = bounded_wait_s(bars_s + 8 * (LY::V_EMPTY + s), ((j / VS) & 1) ^ 1, abort_s, status, 0xa10 + s);
                     if (!ok) return;
-                    mbar_arrive_expect_tx(&bars[V_FULL + s], KV_BYTES);
+                    mbar_arrive_expect_tx(&bars[LY::V_FULL + s], KV_BYTES);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
-                        tma_load_3d(Vs + s * KV_BYTES + c * BN * 128, &tmV, &bars[V_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
+                        tma_load_3d(Vs + s * KV_BYTES + c * BN * 128, &tmV, &bars[LY::V_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
                     v_issued = j + 1;
+                };
+                auto load_bias = [&](int j) {            // of both tiles
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const int s = 2 * (j & 1) + t;
+                        ok = ok && bounded_wait_s(bars_s + 8 * (LY::B_EMPTY + s), ((j >> 1) & 1) ^ 1, abort_s, status, 0xa18 + t);
+                        if (!ok) return;
+                        mbar_arrive_expect_tx(&bars[LY::B_FULL + s], BIAS_BYTES);
+                        tma_load_4d(Bs + s * BIAS_BYTES, &tmBias, &bars[LY::B_FULL + s], j * BN, row0 + t * BM, bias_heads ? bh % H : 0, bias_batches ? bh / H : 0);
+                        b_issued = 2 * j + t + 1;
+                    }
                 };
                 load_q(0);
                 load_k(0);
                 load_q(1);
+                if (BIAS) load_bias(0);
                 if (nsteps > 1) load_k(1);
+                if (BIAS && nsteps > 1) load_bias(1);
                 for (int j = 0; j < nsteps && ok; ++j) {
                     load_v(j);
                     if (ok && j + 2 < nsteps) load_k(j + 2);
+                    if (BIAS && ok && j > 0 && j + 1 < nsteps) load_bias(j + 1);
                 }
                 if (!ok) {
-                    drain_wait(&bars[Q_FULL], 0);
-                    drain_wait(&bars[Q_FULL + 1], 0);
-                    for (int j = k_issued > KS ? k_issued - KS : 0; j < k_issued; ++j) drain_wait(&bars[K_FULL + j % KS], (j / KS) & 1);
-                    for (int j = v_issued > VS ? v_issued - VS : 0; j < v_issued; ++j) drain_wait(&bars[V_FULL + j % VS], (j / VS) & 1);
+                    drain_wait(&bars[LY::Q_FULL], 0);
+                    drain_wait(&bars[LY::Q_FULL + 1], 0);
+                    for (int j = k_issued > KS ? k_issued - KS : 0; j < k_issued; ++j) drain_wait(&bars[LY::K_FULL + j % KS], (j / KS) & 1);
+                    for (int j = v_issued > VS ? v_issued - VS : 0; j < v_issued; ++j) drain_wait(&bars[LY::V_FULL + j % VS], (j / VS) & 1);
+                    if (BIAS)
+                        for (int u = b_issued > 4 ? b_issued - 4 : 0; u < b_issued; ++u) drain_wait(&bars[LY::B_FULL + (u & 3)], (u >> 2) & 1);
                 }
             }
         } else if (warp <= 10) {
@@ -232,29 +278,29 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     for (int k = 0; k < D / 16; ++k)
                         mma_ss(tmem + S_COL(t, j & 1), q_desc + static_cast<uint64_t>(((k / 4) * (BM * 128) + (k % 4) * 32) >> 4),
                                kd + static_cast<uint64_t>(((k / 4) * (BN * 128) + (k % 4) * 32) >> 4), IDESC_S, k > 0);
-                    tc_commit(&bars[S_FULL + 2 * t + (j & 1)]);
-                    tc_commit(&bars[K_EMPTY + j % KS]);
+                    tc_commit(&bars[LY::S_FULL + 2 * t + (j & 1)]);
+                    tc_commit(&bars[LY::K_EMPTY + j % KS]);
                 };
                 auto issue_pv = [&](int j) {             // O_t += P_t(j) V_j, then release the V stage
                     const uint64_t vd = v_desc + static_cast<uint64_t>(((j % VS) * KV_BYTES) >> 4);
 #pragma unroll
                     for (int k = 0; k < BN / 16; ++k)
                         mma_ts(tmem + O_COL(t), tmem + S_COL(t, j & 1) + k * 8, vd + static_cast<uint64_t>((k * 2048) >> 4), IDESC_PV, (j > 0 || k > 0));
-                    tc_commit(&bars[PV_DONE + 2 * t + (j & 1)]);
-                    tc_commit(&bars[V_EMPTY + j % VS]);
+                    tc_commit(&bars[LY::PV_DONE + 2 * t + (j & 1)]);
+                    tc_commit(&bars[LY::V_EMPTY + j % VS]);
                 };
-                wait(Q_FULL + t, 0, 0xa20);
+                wait(LY::Q_FULL + t, 0, 0xa20);
                 for (int j = 0; j < 2 && j < nsteps; ++j) {
-                    wait(K_FULL + j, 0, 0xa21);
+                    wait(LY::K_FULL + j, 0, 0xa21);
                     tc_fence_after();
                     if (ok && elect_one()) issue_s(j);
                     __syncwarp();
                 }
                 for (int j = 0; j < nsteps && ok; ++j) {
                     const bool more = j + 2 < nsteps;
-                    wait(V_FULL + j % VS, (j / VS) & 1, 0xa22);
-                    if (more) wait(K_FULL + (j + 2) % KS, ((j + 2) / KS) & 1, 0xa23);
-                    wait(P_FULL + 2 * t + (j & 1), (j >> 1) & 1, 0xa24);
+                    wait(LY::V_FULL + j % VS, (j / VS) & 1, 0xa22);
+                    if (more) wait(LY::K_FULL + (j + 2) % KS, ((j + 2) / KS) & 1, 0xa23);
+                    wait(LY::P_FULL + 2 * t + (j & 1), (j >> 1) & 1, 0xa24);
                     if (!ok) break;
                     tc_fence_after();
                     // (S(j + 2) overwrites P(j): it goes behind the MMAs that read it)
@@ -265,12 +311,15 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
     } else {
         // ------------------------------------------------------------ softmax + epilogue (warps 0-7)
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
         const int t = warp >> 2;
         const int row = row0 + t * BM + (warp & 3) * 32 + lane;
         const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        const uint32_t my_bars = bars_s + 8 * (S_FULL + 2 * t);       // S_FULL of the tile; P_FULL and PV_DONE 32 and 64 bytes on
-        const bool neg_scale = scale_log2e < 0.f;
+        const uint32_t my_bars = bars_s + 8 * (LY::S_FULL + 2 * t);       // S_FULL of the tile; P_FULL and PV_DONE 32 and 64 bytes on
+        // (bias) the thread's row of its tile; the logits are scaled as they meet the bias
+        const uint32_t brow = smem_u32(Bs) + t * BIAS_BYTES + ((warp & 3) * 32 + lane) * 128;
+        const float unit = BIAS ? 1.f : scale_log2e;
+        const bool neg_scale = !BIAS && scale_log2e < 0.f;
         float m_ref = -INFINITY, l = 0.f;
         bool ok = true;
         const long long rlim = static_cast<long long>(row) + 1 + coff;
@@ -284,7 +333,14 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             uint32_t s[BN];
             tmem_ld_x32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
             tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+            if (BIAS) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * (LY::B_FULL + 2 * (j & 1) + t), (j >> 1) & 1, abort_s, status, 0xa36 + t));
             tc_wait_ld();
+            if (BIAS) {
+                if (!ok) break;
+                add_bias(s, scale_log2e, brow + (j & 1) * (2 * BIAS_BYTES), lane & 7);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + 2 * (j & 1) + t));
+            }
             const int col0 = j * BN;
             const bool tail = col0 + BN > nrow_min;      // (warp-uniform) some row has masked keys in this step
             const int nvalid = nrow > col0 ? (nrow - col0 < BN ? nrow - col0 : BN) : 0;
@@ -296,15 +352,15 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             bool careful = j == 0 || tail;
             float lt = 0.f;
             if (!careful) {
-                lt = exp_store<false>(s, scale_log2e, -m_ref, s_addr, BN);
+                lt = exp_store<false>(s, unit, -m_ref, s_addr, BN);
                 careful = __any_sync(0xffffffffu, !(lt <= OVERFLOW_SUM));
-                if (careful) {           // (the weights went over the first half of the logits only: 32 registers less to keep)
+                if (!BIAS && careful) {  // (the weights went over the first half of the logits only: 32 registers less to keep)
                     tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
                     tc_wait_ld();
                 }
             }
             if (careful) {
-                const float mx = nvalid > 0 ? row_extreme(s, neg_scale) * scale_log2e : -INFINITY;
+                const float mx = nvalid > 0 ? row_extreme(s, neg_scale) * unit : -INFINITY;
                 if (__any_sync(0xffffffffu, mx > m_ref + RESCALE_THRESHOLD)) {
                     const float m_new = fmaxf(m_ref, mx);
                     const float alpha = m_new == -INFINITY ? 1.f : ex2_approx(m_ref - m_new);   // 0 on the row's first keys
@@ -325,7 +381,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     }
                     m_ref = m_new;
                 }
-                lt = exp_store<true>(s, scale_log2e, m_ref == -INFINITY ? 0.f : -m_ref, s_addr, nvalid);
+                lt = exp_store<true>(s, unit, m_ref == -INFINITY ? 0.f : -m_ref, s_addr, nvalid);
             }
             l += lt;
             tc_wait_st();
@@ -371,16 +427,15 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-}  // namespace
-
-int launch_fused_d128(const Problem& p, cudaStream_t st) {
-    if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || p.bias || p.block_mask) return FLAT_ERR_UNSUPPORTED;
+template <bool BIAS>
+int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
+    constexpr int SMEM_BYTES = Layout<BIAS>::SMEM_BYTES;
     CUtensorMap tmQ, tmK, tmV;
     const int BH = p.B * p.H, slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
     if (static_cast<int64_t>(slabs) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
     if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map(&tmK, p.K, BH, p.Nk, D, BN) || !make_map(&tmV, p.V, BH, p.Nk, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<false>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<false, BIAS>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
     // without the causal mask the slabs of a head run side by side and share K and V in L2; with it, those of as many heads as
     // fit L2 together (48 MB of K and V) go longest first: what is left at the end are the short ones
     const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 4);
@@ -395,10 +450,17 @@ int launch_fused_d128(const Problem& p, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false, BIAS>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
                                              p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status,
-                                             static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse);
+                                             static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse, tmB, p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
+}  // namespace
+
+int launch_fused_d128(const Problem& p, const void* bias_map, cudaStream_t st) {
+    if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias_map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
+    return bias_map ? launch<true>(p, *static_cast<const CUtensorMap*>(bias_map), st) : launch<false>(p, CUtensorMap{}, st);
 }
 
 int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q, const int32_t* cu_k, int num_seqs,
@@ -409,10 +471,10 @@ int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* 
     if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
         !make_map_packed(&tmV, V, total_k, H, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<true>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<true, false>>(Layout<false>::SMEM_BYTES)) return FLAT_ERR_CUDA;
     const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535;
     const dim3 grid(group ? num_seqs * H : slabs, group ? slabs : num_seqs * H);
-    fused_d128_kernel<true><<<grid, THREADS, SMEM_BYTES, st>>>(
+    fused_d128_kernel<true, false><<<grid, THREADS, Layout<false>::SMEM_BYTES, st>>>(
         tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), num_seqs * H, H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
         causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr);
     return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;

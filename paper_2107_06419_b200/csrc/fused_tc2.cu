@@ -817,11 +817,12 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
         }
     }
     if (p.bias) {
-        if constexpr (NT == 2 && D == 64) {
-            // bf16 bias with 16-byte aligned rows: the half-row kernel, tiles staged through shared memory by TMA
+        if constexpr (NT == 2) {
+            // bf16 bias with 16-byte aligned rows: tiles staged through shared memory by TMA, in the half-row kernel (d = 64)
+            // or the one with 64-key steps (d = 128: B8 H16 1024^2 244 -> 108 us, B4 H16 4096^2 1,589 -> 612)
             const BiasArg ba = bias_arg(p);
             CUtensorMap tmB;
-            if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) return launch_fused_tc3_bias(p, &tmB, st);
+            if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) return D == 64 ? launch_fused_tc3_bias(p, &tmB, st) : launch_fused_d128(p, &tmB, st);
         }
         if constexpr (NT == 2) {
             if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
@@ -898,7 +899,7 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse);
         return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
     } else {
-        return launch_fused_d128(p, st);                 // (two tiles, d = 128, no bias: a kernel of its own, fused_d128.cu)
+        return launch_fused_d128(p, nullptr, st);                 // (two tiles, d = 128, no bias: a kernel of its own, fused_d128.cu)
     }
 }
 

@@ -20,6 +20,10 @@ CASES = [
     (2, 2, 200, 328, 64, (2, 2), "bf16", None, False, -0.2),
     (2, 2, 130, 301, 64, (1, 2), "bf16", None, False, 0.125),               # rows begin at every second byte
     (2, 2, 130, 302, 128, (2, 1), "bf16", [302, 77], True, 0.1),
+    (2, 3, 257, 520, 128, (1, 3), "bf16", [520, 65], False, 0.1),            # d = 128, staged: nine steps of 64 keys
+    (3, 2, 700, 704, 128, (3, 1), "bf16", [704, 1, 640], True, 0.1),
+    (2, 2, 200, 328, 128, (2, 2), "bf16", None, False, -0.2),
+    (1, 1, 1, 8, 128, (1, 1), "bf16", None, False, 0.1),
     (1, 2, 70, 131, 64, (1, 2), "f32", None, False, 0.125),
     (1, 2, 300, 130, 128, (1, 1), "f32", None, False, 0.1),
     (1, 1, 1, 1, 64, (1, 1), "bf16", None, False, 1.0),
