@@ -93,7 +93,8 @@ int run_fused(const flat::Problem& q, int variant, cudaStream_t st) {
     if (v == FLAT_VARIANT_AUTO) {
         if (!tc_applies(q)) {
             // bf16 with d = 16 or 32: the small-head kernel (B16 H8 1000^2, d = 32: 66 us against 638 on the FFMA kernel).
-            // fp32 tensors: the split-tf32 tensor-core kernel where it applies, else the FFMA kernel
+            // fp32 tensors: the split-tf32 tensor-core kernel where it applies (d = 32, 64, 128; down to one tile of keys
+            // and queries: B1 H4 64^2 d = 128 14 us against 22, B2 H16 4096^2 1.2 ms against 9.5), else the FFMA kernel
             v = flat::tf32_applies(q) ? FLAT_VARIANT_TF32 : flat::small_applies(q) ? FLAT_VARIANT_SMALL : FLAT_VARIANT_SIMT;
         } else if (flat::decode_applies(q)) {
             v = FLAT_VARIANT_DECODE;
@@ -200,7 +201,8 @@ int run_fused(const flat::Problem& q, int variant, cudaStream_t st) {
         g_last_variant = v;
         return rc;
     }
-    if (v == FLAT_VARIANT_TF32 && !flat::tf32_applies(q)) return FLAT_ERR_UNSUPPORTED;
+    // (chosen by the caller: d = 64 only)
+    if (v == FLAT_VARIANT_TF32 && (!flat::tf32_applies(q) || (variant == FLAT_VARIANT_TF32 && q.d != 64))) return FLAT_ERR_UNSUPPORTED;
     if (q.block_mask && (v != FLAT_VARIANT_TC2_SINGLE || q.bias || !tc_applies(q) || q.Nk > 131072)) return FLAT_ERR_UNSUPPORTED;
     g_last_variant = v;
     if (v == FLAT_VARIANT_TC2_SINGLE) {

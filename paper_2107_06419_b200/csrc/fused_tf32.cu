@@ -1,8 +1,8 @@
-// Fused Logit-Softmax-Attend for fp32 tensors on the tensor cores (fp32 in, fp32 out, d = 64).
+// Fused Logit-Softmax-Attend for fp32 tensors on the tensor cores (fp32 in, fp32 out, d = 32, 64, 128).
 //
 // The tensor cores take 32-bit operands only as tf32 (10 mantissa bits), so every fp32 operand x is
-// split into x_hi (x with its low 13 mantissa bits cleared: exactly a tf32 number) and
-// x_lo = x - x_hi (exact in fp32), and each contraction is the sum of three tf32 products
+// split into x_hi (a tf32 number close to x) and x_lo = x - x_hi (exact in fp32), and each contraction is the sum of
+// three tf32 products
 //     a b  ~=  a_lo b_hi + a_hi b_lo + a_hi b_hi          (the dropped a_lo b_lo is 2^-22 of the result)
 // accumulated in fp32.  Both contractions of the path are done this way: S = Q K^T and, per key step,
 // P V with the weights P split the same way.  The accumulation ACROSS key steps is not left to the
@@ -11,8 +11,11 @@
 // streaming softmax then costs nothing extra, and the result does not depend on how the tensor core
 // rounds a 16K-term running sum.
 //
-// Paper mapping (Section 5, 5.1, 5.2): shared outer loops = (batch, head) on blockIdx.y and a tile of
-// 128 query rows on blockIdx.x (R-granularity); Logit and Attend run interleaved over 64-key steps with
+// What bounds it: the tensor pipe at d = 64 and 128 (three products at half the bf16 rate: 85-88 % of it with B2 H16 4096 keys,
+// 552 and 1,180 us), the softmax warps at d = 32 (424 us).  Before, d = 32 and 128 ran on the FFMA kernel: 2,840 and 9,600 us.
+//
+// Paper mapping (Section 5, 5.1, 5.2): shared outer loops = (batch, head) and a tile of 128 query rows on blockIdx.x
+// (R-granularity); Logit and Attend run interleaved over steps of 64 keys (d = 128: 32) with
 // the streaming softmax between them; the logits and weights never leave TMEM.
 //
 // CTA = 512 threads, four warpgroups:
@@ -24,10 +27,12 @@
 //   warps 8-11 converters: warps 8, 9 K tile -> (K_hi in place, K_lo); warps 10, 11 V tile -> transposed
 //              (V^T_hi, V^T_lo), since a tf32 operand must have the contraction index contiguous in shared memory
 //   warp  12   TMA producer (one lane): Q once, K and raw V tiles into rings
-//   warps 13, 14  MMA issuers of the even / odd key steps (one elected lane each): 24 + 24 tcgen05.mma of
-//              128 x 64 x 8 per step, A always from TMEM
+//   warps 13, 14  MMA issuers of the even / odd key steps (one elected lane each): tcgen05.mma with k-slices of 8, A
+//              always from TMEM
 //   warp  15   idle (it completes the warpgroup for the register hand-over)
-// TMEM columns: Q_hi 0, Q_lo 64, S/P_hi 128 + 64 b, P_lo 256 + 64 b, PV 384 + 64 b (b = step parity).
+// TMEM columns: Q_hi d, Q_lo d, then per step parity S / P_hi (as many columns as a step has keys), P_lo and P V (d); at
+// d = 128, where Q takes half of TMEM, steps of 32 keys leave room for both parities of S and P and for one P V buffer:
+// a step's P V waits until the one before has been read, which happens while the pipe works on the logits in between.
 // Every wait is bounded (see tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -45,25 +50,29 @@ using namespace tc;
 namespace {
 
 constexpr int BM = 128;              // query rows per CTA
-constexpr int BN = 64;               // keys per step
-constexpr int D = 64;
 constexpr int KS = 3;                // K ring (each stage: K_hi and K_lo tiles)
 constexpr int VR = 2;                // raw V ring
 constexpr int VS = 3;                // transposed V ring (each stage: V^T_hi and V^T_lo tiles)
-constexpr int TILE = BN * D * 4;     // 16 KB: two panels of 64 rows x 128 bytes
-constexpr int PANEL = 64 * 128;
 constexpr int THREADS = 512;
-constexpr int MERGE_STRIDE = 68;      // floats per row of the merge scratch (64 outputs, m, l, padding: 16-byte rows, no bank conflicts)
 constexpr uint32_t HI_MASK = 0xffffe000u;
+constexpr uint32_t TMEM_COLS = 512;
 
-constexpr uint32_t QH_COL = 0, QL_COL = 64, S_COL = 128, PL_COL = 256, PV_COL = 384, TMEM_COLS = 512;
-
-// shared memory: K_hi[KS] K_lo[KS] Vraw[VR] VT_hi[VS] VT_lo[VS]; the Q tile is staged over VT_hi[0..1]
-constexpr int OFF_KH = 0, OFF_KL = OFF_KH + KS * TILE, OFF_VR = OFF_KL + KS * TILE, OFF_VTH = OFF_VR + VR * TILE,
-              OFF_VTL = OFF_VTH + VS * TILE, TILE_BYTES = OFF_VTL + VS * TILE;
-static_assert(VS * TILE >= BM * D * 4, "the Q tile is staged over the V^T_hi ring");
-static_assert(2 * KS * TILE >= BM * MERGE_STRIDE * 4, "the merge scratch lies over the K rings");
-constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
+template <int D> struct Layout {
+    static constexpr int BN = D == 128 ? 32 : 64;        // keys per step
+    static constexpr int TILE = BN * D * 4;              // K: D/32 panels of BN rows x 128 bytes; V^T: BN/32 panels of D rows
+    static constexpr int PANEL = BN * 128, VT_PANEL = D * 128;
+    static constexpr int MERGE_STRIDE = D + 4;           // floats per row of the merge scratch (outputs, m, l, padding: 16-byte rows, no bank conflicts)
+    static constexpr int PVS = D == 128 ? 1 : 2;         // P V buffers
+    static constexpr uint32_t QH_COL = 0, QL_COL = D, S_COL = 2 * D, PL_COL = S_COL + 2 * BN, PV_COL = PL_COL + 2 * BN;
+    static_assert(PV_COL + PVS * D <= TMEM_COLS, "tensor memory");
+    // shared memory: K_hi[KS] K_lo[KS] Vraw[VR] VT_hi[VS] VT_lo[VS]; the Q tile is staged over the V^T rings
+    static constexpr int OFF_KH = 0, OFF_KL = OFF_KH + KS * TILE, OFF_VR = OFF_KL + KS * TILE, OFF_VTH = OFF_VR + VR * TILE,
+                         OFF_VTL = OFF_VTH + VS * TILE, TILE_BYTES = OFF_VTL + VS * TILE;
+    static_assert(2 * VS * TILE >= BM * D * 4, "the Q tile is staged over the V^T rings");
+    static_assert(2 * KS * TILE >= BM * MERGE_STRIDE * 4, "the merge scratch lies over the K rings");
+    static constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
+    static_assert(SMEM_BYTES <= 232448, "shared memory");
+};
 
 // barriers
 constexpr int Q_FULL = 0, Q_READY = 1, K_FULL = 2, KC_FULL = K_FULL + KS, K_EMPTY = KC_FULL + KS, V_FULL = K_EMPTY + KS,
@@ -79,9 +88,10 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Instruction descriptor for kind::tf32, fp32 accumulator, both operands with the contraction index contiguous.
-constexpr uint32_t IDESC = (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<uint32_t>(BN >> 3) << 17) |
-                           (static_cast<uint32_t>(BM >> 4) << 24);
+// Instruction descriptor for kind::tf32, fp32 accumulator, both operands with the contraction index contiguous, n columns.
+__host__ __device__ constexpr uint32_t idesc_tf32(int n) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(BM >> 4) << 24);
+}
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     uint4 v;
@@ -91,15 +101,34 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 __device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
     asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-__device__ __forceinline__ uint32_t lo_of(uint32_t x) {      // x - x_hi, exact
-    return __float_as_uint(__uint_as_float(x) - __uint_as_float(x & HI_MASK));
+// x_hi and x_lo = x - x_hi (exact).  NEAR: x_hi = x (1 + 0.35 * 2^-10), a third to two thirds of its unit above x, with the low
+// bits cut off: nearly the nearest tf32 number (rounding the product towards zero keeps the largest numbers finite).  The mean
+// square of x_lo is then a third of what cutting x off itself leaves and its mean about zero: with 32 and 128 features the
+// error is that of the FFMA kernel, which ran there before (300 keys, d = 128: rms 4.8e-8 against 4.7e-8, cut off 9.3e-8; 4096
+// keys, d = 32: 9.5e-9 against 3.1e-8).  It costs 2 % of the time there (B2 H16 4096^2: 1,199 us against 1,178, 432 against
+// 424); 12 % at d = 64 (620 against 552), where x is cut off.
+template <bool NEAR>
+__device__ __forceinline__ uint32_t hi_of(uint32_t x) {
+    return (NEAR ? __float_as_uint(__fmul_rz(__uint_as_float(x), 1.00034180f)) : x) & HI_MASK;
+}
+__device__ __forceinline__ uint32_t lo_of(uint32_t x, uint32_t hi) { return __float_as_uint(__uint_as_float(x) - __uint_as_float(hi)); }
+template <bool NEAR>
+__device__ __forceinline__ void split4(const uint4& v, uint4& h, uint4& l) {
+    h = make_uint4(hi_of<NEAR>(v.x), hi_of<NEAR>(v.y), hi_of<NEAR>(v.z), hi_of<NEAR>(v.w));
+    l = make_uint4(lo_of(v.x, h.x), lo_of(v.y, h.y), lo_of(v.z, h.z), lo_of(v.w, h.w));
 }
 
+template <int D>
 __global__ void __launch_bounds__(THREADS, 1)
 fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                  const __grid_constant__ CUtensorMap tmV, float* __restrict__ O, int H, int Nq, int Nk,
-                  float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int32_t* status,
+                  const __grid_constant__ CUtensorMap tmV, float* __restrict__ O, int BH, int H, int Nq, int Nk,
+                  float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int group, int32_t* status,
                   float* __restrict__ lse) {
+    using LY = Layout<D>;
+    constexpr int BN = LY::BN, TILE = LY::TILE, PANEL = LY::PANEL, OFF_KH = LY::OFF_KH, OFF_KL = LY::OFF_KL, OFF_VR = LY::OFF_VR,
+                  OFF_VTH = LY::OFF_VTH, OFF_VTL = LY::OFF_VTL, TILE_BYTES = LY::TILE_BYTES;
+    constexpr bool NEAR = D != 64;
+    constexpr uint32_t QH_COL = LY::QH_COL, QL_COL = LY::QL_COL, S_COL = LY::S_COL, PL_COL = LY::PL_COL, PV_COL = LY::PV_COL;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(base + TILE_BYTES);
@@ -108,8 +137,11 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const uint32_t sb = smem_u32(base);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int bh = blockIdx.y;
-    const int row0 = blockIdx.x * BM;
+    // `group` heads at a time, their tiles side by side, the longest first under the causal mask
+    const int slabs = (Nq + BM - 1) / BM, per = group * slabs, first = static_cast<int>(blockIdx.x) / per * group;
+    const int heads = BH - first < group ? BH - first : group, at = static_cast<int>(blockIdx.x) % per;
+    const int bh = first + at % heads;
+    const int row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * BM;
     int n = Nk;
     if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
     {
@@ -150,8 +182,9 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     ok = bounded_wait(&bars[K_EMPTY + s], ((j / KS) & 1) ^ 1, abort_flag, status, 0x600 + s);
                     if (!ok) return;
                     mbar_arrive_expect_tx(&bars[K_FULL + s], TILE);
-                    tma_load_3d(base + OFF_KH + s * TILE, &tmK, &bars[K_FULL + s], 0, j * BN, bh);
-                    tma_load_3d(base + OFF_KH + s * TILE + PANEL, &tmK, &bars[K_FULL + s], 32, j * BN, bh);
+#pragma unroll
+                    for (int c = 0; c < D / 32; ++c)
+                        tma_load_3d(base + OFF_KH + s * TILE + c * PANEL, &tmK, &bars[K_FULL + s], 32 * c, j * BN, bh);
                     k_issued = j + 1;
                 };
                 auto load_v = [&](int j) {
@@ -159,13 +192,14 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     ok = bounded_wait(&bars[VR_EMPTY + s], ((j / VR) & 1) ^ 1, abort_flag, status, 0x610 + s);
                     if (!ok) return;
                     mbar_arrive_expect_tx(&bars[V_FULL + s], TILE);
-                    tma_load_3d(base + OFF_VR + s * TILE, &tmV, &bars[V_FULL + s], 0, j * BN, bh);
-                    tma_load_3d(base + OFF_VR + s * TILE + PANEL, &tmV, &bars[V_FULL + s], 32, j * BN, bh);
+#pragma unroll
+                    for (int c = 0; c < D / 32; ++c)
+                        tma_load_3d(base + OFF_VR + s * TILE + c * PANEL, &tmV, &bars[V_FULL + s], 32 * c, j * BN, bh);
                     v_issued = j + 1;
                 };
                 mbar_arrive_expect_tx(&bars[Q_FULL], BM * D * 4);
-                tma_load_3d(base + OFF_VTH, &tmQ, &bars[Q_FULL], 0, row0, bh);
-                tma_load_3d(base + OFF_VTH + BM * 128, &tmQ, &bars[Q_FULL], 32, row0, bh);
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) tma_load_3d(base + OFF_VTH + c * BM * 128, &tmQ, &bars[Q_FULL], 32 * c, row0, bh);
                 load_k(0);
                 if (ntiles > 1) load_k(1);
                 for (int j = 0; j < ntiles && ok; ++j) {
@@ -193,20 +227,27 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     if (ok) ok = __all_sync(0xffffffffu, bounded_wait(&bars[bar], parity, abort_flag, status, code));
                     if (ok) tc_fence_after();
                 };
-                // one 128 x 64 x 64 product: eight k-slices of eight (32 bytes of a 128-byte row each)
-                auto product = [&](uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, bool first) {
+                constexpr uint32_t IDESC_S = idesc_tf32(BN), IDESC_PV = idesc_tf32(D);
+                // one product, k-slices of eight (32 bytes of a 128-byte row each): Q K^T (128 x BN x D), P V (128 x D x BN)
+                auto product_s = [&](uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, bool first) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
+                    for (int k = 0; k < D / 8; ++k)
                         mma_tf32_ts(d_tmem, a_tmem + k * 8, b_desc + static_cast<uint64_t>(((k >> 2) * PANEL + (k & 3) * 32) >> 4),
-                                    IDESC, !(first && k == 0));
+                                    IDESC_S, !(first && k == 0));
+                };
+                auto product_pv = [&](uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, bool first) {
+#pragma unroll
+                    for (int k = 0; k < BN / 8; ++k)
+                        mma_tf32_ts(d_tmem, a_tmem + k * 8, b_desc + static_cast<uint64_t>(((k >> 2) * LY::VT_PANEL + (k & 3) * 32) >> 4),
+                                    IDESC_PV, !(first && k == 0));
                 };
                 auto issue_s = [&](int j) {                  // S(j) = Q K_j^T, small terms first; then release the K stage
                     const int ks = j % KS, b = j & 1;
                     if (elect_one()) {
                         const uint64_t st = static_cast<uint64_t>((ks * TILE) >> 4);
-                        product(tmem + S_COL + 64 * b, tmem + QL_COL, kh_desc + st, true);
-                        product(tmem + S_COL + 64 * b, tmem + QH_COL, kl_desc + st, false);
-                        product(tmem + S_COL + 64 * b, tmem + QH_COL, kh_desc + st, false);
+                        product_s(tmem + S_COL + BN * b, tmem + QL_COL, kh_desc + st, true);
+                        product_s(tmem + S_COL + BN * b, tmem + QH_COL, kl_desc + st, false);
+                        product_s(tmem + S_COL + BN * b, tmem + QH_COL, kh_desc + st, false);
                         tc_commit(&bars[S_FULL + b]);
                         tc_commit(&bars[K_EMPTY + ks]);
                     }
@@ -216,9 +257,9 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     const int vs = j % VS, b = j & 1;
                     if (elect_one()) {
                         const uint64_t st = static_cast<uint64_t>((vs * TILE) >> 4);
-                        product(tmem + PV_COL + 64 * b, tmem + PL_COL + 64 * b, vh_desc + st, true);
-                        product(tmem + PV_COL + 64 * b, tmem + S_COL + 64 * b, vl_desc + st, false);
-                        product(tmem + PV_COL + 64 * b, tmem + S_COL + 64 * b, vh_desc + st, false);
+                        product_pv(tmem + PV_COL + (LY::PVS - 1) * D * b, tmem + PL_COL + BN * b, vh_desc + st, true);
+                        product_pv(tmem + PV_COL + (LY::PVS - 1) * D * b, tmem + S_COL + BN * b, vl_desc + st, false);
+                        product_pv(tmem + PV_COL + (LY::PVS - 1) * D * b, tmem + S_COL + BN * b, vh_desc + st, false);
                         tc_commit(&bars[PV_FULL + b]);
                         tc_commit(&bars[VT_EMPTY + vs]);
                     }
@@ -229,7 +270,9 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 if (ok) issue_s(g);
                 for (int j = g; j < ntiles && ok; j += 2) {
                     wait(VT_FULL + j % VS, (j / VS) & 1, 0x630);
-                    wait(PV_FREE + (j & 1), ((j >> 1) & 1) ^ 1, 0x631);
+                    // (the buffer's last use: two steps before, or the step before, of the other issuer)
+                    if (LY::PVS == 2) wait(PV_FREE + (j & 1), ((j >> 1) & 1) ^ 1, 0x631);
+                    else if (j > 0) wait(PV_FREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, 0x631);
                     // (the converted keys of step j + 2 are checked here, ahead of the wait for the weights, so that
                     // the check does not sit between the two batches of products)
                     if (j + 2 < ntiles) wait(KC_FULL + (j + 2) % KS, ((j + 2) / KS) & 1, 0x633);
@@ -253,11 +296,12 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 if (!ok) break;
                 const uint32_t kh = sb + OFF_KH + s * TILE, kl = sb + OFF_KL + s * TILE;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
+                for (int i = 0; i < TILE / 1024; ++i) {
                     const uint32_t off = (ct + 64 * i) * 16;
-                    const uint4 v = lds128(kh + off);
-                    sts128(kl + off, make_uint4(lo_of(v.x), lo_of(v.y), lo_of(v.z), lo_of(v.w)));
-                    sts128(kh + off, make_uint4(v.x & HI_MASK, v.y & HI_MASK, v.z & HI_MASK, v.w & HI_MASK));
+                    uint4 h, l;
+                    split4<NEAR>(lds128(kh + off), h, l);
+                    sts128(kl + off, l);
+                    sts128(kh + off, h);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
@@ -267,7 +311,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             // warps 10, 11: V tile -> transposed V^T_hi, V^T_lo.  4 x 4 blocks: a thread's blocks sit on an XOR
             // diagonal of (key block, feature block), which keeps both the 16-byte reads and the transposed
             // 16-byte writes free of bank conflicts under the 128-byte swizzle.
-            const int DB = warp - 10, u = lane & 7, tq = lane >> 3;
+            const int u = lane & 7, tq = lane >> 3;
             if (ntiles > 0)
                 ok = __all_sync(0xffffffffu, bounded_wait(&bars[Q_READY], 0, abort_flag, status, 0x640));   // (Q has left the V^T ring)
             for (int j = 0; j < ntiles && ok; ++j) {
@@ -275,10 +319,12 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 ok = __all_sync(0xffffffffu, bounded_wait(&bars[V_FULL + r], (j / VR) & 1, abort_flag, status, 0x642));
                 if (ok) ok = __all_sync(0xffffffffu, bounded_wait(&bars[VT_EMPTY + s], ((j / VS) & 1) ^ 1, abort_flag, status, 0x643));
                 if (!ok) break;
-                const uint32_t vr = sb + OFF_VR + r * TILE + DB * PANEL;
+                // 32 x 32 squares (DB: of the features, KB: of the keys) in turn over the two warps
 #pragma unroll
-                for (int KB = 0; KB < 2; ++KB) {
-                    const uint32_t vth = sb + OFF_VTH + s * TILE + KB * PANEL, vtl = sb + OFF_VTL + s * TILE + KB * PANEL;
+                for (int sq = 0; sq < (D / 32) * (BN / 32); sq += 2) {
+                    const int DB = D == 32 ? 0 : D == 64 ? warp - 10 : sq + warp - 10, KB = D == 32 ? warp - 10 : D == 64 ? sq / 2 : 0;
+                    const uint32_t vr = sb + OFF_VR + r * TILE + DB * PANEL;
+                    const uint32_t vth = sb + OFF_VTH + s * TILE + KB * LY::VT_PANEL, vtl = sb + OFF_VTL + s * TILE + KB * LY::VT_PANEL;
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         const int dbc = u ^ (tq + 4 * i);         // feature block (chunk) within the panel; key block = u
@@ -293,8 +339,10 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         for (int c = 0; c < 4; ++c) {
                             const int drow = 32 * DB + 4 * dbc + c;
                             const uint32_t off = drow * 128 + ((u ^ (drow & 7)) << 4);
-                            sts128(vth + off, make_uint4(in[0][c] & HI_MASK, in[1][c] & HI_MASK, in[2][c] & HI_MASK, in[3][c] & HI_MASK));
-                            sts128(vtl + off, make_uint4(lo_of(in[0][c]), lo_of(in[1][c]), lo_of(in[2][c]), lo_of(in[3][c])));
+                            uint4 h, l;
+                            split4<NEAR>(make_uint4(in[0][c], in[1][c], in[2][c], in[3][c]), h, l);
+                            sts128(vth + off, h);
+                            sts128(vtl + off, l);
                         }
                     }
                 }
@@ -320,23 +368,26 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const int nrow_min = __shfl_sync(0xffffffffu, nrow, 0);
         if (ntiles > 0) {
             // Q row -> TMEM, scaled by scale * log2(e) and split: the logits arrive in base-2 units
-            // (each softmax group moves one 32-feature panel of the tile)
+            // (the softmax groups take turns at the 32-feature panels of the tile)
             ok = __all_sync(0xffffffffu, bounded_wait(&bars[Q_FULL], 0, abort_flag, status, 0x650));
             if (ok) {
-                uint32_t hi[32], lo[32];
 #pragma unroll
-                for (int ch = 0; ch < 8; ++ch) {
-                    const uint4 v = lds128(sb + OFF_VTH + g * (BM * 128) + r * 128 + ((ch ^ (r & 7)) << 4));
-                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                for (int pn = g; pn < D / 32; pn += 2) {
+                    uint32_t hi[32], lo[32];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const uint32_t x = __float_as_uint(__uint_as_float(w[e]) * scale_log2e);
-                        hi[ch * 4 + e] = x & HI_MASK;
-                        lo[ch * 4 + e] = lo_of(x);
+                    for (int ch = 0; ch < 8; ++ch) {
+                        const uint4 v = lds128(sb + OFF_VTH + pn * (BM * 128) + r * 128 + ((ch ^ (r & 7)) << 4));
+                        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const uint32_t x = __float_as_uint(__uint_as_float(w[e]) * scale_log2e);
+                            hi[ch * 4 + e] = hi_of<NEAR>(x);
+                            lo[ch * 4 + e] = lo_of(x, hi[ch * 4 + e]);
+                        }
                     }
+                    tmem_st_x32(tl + QH_COL + pn * 32, hi);
+                    tmem_st_x32(tl + QL_COL + pn * 32, lo);
                 }
-                tmem_st_x32(tl + QH_COL + g * 32, hi);
-                tmem_st_x32(tl + QL_COL + g * 32, lo);
                 tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
@@ -347,13 +398,15 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             ok = __all_sync(0xffffffffu, bounded_wait(&bars[PV_FULL + g], (k >> 1) & 1, abort_flag, status, 0x660 + g));
             if (!ok) return;
             tc_fence_after();
+            constexpr int CH = D == 128 ? 16 : 32;           // (128 outputs leave few registers)
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t pv[32];
-                tmem_ld_x32(tl + PV_COL + 64 * g + c * 32, pv);
+            for (int c = 0; c < D; c += CH) {
+                uint32_t pv[CH];
+                if constexpr (CH == 32) tmem_ld_x32(tl + PV_COL + (LY::PVS - 1) * D * g + c, pv);
+                else                    tmem_ld_x16(tl + PV_COL + (LY::PVS - 1) * D * g + c, pv);
                 tc_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 32; ++i) o[c * 32 + i] = fmaf(o[c * 32 + i], alpha_prev, __uint_as_float(pv[i]));
+                for (int i = 0; i < CH; ++i) o[c + i] = fmaf(o[c + i], alpha_prev, __uint_as_float(pv[i]));
             }
             tc_fence_before();
             __syncwarp();
@@ -367,26 +420,26 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             ok = __all_sync(0xffffffffu, bounded_wait(&bars[S_FULL + g], (j >> 1) & 1, abort_flag, status, 0x670 + g));
             if (!ok) break;
             tc_fence_after();
-            uint32_t s[64];
-            tmem_ld_x32(tl + S_COL + 64 * g, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-            tmem_ld_x32(tl + S_COL + 64 * g + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+            uint32_t s[BN];
+#pragma unroll
+            for (int c = 0; c < BN; c += 32) tmem_ld_x32(tl + S_COL + BN * g + c, *reinterpret_cast<uint32_t(*)[32]>(&s[c]));
             tc_wait_ld();
             const int col0 = j * BN;
             const int nvalid = nrow > col0 ? (nrow - col0 < BN ? nrow - col0 : BN) : 0;   // per row
             if (col0 + BN > nrow_min) {                      // (warp-uniform) some row has masked keys in this step
 #pragma unroll
-                for (int i = 0; i < 64; ++i) if (i >= nvalid) s[i] = __float_as_uint(-INFINITY);
+                for (int i = 0; i < BN; ++i) if (i >= nvalid) s[i] = __float_as_uint(-INFINITY);
             }
             float e0 = __uint_as_float(s[0]), e1 = __uint_as_float(s[1]), e2 = __uint_as_float(s[2]), e3 = __uint_as_float(s[3]);
 #pragma unroll
-            for (int i = 4; i < 60; i += 8) {
+            for (int i = 4; i < BN - 4; i += 8) {
                 e0 = max3(e0, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
                 e1 = max3(e1, __uint_as_float(s[i + 2]), __uint_as_float(s[i + 3]));
                 e2 = max3(e2, __uint_as_float(s[i + 4]), __uint_as_float(s[i + 5]));
                 e3 = max3(e3, __uint_as_float(s[i + 6]), __uint_as_float(s[i + 7]));
             }
-            e0 = max3(e0, __uint_as_float(s[60]), __uint_as_float(s[61]));
-            e1 = max3(e1, __uint_as_float(s[62]), __uint_as_float(s[63]));
+            e0 = max3(e0, __uint_as_float(s[BN - 4]), __uint_as_float(s[BN - 3]));
+            e1 = max3(e1, __uint_as_float(s[BN - 2]), __uint_as_float(s[BN - 1]));
             const float m_new = fmaxf(m, fmaxf(fmaxf(e0, e1), fmaxf(e2, e3)));
             // (a row that has seen no valid key yet has no maximum: 0 stands in, its weights are 2^-inf = 0)
             const float m_use = m_new == -INFINITY ? 0.f : m_new;
@@ -395,7 +448,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const uint64_t neg_m2 = pack2(-m_use, -m_use);
             uint64_t lsum0 = 0ull, lsum1 = 0ull;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < BN / 16; ++c) {
                 uint32_t hi[16], lo[16];
 #pragma unroll
                 for (int i = 0; i < 16; i += 2) {
@@ -412,11 +465,11 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     const uint32_t p = hi[i];
-                    hi[i] = p & HI_MASK;
-                    lo[i] = __float_as_uint(__uint_as_float(p) - __uint_as_float(hi[i]));
+                    hi[i] = hi_of<NEAR>(p);
+                    lo[i] = lo_of(p, hi[i]);
                 }
-                tmem_st_x16(tl + S_COL + 64 * g + c * 16, hi);      // P_hi over the logits
-                tmem_st_x16(tl + PL_COL + 64 * g + c * 16, lo);
+                tmem_st_x16(tl + S_COL + BN * g + c * 16, hi);      // P_hi over the logits
+                tmem_st_x16(tl + PL_COL + BN * g + c * 16, lo);
             }
             float l0, l1, l2, l3;
             unpack2(lsum0, l0, l1);
@@ -439,7 +492,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         // Merge of the two streams (both have passed their last P V, so every product that read the K rings
         // has completed and no copy into them is in flight: the scratch lies over them).
-        float* scratch = reinterpret_cast<float*>(base + OFF_KH) + r * MERGE_STRIDE;
+        float* scratch = reinterpret_cast<float*>(base + OFF_KH) + r * LY::MERGE_STRIDE;
         if (g == 1) {
 #pragma unroll
             for (int v = 0; v < D / 4; ++v)
@@ -473,8 +526,8 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// fp32 tensor [BH, N, 64] viewed as 3-D {64, N, BH}; box = 32 floats x rows x 1 (one 128-byte-swizzled panel).
-bool make_map_f32(CUtensorMap* m, const void* ptr, int BH, int N, int box_rows) {
+// fp32 tensor [BH, N, D] viewed as 3-D {D, N, BH}; box = 32 floats x rows x 1 (one 128-byte-swizzled panel).
+bool make_map_f32(CUtensorMap* m, const void* ptr, int BH, int N, int D, int box_rows) {
     EncodeTiledFn enc = get_encode_fn();
     if (!enc) return false;
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(BH)};
@@ -486,26 +539,35 @@ bool make_map_f32(CUtensorMap* m, const void* ptr, int BH, int N, int box_rows) 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+template <int D>
+int launch(const Problem& p, cudaStream_t st) {
+    using LY = Layout<D>;
+    CUtensorMap tmQ, tmK, tmV;
+    const int BH = p.B * p.H, slabs = (p.Nq + BM - 1) / BM;
+    if (static_cast<int64_t>(slabs) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
+    if (!make_map_f32(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map_f32(&tmK, p.K, BH, p.Nk, D, LY::BN) ||
+        !make_map_f32(&tmV, p.V, BH, p.Nk, D, LY::BN))
+        return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_tf32_kernel<D>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+    // without the causal mask the tiles of a head run side by side and share K and V in L2; with it, those of as many heads as
+    // fit L2 together (48 MB of K and V) go longest first: what is left at the end are the short ones
+    const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 8);
+    const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
+    fused_tf32_kernel<D><<<slabs * BH, THREADS, LY::SMEM_BYTES, st>>>(
+        tmQ, tmK, tmV, static_cast<float*>(p.O), BH, p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
+        p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status, p.lse);
+    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
 }  // namespace
 
 bool tf32_applies(const Problem& p) {
-    return p.dtype == FLAT_DTYPE_F32 && p.d == 64 && !p.bias && !p.block_mask;
+    return p.dtype == FLAT_DTYPE_F32 && (p.d == 32 || p.d == 64 || p.d == 128) && !p.bias && !p.block_mask;
 }
 
 int launch_fused_tf32(const Problem& p, cudaStream_t st) {
     if (!tf32_applies(p)) return FLAT_ERR_UNSUPPORTED;
-    CUtensorMap tmQ, tmK, tmV;
-    const int BH = p.B * p.H;
-    if (BH > 65535) return FLAT_ERR_SHAPE;      // (grid y)
-    if (!make_map_f32(&tmQ, p.Q, BH, p.Nq, BM) || !make_map_f32(&tmK, p.K, BH, p.Nk, BN) ||
-        !make_map_f32(&tmV, p.V, BH, p.Nk, BN))
-        return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_tf32_kernel>(SMEM_BYTES)) return FLAT_ERR_CUDA;
-    dim3 grid((p.Nq + BM - 1) / BM, BH);
-    fused_tf32_kernel<<<grid, THREADS, SMEM_BYTES, st>>>(tmQ, tmK, tmV, static_cast<float*>(p.O), p.H, p.Nq, p.Nk,
-                                                         p.scale * 1.4426950408889634f, p.k_valid_len,
-                                                         p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse);
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    return p.d == 32 ? launch<32>(p, st) : p.d == 64 ? launch<64>(p, st) : launch<128>(p, st);
 }
 
 }  // namespace flat

@@ -1,0 +1,65 @@
+"""fp32 tensors with head sizes 32 and 128 (split-tf32 products) at the edges of their key steps and query tiles, against the oracle
+and against the FFMA kernel; masks, lse, values at the ends of the fp32 range."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def run(api, Q, K, V, scale, variant=0, vl=None, causal=False):
+    Qt, Kt, Vt = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (Q, K, V))
+    O = torch.full(Qt.shape, float("nan"), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    lse = torch.full(Qt.shape[:3], float("nan"), device="cuda")
+    api.flat_attn_fwd_ex(Qt, Kt, Vt, O, scale, k_valid_len=None if vl is None else torch.from_numpy(vl).cuda(), status=status,
+                         variant=variant, causal=causal, lse=lse)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    return O.double().cpu().numpy(), lse.double().cpu().numpy()
+
+
+@pytest.mark.parametrize("d", [32, 128])
+@pytest.mark.parametrize("Nk", [1, 31, 32, 33, 63, 64, 65, 96, 128, 129, 333])
+def test_edges(d, Nk):
+    from paper_2107_06419_b200 import api
+    for Nq, causal, vl, scale in ((1, False, None, d ** -0.5), (129, True, None, d ** -0.5), (300, False, [Nk, Nk // 2], -d ** -0.5)):
+        rng = np.random.default_rng(Nq + 7 * Nk + d)
+        Q, K, V = (rng.standard_normal((2, 3, n, d)).astype(np.float32) for n in (Nq, Nk, Nk))
+        vl = None if vl is None else np.array(vl, dtype=np.int32)
+        ref = oracle.attention(Q, K, V, scale, valid_len=vl, causal=causal, want_lse=True)
+        O, lse = run(api, Q, K, V, scale, vl=vl, causal=causal)
+        assert api.flat_attn_last_variant() == api.FLAT_VARIANT_TF32
+        F, _ = run(api, Q, K, V, scale, variant=api.FLAT_VARIANT_SIMT, vl=vl, causal=causal)
+        live = np.isfinite(ref["LSE"])
+        assert np.all(O[~live] == 0.0) and np.all(np.isneginf(lse[~live]))
+        # a logit |q . k| scale is off by at most 2^-20 of sum |q k| scale (three products: 2^-22 dropped, 2^-22 for x_lo as a tf32
+        # number, and the rounding of d sums), a weight by that much in base e, the output by twice that over the largest |v|
+        logit = 2.0 ** -20 * abs(scale) * np.abs(Q).sum(-1).max() * np.abs(K).max()
+        bound = 2 * logit * np.abs(V).max() + 2.0 ** -20 * np.abs(V).max()
+        assert np.max(np.abs(O - ref["O"])) <= bound
+        assert np.max(np.abs(lse[live] - ref["LSE"][live]), initial=0.0) <= logit + 2e-6
+        # on the whole no less exact than the FFMA kernel: its error, and one rounding of the operands to 23 bits
+        rms = lambda e: float(np.sqrt(np.mean(e * e)))
+        assert rms(O - ref["O"]) <= 1.5 * rms(F - ref["O"]) + 2.0 ** -23 * np.abs(V).max() / 4
+
+
+@pytest.mark.parametrize("d", [32, 128])
+def test_ends_of_the_range(d):
+    from paper_2107_06419_b200 import api
+    rng = np.random.default_rng(d)
+    Q, K = (rng.standard_normal((1, 1, n, d)).astype(np.float32) for n in (40, 70))
+    V = rng.standard_normal((1, 1, 70, d)).astype(np.float32)
+    V[..., 0] = np.finfo(np.float32).max                                  # a mean of the largest number
+    V[..., 1] = 1e-38
+    V[..., 2] = 0.0
+    O, _ = run(api, Q, K, V, d ** -0.5)
+    ref = oracle.attention(Q, K, V, d ** -0.5)["O"]
+    assert np.all(np.isfinite(O[..., 1:])) and np.all(O[..., 2] == 0.0)
+    # (the sum of weights in fp32 may pass the largest number by a rounding)
+    big = O[..., 0]
+    assert np.all((np.abs(big / ref[..., 0] - 1) <= 1e-5) | np.isposinf(big))
+    assert np.max(np.abs(O[..., 1] - ref[..., 1])) <= 2.0 ** -10 * 1e-38 + 1e-44
+    assert np.max(np.abs(O[..., 3:] - ref[..., 3:])) <= 2e-5
