@@ -1,7 +1,7 @@
 // Fused Logit-Softmax-Attend for d = 128 (bf16 in, fp32 accumulate, bf16 out): two query tiles of 128 rows per CTA, keys in
 // steps of 64 with the logits of the step after next computed ahead.
 //
-// Paper mapping (Section 5, 5.1, 5.2): shared outer loops = (batch, head) and a slab of 256 query rows (R-granularity);
+// Paper mapping (Section 5, 5.1, 5.2): shared outer loops = items of (batch, head) and a slab of 256 query rows (R-granularity);
 // Logit and Attend interleaved over the key steps with the streaming softmax between them (a reference maximum and a
 // running sum replace the paper's full-row slice on chip; same function).
 //
@@ -21,6 +21,7 @@
 // TMEM columns: S(t, b) 128 t + 64 b (b = step parity), P over the first 32 of them, O_t 256 + 128 t.
 // The softmax takes no row maximum after the first step: any reference gives the exact softmax, and a step whose row sum
 // passes 2^40 is redone with a fresh maximum.  One exponential in four goes through a polynomial on the FMA pipe.
+// MULTI: a CTA walks over items (batch, head, slab of 256 rows); the rings and barriers go on from one to the next.
 // VL: packed batches (Q, O [total_q, H, d], K, V [total_k, H, d]), a CTA per (sequence, head, slab of the longest sequence).
 // Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
@@ -54,12 +55,13 @@ __host__ __device__ constexpr uint32_t O_COL(int t) { return 256u + 128u * t; }
 // S_FULL / P_FULL / PV_DONE [tile][step parity], each once every second step.  (One PV_DONE a tile is not enough: a warp ahead of
 // the others of its tile has its last logits when O += P V of the third last step is done, and would take that one's parity for
 // the last one's.)  B_FULL / B_EMPTY [step parity][tile]: the bias tile / the four softmax warps of the tile have read it.
+// Q_EMPTY / O_FREE [tile], once an item: its logit MMAs are done with the Q tile / its four softmax warps have read the output.
 template <bool BT> struct Layout {
     static constexpr int KS = BT ? 3 : 5, VS = KS;
     static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES + (BT ? 4 * BIAS_BYTES : 0);
     static constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
     static constexpr int Q_FULL = 0, K_FULL = 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS,
-                         P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, B_FULL = PV_DONE + 4, B_EMPTY = B_FULL + 4, NUM_BARS = B_EMPTY + 4;
+                         P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, B_FULL = PV_DONE + 4, B_EMPTY = B_FULL + 4, Q_EMPTY = B_EMPTY + 4, O_FREE = Q_EMPTY + 2, NUM_BARS = O_FREE + 2;
     static_assert(SMEM_BYTES <= 232448 && NUM_BARS * 8 + 8 <= 512, "shared memory");
 };
 
@@ -127,7 +129,12 @@ __device__ __forceinline__ float row_extreme(const uint32_t (&s)[BN], bool small
 }
 
 // BIAS: the bias tiles (bf16, rows on 16-byte boundaries) come through TMA, one per query tile and step, two ahead.
-template <bool VL, bool BIAS>
+struct Item {
+    int bh, row0, n, nsteps, coff;                       // n: keys that any row of the slab sees; coff: Nk - Nq (2^30: no causal mask)
+    int head, q_tok0, k_tok0, q_rows;                    // (packed batches)
+};
+
+template <bool VL, bool BIAS, bool MULTI>
 __global__ void __launch_bounds__(THREADS, 1)
 fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                   __nv_bfloat16* __restrict__ O, int BH, int H, int Nq, int Nk, float scale_log2e, const int32_t* __restrict__ valid_len,
@@ -147,30 +154,48 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    int bh, row0, n = Nk;
-    int head = 0, q_tok0 = 0, k_tok0 = 0, q_rows = 0;    // (packed batches only)
+    // The CTA's r-th item: (batch, head, slab of 256 rows). (Packed batches: one.)
+    auto get_item = [&](int r, Item& it) -> bool {
+        if (!MULTI && r > 0) return false;
+        it.n = Nk;
+        it.coff = coff;
+        if (VL) {
+            // the slabs of a sequence side by side; under the causal mask the last slabs (the longest) of all sequences first
+            it.bh = group ? blockIdx.x : blockIdx.y;
+            it.row0 = static_cast<int>(group ? gridDim.y - 1 - blockIdx.y : blockIdx.x) * (2 * BM);
+            const int s = it.bh / H;
+            it.head = it.bh - s * H;
+            const int q0 = cu_q[s], ql = cu_q[s + 1] - q0, k0 = cu_k[s], kl = cu_k[s + 1] - k0;
+            if (it.row0 >= ql) return false;
+            it.q_tok0 = q0 + it.row0; it.k_tok0 = k0; it.q_rows = ql - it.row0;
+            it.n = kl < 0 ? 0 : kl;
+            if (coff < (1 << 29)) it.coff = kl - ql;
+        } else {
+            // `group` heads at a time, their slabs side by side, the longest first under the causal mask; CTAs with several
+            // items take them forth and back
+            const unsigned at0 = r * gridDim.x + ((r & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+            const int slabs = (Nq + 2 * BM - 1) / (2 * BM), per = group * slabs;
+            if (at0 >= static_cast<unsigned>(BH * slabs)) return false;
+            const int pos = at0;
+            const int first = pos / per * group, heads = BH - first < group ? BH - first : group, at = pos % per;
+            it.bh = first + at % heads;
+            it.row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * (2 * BM);
+            if (valid_len) { const int v = valid_len[it.bh / H]; it.n = v < 0 ? 0 : (v > Nk ? Nk : v); }
+        }
+        // Causal mask (coff = Nk - Nq; 2^30 = none): row r sees keys j < r + 1 + coff, so the last row bounds the slab's keys
+        const long long lim = static_cast<long long>(it.row0) + 2 * BM + it.coff;
+        if (lim < it.n) it.n = lim < 0 ? 0 : static_cast<int>(lim);
+        it.nsteps = (it.n + BN - 1) / BN;
+        return true;
+    };
     if (VL) {
-        // the slabs of a sequence side by side; under the causal mask the last slabs (the longest) of all sequences first
-        bh = group ? blockIdx.x : blockIdx.y;
-        row0 = static_cast<int>(group ? gridDim.y - 1 - blockIdx.y : blockIdx.x) * (2 * BM);
-        const int s = bh / H;
-        head = bh - s * H;
-        const int q0 = cu_q[s], ql = cu_q[s + 1] - q0, k0 = cu_k[s], kl = cu_k[s + 1] - k0;
-        if (row0 >= ql) return;                          // (the whole CTA: nothing is set up yet)
-        q_tok0 = q0 + row0; k_tok0 = k0; q_rows = ql - row0;
-        n = kl < 0 ? 0 : kl;
-        if (coff < (1 << 29)) coff = kl - ql;
-    } else {
-        // `group` heads at a time, their slabs side by side, the longest first under the causal mask
-        const int slabs = (Nq + 2 * BM - 1) / (2 * BM), per = group * slabs, first = static_cast<int>(blockIdx.x) / per * group;
-        const int heads = BH - first < group ? BH - first : group, at = static_cast<int>(blockIdx.x) % per;
-        bh = first + at % heads;
-        row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * (2 * BM);
+        Item it;
+        if (!get_item(0, it)) return;                    // (the whole CTA: nothing is set up yet)
     }
 
     if (threadIdx.x == 256) {
         for (int i = 0; i < LY::NUM_BARS; ++i)
-            mbar_init(&bars[i], (i >= LY::P_FULL && i < LY::PV_DONE) || i >= LY::B_EMPTY ? 4
+            mbar_init(&bars[i], (i >= LY::P_FULL && i < LY::PV_DONE) || (i >= LY::B_EMPTY && i < LY::Q_EMPTY) || i >= LY::O_FREE ? 4
                                 : (i >= LY::K_EMPTY && i < LY::V_FULL) || (i >= LY::V_EMPTY && i < LY::S_FULL) ? 2 : 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -184,76 +209,79 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (!VL) {
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
     }
     const uint32_t tmem = *tmem_slot;
-    {
-        // Causal mask (coff = Nk - Nq; 2^30 = none): row r sees keys j < r + 1 + coff, so the last row bounds the CTA's keys
-        const long long lim = static_cast<long long>(row0) + 2 * BM + coff;
-        if (lim < n) n = lim < 0 ? 0 : static_cast<int>(lim);
-    }
-    const int nsteps = (n + BN - 1) / BN;
     const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         if (warp == 8) {
             // ------------------------------------------------------------ TMA producer
-            if (lane == 0 && nsteps > 0) {
+            if (lane == 0) {
                 prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
                 bool ok = true;
-                int k_issued = 0, v_issued = 0, b_issued = 0;
+                int q_issued[2] = {0, 0}, k_issued = 0, v_issued = 0, b_issued = 0;
+                Item it;
+                int J0 = 0, q = 0;                       // key steps / items with keys so far
                 auto load_q = [&](int t) {
+                    if (MULTI) ok = ok && bounded_wait_s(bars_s + 8 * (LY::Q_EMPTY + t), (q & 1) ^ 1, abort_s, status, 0xa40 + t);
+                    if (!ok) return;
                     mbar_arrive_expect_tx(&bars[LY::Q_FULL + t], Q_BYTES);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
-                        tma_load_3d(Qs + t * Q_BYTES + c * BM * 128, &tmQ, &bars[LY::Q_FULL + t], c * 64, VL ? head : row0 + t * BM, VL ? q_tok0 + t * BM : bh);
+                        tma_load_3d(Qs + t * Q_BYTES + c * BM * 128, &tmQ, &bars[LY::Q_FULL + t], c * 64, VL ? it.head : it.row0 + t * BM, VL ? it.q_tok0 + t * BM : it.bh);
+                    q_issued[t] = q + 1;
                 };
                 auto load_k = [&](int j) {
-                    const int s = j % KS;
-                    ok = bounded_wait_s(bars_s + 8 * (LY::K_EMPTY + s), ((j / KS) & 1) ^ 1, abort_s, status, 0xa00 + s);
+                    const int J = J0 + j, s = J % KS;
+                    ok = ok && bounded_wait_s(bars_s + 8 * (LY::K_EMPTY + s), ((J / KS) & 1) ^ 1, abort_s, status, 0xa00 + s);
                     if (!ok) return;
                     mbar_arrive_expect_tx(&bars[LY::K_FULL + s], KV_BYTES);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
-                        tma_load_3d(Ks + s * KV_BYTES + c * BN * 128, &tmK, &bars[LY::K_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
-                    k_issued = j + 1;
+                        tma_load_3d(Ks + s * KV_BYTES + c * BN * 128, &tmK, &bars[LY::K_FULL + s], c * 64, VL ? it.head : j * BN, VL ? it.k_tok0 + j * BN : it.bh);
+                    k_issued = J + 1;
                 };
                 auto load_v = [&](int j) {
-                    const int s = j % VS;
-                    ok = bounded_wait_s(bars_s + 8 * (LY::V_EMPTY + s), ((j / VS) & 1) ^ 1, abort_s, status, 0xa10 + s);
+                    const int J = J0 + j, s = J % VS;
+                    ok = ok && bounded_wait_s(bars_s + 8 * (LY::V_EMPTY + s), ((J / VS) & 1) ^ 1, abort_s, status, 0xa10 + s);
                     if (!ok) return;
                     mbar_arrive_expect_tx(&bars[LY::V_FULL + s], KV_BYTES);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
-                        tma_load_3d(Vs + s * KV_BYTES + c * BN * 128, &tmV, &bars[LY::V_FULL + s], c * 64, VL ? head : j * BN, VL ? k_tok0 + j * BN : bh);
-                    v_issued = j + 1;
+                        tma_load_3d(Vs + s * KV_BYTES + c * BN * 128, &tmV, &bars[LY::V_FULL + s], c * 64, VL ? it.head : j * BN, VL ? it.k_tok0 + j * BN : it.bh);
+                    v_issued = J + 1;
                 };
                 auto load_bias = [&](int j) {            // of both tiles
+                    const int J = J0 + j;
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
-                        const int s = 2 * (j & 1) + t;
-                        ok = ok && bounded_wait_s(bars_s + 8 * (LY::B_EMPTY + s), ((j >> 1) & 1) ^ 1, abort_s, status, 0xa18 + t);
+                        const int s = 2 * (J & 1) + t;
+                        ok = ok && bounded_wait_s(bars_s + 8 * (LY::B_EMPTY + s), ((J >> 1) & 1) ^ 1, abort_s, status, 0xa18 + t);
                         if (!ok) return;
                         mbar_arrive_expect_tx(&bars[LY::B_FULL + s], BIAS_BYTES);
-                        tma_load_4d(Bs + s * BIAS_BYTES, &tmBias, &bars[LY::B_FULL + s], j * BN, row0 + t * BM, bias_heads ? bh % H : 0, bias_batches ? bh / H : 0);
-                        b_issued = 2 * j + t + 1;
+                        tma_load_4d(Bs + s * BIAS_BYTES, &tmBias, &bars[LY::B_FULL + s], j * BN, it.row0 + t * BM, bias_heads ? it.bh % H : 0, bias_batches ? it.bh / H : 0);
+                        b_issued = 2 * J + t + 1;
                     }
                 };
-                load_q(0);
-                load_k(0);
-                load_q(1);
-                if (BIAS) load_bias(0);
-                if (nsteps > 1) load_k(1);
-                if (BIAS && nsteps > 1) load_bias(1);
-                for (int j = 0; j < nsteps && ok; ++j) {
-                    load_v(j);
-                    if (ok && j + 2 < nsteps) load_k(j + 2);
-                    if (BIAS && ok && j > 0 && j + 1 < nsteps) load_bias(j + 1);
+                for (int r = 0; ok && get_item(r, it); ++r) {
+                    if (it.nsteps == 0) continue;
+                    load_q(0);
+                    load_k(0);
+                    load_q(1);
+                    if (BIAS) load_bias(0);
+                    if (it.nsteps > 1) load_k(1);
+                    if (BIAS && it.nsteps > 1) load_bias(1);
+                    for (int j = 0; j < it.nsteps && ok; ++j) {
+                        load_v(j);
+                        if (j + 2 < it.nsteps) load_k(j + 2);
+                        if (BIAS && j > 0 && j + 1 < it.nsteps) load_bias(j + 1);
+                    }
+                    if (MULTI) { J0 += it.nsteps; ++q; }
                 }
                 if (!ok) {
-                    drain_wait(&bars[LY::Q_FULL], 0);
-                    drain_wait(&bars[LY::Q_FULL + 1], 0);
+                    for (int t = 0; t < 2; ++t)
+                        if (q_issued[t] > 0) drain_wait(&bars[LY::Q_FULL + t], (q_issued[t] - 1) & 1);
                     for (int j = k_issued > KS ? k_issued - KS : 0; j < k_issued; ++j) drain_wait(&bars[LY::K_FULL + j % KS], (j / KS) & 1);
                     for (int j = v_issued > VS ? v_issued - VS : 0; j < v_issued; ++j) drain_wait(&bars[LY::V_FULL + j % VS], (j / VS) & 1);
                     if (BIAS)
@@ -263,7 +291,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         } else if (warp <= 10) {
             // ------------------------------------------------------------ MMA issuer of tile t (whole warp walks, one lane issues)
             const int t = warp - 9;
-            if (nsteps > 0) {
+            {
                 constexpr uint32_t IDESC_S = make_idesc_bf16(BM, BN, 0, 0), IDESC_PV = make_idesc_bf16(BM, D, 0, 1);
                 const uint64_t q_desc = make_smem_desc_sw128(smem_u32(Qs) + t * Q_BYTES, 16, 1024);
                 const uint64_t k_desc = make_smem_desc_sw128(smem_u32(Ks), 16, 1024);
@@ -272,7 +300,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 auto wait = [&](int bar, uint32_t parity, int code) {
                     if (ok) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * bar, parity, abort_s, status, code));
                 };
-                auto issue_s = [&](int j) {              // S_t(j) = Q_t K_j^T, then release the K stage
+                auto issue_s = [&](int j, bool last) {   // S_t(j) = Q_t K_j^T, then release the K stage
                     const uint64_t kd = k_desc + static_cast<uint64_t>(((j % KS) * KV_BYTES) >> 4);
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k)
@@ -280,32 +308,42 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                                kd + static_cast<uint64_t>(((k / 4) * (BN * 128) + (k % 4) * 32) >> 4), IDESC_S, k > 0);
                     tc_commit(&bars[LY::S_FULL + 2 * t + (j & 1)]);
                     tc_commit(&bars[LY::K_EMPTY + j % KS]);
+                    if (MULTI && last) tc_commit(&bars[LY::Q_EMPTY + t]);
                 };
-                auto issue_pv = [&](int j) {             // O_t += P_t(j) V_j, then release the V stage
+                auto issue_pv = [&](int j, bool first) { // O_t += P_t(j) V_j, then release the V stage
                     const uint64_t vd = v_desc + static_cast<uint64_t>(((j % VS) * KV_BYTES) >> 4);
 #pragma unroll
                     for (int k = 0; k < BN / 16; ++k)
-                        mma_ts(tmem + O_COL(t), tmem + S_COL(t, j & 1) + k * 8, vd + static_cast<uint64_t>((k * 2048) >> 4), IDESC_PV, (j > 0 || k > 0));
+                        mma_ts(tmem + O_COL(t), tmem + S_COL(t, j & 1) + k * 8, vd + static_cast<uint64_t>((k * 2048) >> 4), IDESC_PV, (!first || k > 0));
                     tc_commit(&bars[LY::PV_DONE + 2 * t + (j & 1)]);
                     tc_commit(&bars[LY::V_EMPTY + j % VS]);
                 };
-                wait(LY::Q_FULL + t, 0, 0xa20);
-                for (int j = 0; j < 2 && j < nsteps; ++j) {
-                    wait(LY::K_FULL + j, 0, 0xa21);
-                    tc_fence_after();
-                    if (ok && elect_one()) issue_s(j);
-                    __syncwarp();
-                }
-                for (int j = 0; j < nsteps && ok; ++j) {
-                    const bool more = j + 2 < nsteps;
-                    wait(LY::V_FULL + j % VS, (j / VS) & 1, 0xa22);
-                    if (more) wait(LY::K_FULL + (j + 2) % KS, ((j + 2) / KS) & 1, 0xa23);
-                    wait(LY::P_FULL + 2 * t + (j & 1), (j >> 1) & 1, 0xa24);
-                    if (!ok) break;
-                    tc_fence_after();
-                    // (S(j + 2) overwrites P(j): it goes behind the MMAs that read it)
-                    if (elect_one()) { issue_pv(j); if (more) issue_s(j + 2); }
-                    __syncwarp();
+                Item it;
+                int J = 0, q = 0;                        // the item's first key step of all; items with keys so far
+                for (int r = 0; ok && get_item(r, it); ++r) {
+                    const int n = it.nsteps;
+                    if (n == 0) continue;
+                    wait(LY::Q_FULL + t, q & 1, 0xa20);
+                    for (int j = 0; j < 2 && j < n; ++j) {
+                        wait(LY::K_FULL + (J + j) % KS, ((J + j) / KS) & 1, 0xa21);
+                        tc_fence_after();
+                        if (ok && elect_one()) issue_s(J + j, j == n - 1);
+                        __syncwarp();
+                    }
+                    for (int j = 0; j < n && ok; ++j) {
+                        const int g = J + j;
+                        const bool more = j + 2 < n;
+                        wait(LY::V_FULL + g % VS, (g / VS) & 1, 0xa22);
+                        if (more) wait(LY::K_FULL + (g + 2) % KS, ((g + 2) / KS) & 1, 0xa23);
+                        if (MULTI && j == 0) wait(LY::O_FREE + t, (q & 1) ^ 1, 0xa25);
+                        wait(LY::P_FULL + 2 * t + (g & 1), (g >> 1) & 1, 0xa24);
+                        if (!ok) break;
+                        tc_fence_after();
+                        // (S(j + 2) overwrites P(j): it goes behind the MMAs that read it)
+                        if (elect_one()) { issue_pv(g, j == 0); if (more) issue_s(g + 2, j + 3 == n); }
+                        __syncwarp();
+                    }
+                    if (MULTI) { J += n; ++q; }
                 }
             }
         }
@@ -313,33 +351,37 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // ------------------------------------------------------------ softmax + epilogue (warps 0-7)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
         const int t = warp >> 2;
-        const int row = row0 + t * BM + (warp & 3) * 32 + lane;
         const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const uint32_t my_bars = bars_s + 8 * (LY::S_FULL + 2 * t);       // S_FULL of the tile; P_FULL and PV_DONE 32 and 64 bytes on
         // (bias) the thread's row of its tile; the logits are scaled as they meet the bias
         const uint32_t brow = smem_u32(Bs) + t * BIAS_BYTES + ((warp & 3) * 32 + lane) * 128;
         const float unit = BIAS ? 1.f : scale_log2e;
         const bool neg_scale = !BIAS && scale_log2e < 0.f;
-        float m_ref = -INFINITY, l = 0.f;
         bool ok = true;
-        const long long rlim = static_cast<long long>(row) + 1 + coff;
+        Item it;
+        int J = 0;                                       // the item's first key step of all
+        for (int r = 0; ok && get_item(r, it); ++r) {
+        const int n = it.n, nsteps = it.nsteps, row = it.row0 + t * BM + (warp & 3) * 32 + lane;
+        float m_ref = -INFINITY, l = 0.f;
+        const long long rlim = static_cast<long long>(row) + 1 + it.coff;
         const int nrow = rlim < n ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : n;
         const int nrow_min = __shfl_sync(0xffffffffu, nrow, 0);
         for (int j = 0; j < nsteps; ++j) {
-            const uint32_t s_addr = tl + S_COL(t, j & 1);
-            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 8 * (j & 1), (j >> 1) & 1, abort_s, status, 0xa30 + t));
+            const int g = J + j;
+            const uint32_t s_addr = tl + S_COL(t, g & 1);
+            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 8 * (g & 1), (g >> 1) & 1, abort_s, status, 0xa30 + t));
             if (!ok) break;
             tc_fence_after();
             uint32_t s[BN];
             tmem_ld_x32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
             tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-            if (BIAS) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * (LY::B_FULL + 2 * (j & 1) + t), (j >> 1) & 1, abort_s, status, 0xa36 + t));
+            if (BIAS) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * (LY::B_FULL + 2 * (g & 1) + t), (g >> 1) & 1, abort_s, status, 0xa36 + t));
             tc_wait_ld();
             if (BIAS) {
                 if (!ok) break;
-                add_bias(s, scale_log2e, brow + (j & 1) * (2 * BIAS_BYTES), lane & 7);
+                add_bias(s, scale_log2e, brow + (g & 1) * (2 * BIAS_BYTES), lane & 7);
                 __syncwarp();
-                if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + 2 * (j & 1) + t));
+                if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + 2 * (g & 1) + t));
             }
             const int col0 = j * BN;
             const bool tail = col0 + BN > nrow_min;      // (warp-uniform) some row has masked keys in this step
@@ -366,7 +408,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     const float alpha = m_new == -INFINITY ? 1.f : ex2_approx(m_ref - m_new);   // 0 on the row's first keys
                     l *= alpha;
                     if (j > 0) {
-                        ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((j - 1) & 1), ((j - 1) >> 1) & 1, abort_s, status, 0xa32 + t));
+                        ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_s, status, 0xa32 + t));
                         if (!ok) break;
                         tc_fence_after();
 #pragma unroll 1                          // (rare; unrolled, its registers made the common path spill: 428 -> 482 us)
@@ -387,28 +429,34 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_s(my_bars + 32 + 8 * (j & 1));
+            if (lane == 0) mbar_arrive_s(my_bars + 32 + 8 * (g & 1));
         }
         if (ok && nsteps > 0)
-            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((nsteps - 1) & 1), ((nsteps - 1) >> 1) & 1, abort_s, status, 0xa34 + t));
+            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((J + nsteps - 1) & 1), ((J + nsteps - 1) >> 1) & 1, abort_s, status, 0xa34 + t));
+        if (MULTI) J += nsteps;
         if (ok) {
             const float inv = l > 0.f ? 1.f / l : 0.f;
             if (!VL && lse && row < Nq)
-                lse[static_cast<int64_t>(bh) * Nq + row] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
+                lse[static_cast<int64_t>(it.bh) * Nq + row] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
             tc_fence_after();
-            __nv_bfloat16* orow = VL ? O + ((static_cast<int64_t>(q_tok0) + (row - row0)) * H + head) * D
-                                     : O + (static_cast<int64_t>(bh) * Nq + row) * D;
+            __nv_bfloat16* orow = VL ? O + ((static_cast<int64_t>(it.q_tok0) + (row - it.row0)) * H + it.head) * D
+                                     : O + (static_cast<int64_t>(it.bh) * Nq + row) * D;
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t r[32];
                 if (nsteps > 0) {
                     tmem_ld_x32(tl + O_COL(t) + c * 32, r);
                     tc_wait_ld();
+                    if (MULTI && c == D / 32 - 1) {      // the next item may write its output
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::O_FREE + t));
+                    }
                 } else {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) r[i] = 0u;      // no valid key: O = 0
                 }
-                if (VL ? row - row0 < q_rows : row < Nq) {
+                if (VL ? row - it.row0 < it.q_rows : row < Nq) {
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
                         uint4 w;
@@ -421,13 +469,14 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
             }
         }
+        }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <bool BIAS>
+template <bool BIAS, bool MULTI>
 int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
     constexpr int SMEM_BYTES = Layout<BIAS>::SMEM_BYTES;
     CUtensorMap tmQ, tmK, tmV;
@@ -435,13 +484,13 @@ int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
     if (static_cast<int64_t>(slabs) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
     if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map(&tmK, p.K, BH, p.Nk, D, BN) || !make_map(&tmV, p.V, BH, p.Nk, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<false, BIAS>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<false, BIAS, MULTI>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
     // without the causal mask the slabs of a head run side by side and share K and V in L2; with it, those of as many heads as
     // fit L2 together (48 MB of K and V) go longest first: what is left at the end are the short ones
     const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 4);
     const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(slabs) * BH);
+    cfg.gridDim = dim3(MULTI ? device_sm_count() : slabs * BH);
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = st;
@@ -450,7 +499,7 @@ int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false, BIAS>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false, BIAS, MULTI>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
                                              p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status,
                                              static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse, tmB, p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
@@ -460,7 +509,20 @@ int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
 
 int launch_fused_d128(const Problem& p, const void* bias_map, cudaStream_t st) {
     if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias_map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
-    return bias_map ? launch<true>(p, *static_cast<const CUtensorMap*>(bias_map), st) : launch<false>(p, CUtensorMap{}, st);
+    // Short items: one CTA per SM that takes them in turn, so that an item's first loads and logits overlap the last one's output
+    // (us, against a CTA per item: B32 H16 128^2 35 -> 27, 256^2 52 -> 46, 512^2 109 -> 94, 768^2 192 -> 177, B8 H16 1024^2 91 ->
+    // 89).  Its key steps are a few per cent slower (H8 16K^2 955 -> 1,030, B2 H16 2048^2 79 -> 80): up to 1024 keys.  Dealt in
+    // advance, so not for items of unknown length (key counts), and under the causal mask, where the hardware's handing out of
+    // the longest first balances better, only with more items per SM than slabs per head (B16 H16 1024^2, 6.9 items and 4 slabs:
+    // 127 -> 116, B32 H16 2048^2, 28 and 8: 638 -> 613; B8 H16 1024^2, 3.5 and 4: 72 -> 75; B4 H16 4096^2, 6.9 and 16: 269 -> 292).
+    const int sms = device_sm_count(), slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
+    const int64_t items = static_cast<int64_t>(slabs) * p.B * p.H;
+    const bool several = items > sms && !p.k_valid_len && (p.causal ? p.Nk <= 2048 && items > static_cast<int64_t>(slabs) * sms : p.Nk <= 1024);
+    if (bias_map) {
+        const CUtensorMap& tmB = *static_cast<const CUtensorMap*>(bias_map);
+        return several ? launch<true, true>(p, tmB, st) : launch<true, false>(p, tmB, st);
+    }
+    return several ? launch<false, true>(p, CUtensorMap{}, st) : launch<false, false>(p, CUtensorMap{}, st);
 }
 
 int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q, const int32_t* cu_k, int num_seqs,
@@ -471,10 +533,10 @@ int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* 
     if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
         !make_map_packed(&tmV, V, total_k, H, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<true, false>>(Layout<false>::SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<true, false, false>>(Layout<false>::SMEM_BYTES)) return FLAT_ERR_CUDA;
     const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535;
     const dim3 grid(group ? num_seqs * H : slabs, group ? slabs : num_seqs * H);
-    fused_d128_kernel<true, false><<<grid, THREADS, Layout<false>::SMEM_BYTES, st>>>(
+    fused_d128_kernel<true, false, false><<<grid, THREADS, Layout<false>::SMEM_BYTES, st>>>(
         tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), num_seqs * H, H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
         causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr);
     return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;

@@ -61,3 +61,26 @@ def test_d128_packed_edges(causal):
         check_bf16(got, ref, "packed d128")
         assert first is None or np.array_equal(got, first)
         first = got
+
+
+@pytest.mark.parametrize("case", [(19, 20, 300, 1, False), (10, 16, 257, 64, False), (10, 16, 256, 130, False), (5, 31, 300, 200, True),
+                                  (13, 12, 100, 333, True)], ids=str)
+def test_d128_several_items_per_cta(case):
+    """More items than SMs: CTAs take several in turn (with one, two and more key steps; rows without keys under the causal mask)."""
+    from paper_2107_06419_b200 import api
+    B, H, Nq, Nk, causal = case
+    rng = np.random.default_rng(Nq + Nk)
+    Qb, Kb, Vb = rand_bits(rng, (B, H, Nq, 128)), rand_bits(rng, (B, H, Nk, 128)), rand_bits(rng, (B, H, Nk, 128))
+    ref = oracle.attention(Qb, Kb, Vb, 0.09, causal=causal, want_lse=True)
+    live = np.isfinite(ref["LSE"])
+    Q, K, V = bf16_tensor(Qb), bf16_tensor(Kb), bf16_tensor(Vb)
+    for _ in range(3):
+        O = torch.full(Q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((B, H, Nq), float("nan"), device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        api.flat_attn_fwd_ex(Q, K, V, O, 0.09, status=status, causal=causal, lse=lse)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        got, lg = bf16_to_f64(O), lse.cpu().numpy()
+        check_bf16(got, ref["O"], "several items")
+        assert np.all(got[~live] == 0.0) and np.all(np.isneginf(lg[~live])) and np.all(np.abs(lg[live] - ref["LSE"][live]) <= 1e-3)
