@@ -485,13 +485,11 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             // this group's last step
             const int last = ntiles - 1 - ((ntiles - 1 - g) & 1);   // largest j < ntiles with j % 2 == g (negative: none)
             if (ok && last >= 0) accumulate(last);
-            // (a single key step leaves the odd group without work: it still waits for that step's products,
-            // which read the K ring, before it touches the scratch below)
-            if (ok && last < 0 && ntiles > 0)
-                ok = __all_sync(0xffffffffu, bounded_wait(&bars[PV_FULL + 0], 0, abort_flag, status, 0x680));
         }
-        // Merge of the two streams (both have passed their last P V, so every product that read the K rings
-        // has completed and no copy into them is in flight: the scratch lies over them).
+        // Merge of the two streams.  The scratch lies over the K rings: the odd group must not write it before the even group has
+        // passed its last P V too (with an odd number of key steps that one's logits are still to be computed from them when the
+        // odd group is done); after that every product has completed and no copy is in flight.
+        asm volatile("bar.sync 1, 256;" ::: "memory");
         float* scratch = reinterpret_cast<float*>(base + OFF_KH) + r * LY::MERGE_STRIDE;
         if (g == 1) {
 #pragma unroll

@@ -63,3 +63,19 @@ def test_ends_of_the_range(d):
     assert np.all((np.abs(big / ref[..., 0] - 1) <= 1e-5) | np.isposinf(big))
     assert np.max(np.abs(O[..., 1] - ref[..., 1])) <= 2.0 ** -10 * 1e-38 + 1e-44
     assert np.max(np.abs(O[..., 3:] - ref[..., 3:])) <= 2e-5
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+def test_odd_number_of_key_steps(d):
+    """The stream of the odd key steps ends before the last even one: many times over, the same results."""
+    from paper_2107_06419_b200 import api
+    rng = np.random.default_rng(d)
+    Nk = 5 * (32 if d == 128 else 64) - 40
+    Q, K, V = (rng.standard_normal((6, 12, n, d)).astype(np.float32) for n in (300, Nk, Nk))
+    ref = oracle.attention(Q, K, V, d ** -0.5)["O"]
+    first = None
+    for _ in range(10):
+        O, _ = run(api, Q, K, V, d ** -0.5)
+        assert np.max(np.abs(O - ref)) <= 2e-5
+        assert first is None or np.array_equal(O, first)
+        first = O
