@@ -68,7 +68,14 @@ int check_params(const flat_attn_params_t* p);
 int launch_fused_simt(const Problem& p, cudaStream_t st);
 int launch_naive(const Problem& p, void* L, void* A, cudaStream_t st);
 int launch_fused_tc(const Problem& p, cudaStream_t st);
-int launch_fused_d128(const Problem& p, const void* bias_map, cudaStream_t st);    // (bf16, d = 128, no pruning map; with a bias its tensor map: {Nk, Nq, heads, batches}, boxes of 64 x 128)
+// A bf16 bias's tensor map (a CUtensorMap): {Nk, Nq, heads, batches} in boxes of 64 x 128, or, shifted_rows >= 0 (the rows in whole
+// groups of eight), as load_shifted_bias wants it in boxes of SHIFTED_WIDTH(d) x 16.
+struct BiasMap {
+    const void* map;
+    int shifted_rows;
+};
+__host__ __device__ constexpr int SHIFTED_WIDTH(int d) { return d == 64 ? 192 : 128; }     // (a key step, 8 columns of rounding, 56 of the phases)
+int launch_fused_d128(const Problem& p, const BiasMap& bias, cudaStream_t st);         // (bf16, d = 128, no pruning map)
 int launch_fused_tc2(const Problem& p, cudaStream_t st);      // (also the tensor-core kernel for calls with a bias)
 // (only_if_resident: sixteen-CTA clusters only when all clusters of the launch can run at the same time; else
 // FLAT_ERR_UNSUPPORTED)
@@ -76,7 +83,7 @@ int launch_fused_tc2_single(const Problem& p, cudaStream_t st, int key_split = 1
 // The same tile worked on by two warpgroups that take alternate key tiles (bf16, d = 64, dense; key_split 1, 2, 4, 8).
 int launch_fused_tc2_halves(const Problem& p, cudaStream_t st, int key_split = 1, bool only_if_resident = false);   // (key_split 1, 2, 4, 8, 16)   // (d = 64; with a block mask also d = 128; key_split 2 / 4: the keys of a tile over a CTA cluster)
 int launch_fused_tc3(const Problem& p, cudaStream_t st);
-int launch_fused_tc3_bias(const Problem& p, const void* bias_map, cudaStream_t st);   // (bias_map: a CUtensorMap)
+int launch_fused_tc3_bias(const Problem& p, const BiasMap& bias, cudaStream_t st);
 // How the last launch_fused_tc3 of this host thread dealt its items (FLAT_SCHEDULE_*; 0 before any).
 extern thread_local int g_last_schedule;
 bool tf32_applies(const Problem& p);               // fp32, d = 64, no bias, no pruning map

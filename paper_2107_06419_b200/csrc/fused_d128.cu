@@ -48,17 +48,17 @@ constexpr int POLY_LANE = 3;         // element index mod 4 that takes the polyn
 constexpr float OVERFLOW_SUM = 1.0995116e12f;   // 2^40
 
 constexpr int Q_BYTES = BM * D * 2, KV_BYTES = BN * D * 2;
-constexpr int BIAS_BYTES = BM * BN * 2;   // a bias tile: 128 rows of 64 values
 __host__ __device__ constexpr uint32_t S_COL(int t, int b) { return 128u * t + 64u * b; }
 __host__ __device__ constexpr uint32_t O_COL(int t) { return 256u + 128u * t; }
-// Ring depths and barriers.  BT: with two bias tiles per query tile, which take the room of two K and two V stages.
+// Ring depths and barriers.  BT: with two bias tiles per query tile (2: one twice as large), which take the room of two K and two V stages.
 // S_FULL / P_FULL / PV_DONE [tile][step parity], each once every second step.  (One PV_DONE a tile is not enough: a warp ahead of
 // the others of its tile has its last logits when O += P V of the third last step is done, and would take that one's parity for
 // the last one's.)  B_FULL / B_EMPTY [step parity][tile]: the bias tile / the four softmax warps of the tile have read it.
 // Q_EMPTY / O_FREE [tile], once an item: its logit MMAs are done with the Q tile / its four softmax warps have read the output.
-template <bool BT> struct Layout {
+template <int BT> struct Layout {
     static constexpr int KS = BT ? 3 : 5, VS = KS;
-    static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES + (BT ? 4 * BIAS_BYTES : 0);
+    static constexpr int BIAS_BYTES = BT == 2 ? BM * SHIFTED_WIDTH(D) * 2 : BM * BN * 2;   // a bias tile: 128 rows of 64 values (2: of 128)
+    static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES + (BT == 2 ? 2 : BT ? 4 : 0) * BIAS_BYTES;
     static constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
     static constexpr int Q_FULL = 0, K_FULL = 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS,
                          P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, B_FULL = PV_DONE + 4, B_EMPTY = B_FULL + 4, Q_EMPTY = B_EMPTY + 4, O_FREE = Q_EMPTY + 2, NUM_BARS = O_FREE + 2;
@@ -100,12 +100,26 @@ __device__ __forceinline__ float exp_store(const uint32_t (&s)[BN], float scale_
 
 // s = s * scale * log2(e) + bias * log2(e), base-2 units; `brow`: shared-window address of the thread's 128-byte row of the bias
 // tile, rx: the row's place in the swizzle.
+// 2: `rx` is what the row is to be shifted by.
+template <int BIAS>
 __device__ __forceinline__ void add_bias(uint32_t (&s)[BN], float scale_log2e, uint32_t brow, int rx) {
     const uint64_t scale2 = pack2(scale_log2e, scale_log2e), log2e2 = pack2(1.4426950408889634f, 1.4426950408889634f);
+    uint32_t two[8];
+    auto piece = [&](int c, uint32_t& w0, uint32_t& w1, uint32_t& w2, uint32_t& w3) {
+        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3) : "r"(brow + ((BIAS == 2 ? c : c ^ rx) << 4)) : "memory");
+    };
+    if (BIAS == 2) piece(0, two[4], two[5], two[6], two[7]);
 #pragma unroll
     for (int c = 0; c < BN / 8; ++c) {
         uint32_t w[4];
-        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + ((c ^ rx) << 4)) : "memory");
+        if (BIAS == 2) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) two[e] = two[4 + e];
+            piece(c + 1, two[4], two[5], two[6], two[7]);
+            shift8(two, rx, w);
+        } else {
+            piece(c, w[0], w[1], w[2], w[3]);
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int i = c * 8 + 2 * e;
@@ -134,14 +148,15 @@ struct Item {
     int head, q_tok0, k_tok0, q_rows;                    // (packed batches)
 };
 
-template <bool VL, bool BIAS, bool MULTI>
+template <bool VL, int BIAS, bool MULTI>
 __global__ void __launch_bounds__(THREADS, 1)
 fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                   __nv_bfloat16* __restrict__ O, int BH, int H, int Nq, int Nk, float scale_log2e, const int32_t* __restrict__ valid_len,
                   int coff, int group, int32_t* status, const int32_t* __restrict__ cu_q, const int32_t* __restrict__ cu_k,
                   float* __restrict__ lse, const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}, int bias_heads = 0,
-                  int bias_batches = 0) {
+                  int bias_batches = 0, const ShiftedBias sb = ShiftedBias{}) {
     using LY = Layout<BIAS>;
+    constexpr int BIAS_BYTES = LY::BIAS_BYTES;
     constexpr int KS = LY::KS, VS = LY::VS;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -188,6 +203,8 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         it.nsteps = (it.n + BN - 1) / BN;
         return true;
     };
+    // (bias, shifted) the slab's first row among all rows of the bias
+    auto bias_row = [&](const Item& it) { return ((bias_batches ? it.bh / H : 0) * (bias_heads ? H : 1) + (bias_heads ? it.bh % H : 0)) * Nq + it.row0; };
     if (VL) {
         Item it;
         if (!get_item(0, it)) return;                    // (the whole CTA: nothing is set up yet)
@@ -256,11 +273,14 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     const int J = J0 + j;
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
-                        const int s = 2 * (J & 1) + t;
-                        ok = ok && bounded_wait_s(bars_s + 8 * (LY::B_EMPTY + s), ((J >> 1) & 1) ^ 1, abort_s, status, 0xa18 + t);
+                        const int s = BIAS == 2 ? t : 2 * (J & 1) + t;
+                        ok = ok && bounded_wait_s(bars_s + 8 * (LY::B_EMPTY + s), ((BIAS == 2 ? J : J >> 1) & 1) ^ 1, abort_s, status, 0xa18 + t);
                         if (!ok) return;
                         mbar_arrive_expect_tx(&bars[LY::B_FULL + s], BIAS_BYTES);
-                        tma_load_4d(Bs + s * BIAS_BYTES, &tmBias, &bars[LY::B_FULL + s], j * BN, it.row0 + t * BM, bias_heads ? it.bh % H : 0, bias_batches ? it.bh / H : 0);
+                        if (BIAS == 2)
+                            load_shifted_bias<SHIFTED_WIDTH(D)>(Bs + s * BIAS_BYTES, &tmBias, &bars[LY::B_FULL + s], bias_row(it) + t * BM, j * BN, Nk);
+                        else
+                            tma_load_4d(Bs + s * BIAS_BYTES, &tmBias, &bars[LY::B_FULL + s], j * BN, it.row0 + t * BM, bias_heads ? it.bh % H : 0, bias_batches ? it.bh / H : 0);
                         b_issued = 2 * J + t + 1;
                     }
                 };
@@ -271,11 +291,11 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     load_q(1);
                     if (BIAS) load_bias(0);
                     if (it.nsteps > 1) load_k(1);
-                    if (BIAS && it.nsteps > 1) load_bias(1);
+                    if (BIAS == 1 && it.nsteps > 1) load_bias(1);
                     for (int j = 0; j < it.nsteps && ok; ++j) {
                         load_v(j);
                         if (j + 2 < it.nsteps) load_k(j + 2);
-                        if (BIAS && j > 0 && j + 1 < it.nsteps) load_bias(j + 1);
+                        if (BIAS && (BIAS == 2 || j > 0) && j + 1 < it.nsteps) load_bias(j + 1);
                     }
                     if (MULTI) { J0 += it.nsteps; ++q; }
                 }
@@ -285,7 +305,9 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     for (int j = k_issued > KS ? k_issued - KS : 0; j < k_issued; ++j) drain_wait(&bars[LY::K_FULL + j % KS], (j / KS) & 1);
                     for (int j = v_issued > VS ? v_issued - VS : 0; j < v_issued; ++j) drain_wait(&bars[LY::V_FULL + j % VS], (j / VS) & 1);
                     if (BIAS)
-                        for (int u = b_issued > 4 ? b_issued - 4 : 0; u < b_issued; ++u) drain_wait(&bars[LY::B_FULL + (u & 3)], (u >> 2) & 1);
+                        for (int u = b_issued > 4 ? b_issued - 4 : 0; u < b_issued; ++u)
+                            if (BIAS == 1) drain_wait(&bars[LY::B_FULL + (u & 3)], (u >> 2) & 1);
+                            else if (u + 2 >= b_issued) drain_wait(&bars[LY::B_FULL + (u & 1)], (u >> 1) & 1);
                 }
             }
         } else if (warp <= 10) {
@@ -354,7 +376,8 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const uint32_t my_bars = bars_s + 8 * (LY::S_FULL + 2 * t);       // S_FULL of the tile; P_FULL and PV_DONE 32 and 64 bytes on
         // (bias) the thread's row of its tile; the logits are scaled as they meet the bias
-        const uint32_t brow = smem_u32(Bs) + t * BIAS_BYTES + ((warp & 3) * 32 + lane) * 128;
+        uint32_t brow = smem_u32(Bs) + t * BIAS_BYTES + ((warp & 3) * 32 + lane) * 128;
+        int rx = lane & 7;
         const float unit = BIAS ? 1.f : scale_log2e;
         const bool neg_scale = !BIAS && scale_log2e < 0.f;
         bool ok = true;
@@ -362,6 +385,12 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         int J = 0;                                       // the item's first key step of all
         for (int r = 0; ok && get_item(r, it); ++r) {
         const int n = it.n, nsteps = it.nsteps, row = it.row0 + t * BM + (warp & 3) * 32 + lane;
+        const int brR = BIAS == 2 ? bias_row(it) + t * BM + (warp & 3) * 32 + lane : 0;
+        const bool own_copy = BIAS == 2 && brR >= sb.full && row < Nq;      // (a row beyond the last whole group of eight)
+        if (BIAS == 2) {
+            brow = smem_u32(Bs) + t * BIAS_BYTES + shifted_row<SHIFTED_WIDTH(D)>(brR, bias_row(it) + t * BM);
+            rx = shifted_by(brR, Nk);
+        }
         float m_ref = -INFINITY, l = 0.f;
         const long long rlim = static_cast<long long>(row) + 1 + it.coff;
         const int nrow = rlim < n ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : n;
@@ -375,13 +404,14 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             uint32_t s[BN];
             tmem_ld_x32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
             tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-            if (BIAS) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * (LY::B_FULL + 2 * (g & 1) + t), (g >> 1) & 1, abort_s, status, 0xa36 + t));
+            if (BIAS) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * (LY::B_FULL + (BIAS == 2 ? t : 2 * (g & 1) + t)), (BIAS == 2 ? g : g >> 1) & 1, abort_s, status, 0xa36 + t));
             tc_wait_ld();
             if (BIAS) {
                 if (!ok) break;
-                add_bias(s, scale_log2e, brow + (g & 1) * (2 * BIAS_BYTES), lane & 7);
+                if (BIAS == 2 && own_copy) copy_bias_row(sb.p + static_cast<int64_t>(brR) * Nk + j * BN, brow + rx, Nk - j * BN < BN ? Nk - j * BN : BN);
+                add_bias<BIAS>(s, scale_log2e, brow + (BIAS == 2 ? 0 : (g & 1) * (2 * BIAS_BYTES)), rx);
                 __syncwarp();
-                if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + 2 * (g & 1) + t));
+                if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + (BIAS == 2 ? t : 2 * (g & 1) + t)));
             }
             const int col0 = j * BN;
             const bool tail = col0 + BN > nrow_min;      // (warp-uniform) some row has masked keys in this step
@@ -476,8 +506,8 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <bool BIAS, bool MULTI>
-int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
+template <int BIAS, bool MULTI>
+int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStream_t st) {
     constexpr int SMEM_BYTES = Layout<BIAS>::SMEM_BYTES;
     CUtensorMap tmQ, tmK, tmV;
     const int BH = p.B * p.H, slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
@@ -501,14 +531,15 @@ int launch(const Problem& p, const CUtensorMap& tmB, cudaStream_t st) {
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false, BIAS, MULTI>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
                                              p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status,
-                                             static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse, tmB, p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0);
+                                             static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse, tmB, p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0,
+                                             ShiftedBias{static_cast<const uint16_t*>(p.bias), shifted_rows});
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
 }  // namespace
 
-int launch_fused_d128(const Problem& p, const void* bias_map, cudaStream_t st) {
-    if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias_map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
+int launch_fused_d128(const Problem& p, const BiasMap& bias, cudaStream_t st) {
+    if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias.map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
     // Short items: one CTA per SM that takes them in turn, so that an item's first loads and logits overlap the last one's output
     // (us, against a CTA per item: B32 H16 128^2 35 -> 27, 256^2 52 -> 46, 512^2 109 -> 94, 768^2 192 -> 177, B8 H16 1024^2 91 ->
     // 89).  Its key steps are a few per cent slower (H8 16K^2 955 -> 1,030, B2 H16 2048^2 79 -> 80): up to 1024 keys.  Dealt in
@@ -518,11 +549,13 @@ int launch_fused_d128(const Problem& p, const void* bias_map, cudaStream_t st) {
     const int sms = device_sm_count(), slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
     const int64_t items = static_cast<int64_t>(slabs) * p.B * p.H;
     const bool several = items > sms && !p.k_valid_len && (p.causal ? p.Nk <= 2048 && items > static_cast<int64_t>(slabs) * sms : p.Nk <= 1024);
-    if (bias_map) {
-        const CUtensorMap& tmB = *static_cast<const CUtensorMap*>(bias_map);
-        return several ? launch<true, true>(p, tmB, st) : launch<true, false>(p, tmB, st);
+    const int sr = bias.shifted_rows;
+    if (bias.map) {
+        const CUtensorMap& tmB = *static_cast<const CUtensorMap*>(bias.map);
+        if (sr >= 0) return several ? launch<2, true>(p, tmB, sr, st) : launch<2, false>(p, tmB, sr, st);
+        return several ? launch<1, true>(p, tmB, sr, st) : launch<1, false>(p, tmB, sr, st);
     }
-    return several ? launch<false, true>(p, CUtensorMap{}, st) : launch<false, false>(p, CUtensorMap{}, st);
+    return several ? launch<0, true>(p, CUtensorMap{}, sr, st) : launch<0, false>(p, CUtensorMap{}, sr, st);
 }
 
 int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q, const int32_t* cu_k, int num_seqs,
@@ -533,10 +566,10 @@ int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* 
     if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
         !make_map_packed(&tmV, V, total_k, H, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<true, false, false>>(Layout<false>::SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<true, 0, false>>(Layout<0>::SMEM_BYTES)) return FLAT_ERR_CUDA;
     const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535;
     const dim3 grid(group ? num_seqs * H : slabs, group ? slabs : num_seqs * H);
-    fused_d128_kernel<true, false, false><<<grid, THREADS, Layout<false>::SMEM_BYTES, st>>>(
+    fused_d128_kernel<true, 0, false><<<grid, THREADS, Layout<0>::SMEM_BYTES, st>>>(
         tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), num_seqs * H, H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
         causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr);
     return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;

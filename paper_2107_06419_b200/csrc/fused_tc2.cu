@@ -820,9 +820,19 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
         if constexpr (NT == 2) {
             // bf16 bias with 16-byte aligned rows: tiles staged through shared memory by TMA, in the half-row kernel (d = 64)
             // or the one with 64-key steps (d = 128: B8 H16 1024^2 244 -> 108 us, B4 H16 4096^2 1,589 -> 612)
+            // rows at any alignment the same way, shifted (ShiftedBias); broken strides, a base that is not aligned itself and
+            // float32 values go on to the kernel below
             const BiasArg ba = bias_arg(p);
             CUtensorMap tmB;
-            if (ba.vec && !ba.f32 && make_bias_map(&tmB, p)) return D == 64 ? launch_fused_tc3_bias(p, &tmB, st) : launch_fused_d128(p, &tmB, st);
+            BiasMap bm{&tmB, -1};
+            const int64_t plane = static_cast<int64_t>(p.Nq) * p.Nk, rows = static_cast<int64_t>(p.Nq) * (p.bias_sh ? p.H : 1) * (p.bias_sb ? p.B : 1);
+            bool staged = ba.vec && !ba.f32 && make_bias_map(&tmB, p);
+            if (!staged && !ba.f32 && (reinterpret_cast<uintptr_t>(p.bias) & 15u) == 0 && p.Nk >= 32 && p.Nk < (1 << 27) && rows >= 8 &&
+                rows < (1 << 30) && (!p.bias_sh || p.bias_sh == plane) && (!p.bias_sb || p.bias_sb == (p.bias_sh ? p.H * plane : plane))) {
+                bm.shifted_rows = static_cast<int>(rows & ~7ll);
+                staged = make_shifted_bias_map(&tmB, p.bias, rows / 8, p.Nk, SHIFTED_WIDTH(D));
+            }
+            if (staged) return D == 64 ? launch_fused_tc3_bias(p, bm, st) : launch_fused_d128(p, bm, st);
         }
         if constexpr (NT == 2) {
             if (!ensure_dynamic_smem<fused_tc2_kernel<D, NT, true>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
@@ -899,7 +909,7 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse);
         return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
     } else {
-        return launch_fused_d128(p, nullptr, st);                 // (two tiles, d = 128, no bias: a kernel of its own, fused_d128.cu)
+        return launch_fused_d128(p, BiasMap{nullptr, -1}, st);                 // (two tiles, d = 128, no bias: a kernel of its own, fused_d128.cu)
     }
 }
 

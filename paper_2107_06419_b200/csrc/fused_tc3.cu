@@ -71,18 +71,20 @@ constexpr unsigned PRODUCER_SLEEP = 400; // ns between the TMA producer's probes
 constexpr int D = 64;                // head size of this kernel
 constexpr int UNITS_MAX = 1024;      // packed batches: most (sequence, slab) units (and sequences) that are sorted (see Sched)
 
-// BT: with a ring of three bias tiles (128 x 128 bf16, two panels of 64 columns), which leaves room for shallower K and V rings.
-template <bool BT> struct Layout {
+// BT: with a ring of three bias tiles (128 x 128 bf16, two panels of 64 columns; 2: one tile of 128 x 192 per query tile), which
+// leaves room for shallower K and V rings.
+template <int BT> struct Layout {
     static constexpr int KS = BT ? 3 : 4;                // K ring depth (S runs 1.5 key steps ahead of P V)
     static constexpr int VS = BT ? 2 : 3;                // V ring depth
-    static constexpr int BIAS_BYTES = BM * BN * 2;
+    static constexpr int BS = BT == 2 ? 2 : BT ? 3 : 0;  // bias stages
+    static constexpr int BIAS_BYTES = BT == 2 ? BM * SHIFTED_WIDTH(D) * 2 : BM * BN * 2;
     static constexpr int SOFT_WARPS = 16;
     static constexpr int THREADS = 32 * SOFT_WARPS + 128;
     static constexpr uint32_t TMEM_COLS = 512;
     static constexpr int Q_BYTES = BM * D * 2;           // one query tile
     static constexpr int KV_BYTES = BN * D * 2;
     static constexpr int BIAS_OFF = 2 * Q_BYTES + (KS + VS) * KV_BYTES;
-    static constexpr int TILE_BYTES = BIAS_OFF + (BT ? 3 * BIAS_BYTES : 0);
+    static constexpr int TILE_BYTES = BIAS_OFF + BS * BIAS_BYTES;
     static constexpr int XCH_BYTES = 2 * 2 * 2 * BM * 4; // [maximum | row sum][tile][half][row] floats
     static constexpr int SMEM_BYTES = TILE_BYTES + XCH_BYTES + 512 + 512 + 1024;   // (.. barriers, the even deal's table, alignment)
     static constexpr int VL_SMEM_BYTES = SMEM_BYTES + UNITS_MAX * 28 + 128;        // (packed batches: the table of units and what sorting it takes)
@@ -100,12 +102,12 @@ template <bool BT> struct Layout {
     static constexpr int S_FULL = V_EMPTY + VS, P_FULL = S_FULL + 6, PV_DONE = P_FULL + 6;
     static constexpr int Q_EMPTY = PV_DONE + 6;          // [2] the item's logit MMAs are done with the Q tile
     // (BT) B_FULL / B_EMPTY [buffer]: the bias tile of tile-step u is in stage u % 3 / the 8 softmax warps of its tile have
-    // read it, phase u / 3: a stage is filled again only behind its EMPTY, so a waiter is never a phase behind
-    static constexpr int B_FULL = Q_EMPTY + 2, B_EMPTY = B_FULL + (BT ? 3 : 0);
-    static constexpr int NUM_BARS = B_EMPTY + (BT ? 3 : 0);
+    // read it, phase u / 3 (2: stage u % 2, phase u / 2): a stage is filled again only behind its EMPTY, so a waiter is never a phase behind
+    static constexpr int B_FULL = Q_EMPTY + 2, B_EMPTY = B_FULL + BS;
+    static constexpr int NUM_BARS = B_EMPTY + BS;
     static_assert(SMEM_BYTES <= 232448 && NUM_BARS * 8 + 8 <= 512, "shared memory");
 };
-using L3 = Layout<false>;
+using L3 = Layout<0>;
 
 __device__ __forceinline__ float half_max(const uint32_t (&s)[HN]) {
     float e0 = __uint_as_float(s[0]), e1 = __uint_as_float(s[1]), e2 = __uint_as_float(s[2]), e3 = __uint_as_float(s[3]);
@@ -236,15 +238,32 @@ __device__ __forceinline__ void exp_pack32(const uint32_t (&r)[32], float scale_
     }
 }
 
+// (bias) the 16-byte piece c of the thread's row; 2: eight values out of two pieces, of which two[4..7] is the first already
+__device__ __forceinline__ void lds_v4(uint32_t (&w)[8], int at, uint32_t addr) {
+    asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[at]), "=r"(w[at + 1]), "=r"(w[at + 2]), "=r"(w[at + 3]) : "r"(addr) : "memory");
+}
+template <int BIAS>
+__device__ __forceinline__ void bias_piece(uint32_t (&two)[8], uint32_t (&w)[4], uint32_t brow, int c, int rx) {
+    if (BIAS == 2) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) two[e] = two[4 + e];
+        lds_v4(two, 4, brow + ((c + 1) << 4));
+        shift8(two, rx, w);
+    } else {
+        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + ((c ^ rx) << 4)) : "memory");
+    }
+}
 // (bias) r = r * scale * log2(e) + bias * log2(e) for 32 logits of a row: base-2 units.  `brow`: shared-window address of
 // the row in its panel of the staged tile; C0: first of its eight 16-byte chunks; rx: the row's place in the swizzle.
-template <int C0>
+template <int C0, int BIAS>
 __device__ __forceinline__ void add_bias32(uint32_t (&r)[32], float scale_log2e, uint32_t brow, int rx) {
     const uint64_t scale2 = pack2(scale_log2e, scale_log2e), log2e2 = pack2(1.4426950408889634f, 1.4426950408889634f);
+    uint32_t two[8];
+    if (BIAS == 2) lds_v4(two, 4, brow + (C0 << 4));
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         uint32_t w[4];
-        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + (((C0 + c) ^ rx) << 4)) : "memory");
+        bias_piece<BIAS>(two, w, brow, C0 + c, rx);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int i = c * 8 + 2 * e;
@@ -257,13 +276,15 @@ __device__ __forceinline__ void add_bias32(uint32_t (&r)[32], float scale_log2e,
     }
 }
 // The same with the reference taken off: x2 = pairs of r * scale + bias * log2(e) + neg_m.
-template <int C0>
+template <int C0, int BIAS>
 __device__ __forceinline__ void scale_bias32(const uint32_t (&r)[32], uint64_t scale2, uint64_t neg_m2, uint32_t brow, int rx, uint64_t (&x2)[16]) {
     const uint64_t log2e2 = pack2(1.4426950408889634f, 1.4426950408889634f);
+    uint32_t two[8];
+    if (BIAS == 2) lds_v4(two, 4, brow + (C0 << 4));
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         uint32_t w[4];
-        asm volatile("ld.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(brow + (((C0 + c) ^ rx) << 4)) : "memory");
+        bias_piece<BIAS>(two, w, brow, C0 + c, rx);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int i = c * 4 + e;
@@ -666,14 +687,15 @@ __device__ __forceinline__ int fill_units(const Sched& sc, uint4* tab, int seqs)
 // the plain kernel: 100 instructions per 64 logits (eight 16-byte loads, unpacking, one packed FMA a pair) in the kernel
 // whose exponent unit, not its issue slots, is the bound.  Before, the bias was read by the kernel with one softmax
 // thread per row (fused_tc2.cu), 6,500 cycles a key step: B8 H16 1024 x 1024 110 us, 70 here; B16 H16 4096 x 4096 2.55 ms, 1.63 here.
-template <bool VL, bool WLSE = false, bool SPLIT = false, bool BIAS = false>
+template <bool VL, bool WLSE = false, bool SPLIT = false, int BIAS = 0>
 __global__ void __launch_bounds__(L3::THREADS, 1)
 fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, int H, int Nq, int Nk,
                  int items, int slabs, float scale_log2e, const int32_t* __restrict__ valid_len, int coff,
                  int32_t* status, int wide_stores, int paired, const int32_t* __restrict__ cu_q,
                  const int32_t* __restrict__ cu_k, float* __restrict__ lse, const EvenDeal ed,
-                 const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}, int bias_heads = 0, int bias_batches = 0) {
+                 const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}, int bias_heads = 0, int bias_batches = 0,
+                 const ShiftedBias sb = ShiftedBias{}) {
     using LY = Layout<BIAS>;
     static_assert(!BIAS || (!VL && !SPLIT), "the bias is read by the plain dense kernel");
     static_assert(!SPLIT || (!VL && !WLSE), "the even deal is built for the plain dense forward kernel only");
@@ -682,6 +704,8 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // one CTA per slot: a slot past the end of its sequence leaves before anything is set up
         if (get_item<VL>(0, sc).skip) return;
     }
+    // (bias, shifted) the item's first row among all rows of the bias
+    auto bias_row = [&](const Item& it) { return ((bias_batches ? it.bh / H : 0) * (bias_heads ? H : 1) + (bias_heads ? it.bh % H : 0)) * Nq + it.row0; };
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* Qs = base;                                  // 2 tiles
@@ -805,11 +829,14 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             auto load_b = [&](const Item& it, int J, int j) {
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
-                    const int g = 2 * J + t, s = g % 3;
-                    if (ok) ok = bounded_wait_s<PRODUCER_SLEEP>(bars_s + 8 * (LY::B_EMPTY + s), ((g / 3) & 1) ^ 1, abort_s, status, 0x130 + t);
+                    const int g = 2 * J + t, s = BIAS == 2 ? t : g % 3;
+                    if (ok) ok = bounded_wait_s<PRODUCER_SLEEP>(bars_s + 8 * (LY::B_EMPTY + s), ((BIAS == 2 ? J : g / 3) & 1) ^ 1, abort_s, status, 0x130 + t);
                     if (!ok) return;
                     uint8_t* dst = base + LY::BIAS_OFF + s * LY::BIAS_BYTES;
                     mbar_arrive_expect_tx(&bars[LY::B_FULL + s], LY::BIAS_BYTES);
+                    if (BIAS == 2)
+                        load_shifted_bias<SHIFTED_WIDTH(D)>(dst, &tmBias, &bars[LY::B_FULL + s], bias_row(it) + t * BM, j * BN, Nk);
+                    else
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
                         tma_load_4d(dst + c * BM * 128, &tmBias, &bars[LY::B_FULL + s], j * BN + c * 64, it.row0 + t * BM,
@@ -841,7 +868,8 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             }
             if (!ok) {
                 if (BIAS)
-                    for (int g = b_issued > 3 ? b_issued - 3 : 0; g < b_issued; ++g) drain_wait(&bars[LY::B_FULL + g % 3], (g / 3) & 1);
+                    for (int g = b_issued > 3 ? b_issued - 3 : 0; g < b_issued; ++g) if (BIAS == 1) drain_wait(&bars[LY::B_FULL + g % 3], (g / 3) & 1);
+                        else if (g + 2 >= b_issued) drain_wait(&bars[LY::B_FULL + (g & 1)], (g >> 1) & 1);
                 for (int t = 0; t < 2; ++t)
                     if (q_loaded[t] > 0) drain_wait(&bars[LY::Q_FULL + t], (q_loaded[t] - 1) & 1);
                 for (int J = k_issued > LY::KS ? k_issued - LY::KS : 0; J < k_issued; ++J)
@@ -934,7 +962,8 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // (bias) the thread's row in stage 0's panel of this key half; logits are scaled as they meet the bias, so the routines
         // below go on with scale 1
         const uint32_t brow0 = smem_u32(base + LY::BIAS_OFF) + h * (BM * 128) + (q * 32 + lane) * 128;
-        const int rx = lane & 7;
+        int rx = lane & 7;
+        uint32_t browi = 0;                              // (shifted) the same, for the item; rx: what to shift by
         const float sc1 = BIAS ? 1.f : scale_log2e;
         bool ok = true;
         int b = t;                                       // buffer of tile-step g = 2 J + t: g % 3
@@ -956,6 +985,12 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         const int nrow_item = rlim < it.n ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : it.n;
         const int nrow = SPLIT ? (nrow_item > it.tile0 * BN ? nrow_item - it.tile0 * BN : 0) : nrow_item;
         const int nrow_min = __shfl_sync(0xffffffffu, nrow, 0);
+        const int bR = BIAS == 2 ? bias_row(it) + t * BM + q * 32 + lane : 0;
+        const bool own_copy = BIAS == 2 && bR >= sb.full && it.row0 + t * BM + q * 32 + lane < Nq;   // (beyond the last whole group of eight rows)
+        if (BIAS == 2) {
+            browi = smem_u32(base + LY::BIAS_OFF) + t * LY::BIAS_BYTES + h * (HN * 2) + shifted_row<SHIFTED_WIDTH(D)>(bR, bias_row(it) + t * BM);
+            rx = shifted_by(bR, Nk);
+        }
         float l = 0.f;
         const bool exact_first = !first_item_done || sc.coff < (1 << 29) || it.n < BN;   // (the same for all warps)
         first_item_done = true;
@@ -967,11 +1002,12 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             // partner (reading TMEM that may not be ready is harmless, nothing is stored), so that the
             // two always pass the same sequence of named barriers and leave together.
             ok = bounded_wait_s(bars_s + 8 * (LY::S_FULL + t * 3 + b), xph, abort_s, status, 0x300 + t);
-            if (BIAS && ok) ok = bounded_wait_s(bars_s + 8 * (LY::B_FULL + b), static_cast<uint32_t>(g / 3) & 1u, abort_s, status, 0x340 + t);
+            if (BIAS && ok) ok = bounded_wait_s(bars_s + 8 * (LY::B_FULL + (BIAS == 2 ? t : b)), static_cast<uint32_t>(BIAS == 2 ? g / 2 : g / 3) & 1u, abort_s, status, 0x340 + t);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
-            const uint32_t brow = brow0 + (BIAS ? b * LY::BIAS_BYTES : 0);
+            const uint32_t brow = BIAS == 2 ? browi : brow0 + (BIAS ? b * LY::BIAS_BYTES : 0);
             const int col0 = j * BN + h * HN;
+            if (BIAS == 2 && own_copy && col0 < Nk) copy_bias_row(sb.p + static_cast<int64_t>(bR) * Nk + col0, brow + rx, Nk - col0 < HN ? Nk - col0 : HN);
             const bool tail = col0 + HN > nrow_min;      // (warp-uniform) some row has masked keys in this step
             const int nvalid = nrow > col0 ? (nrow - col0 < HN ? nrow - col0 : HN) : 0;   // per row
             // p = 2^(scale*s - m_ref); row sum in fp32 from the unrounded p; P rounded to bf16.  Any
@@ -989,11 +1025,11 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 tmem_ld_x32(s_addr, r);
                 tc_wait_ld();
                 if (tail) {
-                    if (BIAS) add_bias32<0>(r, scale_log2e, brow, rx);
+                    if (BIAS) add_bias32<0, BIAS>(r, scale_log2e, brow, rx);
                     exp_pack32<true, false>(r, sc1, -m_ref, nvalid, ls, pk[0]);
                     tmem_ld_x32(s_addr + 32, r);
                     tc_wait_ld();
-                    if (BIAS) add_bias32<4>(r, scale_log2e, brow, rx);
+                    if (BIAS) add_bias32<4, BIAS>(r, scale_log2e, brow, rx);
                     exp_pack32<true, false>(r, sc1, -m_ref, nvalid - 32, ls, pk[1]);
                     lt = (ls[0] + ls[1]) + (ls[2] + ls[3]);
                 } else {
@@ -1001,12 +1037,12 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     uint64_t l2[2] = {0ull, 0ull};
                     uint64_t x2[16];
                     float xmax = 0.f;
-                    if (BIAS) scale_bias32<0>(r, scale2, neg_m2, brow, rx, x2);
+                    if (BIAS) scale_bias32<0, BIAS>(r, scale2, neg_m2, brow, rx, x2);
                     else      scale32(r, scale2, neg_m2, x2);
                     tmem_ld_x32(s_addr + 32, r);         // the second 32 logits arrive during the first 32 exponentials
                     exp_pack_x2<USE_POLY, SPLIT ? POLY_PAIRS_SA : POLY_PAIRS_A>(x2, l2, xmax, pk[0]);
                     tc_wait_ld();
-                    if (BIAS) scale_bias32<4>(r, scale2, neg_m2, brow, rx, x2);
+                    if (BIAS) scale_bias32<4, BIAS>(r, scale2, neg_m2, brow, rx, x2);
                     else      scale32(r, scale2, neg_m2, x2);
                     exp_pack_x2<USE_POLY, SPLIT ? POLY_PAIRS_SB : POLY_PAIRS_B>(x2, l2, xmax, pk[1]);
                     float a, b2, c, d2;
@@ -1030,8 +1066,8 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
                     tc_wait_ld();
                     if (BIAS) {
-                        add_bias32<0>(*reinterpret_cast<uint32_t(*)[32]>(&s[0]), scale_log2e, brow, rx);
-                        add_bias32<4>(*reinterpret_cast<uint32_t(*)[32]>(&s[32]), scale_log2e, brow, rx);
+                        add_bias32<0, BIAS>(*reinterpret_cast<uint32_t(*)[32]>(&s[0]), scale_log2e, brow, rx);
+                        add_bias32<4, BIAS>(*reinterpret_cast<uint32_t(*)[32]>(&s[32]), scale_log2e, brow, rx);
                     }
                     if (tail) {
                         const uint32_t excl = __float_as_uint(neg_scale ? INFINITY : -INFINITY);
@@ -1080,7 +1116,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                         uint32_t r[32];
                         tmem_ld_x32(s_addr + c * 32, r);
                         tc_wait_ld();
-                        if (BIAS) { if (c == 0) add_bias32<0>(r, scale_log2e, brow, rx); else add_bias32<4>(r, scale_log2e, brow, rx); }
+                        if (BIAS) { if (c == 0) add_bias32<0, BIAS>(r, scale_log2e, brow, rx); else add_bias32<4, BIAS>(r, scale_log2e, brow, rx); }
                         // (every pair so far switched off by the bias: 0 stands in for the reference, the weights are 2^-inf)
                         exp_pack32<true, false>(r, sc1, BIAS && m_ref == -INFINITY ? 0.f : -m_ref, nvalid - c * 32, ls, pk[c]);
                     }
@@ -1107,7 +1143,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             // careful path waits for anything)
             if (careful && pair_any(pair_id, !ok)) ok = false;
             if (!ok) break;
-            if (BIAS && lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + b));   // (behind the vote, which both warps' reads precede)
+            if (BIAS && lane == 0) mbar_arrive_s(bars_s + 8 * (LY::B_EMPTY + (BIAS == 2 ? t : b)));   // (behind the vote, which both warps' reads precede)
             tmem_st_x16(s_addr, pk[0]);
             tmem_st_x16(s_addr + 16, pk[1]);
             l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
@@ -1356,7 +1392,7 @@ int launch_tc3(const Problem& p, cudaStream_t st) {
         kern, grid, LY::SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, static_cast<int>(slots), slabs,
         p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
         (reinterpret_cast<uintptr_t>(p.O) & 31) == 0 ? 1 : 0, paired, static_cast<const int32_t*>(nullptr),
-        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{}, CUtensorMap{}, 0, 0);
+        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{}, CUtensorMap{}, 0, 0, ShiftedBias{});
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
@@ -1396,19 +1432,20 @@ int launch_fused_tc3_varlen(const void* Q, const void* K, const void* V, void* O
     const cudaError_t e = launch_pdl(
         fused_tc3_kernel<true>, grid, LY::VL_SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, num_seqs,
         static_cast<int>(most), slabs, scale * 1.4426950408889634f, static_cast<const int32_t*>(nullptr), causal ? 0 : (1 << 30), status,
-        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, sorted ? 1 : 0, cu_q, cu_k, static_cast<float*>(nullptr), ed, CUtensorMap{}, 0, 0);
+        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, sorted ? 1 : 0, cu_q, cu_k, static_cast<float*>(nullptr), ed, CUtensorMap{}, 0, 0, ShiftedBias{});
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
-// The same kernel with a bf16 bias, whose tensor map ({Nk, Nq, heads, batches}, boxes of 64 x 128) the caller has made.
-int launch_fused_tc3_bias(const Problem& p, const void* bias_map, cudaStream_t st) {
-    using LY = Layout<true>;
+// The same kernel with a bf16 bias, whose tensor map the caller has made.
+template <int BIAS>
+static int launch_tc3_bias(const Problem& p, const BiasMap& bias, cudaStream_t st) {
+    using LY = Layout<BIAS>;
     CUtensorMap tmQ, tmK, tmV;
     const int BH = p.B * p.H;
     if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map(&tmK, p.K, BH, p.Nk, D, BN) || !make_map(&tmV, p.V, BH, p.Nk, D, BN))
         return FLAT_ERR_CUDA;
-    if (!(p.lse ? ensure_dynamic_smem<fused_tc3_kernel<false, true, false, true>>(LY::SMEM_BYTES)
-                : ensure_dynamic_smem<fused_tc3_kernel<false, false, false, true>>(LY::SMEM_BYTES)))
+    if (!(p.lse ? ensure_dynamic_smem<fused_tc3_kernel<false, true, false, BIAS>>(LY::SMEM_BYTES)
+                : ensure_dynamic_smem<fused_tc3_kernel<false, false, false, BIAS>>(LY::SMEM_BYTES)))
         return FLAT_ERR_CUDA;
     const int slabs = (p.Nq + 2 * BM - 1) / (2 * BM), sms = device_sm_count();
     const int64_t items = static_cast<int64_t>(slabs) * BH;
@@ -1417,12 +1454,17 @@ int launch_fused_tc3_bias(const Problem& p, const void* bias_map, cudaStream_t s
     const int64_t slots = paired ? static_cast<int64_t>((slabs + 1) & ~1) * BH : items;
     if (slots > 0x7fffffff) return FLAT_ERR_SHAPE;
     const cudaError_t e = launch_pdl(
-        p.lse ? fused_tc3_kernel<false, true, false, true> : fused_tc3_kernel<false, false, false, true>,
+        p.lse ? fused_tc3_kernel<false, true, false, BIAS> : fused_tc3_kernel<false, false, false, BIAS>,
         static_cast<int>(persistent ? sms : items), LY::SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk,
         static_cast<int>(slots), slabs, p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), p.status,
         (reinterpret_cast<uintptr_t>(p.O) & 31) == 0 ? 1 : 0, paired, static_cast<const int32_t*>(nullptr),
-        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{}, *static_cast<const CUtensorMap*>(bias_map), p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0);
+        static_cast<const int32_t*>(nullptr), p.lse, EvenDeal{}, *static_cast<const CUtensorMap*>(bias.map), p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0,
+        ShiftedBias{static_cast<const uint16_t*>(p.bias), bias.shifted_rows});
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
+int launch_fused_tc3_bias(const Problem& p, const BiasMap& bias, cudaStream_t st) {
+    return bias.shifted_rows >= 0 ? launch_tc3_bias<2>(p, bias, st) : launch_tc3_bias<1>(p, bias, st);
 }
 
 int launch_fused_tc3(const Problem& p, cudaStream_t st) {

@@ -155,5 +155,60 @@ inline bool make_map_packed(CUtensorMap* m, const void* ptr, int64_t tokens, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// A bias whose rows begin at any alignment, staged by TMA all the same.  Row R of all its rows (heads and batches after one
+// another, Nk bf16 each) lies in group R / 8 of eight rows, groups that are 16 Nk bytes apart: a tensor map {8 Nk, groups} brings
+// the rows of one phase R % 8 = b with boxes of 16 groups, from a column rounded down to 16 bytes, and 8 b columns further left
+// still: in shared memory (SHIFT_ROW = 2 x box width = 0 mod 128 bytes a row) rows of different phase then start 16 bytes apart and
+// the 16-byte reads of a warp's rows meet no bank conflict.  What is left, 0 to 14 bytes, a thread shifts in registers.  Rows
+// beyond the last whole group (`full`: rows in whole groups) come from device memory, copied by the row's own thread.
+// Measured, against 16-byte pieces straight from device memory (us): d = 64, B8 H16 1001^2 293 -> 115 (no bias: 59; 1024^2, where
+// nothing is to be shifted: 80), B6 H8 2770^2 1,057 -> 278; d = 128, B8 H16 1001^2 367 -> 153, B3 H12 3247^2 1,380 -> 450.  Bound
+// by the shifts (15 instructions per 8 values) and the one stage per query tile that its width leaves room for.
+struct ShiftedBias {
+    const uint16_t* p;
+    int full;
+};
+// Boxes for the tile of 128 rows from row g0 of all and the keys from column col.
+template <int WIDTH>
+__device__ __forceinline__ void load_shifted_bias(uint8_t* dst, const void* tmap, uint64_t* bar, int g0, int col, int Nk) {
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+        ptx::tma_load_3d(dst + b * 16 * WIDTH * 2, tmap, bar, ((b * Nk + col) & ~7) - 8 * b, (g0 + ((b - g0) & 7)) >> 3, 0);
+}
+// Byte offset of row R's first 16-byte piece in a tile from row g0 on, and the bytes from there to its first value (any column
+// that is a multiple of 8).
+template <int WIDTH>
+__device__ __forceinline__ uint32_t shifted_row(int R, int g0) {
+    const int b = R & 7;
+    return (b * 16 + (R >> 3) - ((g0 + ((b - g0) & 7)) >> 3)) * (WIDTH * 2) + 16 * b;
+}
+__device__ __forceinline__ uint32_t shifted_by(int R, int Nk) { return 2 * (((R & 7) * Nk) & 7); }
+// Eight values from two 16-byte pieces.
+__device__ __forceinline__ void shift8(const uint32_t (&w)[8], uint32_t by, uint32_t (&o)[4]) {
+    uint32_t a[6], c[5];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a[k] = by & 8 ? w[k + 2] : w[k];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) c[k] = by & 4 ? a[k + 1] : a[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[k] = __funnelshift_r(c[k], c[k + 1], (by & 2) * 8);
+}
+// `n` values of a row into its place.
+static __device__ __noinline__ void copy_bias_row(const uint16_t* src, uint32_t dst, int n) {
+    for (int i = 0; i < n; ++i) asm volatile("st.shared::cta.u16 [%0], %1;" ::"r"(dst + 2 * i), "h"(src[i]) : "memory");
+    ptx::fence_proxy_async_smem();       // (the tile's next copy follows)
+}
+inline bool make_shifted_bias_map(CUtensorMap* m, const void* ptr, int64_t groups, int Nk, int width) {
+    EncodeTiledFn enc = get_encode_fn();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {static_cast<cuuint64_t>(Nk) * 8, static_cast<cuuint64_t>(groups), 1};
+    cuuint64_t strides[2] = {static_cast<cuuint64_t>(Nk) * 16, static_cast<cuuint64_t>(Nk) * 16 * groups};
+    cuuint32_t box[3] = {static_cast<cuuint32_t>(width), 16, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace tc
 }  // namespace flat

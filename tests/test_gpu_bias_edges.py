@@ -19,6 +19,15 @@ CASES = [
     (8, 40, 600, 600, 64, (1, 1), "bf16", None, True, 0.125),               # persistent, complementary slabs
     (2, 2, 200, 328, 64, (2, 2), "bf16", None, False, -0.2),
     (2, 2, 130, 301, 64, (1, 2), "bf16", None, False, 0.125),               # rows begin at every second byte
+    (1, 1, 129, 33, 64, (1, 1), "bf16", None, False, 0.125),                # the rows end within a group of eight
+    (3, 5, 257, 517, 64, (3, 5), "bf16", [517, 3, 400], True, 0.125),
+    (2, 3, 700, 131, 64, (2, 1), "bf16", None, False, -0.2),
+    (9, 20, 401, 203, 64, (1, 20), "bf16", None, True, 0.125),              # persistent
+    (9, 20, 301, 130, 64, (1, 1), "bf16", None, False, 0.125),
+    (2, 3, 257, 519, 128, (1, 3), "bf16", [519, 65], False, 0.1),           # d = 128
+    (3, 5, 260, 1001, 128, (3, 5), "bf16", None, True, 0.1),
+    (9, 20, 301, 131, 128, (1, 20), "bf16", None, False, 0.1),              # several items a CTA
+    (1, 2, 9, 30, 128, (1, 2), "bf16", None, False, 0.1),                   # too small for it
     (2, 2, 130, 302, 128, (2, 1), "bf16", [302, 77], True, 0.1),
     (2, 3, 257, 520, 128, (1, 3), "bf16", [520, 65], False, 0.1),            # d = 128, staged: nine steps of 64 keys
     (3, 2, 700, 704, 128, (3, 1), "bf16", [704, 1, 640], True, 0.1),
