@@ -68,7 +68,9 @@ enum {
     FLAT_VARIANT_TC = 2,       /* tcgen05 + TMEM + TMA kernel, one 128-row tile per CTA:
                                   bf16, d in {64,128}                                          */
     FLAT_VARIANT_TC2 = 3,      /* same, two 128-row tiles per CTA ping-ponging on the tensor
-                                  pipe (the default for problems that fill the GPU)            */
+                                  pipe (the default for problems that fill the GPU; d = 128:
+                                  steps of 64 keys; with a bf16 bias at d = 64 the pipeline of
+                                  TC3, still reported as this)                                 */
     FLAT_VARIANT_TC2_SINGLE = 4, /* the TC2 pipeline with one 128-row tile per CTA and two CTAs
                                   per SM: bf16, d = 64 only                                    */
     FLAT_VARIANT_TC3 = 5,      /* two tiles per CTA, the softmax of every row split over two
@@ -80,7 +82,7 @@ enum {
     FLAT_VARIANT_TF32 = 7,     /* fp32 tensors on the tensor cores: every operand split into a tf32
                                   head and an fp32 remainder, each contraction three tf32 products,
                                   running sums in fp32 registers: fp32, d = 64, no bias, no
-                                  pruning map (what AUTO picks there)                            */
+                                  pruning map (what AUTO picks there, and at d = 32 and 128)     */
     FLAT_VARIANT_TC2_SPLIT2 = 8, /* TC2_SINGLE with the keys of every query tile split over a cluster
                                   of two CTAs, whose partial softmaxes are merged through
                                   distributed shared memory: bf16, d in {64,128}, no bias, no pruning map;

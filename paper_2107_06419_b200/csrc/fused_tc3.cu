@@ -1362,12 +1362,15 @@ int launch_tc3(const Problem& p, cudaStream_t st) {
     const int64_t slots = paired ? static_cast<int64_t>((slabs + 1) & ~1) * BH : items;
     if (slots > 0x7fffffff) return FLAT_ERR_SHAPE;
     const int grid = static_cast<int>(persistent ? sms : items);
-    // Too few items for the fixed deal: whole items handed out by the hardware leave SMs idle when the items differ
-    // in length (key-padding masks) or when the last round is mostly empty; the key steps are dealt evenly instead
-    // (EvenDeal), if the average share is long enough to carry the two extra item boundaries.
-    if (!persistent && !p.causal && !p.lse && p.B <= DEAL_MAX_B && sms <= WS_MAX_CTAS && items > 0) {
+    // Whole items leave SMs idle when there are few of them and they differ in length (key-padding masks), or when the last round
+    // is mostly empty; the key steps are dealt evenly instead (EvenDeal), if the average share is long enough.  Of equal items
+    // the longest CTA takes ceil(items / SMs) x key steps; the deal's the average and what measures as 5 % and 10 steps more (the
+    // two extra item boundaries, the merge).  On either side of that line (us, whole items / dealt; items per SM, key steps):
+    // H5 16K^2 2.16, 128: 496 / 363; B2 H10 4096^2 2.16, 32: 124 / 108; B2 H8 8192^2 3.46, 64: 318 / 297; B2 H6 4930^2 1.62, 39:
+    // 105 / 101; B4 H8 3000^2 2.59, 24: 97 / 100; B7 H12 1500^2 3.41, 12: 71 / 73; H17 4096^2 1.84, 32: 88 / 93.
+    if (!p.causal && !p.lse && p.B <= DEAL_MAX_B && sms <= WS_MAX_CTAS && items > 0) {
         const int64_t nt = (p.Nk + BN - 1) / BN, rounds = (items + sms - 1) / sms;
-        const bool ragged = p.k_valid_len != nullptr || 4 * items < 3 * rounds * sms;   // (unmasked: under three quarters of the rounds filled)
+        const bool ragged = p.k_valid_len ? !persistent : 21 * items * nt + 200 * sms < 20 * rounds * nt * sms;
         // teams of `slabs` CTAs if they fill nine SMs in ten; single items only where K and V of all heads stay in L2
         EvenDeal ed{};
         const bool teams_fit = slabs <= sms && 10 * ((sms / slabs) * slabs) >= 9 * sms;
