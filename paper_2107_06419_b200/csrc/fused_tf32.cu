@@ -63,6 +63,10 @@ template <int D> struct Layout {
     static constexpr int PANEL = BN * 128, VT_PANEL = D * 128;
     static constexpr int MERGE_STRIDE = D + 4;           // floats per row of the merge scratch (outputs, m, l, padding: 16-byte rows, no bank conflicts)
     static constexpr int PVS = D == 128 ? 1 : 2;         // P V buffers
+    // registers after the hand-over, of the 512 x 128 of the launch (d = 64 with 192 / 80 / 48: the converters spill, 548 us
+    // against 532 on B2 H16 4096^2)
+    static constexpr int SOFT_REGS = D == 128 ? 192 : 176, CONVERT_REGS = D == 128 ? 80 : 104, ISSUE_REGS = D == 128 ? 48 : 56;
+    static_assert(256 * SOFT_REGS + 128 * CONVERT_REGS + 128 * ISSUE_REGS <= THREADS * 128, "register hand-over");
     static constexpr uint32_t QH_COL = 0, QL_COL = D, S_COL = 2 * D, PL_COL = S_COL + 2 * BN, PV_COL = PL_COL + 2 * BN;
     static_assert(PV_COL + PVS * D <= TMEM_COLS, "tensor memory");
     // shared memory: K_hi[KS] K_lo[KS] Vraw[VR] VT_hi[VS] VT_lo[VS]; the Q tile is staged over the V^T rings
@@ -142,16 +146,6 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const int heads = BH - first < group ? BH - first : group, at = static_cast<int>(blockIdx.x) % per;
     const int bh = first + at % heads;
     const int row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * BM;
-    int n = Nk;
-    if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
-    {
-        // Causal mask (coff = Nk - Nq; 2^30 = none): row r sees keys j < r + 1 + coff, so the CTA's
-        // last row bounds the keys of all its rows.
-        const long long lim = static_cast<long long>(row0) + BM + coff;
-        if (lim < n) n = lim < 0 ? 0 : static_cast<int>(lim);
-    }
-    const int ntiles = (n + BN - 1) / BN;
-
     if (threadIdx.x == 384) {
         for (int i = 0; i < NUM_BARS; ++i) {
             if (i == Q_READY) { mbar_init(&bars[i], 8); continue; }
@@ -168,9 +162,22 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // (launched with programmatic stream serialization: this set-up overlaps the tail of the previous kernel of the stream, and
+    // nothing in device memory is touched before that one has finished)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int n = Nk;
+    if (valid_len) { n = valid_len[bh / H]; n = n < 0 ? 0 : (n > Nk ? Nk : n); }
+    {
+        // Causal mask (coff = Nk - Nq; 2^30 = none): row r sees keys j < r + 1 + coff, so the CTA's
+        // last row bounds the keys of all its rows.
+        const long long lim = static_cast<long long>(row0) + BM + coff;
+        if (lim < n) n = lim < 0 ? 0 : static_cast<int>(lim);
+    }
+    const int ntiles = (n + BN - 1) / BN;
 
     if (warp >= 12) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(LY::ISSUE_REGS));
         if (warp == 12) {
             // ------------------------------------------------------------ TMA producer
             if (lane == 0 && ntiles > 0) {
@@ -285,7 +292,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
     } else if (warp >= 8) {
         // ------------------------------------------------------------ converters (warps 8-11)
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(LY::CONVERT_REGS));
         bool ok = true;
         if (warp < 10) {
             // warps 8, 9: K tile -> K_hi (in place) and K_lo, element by element
@@ -353,7 +360,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
     } else {
         // ------------------------------------------------------------ softmax + output (warps 0-7)
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(LY::SOFT_REGS));
         const int g = warp >> 2;                             // 0: even key steps, 1: odd key steps (= TMEM buffer)
         const int r = (warp & 3) * 32 + lane;                // row of the tile <-> TMEM lane
         const int row = row0 + r;
@@ -398,12 +405,11 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             ok = __all_sync(0xffffffffu, bounded_wait(&bars[PV_FULL + g], (k >> 1) & 1, abort_flag, status, 0x660 + g));
             if (!ok) return;
             tc_fence_after();
-            constexpr int CH = D == 128 ? 16 : 32;           // (128 outputs leave few registers)
+            constexpr int CH = 16;                           // (32 at a time: d = 64 1 % slower, d = 128 spills)
 #pragma unroll
             for (int c = 0; c < D; c += CH) {
                 uint32_t pv[CH];
-                if constexpr (CH == 32) tmem_ld_x32(tl + PV_COL + (LY::PVS - 1) * D * g + c, pv);
-                else                    tmem_ld_x16(tl + PV_COL + (LY::PVS - 1) * D * g + c, pv);
+                tmem_ld_x16(tl + PV_COL + (LY::PVS - 1) * D * g + c, pv);
                 tc_wait_ld();
 #pragma unroll
                 for (int i = 0; i < CH; ++i) o[c + i] = fmaf(o[c + i], alpha_prev, __uint_as_float(pv[i]));
@@ -551,10 +557,19 @@ int launch(const Problem& p, cudaStream_t st) {
     // fit L2 together (48 MB of K and V) go longest first: what is left at the end are the short ones
     const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 8);
     const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
-    fused_tf32_kernel<D><<<slabs * BH, THREADS, LY::SMEM_BYTES, st>>>(
-        tmQ, tmK, tmV, static_cast<float*>(p.O), BH, p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
-        p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status, p.lse);
-    return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(slabs) * BH);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = LY::SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_tf32_kernel<D>, tmQ, tmK, tmV, static_cast<float*>(p.O), BH, p.H, p.Nq, p.Nk,
+                                             p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status, p.lse);
+    return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
 }  // namespace
