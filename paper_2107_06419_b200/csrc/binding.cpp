@@ -6,8 +6,9 @@
 // object).
 //
 // Every function answers with the library's return code, or with -1 where an argument is not of the plain form it
-// handles (not exactly a torch.Tensor, wrong type, shape or device, not contiguous, an object that is no number):
-// nothing was launched then, and api.py goes its long way, whose checks say what is wrong.
+// handles (not exactly a torch.Tensor, wrong type, shape or device, not contiguous, an object that is no number; a tensor
+// that has no memory to point at, which torch reports by a C++ exception: those of vmap, grad and tracing): nothing was
+// launched then, and api.py goes its long way, whose checks say what is wrong.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -76,12 +77,16 @@ struct Args {
         PyObject* o = next();
         if (bad) return nullptr;
         if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-        if (PyLong_CheckExact(o)) return PyLong_AsVoidPtr(o);
+        if (PyLong_CheckExact(o)) return address(o);
         PyObject* s = PyObject_GetAttrString(o, "cuda_stream");
         if (!s) { PyErr_Clear(); bad = true; return nullptr; }
-        void* p = PyLong_Check(s) ? PyLong_AsVoidPtr(s) : nullptr;
-        bad = !PyLong_Check(s);
+        void* p = address(s);
         Py_DECREF(s);
+        return p;
+    }
+    void* address(PyObject* o) {
+        void* p = PyLong_Check(o) ? PyLong_AsVoidPtr(o) : nullptr;
+        if (!PyLong_Check(o) || PyErr_Occurred()) { PyErr_Clear(); bad = true; }
         return p;
     }
     void end() { if (i != n) bad = true; }
@@ -93,7 +98,8 @@ inline PyObject* no() { return PyLong_FromLong(-1); }
 template <typename T> inline T* at_(const at::Tensor* t) { return t ? static_cast<T*>(t->data_ptr()) : nullptr; }
 inline void* ptr(const at::Tensor* t) { return at_<void>(t); }
 
-// Runs `call` without the interpreter lock (the driver may block in a launch) and answers with its code.
+// Runs `call`, which throws nothing (pointers are taken from the tensors before it), without the interpreter lock (the
+// driver may block in a launch) and answers with its code.
 template <typename F> PyObject* run(F&& call) {
     int rc;
     Py_BEGIN_ALLOW_THREADS
@@ -215,10 +221,11 @@ PyObject* varlen_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
     if (!is(*K, {tk, H, d}) || !is(*V, {tk, H, d}) || !is(*O, {tq, H, d}) || ck->size(0) != seqs + 1 || seqs < 1 ||
         !small(seqs) || !small(H) || !small(d))
         return no();
+    void *q = ptr(Q), *k = ptr(K), *v = ptr(V), *o = ptr(O);
+    const int32_t *cuq = at_<const int32_t>(cq), *cuk = at_<const int32_t>(ck);
     return run([&] {
-        return flat_attn_varlen_fwd(ptr(Q), ptr(K), ptr(V), ptr(O), at_<const int32_t>(cq), at_<const int32_t>(ck),
-                                    static_cast<int>(seqs), static_cast<int>(H), static_cast<int>(d), tq, tk, longest,
-                                    scale, causal, status, st);
+        return flat_attn_varlen_fwd(q, k, v, o, cuq, cuk, static_cast<int>(seqs), static_cast<int>(H), static_cast<int>(d), tq, tk,
+                                    longest, scale, causal, status, st);
     });
 }
 
@@ -237,10 +244,10 @@ PyObject* layer_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
     if (!small(B) || !small(H) || !small(N) || !small(d) || !small(Dm) || !is(*X, {B, N, Dm}) || !is(*Wqkv, {3 * H * d, Dm}) ||
         !is(*Wo, {Dm, H * d}) || !is(*Y, {B, N, Dm}) || !is(*K, {B, H, N, d}) || !is(*V, {B, H, N, d}) || !is(*O, {B, H, N, d}))
         return no();
+    void *x = ptr(X), *wqkv = ptr(Wqkv), *wo = ptr(Wo), *y = ptr(Y), *q = ptr(Q), *k = ptr(K), *v = ptr(V), *o = ptr(O);
     return run([&] {
-        return flat_attn_layer_fwd(ptr(X), ptr(Wqkv), ptr(Wo), ptr(Y), ptr(Q), ptr(K), ptr(V), ptr(O), static_cast<int>(B),
-                                   static_cast<int>(N), static_cast<int>(H), static_cast<int>(d), static_cast<int>(Dm), scale,
-                                   causal, status, st);
+        return flat_attn_layer_fwd(x, wqkv, wo, y, q, k, v, o, static_cast<int>(B), static_cast<int>(N), static_cast<int>(H),
+                                   static_cast<int>(d), static_cast<int>(Dm), scale, causal, status, st);
     });
 }
 
@@ -255,9 +262,8 @@ PyObject* fc_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {    // X, W, Y
     if (W->size(1) != K || Y->size(-1) != Nout || !X->sizes().slice(0, X->dim() - 1).equals(Y->sizes().slice(0, Y->dim() - 1)) ||
         M < 1 || !small(M) || !small(K) || !small(Nout))
         return no();
-    return run([&] {
-        return flat_fc_fwd(ptr(X), ptr(W), ptr(Y), static_cast<int>(M), static_cast<int>(K), static_cast<int>(Nout), status, st);
-    });
+    void *x = ptr(X), *w = ptr(W), *y = ptr(Y);
+    return run([&] { return flat_fc_fwd(x, w, y, static_cast<int>(M), static_cast<int>(K), static_cast<int>(Nout), status, st); });
 }
 
 PyObject* layernorm_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {   // X, gamma, beta, Y, eps, residual, stream
@@ -271,10 +277,22 @@ PyObject* layernorm_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {   // X
     const int64_t D = X->size(-1), M = D > 0 ? X->numel() / D : 0;
     if (!small(D) || M < 1 || !is(*g, {D}) || !is(*b, {D}) || !Y->sizes().equals(X->sizes()) || (R && !R->sizes().equals(X->sizes())))
         return no();
-    return run([&] { return flat_layernorm_fwd(ptr(X), ptr(R), ptr(g), ptr(b), ptr(Y), M, static_cast<int>(D), eps, st); });
+    void *x = ptr(X), *r = ptr(R), *gamma = ptr(g), *beta = ptr(b), *y = ptr(Y);
+    return run([&] { return flat_layernorm_fwd(x, r, gamma, beta, y, M, static_cast<int>(D), eps, st); });
 }
 
-#define FAST(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(f)), METH_FASTCALL, nullptr}
+// The functions as Python sees them: no C++ exception leaves them.
+typedef PyObject* Fast(PyObject*, PyObject* const*, Py_ssize_t);
+template <Fast* F> PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t n) {
+    try {
+        return F(self, args, n);
+    } catch (...) {
+        PyErr_Clear();
+        return no();
+    }
+}
+
+#define FAST(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(guarded<f>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {FAST(fwd), FAST(fwd_ex), FAST(bwd_ex), FAST(varlen_fwd), FAST(layer_fwd), FAST(fc_fwd),
                          FAST(layernorm_fwd), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
