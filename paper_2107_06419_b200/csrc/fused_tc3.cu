@@ -320,6 +320,7 @@ struct Item {
 // tile would come from DRAM once per slab (measured: no gain at all on the masked workload).  So the unit that is
 // dealt is the head -- all its slabs -- and a team of `team` = slabs CTAs takes a range of head key steps, member
 // s of the team working on slab s; team = 1 deals single items.
+// (Packed batches have no such deal; `team` and `epoch` carry what launch_fused_tc3_varlen says there.)
 struct EvenDeal {
     int team;
     int epoch;
@@ -700,8 +701,11 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     static_assert(!BIAS || (!VL && !SPLIT), "the bias is read by the plain dense kernel");
     static_assert(!SPLIT || (!VL && !WLSE), "the even deal is built for the plain dense forward kernel only");
     Sched sc{items, slabs, H, Nk, valid_len, coff, paired, cu_q, cu_k, nullptr, BIAS && !bias_batches ? items / (H * (paired ? (slabs + 1) & ~1 : slabs)) : 0, ed};
-    if (VL && !paired && static_cast<int>(gridDim.x) == items) {
-        // one CTA per slot: a slot past the end of its sequence leaves before anything is set up
+    if (VL && ed.epoch) {
+        // One CTA per slot: a slot past the end of its sequence leaves before anything is set up.  The offsets may be what
+        // the previous kernel of the stream writes, so that one is waited for first.  (The next kernel is let go behind the
+        // set-up only, as ever: one that got the tensor memory before a CTA of this grid would hold it until the grid ends.)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         if (get_item<VL>(0, sc).skip) return;
     }
     // (bias, shifted) the item's first row among all rows of the bias
@@ -777,8 +781,8 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     // (launched with programmatic stream serialization: this set-up overlaps the tail of the previous kernel of the stream,
-    // and nothing in device memory is touched before that one has finished.  Not the even deal: its launches have an event
-    // between them, which forbids the overlap.)
+    // and nothing in device memory is touched before that one has finished (packed batches with empty slots have waited
+    // above).  Not the even deal: its launches have an event between them, which forbids the overlap.)
     if (!SPLIT) {
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1431,6 +1435,7 @@ int launch_fused_tc3_varlen(const void* Q, const void* K, const void* V, void* O
     const int grid = static_cast<int>(persistent && most > sms ? sms : most);
     EvenDeal ed{};
     ed.team = static_cast<int>(static_cast<unsigned>(((1ull << 32) + H - 1) / H));   // (see unit_of)
+    ed.epoch = !persistent && !equal;                    // (a CTA per slot, some of them past the end of their sequence)
     g_last_schedule = persistent ? FLAT_SCHEDULE_PERSISTENT : FLAT_SCHEDULE_ITEMS;
     const cudaError_t e = launch_pdl(
         fused_tc3_kernel<true>, grid, LY::VL_SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, num_seqs,
