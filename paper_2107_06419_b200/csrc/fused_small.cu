@@ -18,7 +18,8 @@
 // Measured: B16 H8 1000 x 1000 at d = 32: 66 us (1.9e12 pairs/s, 0.42 of the exponential unit; 1024 CTAs are 3.5 rounds of
 // the 296 that run at a time) against 638 us of the FFMA kernel, which keeps the fp32 tensors and the calls with a bias.
 // Reference maximum as in the two-tile kernel: exact on the first and on masked steps, kept otherwise, a step whose row
-// sum passes 2^40 is redone with a fresh one.  Every wait is bounded; on expiry the CTA ends cleanly and reports a code.
+// sum passes 2^40 is redone with a fresh one.  A row that does not come out finite (infinite or very large values) is computed
+// again without the split (plain_row).  Every wait is bounded; on expiry the CTA ends cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -105,8 +106,8 @@ __device__ __forceinline__ float exp_store_split(const uint32_t (&s)[BN], float 
 template <int D>
 __global__ void __launch_bounds__(SMALL_THREADS, 2)
 fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, int H, int Nq, int Nk,
-                   float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int32_t* status,
+                   const __grid_constant__ CUtensorMap tmV, const __nv_bfloat16* Q, const __nv_bfloat16* K, const __nv_bfloat16* V,
+                   __nv_bfloat16* O, int H, int Nq, int Nk, float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int32_t* status,
                    float* __restrict__ lse) {
     using LY = LS<D>;
     extern __shared__ uint8_t smem_raw[];
@@ -317,6 +318,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 lse[static_cast<int64_t>(bh) * Nq + row] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
             tc_fence_after();
             __nv_bfloat16* orow = O + (static_cast<int64_t>(bh) * Nq + row) * D;
+            uint64_t zero[2] = {0ull, 0ull};             // (NaN once a result is not finite)
 #pragma unroll
             for (int c = 0; c < D / 16; ++c) {
                 uint32_t r[16];
@@ -327,6 +329,9 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 #pragma unroll
                     for (int i = 0; i < 16; ++i) r[i] = 0u;      // no valid key: O = 0
                 }
+#pragma unroll
+                for (int i = 0; i < 16; i += 2)
+                    zero[(i >> 1) & 1] = fma2(pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), 0ull, zero[(i >> 1) & 1]);
                 if (row < Nq) {
 #pragma unroll
                     for (int v = 0; v < 2; ++v) {
@@ -338,6 +343,17 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         *reinterpret_cast<uint4*>(orow + c * 16 + v * 8) = w;
                     }
                 }
+            }
+            float z0, z1;
+            unpack2(add2(zero[0], zero[1]), z0, z1);
+            unsigned again = __ballot_sync(0xffffffffu, row < Nq && z0 + z1 != 0.f);
+            while (again) {
+                const int at = __ffs(again) - 1;
+                again &= again - 1;
+                __syncwarp();                            // (the row's own thread has stored it)
+                const int64_t r = static_cast<int64_t>(bh) * Nq + row0 + warp * 32 + at;
+                plain_row<__nv_bfloat16, D>(Q + r * D, K + static_cast<int64_t>(bh) * Nk * D, V + static_cast<int64_t>(bh) * Nk * D, O + r * D,
+                                            lse ? lse + r : nullptr, __shfl_sync(0xffffffffu, nrow, at), scale_log2e);
             }
         }
     }
@@ -378,8 +394,9 @@ int launch_small_d(const Problem& p, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_small_kernel<D>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq,
-                                             p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_small_kernel<D>, tmQ, tmK, tmV, static_cast<const __nv_bfloat16*>(p.Q),
+                                             static_cast<const __nv_bfloat16*>(p.K), static_cast<const __nv_bfloat16*>(p.V),
+                                             static_cast<__nv_bfloat16*>(p.O), p.H, p.Nq, p.Nk, p.scale * 1.4426950408889634f, p.k_valid_len,
                                              p.causal ? p.Nk - p.Nq : (1 << 30), p.status, p.lse);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }

@@ -110,6 +110,68 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// One query row in plain fp32 FMAs, keys 0 .. nkeys - 1, by a whole warp: for the rows whose result from split operands is not
+// finite.  An infinity splits into a head and a remainder that is no number, and a weight of up to 2^40 (reference maxima are
+// kept while they serve) may carry a large value past the largest number; without either, infinite values give infinite
+// features and large ones their mean.  A warp takes 32 keys at a time: a lane one key's logit, then each lane d / 32 features.
+// Two to three times the time of the FFMA kernel if it came to every row.
+__device__ __forceinline__ void floats16(const float* p, float (&f)[4]) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+}
+__device__ __forceinline__ void floats16(const __nv_bfloat16* p, float (&f)[8]) {
+    const uint4 v = *reinterpret_cast<const uint4*>(p);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { f[2 * e] = __uint_as_float(w[e] << 16); f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+}
+template <typename T, int D>
+static __device__ __noinline__ void plain_row(const T* q, const T* K, const T* V, T* o, float* lse, int nkeys, float scale_log2e) {
+    constexpr int N = 16 / sizeof(T), F = (D + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    float m = -INFINITY, l = 0.f, acc[F];
+#pragma unroll
+    for (int i = 0; i < F; ++i) acc[i] = 0.f;
+    for (int k0 = 0; k0 < nkeys; k0 += 32) {
+        const bool live = k0 + lane < nkeys;
+        const T* k = K + static_cast<int64_t>(live ? k0 + lane : k0) * D;
+        float x = 0.f;
+#pragma unroll 4
+        for (int t = 0; t < D; t += N) {
+            float a[N], b[N];
+            floats16(q + t, a);
+            floats16(k + t, b);
+#pragma unroll
+            for (int e = 0; e < N; ++e) x = fmaf(a[e], b[e], x);
+        }
+        x = live ? x * scale_log2e : -INFINITY;
+        float mx = x;
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+        const float m_new = fmaxf(m, mx), m_use = m_new == -INFINITY ? 0.f : m_new;
+        const float alpha = exp2f(m - m_use), p = exp2f(x - m_use);
+        float sum = p;
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, s);
+        l = l * alpha + sum;
+        m = m_new;
+#pragma unroll
+        for (int i = 0; i < F; ++i) acc[i] *= alpha;
+        const int n = nkeys - k0 < 32 ? nkeys - k0 : 32;
+        for (int j = 0; j < n; ++j) {
+            const float pj = __shfl_sync(0xffffffffu, p, j);
+#pragma unroll
+            for (int i = 0; i < F; ++i)
+                if (lane + 32 * i < D) acc[i] = fmaf(pj, static_cast<float>(V[static_cast<int64_t>(k0 + j) * D + lane + 32 * i]), acc[i]);
+        }
+    }
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+    for (int i = 0; i < F; ++i)
+        if (lane + 32 * i < D) o[lane + 32 * i] = static_cast<T>(acc[i] * inv);
+    if (lse && lane == 0) *lse = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

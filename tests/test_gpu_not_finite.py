@@ -1,0 +1,83 @@
+"""Infinite and very large values: the kernels that split their operands give what plain fp32 arithmetic gives."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def run(api, Q, K, V, scale, variant=0, **kw):
+    O = torch.full_like(Q, float("nan"))
+    lse = torch.full(Q.shape[:3], float("nan"), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    api.flat_attn_fwd_ex(Q, K, V, O, scale, status=status, variant=variant, lse=lse, **kw)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    return O.float(), lse
+
+
+def check(api, Q, K, V, scale, variant, rounding, **kw):
+    """AUTO (which must run `variant`) against the FFMA kernel: the same infinities and NaN, finite values to `rounding` of the
+    largest value a feature has (each is off the exact one by its format's rounding, and by sums in another order)."""
+    O, lse = run(api, Q, K, V, scale, **kw)
+    assert api.flat_attn_last_variant() == variant
+    F, flse = run(api, Q, K, V, scale, variant=api.FLAT_VARIANT_SIMT, **kw)
+    for got, want, size in ((O, F, V.float().nan_to_num(0.0, 0.0, 0.0).abs().amax(2, keepdim=True)), (lse, flse, None)):
+        same = (got == want) | (got.isnan() & want.isnan())
+        ok = got.isfinite() & want.isfinite()
+        bound = rounding * size if size is not None else 4e-5 * (1 + want.abs())
+        near = ok & ((got - want).abs() <= bound)
+        assert bool((same | near).all())
+    return O
+
+
+FORMATS = [(16, torch.bfloat16), (32, torch.bfloat16)]
+
+
+def variant_of(api, dtype):
+    return api.FLAT_VARIANT_SMALL if dtype == torch.bfloat16 else api.FLAT_VARIANT_TF32
+
+
+def rounding_of(dtype):                                  # of one bf16 number (2^-8), or of fp32 sums of a few hundred terms
+    return 2.0 ** -7 if dtype == torch.bfloat16 else 2.0 ** -16
+
+
+@pytest.mark.parametrize("d,dtype", FORMATS)
+@pytest.mark.parametrize("options", [{}, {"causal": True}, {"valid": True}], ids=str)
+def test_infinite_values(d, dtype, options):
+    from paper_2107_06419_b200 import api
+    torch.manual_seed(d)
+    B, H, Nq, Nk = 2, 3, 150, 333
+    Q, K, V = (torch.randn(B, H, n, d, device="cuda").to(dtype) for n in (Nq, Nk, Nk))
+    V[0, 0, 5, 1] = float("inf")
+    V[0, 0, 6, 2] = -float("inf")
+    V[0, 1, 7, 3], V[0, 1, 140, 3] = float("inf"), -float("inf")   # both signs in one feature: NaN where a row sees both
+    V[1, 0, 9, 0] = float("nan")
+    K[1, 1, 20, 4] = float("inf")                        # an infinite logit of either sign
+    Q[1, 2, 30, 5] = -float("inf")
+    kw = {"causal": True} if "causal" in options else {}
+    if "valid" in options:
+        kw["k_valid_len"] = torch.tensor([333, 50], dtype=torch.int32, device="cuda")
+    O = check(api, Q, K, V, d ** -0.5, variant_of(api, dtype), rounding_of(dtype), **kw)
+    assert bool((O[0, 0, :, 1] == float("inf")).all()) and bool((O[0, 0, :, 2] == -float("inf")).all())
+    rest = [c for c in range(d) if c not in (1, 2)]
+    assert bool(O[0, 0][:, rest].isfinite().all())
+
+
+@pytest.mark.parametrize("d,dtype", FORMATS)
+def test_large_values_behind_growing_logits(d, dtype):
+    """A few keys whose logits lie 36 (base 2) above the first ones', with values about 2^100: weight times value passes the largest
+    number, while the sum of the weights stays below the bound that has a step redone."""
+    from paper_2107_06419_b200 import api
+    torch.manual_seed(d + 1)
+    Q = torch.ones(1, 2, 140, d, device="cuda", dtype=dtype)
+    K = torch.zeros(1, 2, 500, d, device="cuda", dtype=dtype)
+    K[:, :, 200:203] = 25.0 / d
+    V = torch.randn(1, 2, 500, d, device="cuda").to(dtype) * 2.0 ** 100
+    O = check(api, Q, K, V, 1.0, variant_of(api, dtype), rounding_of(dtype))
+    assert bool(O.isfinite().all())
+    f64 = lambda t: t.double().cpu().numpy()
+    x = f64(Q)[0] @ f64(K)[0].transpose(0, 2, 1)
+    p = np.exp(x - x.max(-1, keepdims=True))
+    ref = (p / p.sum(-1, keepdims=True)) @ f64(V)[0]
+    assert np.max(np.abs(f64(O)[0] - ref)) <= rounding_of(dtype) * np.abs(f64(V)).max()
