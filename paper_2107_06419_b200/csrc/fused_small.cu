@@ -404,7 +404,8 @@ int launch_small_d(const Problem& p, cudaStream_t st) {
 }  // namespace
 
 bool small_applies(const Problem& p) {
-    return p.dtype == FLAT_DTYPE_BF16 && (p.d == 16 || p.d == 32) && !p.bias && !p.block_mask;
+    // (2^30 keys: the offset that stands for "no causal mask"; what lies beyond is the FFMA kernel's)
+    return p.dtype == FLAT_DTYPE_BF16 && (p.d == 16 || p.d == 32) && !p.bias && !p.block_mask && p.Nk <= (1 << 30);
 }
 
 int launch_fused_small(const Problem& p, cudaStream_t st) {
