@@ -501,13 +501,13 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
             for (int v = 0; v < D / 4; ++v)
                 *reinterpret_cast<float4*>(scratch + 4 * v) = make_float4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
-            scratch[D] = m;
-            scratch[D + 1] = ok ? l : __int_as_float(0x7fc00000);
+            scratch[D] = ok ? m : __int_as_float(0x7fc00000);       // (a maximum is never NaN: max takes the other operand)
+            scratch[D + 1] = l;
         }
         asm volatile("bar.sync 1, 256;" ::: "memory");
         if (g == 0) {
             const float m1 = scratch[D], l1 = scratch[D + 1];
-            if (ok && l1 == l1 && row < Nq) {                // (a group that gave up leaves NaN: no output then)
+            if (ok && m1 == m1 && row < Nq) {                // (a group that gave up leaves NaN: no output then)
                 const float mt = fmaxf(m, m1);
                 const float mu = mt == -INFINITY ? 0.f : mt;
                 const float a0 = ex2_approx(m - mu), a1 = ex2_approx(m1 - mu);

@@ -7,8 +7,8 @@ pytestmark = pytest.mark.gpu
 
 
 def run(api, Q, K, V, scale, variant=0, **kw):
-    O = torch.full_like(Q, float("nan"))
-    lse = torch.full(Q.shape[:3], float("nan"), device="cuda")
+    O = torch.full_like(Q, 7.0)
+    lse = torch.full(Q.shape[:3], 7.0, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     api.flat_attn_fwd_ex(Q, K, V, O, scale, status=status, variant=variant, lse=lse, **kw)
     torch.cuda.synchronize()
@@ -81,3 +81,18 @@ def test_large_values_behind_growing_logits(d, dtype):
     p = np.exp(x - x.max(-1, keepdims=True))
     ref = (p / p.sum(-1, keepdims=True)) @ f64(V)[0]
     assert np.max(np.abs(f64(O)[0] - ref)) <= rounding_of(dtype) * np.abs(f64(V)).max()
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+@pytest.mark.parametrize("key", [5, 70, 100])            # in an even and in an odd key step
+def test_nan_inputs_leave_no_row_unwritten(d, key):
+    """A NaN logit makes its row NaN, as on the FFMA kernel; the row must not keep what the output held before."""
+    from paper_2107_06419_b200 import api
+    torch.manual_seed(key)
+    Q, K, V = (torch.randn(1, 2, n, d, device="cuda") for n in (140, 200, 200))
+    K[0, 0, key, 3] = float("nan")
+    Q[0, 1, 20, 1] = float("nan")
+    O, lse = run(api, Q, K, V, d ** -0.5)
+    F, flse = run(api, Q, K, V, d ** -0.5, variant=api.FLAT_VARIANT_SIMT)
+    assert bool(O[0, 0].isnan().all()) and bool(O[0, 1, 20].isnan().all())
+    assert torch.equal(O.isnan(), F.isnan()) and torch.equal(lse.isinf(), flse.isinf()) and bool((lse[0, 1, :20] != 7.0).all())
