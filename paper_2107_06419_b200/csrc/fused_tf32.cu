@@ -33,6 +33,8 @@
 // TMEM columns: Q_hi d, Q_lo d, then per step parity S / P_hi (as many columns as a step has keys), P_lo and P V (d); at
 // d = 128, where Q takes half of TMEM, steps of 32 keys leave room for both parities of S and P and for one P V buffer:
 // a step's P V waits until the one before has been read, which happens while the pipe works on the logits in between.
+// An infinite operand has no finite remainder: its products are NaN.  At d = 32 and 128 a row that does not come out finite is
+// computed again in plain fp32 (plain_row), which gives what the FFMA kernel gives; at d = 64 it stays NaN.
 // Every wait is bounded (see tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -125,8 +127,8 @@ __device__ __forceinline__ void split4(const uint4& v, uint4& h, uint4& l) {
 template <int D>
 __global__ void __launch_bounds__(THREADS, 1)
 fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                  const __grid_constant__ CUtensorMap tmV, float* __restrict__ O, int BH, int H, int Nq, int Nk,
-                  float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int group, int32_t* status,
+                  const __grid_constant__ CUtensorMap tmV, const float* Q, const float* K, const float* V, float* O, int BH, int H, int Nq,
+                  int Nk, float scale_log2e, const int32_t* __restrict__ valid_len, int coff, int group, int32_t* status,
                   float* __restrict__ lse) {
     using LY = Layout<D>;
     constexpr int BN = LY::BN, TILE = LY::TILE, PANEL = LY::PANEL, OFF_KH = LY::OFF_KH, OFF_KL = LY::OFF_KL, OFF_VR = LY::OFF_VR,
@@ -507,6 +509,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         asm volatile("bar.sync 1, 256;" ::: "memory");
         if (g == 0) {
             const float m1 = scratch[D], l1 = scratch[D + 1];
+            uint64_t zero[2] = {0ull, 0ull};                 // (NaN once a result is not finite)
             if (ok && m1 == m1 && row < Nq) {                // (a group that gave up leaves NaN: no output then)
                 const float mt = fmaxf(m, m1);
                 const float mu = mt == -INFINITY ? 0.f : mt;
@@ -519,8 +522,23 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
                 for (int v = 0; v < D / 4; ++v) {
                     const float4 q = *reinterpret_cast<const float4*>(scratch + 4 * v);
-                    orow[v] = make_float4(o[4 * v] * w0 + q.x * w1, o[4 * v + 1] * w0 + q.y * w1, o[4 * v + 2] * w0 + q.z * w1,
-                                          o[4 * v + 3] * w0 + q.w * w1);
+                    const float4 x = make_float4(o[4 * v] * w0 + q.x * w1, o[4 * v + 1] * w0 + q.y * w1, o[4 * v + 2] * w0 + q.z * w1,
+                                                 o[4 * v + 3] * w0 + q.w * w1);
+                    orow[v] = x;
+                    if (NEAR) { zero[0] = fma2(pack2(x.x, x.y), 0ull, zero[0]); zero[1] = fma2(pack2(x.z, x.w), 0ull, zero[1]); }
+                }
+            }
+            if (NEAR) {                                      // (at d = 64 the row stays as it is)
+                float z0, z1;
+                unpack2(add2(zero[0], zero[1]), z0, z1);
+                unsigned again = __ballot_sync(0xffffffffu, z0 + z1 != 0.f);
+                while (again) {
+                    const int at_lane = __ffs(again) - 1;
+                    again &= again - 1;
+                    __syncwarp();                            // (the row's own thread has stored it)
+                    const int64_t rr = static_cast<int64_t>(bh) * Nq + row0 + warp * 32 + at_lane;
+                    plain_row<float, D>(Q + rr * D, K + static_cast<int64_t>(bh) * Nk * D, V + static_cast<int64_t>(bh) * Nk * D, O + rr * D,
+                                        lse ? lse + rr : nullptr, __shfl_sync(0xffffffffu, nrow, at_lane), scale_log2e);
                 }
             }
         }
@@ -567,7 +585,8 @@ int launch(const Problem& p, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_tf32_kernel<D>, tmQ, tmK, tmV, static_cast<float*>(p.O), BH, p.H, p.Nq, p.Nk,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_tf32_kernel<D>, tmQ, tmK, tmV, static_cast<const float*>(p.Q), static_cast<const float*>(p.K),
+                                             static_cast<const float*>(p.V), static_cast<float*>(p.O), BH, p.H, p.Nq, p.Nk,
                                              p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status, p.lse);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }

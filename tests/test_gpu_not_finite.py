@@ -31,7 +31,7 @@ def check(api, Q, K, V, scale, variant, rounding, **kw):
     return O
 
 
-FORMATS = [(16, torch.bfloat16), (32, torch.bfloat16)]
+FORMATS = [(16, torch.bfloat16), (32, torch.bfloat16), (32, torch.float32), (128, torch.float32)]
 
 
 def variant_of(api, dtype):
