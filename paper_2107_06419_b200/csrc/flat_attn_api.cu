@@ -94,8 +94,12 @@ int run_fused(const flat::Problem& q, int variant, cudaStream_t st) {
         if (!tc_applies(q)) {
             // bf16 with d = 16 or 32: the small-head kernel (B16 H8 1000^2, d = 32: 66 us against 638 on the FFMA kernel).
             // fp32 tensors: the split-tf32 tensor-core kernel where it applies (d = 32, 64, 128; down to one tile of keys
-            // and queries: B1 H4 64^2 d = 128 14 us against 22, B2 H16 4096^2 1.2 ms against 9.5), else the FFMA kernel
-            v = flat::tf32_applies(q) ? FLAT_VARIANT_TF32 : flat::small_applies(q) ? FLAT_VARIANT_SMALL : FLAT_VARIANT_SIMT;
+            // and queries: B1 H4 64^2 d = 128 8.4 us against 13, B2 H16 4096^2 1.2 ms against 9.5), else the FFMA kernel.
+            // d = 32 with one FFMA tile (64 x 64) a head and more heads than SMs is that kernel's too, four CTAs an SM against
+            // one (us, FFMA / tf32: 148 heads 64^2 6.8 / 6.1, 190 8.8 / 10.1, 1024 29 / 37, 1024 of 16^2 25 / 39; one key more,
+            // 1024 heads 64 x 65: 48 / 42; one query more, 65 x 64: 51 / 37)
+            const bool tiny = q.d == 32 && q.Nq <= 64 && q.Nk <= 64 && static_cast<int64_t>(q.B) * q.H > flat::device_sm_count();
+            v = flat::tf32_applies(q) && !tiny ? FLAT_VARIANT_TF32 : flat::small_applies(q) ? FLAT_VARIANT_SMALL : FLAT_VARIANT_SIMT;
         } else if (flat::decode_applies(q)) {
             v = FLAT_VARIANT_DECODE;
         } else {

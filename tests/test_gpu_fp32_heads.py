@@ -79,3 +79,16 @@ def test_odd_number_of_key_steps(d):
         assert np.max(np.abs(O - ref)) <= 2e-5
         assert first is None or np.array_equal(O, first)
         first = O
+
+
+@pytest.mark.parametrize("heads,Nq,Nk,simt", [(16, 64, 64, False), (1024, 64, 64, True), (1024, 1, 16, True), (1024, 64, 65, False),
+                                              (1024, 65, 64, False)])
+def test_many_heads_of_one_tile(heads, Nq, Nk, simt):
+    """d = 32: one FFMA tile a head and more heads than SMs run on the FFMA kernel."""
+    from paper_2107_06419_b200 import api
+    rng = np.random.default_rng(heads + Nq + Nk)
+    Q, K, V = (rng.standard_normal((1, heads, n, 32)).astype(np.float32) for n in (Nq, Nk, Nk))
+    O, lse = run(api, Q, K, V, 32 ** -0.5)
+    assert api.flat_attn_last_variant() == (api.FLAT_VARIANT_SIMT if simt else api.FLAT_VARIANT_TF32)
+    ref = oracle.attention(Q, K, V, 32 ** -0.5, want_lse=True)
+    assert np.max(np.abs(O - ref["O"])) <= 2e-5 and np.max(np.abs(lse - ref["LSE"])) <= 2e-5
