@@ -29,9 +29,9 @@
 // on a carried reference, vanished), in which case both redo the step with a fresh common maximum
 // (the logits are still in TMEM: the vote comes before the weights are stored over them) and O_t, l
 // are rescaled.
-// A second instantiation (VL) runs packed batches of sequences of different lengths: the tensor maps
+// Two more instantiations (VL) run packed batches of sequences of different lengths: the tensor maps
 // then view [tokens, H, d] tensors, an item is (sequence, head, slab) and reads its sequence's
-// offsets from device arrays (see get_item).
+// offsets from device arrays (SLOTS) or from a sorted table in shared memory (SORTED; see Sched).
 // Every wait is bounded (see tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -69,6 +69,7 @@ constexpr unsigned POLY_PAIRS_SA = 0x0900, POLY_PAIRS_SB = 0x0900; // the same f
 constexpr unsigned PRODUCER_SLEEP = 400; // ns between the TMA producer's probes of a full ring (it runs far ahead: its reaction time is immaterial)
 
 constexpr int D = 64;                // head size of this kernel
+constexpr int SLOTS = 1, SORTED = 2; // values of VL (0: dense batches)
 constexpr int UNITS_MAX = 1024;      // packed batches: most (sequence, slab) units (and sequences) that are sorted (see Sched)
 
 // BT: with a ring of three bias tiles (128 x 128 bf16, two panels of 64 columns; 2: one tile of 128 x 192 per query tile), which
@@ -337,19 +338,27 @@ constexpr int WS_MAX_CTAS = 160;
 // items for b = 0 .. B (DEAL_MAX_B batches at most).
 constexpr int DEAL_LO = 0, DEAL_HI = 1, DEAL_FIRST = 2, DEAL_END = 3, DEAL_T = 4, DEAL_TEAM = 5, DEAL_TEAMS = 6, DEAL_PREFIX = 8, DEAL_MAX_B = 64;
 static_assert((DEAL_PREFIX + DEAL_MAX_B + 1) * 4 <= 512, "the deal's table has 512 bytes of shared memory");
-// (packed batches) The table of units in shared memory: first token and number of the query rows from the unit's first one
+// (SORTED) The table of units in shared memory: first token and number of the query rows from the unit's first one
 // on, first token and number of the keys; then the units' first rows.
 __device__ __forceinline__ uint4* unit_table() {
     extern __shared__ uint8_t smem_raw[];
     return reinterpret_cast<uint4*>(((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023)) + L3::TILE_BYTES + L3::XCH_BYTES + 1024);
 }
-// (packed batches) The number of rounds in which this CTA has an item, and the position of the item of a round.
-__device__ __forceinline__ int vl_rounds(int items, int sorted) {
+// (SORTED) The number of rounds in which this CTA has an item, and the position of the item of a round.  The number stays in
+// shared memory, in front of the table, and is read where an item ends: a register that held it through the key steps would be
+// one too many (24 bytes of spills: 32 sequences of 1000 tokens, 16 heads, 187 us against 178).
+__device__ __forceinline__ int unit_rounds(int items) {
     const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x), full = items / G, rest = items - full * G;
-    return full + ((sorted && (full & 1) ? G - 1 - c : c) < rest ? 1 : 0);
+    return full + ((full & 1 ? G - 1 - c : c) < rest ? 1 : 0);
 }
-__device__ __forceinline__ int vl_position(int round, int sorted) {
-    return round * static_cast<int>(gridDim.x) + static_cast<int>(sorted && (round & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+__device__ __forceinline__ int unit_position(int round) {
+    return round * static_cast<int>(gridDim.x) + static_cast<int>(round & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+}
+__device__ __forceinline__ uint32_t rounds_at() { return smem_u32(unit_table()) - 512; }
+__device__ __forceinline__ int stored_rounds() {
+    int v;
+    asm volatile("ld.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(rounds_at()) : "memory");
+    return v;
 }
 // What every role needs to enumerate the items.
 struct Sched {
@@ -357,7 +366,7 @@ struct Sched {
     const int32_t* valid_len;
     int coff;                                            // causal mask: row r sees keys j < r + 1 + coff (coff = Nk - Nq); none: 2^30
     int paired;                                          // 1: items come in pairs of complementary slabs (see get_item)
-    // (packed batches) 1: the units (sequence, slab) are sorted by their number of key steps, longest first, into a table
+    // SORTED: the units (sequence, slab) are sorted by their number of key steps, longest first, into a table
     // in shared memory (fill_units), every unit stands for its H heads, and the CTAs take the items of that order
     // forwards and backwards in turn -- CTA c has items c, 2 G - 1 - c, 2 G + c, ... -- so that their shares weigh the
     // same to a few per cent (32 sequences of 40 to 2000 tokens, 12 heads: 105 us with a CTA per slot of the longest
@@ -480,19 +489,19 @@ __device__ __forceinline__ void deal_finish_merged(const EvenDeal ed, uint32_t o
 }
 // The sequence of item indices of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...; in paired mode the
 // CTA takes PAIRS of consecutive indices (2 c, 2 c + 1), (2 (c + gridDim.x), ...), ...
-template <bool SPLIT = false, bool VL = false>
+template <bool SPLIT = false, int VL = 0>
 __device__ __forceinline__ int first_item(const Sched& sc) {
     if (SPLIT) return sc.deal[DEAL_FIRST];
-    if (VL) return 0;
+    if (VL == SORTED) return 0;
     return sc.paired ? 2 * blockIdx.x : blockIdx.x;
 }
-template <bool SPLIT = false, bool VL = false>
+template <bool SPLIT = false, int VL = 0>
 __device__ __forceinline__ int next_item(int idx, const Sched& sc) {
     if (SPLIT) return idx + sc.deal[DEAL_TEAM];
-    if (VL) return idx + 1;
+    if (VL == SORTED) return idx + 1;
     return sc.paired ? ((idx & 1) ? idx - 1 + 2 * static_cast<int>(gridDim.x) : idx + 1) : idx + static_cast<int>(gridDim.x);
 }
-// (packed batches, sorted) The unit of the item at position `pos`: pos / H by the reciprocal that the launcher gives
+// (SORTED) The unit of the item at position `pos`: pos / H by the reciprocal that the launcher gives
 // in ed.team (exact: pos < 1024 H and H < 2048).
 __device__ __forceinline__ int unit_of(int pos, const Sched& sc) {
     return sc.H == 1 ? pos : static_cast<int>(__umulhi(static_cast<unsigned>(pos), static_cast<unsigned>(sc.ed.team)));
@@ -501,7 +510,7 @@ __device__ __forceinline__ int unit_of(int pos, const Sched& sc) {
 // tokens cu_q[s] .. cu_q[s+1] - 1 of Q and cu_k[s] .. cu_k[s+1] - 1 of K, V.  Item index =
 // (sequence * H + head) * slabs + slab with `slabs` taken from the longest sequence; a slab past the
 // end of its sequence is an empty slot.  The causal offset is that of the sequence.
-template <bool VL, bool SPLIT = false, bool BIAS = false>
+template <int VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ Item get_item(int idx, const Sched& sc) {
     Item it;
     int slab;
@@ -509,8 +518,8 @@ __device__ __forceinline__ Item get_item(int idx, const Sched& sc) {
     it.tile0 = 0;
     if (VL) {
         int ql, k0, kl;
-        idx = vl_position(idx, sc.paired);
-        if (sc.paired) {
+        if (VL == SORTED) {
+            idx = unit_position(idx);
             const int u = unit_of(idx, sc);
             it.head = idx - u * sc.H;
             const uint32_t at = smem_u32(unit_table());
@@ -586,21 +595,21 @@ struct Cursor {
     Item it;
     bool valid;
 };
-template <bool VL, bool SPLIT = false, bool BIAS = false>
+template <int VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ void cursor_seek(Cursor& c, const Sched& sc) {
     c.valid = false;
-    while (c.idx < sc.items) {
+    while (c.idx < (VL == SORTED ? stored_rounds() : sc.items)) {
         c.it = get_item<VL, SPLIT, BIAS>(c.idx, sc);
         if (c.it.ntiles > 0) { c.valid = true; return; }
         c.idx = next_item<SPLIT, VL>(c.idx, sc);
     }
 }
-template <bool VL, bool SPLIT = false, bool BIAS = false>
+template <int VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ void cursor_init(Cursor& c, const Sched& sc) {
     c.idx = first_item<SPLIT, VL>(sc); c.j = 0; c.J = 0; c.q = 0;
     cursor_seek<VL, SPLIT, BIAS>(c, sc);
 }
-template <bool VL, bool SPLIT = false, bool BIAS = false>
+template <int VL, bool SPLIT = false, bool BIAS = false>
 __device__ __forceinline__ void cursor_next(Cursor& c, const Sched& sc) {
     ++c.j; ++c.J;
     if (c.j == c.it.ntiles) {
@@ -688,7 +697,7 @@ __device__ __forceinline__ int fill_units(const Sched& sc, uint4* tab, int seqs)
 // the plain kernel: 100 instructions per 64 logits (eight 16-byte loads, unpacking, one packed FMA a pair) in the kernel
 // whose exponent unit, not its issue slots, is the bound.  Before, the bias was read by the kernel with one softmax
 // thread per row (fused_tc2.cu), 6,500 cycles a key step: B8 H16 1024 x 1024 110 us, 70 here; B16 H16 4096 x 4096 2.55 ms, 1.63 here.
-template <bool VL, bool WLSE = false, bool SPLIT = false, int BIAS = 0>
+template <int VL, bool WLSE = false, bool SPLIT = false, int BIAS = 0>
 __global__ void __launch_bounds__(L3::THREADS, 1)
 fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, int H, int Nq, int Nk,
@@ -701,7 +710,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     static_assert(!BIAS || (!VL && !SPLIT), "the bias is read by the plain dense kernel");
     static_assert(!SPLIT || (!VL && !WLSE), "the even deal is built for the plain dense forward kernel only");
     Sched sc{items, slabs, H, Nk, valid_len, coff, paired, cu_q, cu_k, nullptr, BIAS && !bias_batches ? items / (H * (paired ? (slabs + 1) & ~1 : slabs)) : 0, ed};
-    if (VL && ed.epoch) {
+    if (VL == SLOTS && ed.epoch) {
         // One CTA per slot: a slot past the end of its sequence leaves before anything is set up.  The offsets may be what
         // the previous kernel of the stream writes, so that one is waited for first.  (The next kernel is let go behind the
         // set-up only, as ever: one that got the tensor memory before a CTA of this grid would hold it until the grid ends.)
@@ -787,7 +796,12 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
-    if (VL) sc.items = items = vl_rounds(paired ? fill_units(sc, unit_table(), Nk) * H : items, paired);
+    if (VL == SORTED) {
+        const int rounds = unit_rounds(fill_units(sc, unit_table(), Nk) * H);
+        if (threadIdx.x == 0) asm volatile("st.shared::cta.s32 [%0], %1;" ::"r"(rounds_at()), "r"(rounds) : "memory");
+        __syncthreads();
+    }
+    auto more = [&](int idx) { return idx < (VL == SORTED ? stored_rounds() : items); };
     if (SPLIT) { sc.deal = deal; sc.items = deal[DEAL_END]; items = deal[DEAL_END]; }
 
     if (warp >= LY::SOFT_WARPS) {
@@ -849,7 +863,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 }
             };
             int J0 = 0, q = 0;
-            for (int idx = first_item<SPLIT, VL>(sc); idx < items && ok; idx = next_item<SPLIT, VL>(idx, sc)) {
+            for (int idx = first_item<SPLIT, VL>(sc); more(idx) && ok; idx = next_item<SPLIT, VL>(idx, sc)) {
                 const Item it = get_item<VL, SPLIT, BIAS>(idx, sc);
                 if (it.ntiles == 0) continue;
                 // tile of query rows r.. / of keys of step j
@@ -978,7 +992,7 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // of the CTA and items whose first step is partly masked start from an exact maximum.
         float m_ref = -INFINITY;
         bool first_item_done = false;
-        for (int idx = first_item<SPLIT, VL>(sc); idx < items; idx = next_item<SPLIT, VL>(idx, sc)) {
+        for (int idx = first_item<SPLIT, VL>(sc); more(idx); idx = next_item<SPLIT, VL>(idx, sc)) {
         const Item it = get_item<VL, SPLIT, BIAS>(idx, sc);
         if (it.skip) continue;
         const int ntiles = it.ntiles;
@@ -1186,17 +1200,12 @@ fused_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             }
         }
         {
-            // (packed batches: the rows are looked up again, so that they do not live in registers through the key steps)
-            int tok0 = 0, rows = 0, head = 0;
-            if (VL) {
-                if (paired) {
-                    const int pos = vl_position(idx, paired), u = unit_of(pos, sc);
-                    head = pos - u * H;
-                    asm volatile("ld.shared::cta.v2.s32 {%0, %1}, [%2];" : "=r"(tok0), "=r"(rows) : "r"(smem_u32(unit_table()) + 16 * u) : "memory");
-                } else {
-                    const Item ie = get_item<VL, SPLIT>(idx, sc);
-                    tok0 = ie.q_tok0; rows = ie.q_rows; head = ie.head;
-                }
+            // (SORTED: the rows are looked up again, so that they do not live in registers through the key steps)
+            int tok0 = it.q_tok0, rows = it.q_rows, head = it.head;
+            if (VL == SORTED) {
+                const int pos = unit_position(idx), u = unit_of(pos, sc);
+                head = pos - u * H;
+                asm volatile("ld.shared::cta.v2.s32 {%0, %1}, [%2];" : "=r"(tok0), "=r"(rows) : "r"(smem_u32(unit_table()) + 16 * u) : "memory");
             }
             const int row = (VL ? 0 : it.row0) + t * BM + q * 32 + lane;   // (packed batches: counted from the slab's first)
             const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -1416,31 +1425,37 @@ int launch_fused_tc3_varlen(const void* Q, const void* K, const void* V, void* O
     if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
         !make_map_packed(&tmV, V, total_k, H, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_tc3_kernel<true>>(LY::VL_SMEM_BYTES)) return FLAT_ERR_CUDA;
     const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM);
     const int64_t items = static_cast<int64_t>(slabs) * num_seqs * H;
     if (items > 0x7fffffff) return FLAT_ERR_SHAPE;
     const int sms = device_sm_count();
-    // Persistent CTAs on sorted units (see Sched) where the table holds them all: a sequence has at most one slab more
-    // than its share of the tokens fills.  Otherwise the slots of the longest sequence's grid, by fixed deal while they
-    // are short, or one CTA each, handed out by the hardware as SMs become free (8 sequences of 3.9K-14.5K tokens: 2.81 ms
-    // against 2.89 by fixed deal, causal 1.61 against 1.86).
-    const int64_t units = total_q / (2 * BM) + num_seqs < static_cast<int64_t>(slabs) * num_seqs ? total_q / (2 * BM) + num_seqs
-                                                                                                  : static_cast<int64_t>(slabs) * num_seqs;
-    // (sequences of one length need no order: the table costs about 2 us a launch)
-    const bool equal = !causal && total_q == static_cast<int64_t>(num_seqs) * max_seqlen_q;
-    const bool sorted = units <= UNITS_MAX && num_seqs <= UNITS_MAX && H < 2048 && !equal;
-    const bool persistent = sorted || (items >= 8 * static_cast<int64_t>(sms) && slabs < 8);
+    // Persistent CTAs on sorted units (see Sched) where the table holds them all (a sequence has at most one slab more than its
+    // share of the tokens fills) and there is more than one item per SM.  Otherwise the slots of the longest sequence's grid, by
+    // fixed deal while they are short, or one CTA each, handed out by the hardware as SMs become free (8 sequences of 3.9K-14.5K
+    // tokens: 2.81 ms against 2.89 by fixed deal, causal 1.61 against 1.86).  Slots that all weigh the same -- sequences of one
+    // length, without the causal mask or of one slab -- need no order and go by fixed deal (us, sorted / fixed deal / a CTA per
+    // slot: 100 of 256 tokens, 16 heads 59 / 54 / 53, causal 75 / 68 / 67; 64 of 128, 8 heads 18.6 / 16.1 / 23.9; 16 of 512, 8
+    // heads 19.6 / 18.8 / 21.5; 2 of 8192, 16 heads 574 / 558 / 577).  The table costs 1 us: with one item per SM or less it is
+    // left out (4 of 40 to 200 tokens, 4 heads 8.5 us sorted, 7.5 by slots; 8 of 40 to 512, 12 heads, 156 items 13.0 and 16.1).
+    const int64_t all = static_cast<int64_t>(slabs) * num_seqs, bound = total_q / (2 * BM) + num_seqs, units = bound < all ? bound : all;
+    const bool one_length = total_q == static_cast<int64_t>(num_seqs) * max_seqlen_q;
+    const bool alike = one_length && total_k == total_q && (!causal || slabs == 1);
+    const bool sorted = !alike && units * H > sms && units <= UNITS_MAX && num_seqs <= UNITS_MAX && H < 2048;
+    const bool persistent = sorted || (alike ? items > sms : items >= 8 * static_cast<int64_t>(sms) && slabs < 8);
     const int64_t most = sorted ? units * H : items;
     const int grid = static_cast<int>(persistent && most > sms ? sms : most);
     EvenDeal ed{};
     ed.team = static_cast<int>(static_cast<unsigned>(((1ull << 32) + H - 1) / H));   // (see unit_of)
-    ed.epoch = !persistent && !equal;                    // (a CTA per slot, some of them past the end of their sequence)
+    // a CTA per slot, some of them past the end of their sequence, and not all at the same time: those leave at once
+    ed.epoch = !persistent && items > sms && !one_length;
     g_last_schedule = persistent ? FLAT_SCHEDULE_PERSISTENT : FLAT_SCHEDULE_ITEMS;
+    const int bytes = sorted ? LY::VL_SMEM_BYTES : LY::SMEM_BYTES;
+    if (!(sorted ? ensure_dynamic_smem<fused_tc3_kernel<SORTED>>(bytes) : ensure_dynamic_smem<fused_tc3_kernel<SLOTS>>(bytes))) return FLAT_ERR_CUDA;
     const cudaError_t e = launch_pdl(
-        fused_tc3_kernel<true>, grid, LY::VL_SMEM_BYTES, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H, max_seqlen_q, num_seqs,
-        static_cast<int>(most), slabs, scale * 1.4426950408889634f, static_cast<const int32_t*>(nullptr), causal ? 0 : (1 << 30), status,
-        (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, sorted ? 1 : 0, cu_q, cu_k, static_cast<float*>(nullptr), ed, CUtensorMap{}, 0, 0, ShiftedBias{});
+        sorted ? fused_tc3_kernel<SORTED> : fused_tc3_kernel<SLOTS>, grid, bytes, st, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), H,
+        max_seqlen_q, num_seqs, static_cast<int>(most), slabs, scale * 1.4426950408889634f, static_cast<const int32_t*>(nullptr),
+        causal ? 0 : (1 << 30), status, (reinterpret_cast<uintptr_t>(O) & 31) == 0 ? 1 : 0, 0, cu_q, cu_k, static_cast<float*>(nullptr), ed,
+        CUtensorMap{}, 0, 0, ShiftedBias{});
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
