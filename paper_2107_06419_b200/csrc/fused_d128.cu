@@ -22,7 +22,8 @@
 // The softmax takes no row maximum after the first step: any reference gives the exact softmax, and a step whose row sum
 // passes 2^40 is redone with a fresh maximum.  One exponential in four goes through a polynomial on the FMA pipe.
 // MULTI: a CTA walks over items (batch, head, slab of 256 rows); the rings and barriers go on from one to the next.
-// VL: packed batches (Q, O [total_q, H, d], K, V [total_k, H, d]), a CTA per (sequence, head, slab of the longest sequence).
+// VL: packed batches (Q, O [total_q, H, d], K, V [total_k, H, d]), an item per (sequence, head, slab of the longest sequence): a
+// CTA each, or (MULTI, sequences of one length) by fixed deal.
 // Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -169,21 +170,28 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    // The CTA's r-th item: (batch, head, slab of 256 rows). (Packed batches: one.)
+    // The CTA's r-th item: (batch, head, slab of 256 rows).
     auto get_item = [&](int r, Item& it) -> bool {
         if (!MULTI && r > 0) return false;
         it.n = Nk;
         it.coff = coff;
         if (VL) {
-            // the slabs of a sequence side by side; under the causal mask the last slabs (the longest) of all sequences first
-            it.bh = group ? blockIdx.x : blockIdx.y;
-            it.row0 = static_cast<int>(group ? gridDim.y - 1 - blockIdx.y : blockIdx.x) * (2 * BM);
+            if (MULTI) {
+                const unsigned pos = r * gridDim.x + blockIdx.x, slabs = (Nq + 2 * BM - 1) / (2 * BM);
+                if (pos >= BH * slabs) return false;
+                it.bh = pos / slabs;
+                it.row0 = static_cast<int>(pos % slabs) * (2 * BM);
+            } else {
+                // the slabs of a sequence side by side; under the causal mask the last slabs (the longest) of all sequences first
+                it.bh = group ? blockIdx.x : blockIdx.y;
+                it.row0 = static_cast<int>(group ? gridDim.y - 1 - blockIdx.y : blockIdx.x) * (2 * BM);
+            }
             const int s = it.bh / H;
             it.head = it.bh - s * H;
             const int q0 = cu_q[s], ql = cu_q[s + 1] - q0, k0 = cu_k[s], kl = cu_k[s + 1] - k0;
-            if (it.row0 >= ql) return false;
+            if (!MULTI && it.row0 >= ql) return false;
             it.q_tok0 = q0 + it.row0; it.k_tok0 = k0; it.q_rows = ql - it.row0;
-            it.n = kl < 0 ? 0 : kl;
+            it.n = kl < 0 || it.q_rows <= 0 ? 0 : kl;
             if (coff < (1 << 29)) it.coff = kl - ql;
         } else {
             // `group` heads at a time, their slabs side by side, the longest first under the causal mask; CTAs with several
@@ -205,7 +213,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     };
     // (bias, shifted) the slab's first row among all rows of the bias
     auto bias_row = [&](const Item& it) { return ((bias_batches ? it.bh / H : 0) * (bias_heads ? H : 1) + (bias_heads ? it.bh % H : 0)) * Nq + it.row0; };
-    if (VL) {
+    if (VL && !MULTI) {
         Item it;
         if (!get_item(0, it)) return;                    // (the whole CTA: nothing is set up yet)
     }
@@ -566,12 +574,21 @@ int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* 
     if (!make_map_packed(&tmQ, Q, total_q, H, D, BM) || !make_map_packed(&tmK, K, total_k, H, D, BN) ||
         !make_map_packed(&tmV, V, total_k, H, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<true, 0, false>>(Layout<0>::SMEM_BYTES)) return FLAT_ERR_CUDA;
-    const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535;
-    const dim3 grid(group ? num_seqs * H : slabs, group ? slabs : num_seqs * H);
-    fused_d128_kernel<true, 0, false><<<grid, THREADS, Layout<0>::SMEM_BYTES, st>>>(
+    const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535, sms = device_sm_count();
+    const int64_t items = static_cast<int64_t>(slabs) * num_seqs * H;
+    // Items that all weigh the same -- sequences of one length, without the causal mask or of one slab -- several per CTA, up to
+    // launch_fused_d128's bound and from three per SM on (us, a CTA each / dealt: 100 of 256 tokens, 16 heads 146 / 129, causal
+    // 142 / 116; 64 of 128, 8 heads 26.3 / 20.7; 64 of 64, 16 heads 36 / 22; 32 of 1000, 16 heads 281 / 275; with 1.7 and 2.6 per
+    // SM, 16 of 512, 8 heads 26.5 / 27.5, 16 of 300, 12 heads 33.1 / 35.4).
+    const bool alike = total_q == static_cast<int64_t>(num_seqs) * max_seqlen_q && total_k == total_q && (!causal || slabs == 1);
+    const bool several = alike && items >= 3 * static_cast<int64_t>(sms) && items <= 0x7fffffff && max_seqlen_q <= 1024;
+    if (!(several ? ensure_dynamic_smem<fused_d128_kernel<true, 0, true>>(Layout<0>::SMEM_BYTES)
+                  : ensure_dynamic_smem<fused_d128_kernel<true, 0, false>>(Layout<0>::SMEM_BYTES)))
+        return FLAT_ERR_CUDA;
+    const dim3 grid(several ? sms : group ? num_seqs * H : slabs, several ? 1 : group ? slabs : num_seqs * H);
+    (several ? fused_d128_kernel<true, 0, true> : fused_d128_kernel<true, 0, false>)<<<grid, THREADS, Layout<0>::SMEM_BYTES, st>>>(
         tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), num_seqs * H, H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
-        causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr);
+        causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr, CUtensorMap{}, 0, 0, ShiftedBias{});
     return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
