@@ -1380,10 +1380,14 @@ int launch_tc3(const Problem& p, cudaStream_t st) {
     // the longest CTA takes ceil(items / SMs) x key steps; the deal's the average and what measures as 5 % and 10 steps more (the
     // two extra item boundaries, the merge).  On either side of that line (us, whole items / dealt; items per SM, key steps):
     // H5 16K^2 2.16, 128: 496 / 363; B2 H10 4096^2 2.16, 32: 124 / 108; B2 H8 8192^2 3.46, 64: 318 / 297; B2 H6 4930^2 1.62, 39:
-    // 105 / 101; B4 H8 3000^2 2.59, 24: 97 / 100; B7 H12 1500^2 3.41, 12: 71 / 73; H17 4096^2 1.84, 32: 88 / 93.
+    // 105 / 101; B4 H8 3000^2 2.59, 24: 97 / 100; B7 H12 1500^2 3.41, 12: 71 / 73; H17 4096^2 1.84, 32: 88 / 93.  Where there are
+    // less than one and a half items per SM, one of them per CTA otherwise, the deal costs less (3 to 7 steps) and is taken in any case:
+    // B3 H12 1500^2 1.46, 12: 40.5 / 37.3; H30 1600^2 1.42, 13: 42.5 / 41.2; B2 H13 1800^2 1.41, 15: 47.5 / 45.8; H26 2048^2 1.41,
+    // 16: 49.3 / 47.3 (H35 1536^2 1.42, 12: 39.8 / 41.2; B1 H40 1500^2, 1.62, 12: 40.5 / 43.2).
     if (!p.causal && !p.lse && p.B <= DEAL_MAX_B && sms <= WS_MAX_CTAS && items > 0) {
         const int64_t nt = (p.Nk + BN - 1) / BN, rounds = (items + sms - 1) / sms;
-        const bool ragged = p.k_valid_len ? !persistent : 21 * items * nt + 200 * sms < 20 * rounds * nt * sms;
+        const bool ragged = p.k_valid_len ? !persistent
+                                          : (!persistent && 4 * items < 3 * rounds * sms) || 21 * items * nt + 200 * sms < 20 * rounds * nt * sms;
         // teams of `slabs` CTAs if they fill nine SMs in ten; single items only where K and V of all heads stay in L2
         EvenDeal ed{};
         const bool teams_fit = slabs <= sms && 10 * ((sms / slabs) * slabs) >= 9 * sms;

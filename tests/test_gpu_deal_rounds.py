@@ -31,3 +31,21 @@ def test_deal_of_equal_items(case):
         check_bf16(bf16_to_f64(O.reshape(-1, 64)[torch.from_numpy(rows).cuda()]), ref, "deal")
         assert first is None or torch.equal(O, first)
         first = O
+
+
+@pytest.mark.parametrize("B,H,N,dealt", [(3, 12, 1500, True), (1, 26, 2048, True), (1, 30, 1600, True), (1, 40, 1500, False), (1, 17, 4096, False)])
+def test_line_of_the_deal(B, H, N, dealt):
+    """Less than one and a half items per SM: dealt; above, with few key steps: whole."""
+    from paper_2107_06419_b200 import api
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the expected choices are those of a 148-SM GPU")
+    torch.manual_seed(N)
+    Q, K, V = (torch.randn(B, H, N, 64, device="cuda").to(torch.bfloat16) for _ in range(3))
+    O = torch.full_like(Q, float("nan"))
+    torch.cuda.synchronize()
+    api.flat_attn_fwd(Q, K, V, O, 0.125)
+    torch.cuda.synchronize()
+    assert api.flat_attn_last_variant() == api.FLAT_VARIANT_TC3
+    assert (api.flat_attn_last_schedule() == api.FLAT_SCHEDULE_EVEN_DEAL) == dealt
+    ref = torch.softmax(Q.float() @ K.float().transpose(2, 3) * 0.125, -1) @ V.float()
+    assert float((O.float() - ref).abs().max()) <= 2e-2  # (the parity bar of bf16 results)
