@@ -310,7 +310,15 @@ def flat_attn_bwd_ex(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, k_valid_len=
 
 def flat_attn_bwd(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, stream=None):
     """flat_attn_bwd_ex without masks and without a status word."""
-    return flat_attn_bwd_ex(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, stream=stream)
+    rc = _binding.bwd(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, stream)
+    if rc >= 0:
+        if rc:
+            raise FlatAttnError(rc)
+        return dQ, dK, dV
+    p = _bwd_params(Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, None, None, False)
+    _check(_lib.flat_attn_bwd(p.Q, p.K, p.V, p.O, p.dO, p.lse, p.dQ, p.dK, p.dV, p.delta, p.B, p.H, p.Nq, p.Nk, p.d,
+                              p.scale, _stream_ptr(stream)))
+    return dQ, dK, dV
 
 
 def flat_attn_naive_fwd(Q, K, V, O, L, A, scale, stream=None):

@@ -134,7 +134,7 @@ PyObject* fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {       // Q, K, V
     void* st = a.stream();
     a.end();
     if (a.bad) return no();
-    return run([&] { return flat_attn_fwd_ex(&p, st); });
+    return run([&] { return flat_attn_fwd(p.Q, p.K, p.V, p.O, p.B, p.H, p.Nq, p.Nk, p.d, p.scale, st); });
 }
 
 PyObject* fwd_ex(PyObject*, PyObject* const* args, Py_ssize_t n) {
@@ -180,29 +180,45 @@ PyObject* fwd_ex(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return run([&] { return flat_attn_fwd_ex(&p, st); });
 }
 
-PyObject* bwd_ex(PyObject*, PyObject* const* args, Py_ssize_t n) {
-    // Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, k_valid_len, status, causal, stream
-    Args a{args, n};
+// Q, K, V, O, dO, lse, dQ, dK, dV, delta, scale, [k_valid_len, status, causal,] stream
+bool bwd_args(Args& a, bool ex, flat_attn_bwd_params_t& p, void*& st) {
     flat_attn_params_t f{};
-    if (!qkvo(a, at::kBFloat16, f)) return no();
+    if (!qkvo(a, at::kBFloat16, f)) return false;
     const at::Tensor *dO = a.bf16(), *lse = a.tensor(at::kFloat), *dQ = a.bf16(), *dK = a.bf16(), *dV = a.bf16(),
                      *delta = a.tensor(at::kFloat);
-    flat_attn_bwd_params_t p{};
     p.scale = static_cast<float>(a.number());
-    const at::Tensor* valid = a.tensor(at::kInt, true);
-    p.status = a.status();
-    p.causal = a.truth();
-    void* st = a.stream();
+    const at::Tensor* valid = ex ? a.tensor(at::kInt, true) : nullptr;
+    p.status = ex ? a.status() : nullptr;
+    p.causal = ex ? a.truth() : 0;
+    st = a.stream();
     a.end();
     if (a.bad || !is(*dO, {f.B, f.H, f.Nq, f.d}) || !is(*dQ, {f.B, f.H, f.Nq, f.d}) || !is(*dK, {f.B, f.H, f.Nk, f.d}) ||
         !is(*dV, {f.B, f.H, f.Nk, f.d}) || !is(*lse, {f.B, f.H, f.Nq}) || !is(*delta, {f.B, f.H, f.Nq}) ||
         (valid && !is(*valid, {f.B})))
-        return no();
+        return false;
     p.Q = f.Q; p.K = f.K; p.V = f.V; p.O = f.O;
     p.dO = ptr(dO); p.dQ = ptr(dQ); p.dK = ptr(dK); p.dV = ptr(dV);
     p.lse = at_<const float>(lse); p.delta = at_<float>(delta);
     p.B = f.B; p.H = f.H; p.Nq = f.Nq; p.Nk = f.Nk; p.d = f.d;
     p.k_valid_len = at_<const int32_t>(valid);
+    return true;
+}
+
+PyObject* bwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    Args a{args, n};
+    flat_attn_bwd_params_t p{};
+    void* st = nullptr;
+    if (!bwd_args(a, false, p, st)) return no();
+    return run([&] {
+        return flat_attn_bwd(p.Q, p.K, p.V, p.O, p.dO, p.lse, p.dQ, p.dK, p.dV, p.delta, p.B, p.H, p.Nq, p.Nk, p.d, p.scale, st);
+    });
+}
+
+PyObject* bwd_ex(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    Args a{args, n};
+    flat_attn_bwd_params_t p{};
+    void* st = nullptr;
+    if (!bwd_args(a, true, p, st)) return no();
     return run([&] { return flat_attn_bwd_ex(&p, st); });
 }
 
@@ -293,7 +309,7 @@ template <Fast* F> PyObject* guarded(PyObject* self, PyObject* const* args, Py_s
 }
 
 #define FAST(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(guarded<f>)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {FAST(fwd), FAST(fwd_ex), FAST(bwd_ex), FAST(varlen_fwd), FAST(layer_fwd), FAST(fc_fwd),
+PyMethodDef methods[] = {FAST(fwd), FAST(fwd_ex), FAST(bwd), FAST(bwd_ex), FAST(varlen_fwd), FAST(layer_fwd), FAST(fc_fwd),
                          FAST(layernorm_fwd), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
