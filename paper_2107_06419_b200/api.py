@@ -11,8 +11,8 @@ PyTorch is used for); every computation happens inside the library's kernels.
 from __future__ import annotations
 
 import ctypes
-import glob
 import os
+import sysconfig
 
 import torch
 
@@ -26,10 +26,16 @@ if not os.path.exists(LIB_PATH):
 
 _lib = ctypes.CDLL(LIB_PATH)
 
-if not glob.glob(os.path.join(_HERE, "_binding*.so")):
-    raise ImportError("the extension module _binding is not built (run `python -m paper_2107_06419_b200.build`)")
+_REBUILD = " (run `python -m paper_2107_06419_b200.build`)"
+if not os.path.exists(os.path.join(_HERE, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))):
+    raise ImportError("the extension module _binding is not built for this Python" + _REBUILD)
 
-from . import _binding  # noqa: E402  (after the library that it calls)
+try:
+    from . import _binding  # noqa: E402  (after the library that it calls)
+except ImportError as e:
+    raise ImportError("the extension module _binding does not load: %s%s" % (e, _REBUILD)) from e
+if ("torch %s," % torch.__version__) not in _binding.built_for:
+    raise ImportError("the extension module _binding is a %s, this is torch %s%s" % (_binding.built_for, torch.__version__, _REBUILD))
 
 FLAT_OK = 0
 FLAT_DTYPE_BF16, FLAT_DTYPE_F32 = 0, 1

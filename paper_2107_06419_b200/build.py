@@ -21,7 +21,8 @@ def nvcc_path() -> str:
     raise RuntimeError("nvcc not found: libflat_attn.so cannot be built")
 
 
-BINDING = os.path.join(HERE, "_binding.so")
+BINDING = os.path.join(HERE, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))   # (the name says which Python it is for)
+BINDING_FLAGS = ["-O2", "-std=c++17", "-shared", "-fPIC"]
 
 
 def _older(target: str, deps) -> bool:
@@ -46,6 +47,19 @@ def build_library(verbose: bool = False) -> None:
     os.replace(tmp, LIB)
 
 
+def binding_key() -> str:
+    """What the extension module is compiled against: it reads torch's tensors through torch's C++ headers and libraries."""
+    import torch
+    return "flat_attn binding for torch %s, %s" % (torch.__version__, " ".join(BINDING_FLAGS))
+
+
+def binding_is_stale() -> bool:
+    if _older(BINDING, [os.path.join(CSRC, "binding.cpp"), os.path.join(HERE, "..", "include", "flat_attn.h")]):
+        return True
+    with open(BINDING, "rb") as f:                       # (the module holds its key as a string)
+        return binding_key().encode() not in f.read()
+
+
 def build_binding() -> None:
     """The extension module next to the library, which it is linked against (found through its own folder)."""
     import torch
@@ -53,17 +67,17 @@ def build_binding() -> None:
     include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include"), sysconfig.get_paths()["include"]]
     tmp = BINDING + ".%d.tmp" % os.getpid()
-    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC"] + ["-I" + d for d in include]
-                          + [os.path.join(CSRC, "binding.cpp"), "-o", tmp, "-L" + os.path.join(root, "lib"), "-lc10",
-                             "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L" + HERE, "-l:libflat_attn.so",
-                             "-Wl,-rpath,$ORIGIN"])
+    subprocess.check_call(["g++"] + BINDING_FLAGS + ["-I" + d for d in include] + ['-DBINDING_KEY="%s"' % binding_key(),
+                          os.path.join(CSRC, "binding.cpp"), "-o", tmp, "-L" + os.path.join(root, "lib"), "-lc10",
+                          "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L" + HERE, "-l:libflat_attn.so",
+                          "-Wl,-rpath,$ORIGIN"])
     os.replace(tmp, BINDING)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     if force or is_stale():
         build_library(verbose)
-    if force or _older(BINDING, [os.path.join(CSRC, "binding.cpp"), os.path.join(HERE, "..", "include", "flat_attn.h")]):
+    if force or binding_is_stale():
         build_binding()
     return LIB
 

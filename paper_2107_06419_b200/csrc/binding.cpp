@@ -315,4 +315,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding() { return PyModule_Create(&module); }
+// `built_for`: what the module was compiled against (build.py rebuilds it when that is no longer what is there)
+PyMODINIT_FUNC PyInit__binding() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", BINDING_KEY) != 0) { Py_DECREF(m); return nullptr; }
+    return m;
+}
