@@ -52,17 +52,20 @@ def test_ends_of_the_range(d):
     rng = np.random.default_rng(d)
     Q, K = (rng.standard_normal((1, 1, n, d)).astype(np.float32) for n in (40, 70))
     V = rng.standard_normal((1, 1, 70, d)).astype(np.float32)
-    V[..., 0] = np.finfo(np.float32).max                                  # a mean of the largest number
+    big = np.finfo(np.float32).max
+    V[..., 0] = big / 128                                # (70 weights of at most 1 each: no partial sum passes the largest number)
     V[..., 1] = 1e-38
     V[..., 2] = 0.0
     O, _ = run(api, Q, K, V, d ** -0.5)
     ref = oracle.attention(Q, K, V, d ** -0.5)["O"]
-    assert np.all(np.isfinite(O[..., 1:])) and np.all(O[..., 2] == 0.0)
-    # (the sum of weights in fp32 may pass the largest number by a rounding)
-    big = O[..., 0]
-    assert np.all((np.abs(big / ref[..., 0] - 1) <= 1e-5) | np.isposinf(big))
+    assert np.all(np.isfinite(O)) and np.all(O[..., 2] == 0.0)
+    assert np.max(np.abs(O[..., 0] / ref[..., 0] - 1)) <= 1e-5
     assert np.max(np.abs(O[..., 1] - ref[..., 1])) <= 2.0 ** -10 * 1e-38 + 1e-44
     assert np.max(np.abs(O[..., 3:] - ref[..., 3:])) <= 2e-5
+    # one visible key: its values, the largest number of either sign included, whose head must not be rounded to infinity
+    V[..., 0], V[..., 3] = big, -big
+    one, _ = run(api, Q, K, V, d ** -0.5, vl=np.array([1], dtype=np.int32))
+    assert np.all(np.isfinite(one)) and np.max(np.abs(one[..., [0, 3]] / V[0, 0, 0, [0, 3]].astype(np.float64) - 1)) <= 2.0 ** -20
 
 
 @pytest.mark.parametrize("d", [32, 64, 128])
