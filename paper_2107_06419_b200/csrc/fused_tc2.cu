@@ -215,8 +215,8 @@ __device__ __forceinline__ void add_bias_row(uint32_t (&s)[128], float scale_log
 }
 
 // BIAS: a separate instantiation that adds a bias tensor to the scaled logits (dense batches): the softmax
-// thread fetches its row's 128 values of the step straight from device memory -- a bf16 bias adds
-// 2 B H Nq Nk bytes of traffic, four times |Q|+|K|+|V|+|O| on a 4096 x 4096, d = 64 problem.
+// thread fetches its row's 128 values of the step straight from device memory.  For the tensors that are not staged by TMA
+// (launch_tc2_d): fp32 values, and bf16 ones at odd addresses.
 // SPARSE (one tile per CTA): pruned attention.  A byte map over 128 x 128 blocks of the logit matrix says
 // which key tiles the CTA's query tile attends; the CTA compacts its row of the map into a list in shared
 // memory and every role walks that list instead of 0, 1, 2, ...: pruned key tiles are neither loaded nor
@@ -471,23 +471,6 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         const int nrow_min = __shfl_sync(0xffffffffu, nrow, 0);
         if (LY::TURNS && t == 1 && lane == 0) mbar_arrive(&bars[LY::TURN + (warp & 3)]);   // tile A goes first
         for (int j = 0; j < nt_t; ++j) {
-            // (bias, the common case of an aligned bf16 tensor: the row's 128 values of this step are fetched
-            // before the wait for the logits, so that the two latencies overlap)
-            uint32_t bpk[BIAS ? 64 : 1];
-            bool bias_ready = false;
-            if (BIAS) {
-                if (bias.vec && !bias.f32 && row < Nq && (j + 1) * BN <= Nk) {
-                    const uint4* g = reinterpret_cast<const uint4*>(
-                        static_cast<const __nv_bfloat16*>(bias.p) + static_cast<long long>(bh / H) * bias.sb +
-                        static_cast<long long>(bh % H) * bias.sh + static_cast<long long>(row) * Nk + j * BN);
-#pragma unroll
-                    for (int v = 0; v < 16; ++v) {
-                        const uint4 w = g[v];
-                        bpk[4 * v] = w.x; bpk[4 * v + 1] = w.y; bpk[4 * v + 2] = w.z; bpk[4 * v + 3] = w.w;
-                    }
-                    bias_ready = true;
-                }
-            }
             ok = bounded_wait(&bars[LY::S_FULL + t], j & 1, abort_flag, status, 0x300 + t);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -506,44 +489,18 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 const long long at = static_cast<long long>(bh / H) * bias.sb + static_cast<long long>(bh % H) * bias.sh +
                                      static_cast<long long>(row) * Nk + col0;
                 const bool in_rows = row < Nq;
-                if (bias_ready) {
+                if (bias.f32 && bias.vec && in_rows && col0 + BN <= Nk) {
 #pragma unroll
-                    for (int i = 0; i < 64; ++i) {
-                        s[2 * i] = __float_as_uint(fmaf(__uint_as_float(s[2 * i]), scale_log2e,
-                                                        __uint_as_float(bpk[i] << 16) * 1.4426950408889634f));
-                        s[2 * i + 1] = __float_as_uint(fmaf(__uint_as_float(s[2 * i + 1]), scale_log2e,
-                                                            __uint_as_float(bpk[i] & 0xffff0000u) * 1.4426950408889634f));
-                    }
-                } else if (bias.vec && in_rows && col0 + BN <= Nk) {
+                    for (int c = 0; c < 32; ++c) {
+                        const float4 w = reinterpret_cast<const float4*>(static_cast<const float*>(bias.p) + at)[c];
+                        const float bv[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {        // sixteen columns at a time (few registers live)
-                        float bv[16];
-                        if (bias.f32) {
-                            const float4* g = reinterpret_cast<const float4*>(static_cast<const float*>(bias.p) + at + c * 16);
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) {
-                                const float4 w = g[v];
-                                bv[4 * v] = w.x; bv[4 * v + 1] = w.y; bv[4 * v + 2] = w.z; bv[4 * v + 3] = w.w;
-                            }
-                        } else {
-                            const uint4* g = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(bias.p) + at + c * 16);
-#pragma unroll
-                            for (int v = 0; v < 2; ++v) {
-                                const uint4 w = g[v];
-                                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    bv[8 * v + 2 * e] = __uint_as_float(ww[e] << 16);
-                                    bv[8 * v + 2 * e + 1] = __uint_as_float(ww[e] & 0xffff0000u);
-                                }
-                            }
-                        }
-#pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            s[c * 16 + i] = __float_as_uint(fmaf(__uint_as_float(s[c * 16 + i]), scale_log2e, bv[i] * 1.4426950408889634f));
+                        for (int i = 0; i < 4; ++i)
+                            s[c * 4 + i] = __float_as_uint(fmaf(__uint_as_float(s[c * 4 + i]), scale_log2e, bv[i] * 1.4426950408889634f));
                     }
                 } else if (in_rows) {
-                    // Rows that begin anywhere.  bf16: aligned 16-byte pieces, two neighbours at a time, shifted into place
+                    // Rows that begin anywhere, and a row's last values.  bf16 (what no tensor map describes: a base off the
+                    // 16-byte grid, strides with gaps): aligned 16-byte pieces, two neighbours at a time, shifted into place
                     // (B8 H16 1001 x 1001: 257 us, 346 value by value; d = 128 334 and 416; staged word by word by one warp 657); fp32: value
                     // by value (487 us against 576).
                     const int count = Nk - col0 < BN ? Nk - col0 : BN;
