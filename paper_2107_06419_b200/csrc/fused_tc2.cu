@@ -502,13 +502,19 @@ fused_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     // Rows that begin anywhere, and a row's last values.  bf16 (what no tensor map describes: a base off the
                     // 16-byte grid, strides with gaps): aligned 16-byte pieces, two neighbours at a time, shifted into place
                     // (B8 H16 1001 x 1001: 257 us, 346 value by value; d = 128 334 and 416; staged word by word by one warp 657); fp32: value
-                    // by value (487 us against 576).
+                    // by value (395 us; through pieces 576 against 487 then).
                     const int count = Nk - col0 < BN ? Nk - col0 : BN;
+                    constexpr int FEW = D == 64 ? 64 : 32;
                     if (bias.f32) {
 #pragma unroll                                           // (fully: the logits must stay in registers)
                         for (int i = 0; i < 128; ++i)
                             s[i] = __float_as_uint(fmaf(__uint_as_float(s[i]), scale_log2e,
                                                         (i < count ? static_cast<const float*>(bias.p)[at + i] : 0.f) * 1.4426950408889634f));
+                    } else if (Nk < FEW) {               // (few values: one by one; B64 H8 20^2 35 us through the pieces, 23 like this)
+#pragma unroll
+                        for (int i = 0; i < FEW; ++i)    // (what lies behind them is masked)
+                            s[i] = __float_as_uint(fmaf(__uint_as_float(s[i]), scale_log2e,
+                                                        (i < count ? __bfloat162float(static_cast<const __nv_bfloat16*>(bias.p)[at + i]) : 0.f) * 1.4426950408889634f));
                     } else {
                         add_bias_row(s, scale_log2e, static_cast<const char*>(bias.p) + at * 2, count, bias);
                     }
@@ -784,7 +790,10 @@ int launch_tc2_d(const Problem& p, cudaStream_t st, int key_split = 1, bool only
             BiasMap bm{&tmB, -1};
             const int64_t plane = static_cast<int64_t>(p.Nq) * p.Nk, rows = static_cast<int64_t>(p.Nq) * (p.bias_sh ? p.H : 1) * (p.bias_sb ? p.B : 1);
             bool staged = ba.vec && !ba.f32 && make_bias_map(&tmB, p);
-            if (!staged && !ba.f32 && (reinterpret_cast<uintptr_t>(p.bias) & 15u) == 0 && p.Nk >= 32 && p.Nk < (1 << 27) && rows >= 8 &&
+            // (few values to a row: one by one in the kernel below while a head has one slab -- us, staged / one by one, d = 64: B64 H8 33^2
+            // 31.9 / 23.8, 63^2 32.0 / 27.4, B8 H16 1000 x 62 33.1 / 37.2; d = 128, B64 H8 33^2 21.8 / 30.8)
+            const bool few = p.Nk < 32 || (D == 64 && p.Nk < 64 && p.Nq <= 2 * BM);
+            if (!staged && !ba.f32 && (reinterpret_cast<uintptr_t>(p.bias) & 15u) == 0 && !few && p.Nk < (1 << 27) && rows >= 8 &&
                 rows < (1 << 30) && (!p.bias_sh || p.bias_sh == plane) && (!p.bias_sb || p.bias_sb == (p.bias_sh ? p.H * plane : plane))) {
                 bm.shifted_rows = static_cast<int>(rows & ~7ll);
                 staged = make_shifted_bias_map(&tmB, p.bias, rows / 8, p.Nk, SHIFTED_WIDTH(D));

@@ -36,6 +36,11 @@ CASES = [
     (1, 2, 70, 131, 64, (1, 2), "f32", None, False, 0.125),
     (1, 2, 300, 130, 128, (1, 1), "f32", None, False, 0.1),
     (1, 1, 1, 1, 64, (1, 1), "bf16", None, False, 1.0),
+    (2, 2, 100, 31, 64, (1, 2), "bf16", [31, 5], False, 0.125),             # few values to a row: read one by one ...
+    (2, 2, 256, 63, 64, (1, 2), "bf16", None, True, -0.2),
+    (2, 2, 257, 63, 64, (2, 1), "bf16", [63, 1], False, 0.125),             # ... staged
+    (1, 2, 100, 65, 64, (1, 2), "bf16", None, True, 0.125),
+    (2, 2, 100, 31, 128, (1, 2), "bf16", [31, 5], True, 0.1),
 ]
 
 
