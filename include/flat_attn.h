@@ -311,8 +311,8 @@ int flat_layernorm_fwd(const void* X, const void* R, const void* gamma, const vo
  * neighbours; to the caller it behaves like work enqueued on `stream`.  The side
  * streams and events are created once per device and host thread and never freed
  * (no device memory is allocated).
- * p->Q, p->K, p->V, p->O and p->k_valid_len are HOST pointers here; p->status and
- * p->lse are still device pointers or NULL.  `workspace` is a caller-owned DEVICE buffer of at
+ * p->Q, p->K, p->V, p->O and p->k_valid_len are HOST pointers here; p->status, p->lse,
+ * p->bias and p->block_mask are still device pointers or NULL.  `workspace` is a caller-owned DEVICE buffer of at
  * least flat_attn_host_workspace_bytes(...) bytes, 256-byte aligned.
  * The operation is that of flat_attn_fwd_ex; the paper has no counterpart for the copies.
  */

@@ -392,6 +392,9 @@ int flat_attn_fwd_host(const flat_attn_params_t* p, void* workspace, size_t work
         sub.Q = dQ + qo; sub.K = dK + ko; sub.V = dV + ko; sub.O = dO + qo;
         if (p->B > 1) { sub.B = u1 - u0; if (sub.k_valid_len) sub.k_valid_len += u0; }
         else          { sub.H = u1 - u0; }
+        const int64_t bias_unit = p->B > 1 ? q.bias_sb : q.bias_sh, map_unit = p->B > 1 ? q.bmask_sb : q.bmask_sh;
+        if (sub.bias) sub.bias = static_cast<const char*>(sub.bias) + u0 * bias_unit * (q.bias_dtype == FLAT_DTYPE_F32 ? 4 : 2);
+        if (sub.block_mask) sub.block_mask += u0 * map_unit;
         if (sub.lse) sub.lse += static_cast<size_t>(u0) * (p->B > 1 ? static_cast<size_t>(p->H) * p->Nq : static_cast<size_t>(p->Nq));
         const int r = run_fused(sub, p->variant, ss);
         if (r != FLAT_OK) return r;
