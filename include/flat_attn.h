@@ -27,8 +27,8 @@
  *   - Return value: FLAT_OK or one of the error codes below.  On an argument
  *     error nothing is launched.  There is no CPU fallback: an unsupported
  *     request is an error.
- *   - Supported sizes: B, H, Nq, Nk >= 1; d in {16, 32, 64, 128} (tensor-core
- *     kernels need d in {64, 128} and bf16); B*H*Nq*Nk and all byte counts must
+ *   - Supported sizes: B, H, Nq, Nk >= 1; d in {16, 32, 64, 128} (which kernel takes
+ *     which of them and which type: FLAT_VARIANT_* below); B*H*Nq*Nk and all byte counts must
  *     fit in 63 bits; B*H <= 65535.
  *   - scale multiplies the logits before the softmax and must be finite.  The
  *     paper does not mention a scale (scale = 1 is its literal text); 1/sqrt(d)
@@ -61,7 +61,7 @@ enum {
 
 enum { FLAT_DTYPE_BF16 = 0, FLAT_DTYPE_F32 = 1 };
 
-/* Kernel choice for the fused path. AUTO picks the tensor-core kernel when it applies. */
+/* Kernel choice for the fused path. AUTO picks the tensor-core kernel that applies and is the fastest for the size. */
 enum {
     FLAT_VARIANT_AUTO = 0,
     FLAT_VARIANT_SIMT = 1,     /* fp32 FFMA kernel, any supported d and dtype                  */
@@ -81,8 +81,11 @@ enum {
                                   softmax over complete rows: bf16, d = 64, Nk <= 512 only      */
     FLAT_VARIANT_TF32 = 7,     /* fp32 tensors on the tensor cores: every operand split into a tf32
                                   head and an fp32 remainder, each contraction three tf32 products,
-                                  running sums in fp32 registers: fp32, d = 64, no bias, no
-                                  pruning map (what AUTO picks there, and at d = 32 and 128)     */
+                                  running sums in fp32 registers: fp32, no bias, no pruning map.
+                                  Asked for by name: d = 64.  AUTO picks it there and at d = 32 and
+                                  128 (d = 32 with at most 64 queries and keys and more heads than
+                                  SMs: SIMT).  An infinite operand gives NaN at d = 64; at d = 32 and
+                                  128 what SIMT gives                                            */
     FLAT_VARIANT_TC2_SPLIT2 = 8, /* TC2_SINGLE with the keys of every query tile split over a cluster
                                   of two CTAs, whose partial softmaxes are merged through
                                   distributed shared memory: bf16, d in {64,128}, no bias, no pruning map;
@@ -131,8 +134,7 @@ typedef struct flat_attn_params {
                                   path only: lse[b,h,i] = log sum_j exp(scale * q_i . k_j) over the
                                   keys that row i sees (natural logarithm; -inf for a row without
                                   any).  It is what flat_attn_bwd needs from the forward pass.
-                                  Written by the SIMT, SMALL, DECODE, TC2, TC2_SINGLE and TC3 kernels (AUTO picks
-                                  among these when it is set); FLAT_ERR_UNSUPPORTED for the others.
+                                  Written by every kernel but TC and RGRAN (FLAT_ERR_UNSUPPORTED there).
                                   The paper has no counterpart (it stops at inference).           */
     const void* bias;          /* optional device tensor added to the SCALED logits before the
                                   softmax (it is not multiplied by `scale`): the relative-position

@@ -123,7 +123,7 @@ int run_fused(const flat::Problem& q, int variant, cudaStream_t st) {
             // d = 128: the two-tile kernel, even when it leaves SMs empty (B2 H8 2048 keys: 0.037 against 0.096 ms
             // on its single-tile predecessor, B16 H8 256 keys: 18.4 against 26.6 us, B8 H8 128 keys: the same).
             else           v = FLAT_VARIANT_TC2;
-            // (the bias is read by the two-tile kernel with one thread per row)
+            // (with a bias: launch_fused_tc2 picks the kernel that stages or reads it)
             if (q.bias) v = FLAT_VARIANT_TC2;
             // (pruned attention runs on the one-tile kernel: a CTA walks the list of its query tile's kept key tiles)
             if (q.block_mask) v = FLAT_VARIANT_TC2_SINGLE;
@@ -205,7 +205,8 @@ int run_fused(const flat::Problem& q, int variant, cudaStream_t st) {
         g_last_variant = v;
         return rc;
     }
-    // (chosen by the caller: d = 64 only)
+    // (asked for by name: d = 64 only, which is what the name has always stood for -- callers that asked for it at other head sizes
+    // were refused and still are; AUTO takes the kernel there by itself)
     if (v == FLAT_VARIANT_TF32 && (!flat::tf32_applies(q) || (variant == FLAT_VARIANT_TF32 && q.d != 64))) return FLAT_ERR_UNSUPPORTED;
     if (q.block_mask && (v != FLAT_VARIANT_TC2_SINGLE || q.bias || !tc_applies(q) || q.Nk > 131072)) return FLAT_ERR_UNSUPPORTED;
     g_last_variant = v;

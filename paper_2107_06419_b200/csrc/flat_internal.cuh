@@ -80,17 +80,18 @@ int launch_fused_tc2(const Problem& p, cudaStream_t st);      // (also the tenso
 // (only_if_resident: sixteen-CTA clusters only when all clusters of the launch can run at the same time; else
 // FLAT_ERR_UNSUPPORTED)
 int launch_fused_tc2_single(const Problem& p, cudaStream_t st, int key_split = 1, bool only_if_resident = false);
-// The same tile worked on by two warpgroups that take alternate key tiles (bf16, d = 64, dense; key_split 1, 2, 4, 8).
-int launch_fused_tc2_halves(const Problem& p, cudaStream_t st, int key_split = 1, bool only_if_resident = false);   // (key_split 1, 2, 4, 8, 16)   // (d = 64; with a block mask also d = 128; key_split 2 / 4: the keys of a tile over a CTA cluster)
+// The same tile worked on by two warpgroups that take alternate key tiles (bf16, d = 64, dense; key_split 1, 2, 4, 8, 16: the keys of
+// a tile over a cluster of as many CTAs).
+int launch_fused_tc2_halves(const Problem& p, cudaStream_t st, int key_split = 1, bool only_if_resident = false);
 int launch_fused_tc3(const Problem& p, cudaStream_t st);
 int launch_fused_tc3_bias(const Problem& p, const BiasMap& bias, cudaStream_t st);
 // How the last launch_fused_tc3 of this host thread dealt its items (FLAT_SCHEDULE_*; 0 before any).
 extern thread_local int g_last_schedule;
-bool tf32_applies(const Problem& p);               // fp32, d = 64, no bias, no pruning map
+bool tf32_applies(const Problem& p);               // fp32, d in {32, 64, 128}, no bias, no pruning map
 int launch_fused_tf32(const Problem& p, cudaStream_t st);     // fp32 tensors through split tf32 products
 bool decode_applies(const Problem& p);             // bf16, d in {64, 128}, at most 16 queries, no bias, no pruning map
 int launch_fused_decode(const Problem& p, cudaStream_t st);
-bool small_applies(const Problem& p);              // bf16, d in {16, 32}, no bias, no pruning map
+bool small_applies(const Problem& p);              // bf16, d in {16, 32}, no bias, no pruning map, at most 2^30 keys
 int launch_fused_small(const Problem& p, cudaStream_t st);
 bool rgran_applies(const Problem& p);              // bf16, d = 64, Nk <= 512
 int launch_fused_rgran(const Problem& p, cudaStream_t st);

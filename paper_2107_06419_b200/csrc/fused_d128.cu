@@ -12,9 +12,11 @@
 // O += P(j) V and S(j + 2), which takes P(j)'s columns, have a whole softmax step to run in.  The price is that a
 // logit MMA of N = 64 with both operands in shared memory takes 48 cycles where its arithmetic takes 32 (A alone is 4 KB of
 // a port of 128 bytes a cycle): 1280 cycles of the pipe per 64 keys of both tiles, against 1024.
-// Measured, against fused_tc2_kernel on the same GPU (us): B4 H16 4096^2 460 -> 428, causal 347 -> 256; H8 64K causal 7,780 ->
-// 6,380 (1,380 TFLOP/s; a cuBLAS GEMM of 8192^3 reaches 1,650 in a burst, 1,395 sustained); B2 H16 3000 causal 120 -> 97; B32
-// H16 512^2 110 -> 106.  The causal gain is also the order: the longest slabs first, so that short ones are left at the end.
+// Measured, against fused_tc2_kernel on the same GPU in the first 20 ms of launches (us): B4 H16 4096^2 460 -> 428, causal 347 ->
+// 256; H8 64K causal 7,780 -> 6,350 (1,386 TFLOP/s; a cuBLAS GEMM of 8192^3 reaches 1,630 in a burst); B2 H16 3000 causal 120 ->
+// 97; B32 H16 512^2 110 -> 106.  After that the power cap takes the clock down: in a second of launches H8 64K causal takes 7,160
+// (1,229 TFLOP/s at 1,462 MHz; cuBLAS sustained 1,376), B4 H16 4096^2 498 at 1,500 MHz.  The causal gain is also the order: the
+// longest slabs first, so that short ones are left at the end.
 //
 // CTA = 384 threads: warps 0-3 / 4-7 softmax of tile A / B (thread = row = TMEM lane), warp 8 TMA producer, warps 9 / 10 MMA
 // issuers of tile A / B (one elected lane), warp 11 idle (it completes the warpgroup for the register hand-over).

@@ -11,8 +11,8 @@
 // among them until the end.  Then the four merge through shared memory and the CTAs of a cluster, which share a
 // head's keys evenly, through distributed shared memory: every CTA leaves (m, l, O) in its own memory, a cluster
 // barrier, and each finishes its share of the outputs from all of them in the order of the ranks (same bits every time).
-// Measured (graph of calls on fresh inputs, key counts uniform in [Nk / 4, Nk]): B16 H16 1 x 8192 d 128 203 -> 101 us (6.5 TB/s), d 64
-// 117 -> 54; sixteen queries 190 -> 104; B32 H32 1 x 2048 181 -> 100; 4 heads x 32768 48 -> 14; B32 H8 1 x 512 29 -> 11.5.
+// Measured (key counts uniform in [Nk / 4, Nk]): B16 H16 1 x 8192 d 128 203 -> 101 us (76,343 keys a head in the 16 batches: 625 MB, 6.2
+// TB/s; all 131,072: 151 us, 7.1 TB/s), d 64 117 -> 52 (80,413 keys: 329 MB, 6.3 TB/s; all: 78 us, 6.8 TB/s); sixteen queries 190 -> 104; B32 H32 1 x 2048 181 -> 100; 4 heads x 32768 48 -> 14; B32 H8 1 x 512 29 -> 11.5.
 //
 // CTA = 160 threads: warps 0-3 as above, warp 4 TMA producer.  Tiles have the 128-byte swizzle; ldmatrix reads eight rows
 // of a panel without bank conflicts.  A warp's logits come out with queries as rows and keys as columns, which is the
@@ -343,9 +343,9 @@ int launch_decode(const Problem& p, cudaStream_t st) {
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
-// How many CTAs share a head, and how deep their rings are.  One round of two CTAs per SM streams at full rate (B16 H16
-// 1 x 8192, d = 128: 6.3 TB/s), so the widest split that stays within it; up to two rounds where a CTA still reads a
-// megabyte, which evens out key counts that differ between the batches (the same case split in two: 6.7 TB/s; short ones
+// How many CTAs share a head, and how deep their rings are.  One round of two CTAs per SM streams at full rate, so the widest split that
+// stays within it; up to two rounds where a CTA still reads a megabyte, which evens out key counts that differ between the batches
+// (B16 H16 1 x 8192, d = 128, 25 to 100 % filled: 6 % less time in halves; short ones
 // pay for their set-up: 512 keys in halves 15.2 us against 11.7).  Sixteen, more than the portable cluster size, only while every CTA
 // has an SM of its own (4 heads x 32768 keys: eight CTAs a head 20.5 us).  Six stages where that is so (8 heads x 32768: 32.2 us
 // against 35.9 with three).

@@ -1,9 +1,11 @@
 // Fused Logit-Softmax-Attend for small heads (bf16 in, fp32 accumulate, bf16 out; d = 16 and 32) on the sm_100a tensor
 // cores: the paper's fused dataflow (Section 5, 5.1, 5.2), one 128-row query tile per CTA, keys streamed in tiles of BN.
 //
-// What bounds it: the exponential unit.  A (query, key) pair costs 4 d FLOP on the tensor pipe -- at d = 32 a quarter of
-// what d = 128 has -- and one exponential whatever the head size (16 per clock and SM: 4.65e12 pairs/s on 148 SMs), so
-// the contractions are nearly free and there is room for the accuracy that the FFMA kernel gave these head sizes
+// What bounds it: the chain of a step in the softmax warps -- logits seen, TMEM load, exponentials and splits, the wait for the last
+// P V, stores, arrival -- with two of them on a scheduler to hide it: the exponential unit is busy 51 % of the time, the issue slots
+// 49 %, the tensor pipe 19 % (counters, B64 H8 1000^2); and 1,024 CTAs are 3.5 rounds of the 296 that run at a time.  A (query, key)
+// pair costs 4 d FLOP on the tensor pipe -- at d = 32 a quarter of what d = 128 has -- and one exponential whatever the head size
+// (16 per clock and SM: 4.65e12 pairs/s on 148 SMs), so the contractions are nearly free and there is room for the accuracy that the FFMA kernel gave these head sizes
 // (weights kept in fp32): a weight p goes to the second contraction as TWO bf16 numbers, its rounded head and the rounded
 // remainder (together 17 bits of mantissa), each with an MMA of its own against the same V, and no exponential takes
 // the polynomial.  Results then sit at the rounding of the bf16 output, as before.
@@ -15,8 +17,7 @@
 // step would wait for MMA, softmax and MMA in turn.)
 // Tiles in shared memory have rows of 2 d bytes with the swizzle of that width (64 or 32 bytes): the canonical K-major
 // (Q, K) and MN-major (V) layouts with one panel.
-// Measured: B16 H8 1000 x 1000 at d = 32: 66 us (1.9e12 pairs/s, 0.42 of the exponential unit; 1024 CTAs are 3.5 rounds of
-// the 296 that run at a time) against 638 us of the FFMA kernel, which keeps the fp32 tensors and the calls with a bias.
+// Measured: B16 H8 1000 x 1000 at d = 32: 65 us (2.0e12 pairs/s, 0.42 of the exponential unit) against 638 us of the FFMA kernel, which keeps the fp32 tensors and the calls with a bias.
 // Reference maximum as in the two-tile kernel: exact on the first and on masked steps, kept otherwise, a step whose row
 // sum passes 2^40 is redone with a fresh one.  A row that does not come out finite (infinite or very large values) is computed
 // again without the split (plain_row).  Every wait is bounded; on expiry the CTA ends cleanly and reports a code.

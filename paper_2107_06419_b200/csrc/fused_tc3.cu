@@ -370,7 +370,7 @@ struct Sched {
     // in shared memory (fill_units), every unit stands for its H heads, and the CTAs take the items of that order
     // forwards and backwards in turn -- CTA c has items c, 2 G - 1 - c, 2 G + c, ... -- so that their shares weigh the
     // same to a few per cent (32 sequences of 40 to 2000 tokens, 12 heads: 105 us with a CTA per slot of the longest
-    // sequence's grid, most of them empty, in the order of the sequences; 81 like this).  An item index is a round then.
+    // sequence's grid, most of them empty, in the order of the sequences; 78 like this).  An item index is a round then.
     const int32_t* cu_q;                                 // packed variable-length batches: first token of every sequence's
     const int32_t* cu_k;                                 // queries / keys in the packed tensors ([sequences + 1] entries)
     const int* deal;                                     // even deal: its table in shared memory

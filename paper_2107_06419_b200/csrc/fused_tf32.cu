@@ -11,8 +11,10 @@
 // streaming softmax then costs nothing extra, and the result does not depend on how the tensor core
 // rounds a 16K-term running sum.
 //
-// What bounds it: the tensor pipe at d = 64 and 128 (three products at half the bf16 rate: 85-88 % of it with B2 H16 4096 keys,
-// 552 and 1,180 us), the softmax warps at d = 32 (424 us).  Before, d = 32 and 128 ran on the FFMA kernel: 2,840 and 9,600 us.
+// What bounds it: the tensor pipe at d = 64 (three products at half the bf16 rate: active 77 % of the time by its counter, and
+// 52 % of the shared-memory port), the chain of a 32-key step at d = 128 (59 %; its softmax warps spill 308 bytes), the softmax
+// warps at d = 32.  B2 H16 4096^2, d = 32 / 64 / 128: 393 / 539 / 1,247 us in the first 20 ms of launches, 412 / 610 / 1,402 in a
+// second of them (the power cap: 1,837, 1,575 and 1,717 MHz).  Before, d = 32 and 128 ran on the FFMA kernel: 2,840 and 9,600 us.
 //
 // Paper mapping (Section 5, 5.1, 5.2): shared outer loops = (batch, head) and a tile of 128 query rows on blockIdx.x
 // (R-granularity); Logit and Attend run interleaved over steps of 64 keys (d = 128: 32) with
@@ -66,7 +68,7 @@ template <int D> struct Layout {
     static constexpr int MERGE_STRIDE = D + 4;           // floats per row of the merge scratch (outputs, m, l, padding: 16-byte rows, no bank conflicts)
     static constexpr int PVS = D == 128 ? 1 : 2;         // P V buffers
     // registers after the hand-over, of the 512 x 128 of the launch (d = 64 with 192 / 80 / 48: the converters spill, 548 us
-    // against 532 on B2 H16 4096^2)
+    // against 532 on B2 H16 4096^2 in short runs)
     static constexpr int SOFT_REGS = D == 128 ? 192 : 176, CONVERT_REGS = D == 128 ? 80 : 104, ISSUE_REGS = D == 128 ? 48 : 56;
     static_assert(256 * SOFT_REGS + 128 * CONVERT_REGS + 128 * ISSUE_REGS <= THREADS * 128, "register hand-over");
     static constexpr uint32_t QH_COL = 0, QL_COL = D, S_COL = 2 * D, PL_COL = S_COL + 2 * BN, PV_COL = PL_COL + 2 * BN;

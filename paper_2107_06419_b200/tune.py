@@ -31,7 +31,7 @@ VARIANTS = {
     api.FLAT_VARIANT_SIMT: "simt: 64-row FFMA tiles",
     api.FLAT_VARIANT_TC: "tc: 128-row CTA, exact running maximum",
     api.FLAT_VARIANT_TC2_SINGLE: "tc2_single: 128-row CTA, two per SM (d = 64)",
-    api.FLAT_VARIANT_TC2: "tc2: 256-row CTA (two tiles ping-pong)",
+    api.FLAT_VARIANT_TC2: "tc2: 256-row CTA (two tiles ping-pong; d = 128: steps of 64 keys)",
     api.FLAT_VARIANT_TC3: "tc3: 256-row CTA, half-row softmax threads, logits three tile-steps ahead (d = 64)",
     api.FLAT_VARIANT_RGRAN: "rgran: whole logit rows on chip, two-pass softmax (d = 64, Nk <= 512)",
     api.FLAT_VARIANT_TC2_SPLIT2: "tc2_split2: 128-row CTA, keys split over a cluster of 2 CTAs",
@@ -43,6 +43,8 @@ VARIANTS = {
     api.FLAT_VARIANT_TC2_HALVES_SPLIT8: "tc2_halves_split8: ... of 8 CTAs",
     api.FLAT_VARIANT_TC2_SPLIT16: "tc2_split16: keys over a cluster of 16 CTAs (d = 128)",
     api.FLAT_VARIANT_TC2_HALVES_SPLIT16: "tc2_halves_split16: two warpgroups per tile, keys over a cluster of 16 CTAs (d = 64)",
+    api.FLAT_VARIANT_SMALL: "small: 128-row CTA, two per SM, weights as two bf16 numbers (d = 16, 32)",
+    api.FLAT_VARIANT_DECODE: "decode: sixteen query rows, keys split over a cluster of up to 16 CTAs (at most 16 queries)",
     api.FLAT_VARIANT_AUTO: "auto (the dispatcher's choice)",
 }
 
