@@ -20,7 +20,7 @@
 // Measured: B16 H8 1000 x 1000 at d = 32: 65 us (2.0e12 pairs/s, 0.42 of the exponential unit) against 638 us of the FFMA kernel, which keeps the fp32 tensors and the calls with a bias.
 // Reference maximum as in the two-tile kernel: exact on the first and on masked steps, kept otherwise, a step whose row
 // sum passes 2^40 is redone with a fresh one.  A row that does not come out finite (infinite or very large values) is computed
-// again without the split (plain_row).  Every wait is bounded; on expiry the CTA ends cleanly and reports a code.
+// again without the split (plain_rows).  Every wait is bounded; on expiry the CTA ends cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -347,15 +347,10 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             float z0, z1;
             unpack2(add2(zero[0], zero[1]), z0, z1);
-            unsigned again = __ballot_sync(0xffffffffu, row < Nq && z0 + z1 != 0.f);
-            while (again) {
-                const int at = __ffs(again) - 1;
-                again &= again - 1;
-                __syncwarp();                            // (the row's own thread has stored it)
-                const int64_t r = static_cast<int64_t>(bh) * Nq + row0 + warp * 32 + at;
-                plain_row<__nv_bfloat16, D>(Q + r * D, K + static_cast<int64_t>(bh) * Nk * D, V + static_cast<int64_t>(bh) * Nk * D, O + r * D,
-                                            lse ? lse + r : nullptr, __shfl_sync(0xffffffffu, nrow, at), scale_log2e);
-            }
+            const unsigned again = __ballot_sync(0xffffffffu, row < Nq && z0 + z1 != 0.f);
+            if (again)
+                plain_rows<__nv_bfloat16, D>(again, static_cast<int64_t>(bh) * Nq + row0 + warp * 32, nrow, Q, K + static_cast<int64_t>(bh) * Nk * D,
+                                             V + static_cast<int64_t>(bh) * Nk * D, O, lse, scale_log2e);
         }
     }
     tc_fence_before();

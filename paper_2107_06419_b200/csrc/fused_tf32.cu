@@ -12,7 +12,7 @@
 // rounds a 16K-term running sum.
 //
 // What bounds it: the tensor pipe at d = 64 (three products at half the bf16 rate: active 77 % of the time by its counter, and
-// 52 % of the shared-memory port), the chain of a 32-key step at d = 128 (59 %; its softmax warps spill 308 bytes), the softmax
+// 52 % of the shared-memory port), the chain of a 32-key step at d = 128 (59 %; its softmax warps spill 312 bytes), the softmax
 // warps at d = 32.  B2 H16 4096^2, d = 32 / 64 / 128: 393 / 539 / 1,247 us in the first 20 ms of launches, 412 / 610 / 1,402 in a
 // second of them (the power cap: 1,837, 1,575 and 1,717 MHz).  Before, d = 32 and 128 ran on the FFMA kernel: 2,840 and 9,600 us.
 //
@@ -36,7 +36,7 @@
 // d = 128, where Q takes half of TMEM, steps of 32 keys leave room for both parities of S and P and for one P V buffer:
 // a step's P V waits until the one before has been read, which happens while the pipe works on the logits in between.
 // An infinite operand has no finite remainder: its products are NaN.  At d = 32 and 128 a row that does not come out finite is
-// computed again in plain fp32 (plain_row), which gives what the FFMA kernel gives; at d = 64 it stays NaN.
+// computed again in plain fp32 (plain_rows), which gives what the FFMA kernel gives; at d = 64 it stays NaN.
 // Every wait is bounded (see tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -533,15 +533,10 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (NEAR) {                                      // (at d = 64 the row stays as it is)
                 float z0, z1;
                 unpack2(add2(zero[0], zero[1]), z0, z1);
-                unsigned again = __ballot_sync(0xffffffffu, z0 + z1 != 0.f);
-                while (again) {
-                    const int at_lane = __ffs(again) - 1;
-                    again &= again - 1;
-                    __syncwarp();                            // (the row's own thread has stored it)
-                    const int64_t rr = static_cast<int64_t>(bh) * Nq + row0 + warp * 32 + at_lane;
-                    plain_row<float, D>(Q + rr * D, K + static_cast<int64_t>(bh) * Nk * D, V + static_cast<int64_t>(bh) * Nk * D, O + rr * D,
-                                        lse ? lse + rr : nullptr, __shfl_sync(0xffffffffu, nrow, at_lane), scale_log2e);
-                }
+                const unsigned again = __ballot_sync(0xffffffffu, z0 + z1 != 0.f);
+                if (again)
+                    plain_rows<float, D>(again, static_cast<int64_t>(bh) * Nq + row0 + warp * 32, nrow, Q, K + static_cast<int64_t>(bh) * Nk * D,
+                                         V + static_cast<int64_t>(bh) * Nk * D, O, lse, scale_log2e);
             }
         }
     }

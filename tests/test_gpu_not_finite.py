@@ -96,3 +96,25 @@ def test_nan_inputs_leave_no_row_unwritten(d, key):
     F, flse = run(api, Q, K, V, d ** -0.5, variant=api.FLAT_VARIANT_SIMT)
     assert bool(O[0, 0].isnan().all()) and bool(O[0, 1, 20].isnan().all())
     assert torch.equal(O.isnan(), F.isnan()) and torch.equal(lse.isinf(), flse.isinf()) and bool((lse[0, 1, :20] != 7.0).all())
+
+
+@pytest.mark.parametrize("d,dtype", FORMATS)
+@pytest.mark.parametrize("rows", [1, 7, 8, 9, 31])
+def test_some_rows_of_a_warp(d, dtype, rows):
+    """As many rows of a warp come out NaN (a NaN in their query) as the second pass takes at a time, less and more; an infinite value
+    under the causal mask is seen by the later rows only."""
+    from paper_2107_06419_b200 import api
+    torch.manual_seed(rows)
+    Q, K, V = (torch.randn(1, 2, 160, d, device="cuda").to(dtype) for _ in range(3))
+    Q[0, 0, 33:33 + rows, 2] = float("nan")
+    V[0, 1, 160 - rows, 3] = float("inf")
+    O, lse = run(api, Q, K, V, d ** -0.5, causal=True)
+    assert api.flat_attn_last_variant() == variant_of(api, dtype)
+    bad = O[0, 0].isnan()
+    assert bool(bad[33:33 + rows].all()) and int(bad.sum()) == rows * d
+    assert int((O[0, 1] == float("inf")).sum()) == rows and bool((O[0, 1, 160 - rows:, 3] == float("inf")).all())
+    ref = torch.softmax((Q.double() @ K.double().transpose(2, 3) * d ** -0.5).masked_fill(
+        torch.ones(160, 160, device="cuda", dtype=torch.bool).triu(1), -float("inf")), -1) @ V.double().nan_to_num(0.0, 0.0, 0.0)
+    ok = O.isfinite()
+    assert int(ok.sum()) == O.numel() - rows * d - rows
+    assert float((O.double() - ref)[ok].abs().max()) <= rounding_of(dtype) * float(V.float().nan_to_num(0.0, 0.0, 0.0).abs().max())
