@@ -7,9 +7,9 @@
 // lse the row-wise log-sum-exp that the forward pass saved, P = exp(S - lse) and delta_i = sum_t dO[i,t] O[i,t]:
 //     dV = P^T dO        dP = dO V^T        dS = P o (dP - delta)        dQ = scale dS K        dK = scale dS^T Q
 // Two launches of one kernel template, no atomics and no workspace beyond delta [B,H,Nq]:
-//   MODE_DQ : one CTA per 128 query rows, streaming key tiles:   S = Q K^T, dP = dO V^T, dQ += dS K.
+//   MODE_DQ : 128 query rows at a time, streaming key tiles:   S = Q K^T, dP = dO V^T, dQ += dS K.
 //             Also computes delta for its rows and writes it for the second launch.
-//   MODE_DKV: one CTA per 128 keys, streaming query tiles:       S^T = K Q^T, dP^T = V dO^T,
+//   MODE_DKV: 128 keys at a time, streaming query tiles:       S^T = K Q^T, dP^T = V dO^T,
 //             dV += P^T dO, dK += dS^T Q.
 // Both are the same program: a stationary pair of tiles (X1, X2) whose rows are the TMEM lanes, a streamed
 // pair (Y1, Y2) whose rows are the columns:  T1 = X1 Y1^T,  T2 = X2 Y2^T  (both operands K-major in shared
@@ -39,10 +39,18 @@
 //    port per tile (a broadcast read is one wavefront per column and warp); instead they join the contractions: one more
 //    slice of 16 contraction indices, (1, 1, 1, 0 ...) on the stationary side and -lse / scale, or -delta, as the sum of
 //    three bf16 numbers (24 bits) on the streamed side, gives T1 = K Q^T - lse / scale and T2 = V dO^T - delta.
-// Measured (both launches): B4 H16 4096 x 4096 d 64 1.265 -> 0.91 ms, B1 H4 16384 d 128 1.80 -> 1.46, B2 H16 3000 d 128
-// causal 0.361 -> 0.291.
+//  * A CTA that has issued the copies of its tile takes over a tile whose CTA has not started (clusterlaunchcontrol), so that
+//    no tile pays for launch, allocation, barrier set-up and first loads (3,500 cycles), and the next tile's operands and T are
+//    under way while this one's gradients are stored.  The stationary tiles come by TMA and go to TMEM from shared memory, and
+//    delta's rows are read side by side: a lane per row, 16 bytes an instruction, took 6,600 (d = 64) and 14,300 cycles (128).
+//    Between two tiles are now 3,300 / 3,800 cycles (dQ / dK dV, d = 64) and 5,800 / 7,100 (d = 128) instead of 11,100 / 6,900
+//    and 20,600 / 11,000; a tile of 4096 rows has 48,000 to 98,000 cycles of steps.
+//  * Waits by whole warps and values that the compiler knows to be the same in all lanes (warp_wait, the shuffles): without
+//    them 3 to 7 % a step.
+// Measured (both launches): B4 H16 4096 x 4096 d 64 905 -> 854 us, causal 548 -> 474; B2 H16 3000 d 128 causal 286 -> 239;
+// B8 H8 512 d 64 39.7 -> 35; B4 H8 256 d 128 26.5 -> 22.
 //
-// CTA = 640 threads: warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four
+// CTA = 640 threads, an item at a time (a tile of the stationary operands): warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four
 // warps per scheduler), warp 16 TMA producer, warp 17 issues the T MMAs and warp 18 the accumulations (where P / dS
 // overlay T, warp 17 issues both), warp 19 writes the slices that carry lse and delta (MODE_DKV).
 // Under the causal mask the tiles of a head differ in length by a factor of their number: the longest tiles of a group of
@@ -76,7 +84,8 @@ template <int D, int MODE> struct BL {
     static constexpr bool SEP = !(D == 128 && DKV);
     static constexpr bool X1_TMEM = !DKV, X2_TMEM = !DKV && D == 64;   // stationary operand in TMEM, else in shared memory
     static constexpr int TILE_BYTES = BT * D * 2;
-    static constexpr int X_BYTES = (X1_TMEM ? 0 : TILE_BYTES) + (X2_TMEM ? 0 : TILE_BYTES);
+    static constexpr bool X_SMEM = !X1_TMEM || !X2_TMEM;                     // some stationary operand is read by MMAs from shared memory
+    static constexpr int X_BYTES = 2 * TILE_BYTES;       // (an operand that goes to TMEM is staged here)
     // Rings of streamed tiles (SEP: whole ones; else halves of 64 rows), deep enough that a copy (one to two microseconds)
     // is under way for every step in work.  MODE_DQ needs Y2 = V for T2 only, so that its slots are free again early.
     static constexpr int PARTS = SEP ? 1 : 2;            // copies per step; also column groups with T, dS and barriers of their own
@@ -87,8 +96,8 @@ template <int D, int MODE> struct BL {
     static constexpr int AUG_BYTES = BT * 32;
     static constexpr int VSTAGES = DKV ? S1 / PARTS : 1;
     static constexpr int AUG_ALL = DKV ? (1 + 2 * VSTAGES) * AUG_BYTES : 0;
-    static constexpr int XCH_BYTES = DKV ? 0 : 4 * BT * 4;                   // delta quarters of MODE_DQ
-    static constexpr int SMEM_BYTES = OPERAND_BYTES + AUG_ALL + XCH_BYTES + 512 + 1024;
+    static constexpr int DELTA_BYTES = DKV ? 0 : 2 * BT * 4;                 // delta of the rows (MODE_DQ), of two items in turn
+    static constexpr int SMEM_BYTES = OPERAND_BYTES + AUG_ALL + DELTA_BYTES + 512 + 1024;
     static_assert(SMEM_BYTES <= 232448, "shared memory");
     static constexpr uint32_t T1_COL = 0, T2_COL = 128, ACC_A_COL = 256, ACC_B_COL = 256 + D;
     static constexpr uint32_t ACC_END = 256 + (DKV ? 2 : 1) * D;
@@ -102,18 +111,29 @@ template <int D, int MODE> struct BL {
     __host__ __device__ static constexpr uint32_t p_store(int g) { return SEP ? P_COL + g * 16 : T1_COL + g * 32; }
     __host__ __device__ static constexpr uint32_t ds_slice(int k) { return ds_store(k / 2) + (k % 2) * 8; }
     __host__ __device__ static constexpr uint32_t p_slice(int k) { return p_store(k / 2) + (k % 2) * 8; }
-    // barriers.  X_FULL: stationary tiles in shared memory; X_TMEM: in TMEM (one arrival per element-wise warp);
+    static_assert(SEP || (p_slice(4) == p_slice(0) + HC && ds_slice(4) == ds_slice(0) + HC && p_slice(7) == p_slice(3) + HC), "halves");
+    // barriers.  Per item: X_FULL: stationary tiles in shared memory; X_TMEM: in TMEM (one arrival per element-wise warp);
+    // X_EMPTY: the T MMAs that read them from shared memory have completed (where none do: warp 17 has seen X_TMEM);
+    // ACC_DONE: everything accumulated; ACC_FREE: the accumulators are in registers; ITEM_FULL / ITEM_EMPTY [2]: the next item
+    // is known / read by every warp.
     // Y_FULL [S1]: the copy's Y1 and Y2 have landed (and, MODE_DKV, warp 19 has written the step's slices);
-    // Y1_EMPTY [S1], Y2_EMPTY [S2] (MODE_DQ): read; ACC_STEP (SEP): the MMAs that read dS, P have completed; ACC_DONE:
-    // everything accumulated; per column group: T_FULL: T1, T2 computed; PD_FULL: dS (and P) written; T_FREE (SEP): T1, T2
+    // Y1_EMPTY [S1], Y2_EMPTY [S2] (MODE_DQ): read; ACC_STEP (SEP): the MMAs that read dS, P have completed;
+    // per column group: T_FULL: T1, T2 computed; PD_FULL: dS (and P) written; T_FREE (SEP): T1, T2
     // taken into registers.  Without SEP warp 18 arrives on PD_FULL, too, once the half's next copy has landed, so that the
     // issuing warp has one barrier to look at.
-    static constexpr int BAR_X_FULL = 0, BAR_X_TMEM = 1, BAR_Y_FULL = 2, BAR_Y1_EMPTY = BAR_Y_FULL + S1,
+    static constexpr int BAR_X_FULL = 0, BAR_X_TMEM = 1, BAR_X_EMPTY = 2, BAR_ACC_FREE = 3, BAR_ITEM_FULL = 4, BAR_ITEM_EMPTY = 6,
+                         BAR_Y_FULL = 8, BAR_Y1_EMPTY = BAR_Y_FULL + S1,
                          BAR_Y2_EMPTY = BAR_Y1_EMPTY + S1, BAR_ACC_STEP = BAR_Y2_EMPTY + S2, BAR_ACC_DONE = BAR_ACC_STEP + 1,
                          BAR_T_FULL = BAR_ACC_DONE + 1, BAR_T_FREE = BAR_T_FULL + PARTS, BAR_PD_FULL = BAR_T_FREE + 1,
                          NUM_BARS = BAR_PD_FULL + PARTS;
     static constexpr int PD_ARRIVALS = SEP ? EW_WARPS : EW_WARPS / 2 + 1;
-    static_assert(NUM_BARS * 8 + 8 <= 512, "barriers");
+    static constexpr int READERS = EW_WARPS + (DKV ? 3 : 2);                 // warps that read an item: all but the producer
+    __host__ __device__ static constexpr int arrivals(int i) {
+        return i == BAR_X_TMEM || i == BAR_ACC_FREE || i == BAR_T_FREE ? EW_WARPS
+               : i == BAR_ITEM_EMPTY || i == BAR_ITEM_EMPTY + 1 ? READERS
+               : i >= BAR_Y_FULL && i < BAR_Y1_EMPTY && DKV ? 2 : i >= BAR_PD_FULL ? PD_ARRIVALS : 1;
+    }
+    static_assert(NUM_BARS * 8 + 8 + 32 <= 512, "barriers");
 };
 
 // Shared-memory descriptor of a slice tile: K-major rows of 32 bytes, 32-byte swizzle, eight rows 256 bytes apart.
@@ -136,6 +156,27 @@ __device__ __forceinline__ float exponent_factor(float scale) {
 
 __device__ __forceinline__ void ew_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
+// Wait by a whole warp, every lane for the barrier that it names.  The warp stays together: its lanes probe and vote as one.
+// (Where each lane loops by itself, the lanes come back one by one after a long wait and what follows starts up to 500
+// cycles late.)
+__device__ __forceinline__ bool warp_wait(uint32_t bar_addr, uint32_t parity, uint32_t abort_addr, int32_t* status, int code) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_s(bar_addr, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 32; ++i)
+            if (__all_sync(0xffffffffu, mbar_try_wait_s(bar_addr, parity))) return true;
+        int aborted;
+        asm volatile("ld.volatile.shared::cta.s32 %0, [%1];" : "=r"(aborted) : "r"(abort_addr) : "memory");
+        if (__any_sync(0xffffffffu, aborted)) return false;
+        if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_CYCLES)) {
+            asm volatile("st.volatile.shared::cta.s32 [%0], %1;" ::"r"(abort_addr), "r"(1) : "memory");
+            if (status) atomicExch(status, code);
+            return false;
+        }
+    }
+}
+
 // X1, X2 / Y1, Y2 by mode:  MODE_DQ: (Q, dO) / (K, V);  MODE_DKV: (K, V) / (Q, dO).
 template <int D, int MODE>
 __global__ void __launch_bounds__(BWD_THREADS, 1)
@@ -149,32 +190,24 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* X1s = base;
-    uint8_t* X2s = X1s + (LY::X1_TMEM ? 0 : LY::TILE_BYTES);
+    uint8_t* X2s = X1s + LY::TILE_BYTES;
     uint8_t* Y1s = base + LY::X_BYTES;                   // rings of streamed tiles
     uint8_t* Y2s = Y1s + LY::S1 * LY::Y_BYTES;
     uint8_t* aug = base + LY::OPERAND_BYTES;             // (MODE_DKV) ones, then per stage -lse / scale and -delta
-    float* xch = reinterpret_cast<float*>(base + LY::OPERAND_BYTES + LY::AUG_ALL);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + LY::OPERAND_BYTES + LY::AUG_ALL + LY::XCH_BYTES);
+    float* dls = reinterpret_cast<float*>(base + LY::OPERAND_BYTES + LY::AUG_ALL);
+    uint8_t* next_item = base + LY::OPERAND_BYTES + LY::AUG_ALL + LY::DELTA_BYTES;           // two answers of 16 bytes
+    uint64_t* bars = reinterpret_cast<uint64_t*>(next_item + 32);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffles here and below tell the compiler that a value is the same in all lanes: the MMA operands, which come from
+    // uniform registers, are then computed there)
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int NX = MODE == MODE_DQ ? Nq : Nk;            // rows of the stationary tensors
-    // CTA -> (head, tile): `group` heads at a time, their tiles side by side, the longest first under the causal mask
-    // (the last query tiles, the first key tiles)
     const int tiles = (NX + BT - 1) / BT;
-    const int per = group * tiles, first_head = static_cast<int>(blockIdx.x) / per * group;
-    const int heads = BH - first_head < group ? BH - first_head : group;
-    const int at = static_cast<int>(blockIdx.x) % per, bh = first_head + at % heads;
-    const int tile = (MODE == MODE_DQ && coff < (1 << 29)) ? tiles - 1 - at / heads : at / heads;
-    const int x0 = tile * BT;                            // first row of the stationary tile (query or key)
 
     if (threadIdx.x == EW_WARPS * 32) {
-        for (int i = 0; i < LY::NUM_BARS; ++i) {
-            const bool y_full = i >= LY::BAR_Y_FULL && i < LY::BAR_Y1_EMPTY;
-            mbar_init(&bars[i], i == LY::BAR_X_TMEM || i == LY::BAR_T_FREE ? EW_WARPS : i >= LY::BAR_PD_FULL ? LY::PD_ARRIVALS
-                                : y_full && LY::DKV ? 2 : 1);
-        }
+        for (int i = 0; i < LY::NUM_BARS; ++i) mbar_init(&bars[i], LY::arrivals(i));
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -195,47 +228,114 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    int nkeys = Nk;                                      // keys of this batch that take part at all
-    if (valid_len) { nkeys = valid_len[bh / H]; nkeys = nkeys < 0 ? 0 : (nkeys > Nk ? Nk : nkeys); }
-    // Range of streamed tiles [y_begin, y_end) that hold at least one visible (query, key) pair.
-    // Causal mask (coff = Nk - Nq; 2^30 = none): query i sees key j iff j <= i + coff.
-    int y_begin = 0, y_end;
-    if (MODE == MODE_DQ) {
-        const long long lim = static_cast<long long>(x0) + BT + coff;          // keys below this for the tile's last row
-        const int n = lim < nkeys ? (lim < 0 ? 0 : static_cast<int>(lim)) : nkeys;
-        y_end = (n + BT - 1) / BT;
-    } else {
-        y_end = x0 < nkeys ? (Nq + BT - 1) / BT : 0;
-        const long long first = static_cast<long long>(x0) - coff;             // first query that sees key x0
-        if (first > 0) y_begin = static_cast<int>(first / BT < y_end ? first / BT : y_end);
-    }
-    const int nsteps = y_end - y_begin;
-    const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
+    const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag)), next_s = smem_u32(next_item);
     auto wait_warp = [&](int bar, uint32_t parity, int code) {
-        return __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * bar, parity, abort_s, status, code));
+        return warp_wait(bars_s + 8 * bar, parity, abort_s, status, code);
     };
-    const int ncopies = LY::PARTS * nsteps;              // copies of the rings: step j, or half g & 1 of step g >> 1
 
-    if (warp == EW_WARPS) {
+    // Item -> (head, tile): `group` heads at a time, their tiles side by side, the longest first under the causal mask
+    // (the last query tiles, the first key tiles); its range of streamed tiles, those with at least one visible (query, key)
+    // pair.  Causal mask (coff = Nk - Nq; 2^30 = none): query i sees key j iff j <= i + coff.
+    int bh, x0, nkeys, y_begin, nsteps;                  // nkeys: keys of this batch that take part at all
+    auto place = [&](int item, int& head, int& row) {
+        const int per = group * tiles, first_head = item / per * group;
+        const int heads = BH - first_head < group ? BH - first_head : group;
+        const int at = item % per;
+        head = first_head + at % heads;
+        row = (MODE == MODE_DQ && coff < (1 << 29) ? tiles - 1 - at / heads : at / heads) * BT;
+    };
+    auto decode = [&](int item) {
+        place(item, bh, x0);
+        nkeys = Nk;
+        if (valid_len) {
+            nkeys = __shfl_sync(0xffffffffu, valid_len[bh / H], 0);
+            nkeys = nkeys < 0 ? 0 : (nkeys > Nk ? Nk : nkeys);
+        }
+        y_begin = 0;
+        int y_end;
+        if (MODE == MODE_DQ) {
+            const long long lim = static_cast<long long>(x0) + BT + coff;      // keys below this for the tile's last row
+            const int n = lim < nkeys ? (lim < 0 ? 0 : static_cast<int>(lim)) : nkeys;
+            y_end = (n + BT - 1) / BT;
+        } else {
+            y_end = x0 < nkeys ? (Nq + BT - 1) / BT : 0;
+            const long long first = static_cast<long long>(x0) - coff;         // first query that sees key x0
+            if (first > 0) y_begin = static_cast<int>(first / BT < y_end ? first / BT : y_end);
+        }
+        nsteps = y_end - y_begin;
+    };
+    // The n-th item (n > 0) that this CTA has taken over from one of the grid that had not started; -1: there was none left,
+    // -2: gave up.  (The reader's fence orders its read before the next answer, which comes through the asynchronous proxy.)
+    auto take_item = [&](int n) {
+        const int slot = (n - 1) & 1;
+        if (!wait_warp(LY::BAR_ITEM_FULL + slot, ((n - 1) >> 1) & 1, 0x570)) return -2;
+        const int item = __shfl_sync(0xffffffffu, clc_answer(next_s + 16 * slot), 0);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (warp != EW_WARPS && lane == 0) mbar_arrive_s(bars_s + 8 * (LY::BAR_ITEM_EMPTY + slot));
+        __syncwarp();
+        return item;
+    };
+
+    // Every role walks the same items; n: the item's number, gs: steps before it, ne: items before it that had steps.
+    // The rings and the phases of the per-step barriers run on over the items.
+    if (warp >= EW_WARPS) {
+      if (warp == EW_WARPS) {
         // ------------------------------------------------------------ TMA producer (lane 0 issues the copies)
-        if (nsteps > 0) {
+        if (lane == 0) { prefetch_tensormap(&tmX1); prefetch_tensormap(&tmX2); prefetch_tensormap(&tmY1); prefetch_tensormap(&tmY2); }
+        // The next item is asked for some steps before the end of this one (six: early enough for what follows, late enough that
+        // no CTA sits on work while another has none) and its stationary rows are brought to L2: the CTAs come to the ends of
+        // their items together, and 64 to 96 KB for every SM at once take 2,500 to 5,500 cycles from DRAM.
+        constexpr int LEAD = 6 * LY::PARTS;
+        bool ok = true;
+        int G = 0, n = 0, xs = 0, asked = 0;             // copies, items, stationary pairs and questions so far
+        auto ask = [&]() {
+            if (n >= 2) ok = wait_warp(LY::BAR_ITEM_EMPTY + (n & 1), ((n >> 1) - 1) & 1, 0x505);
+            if (ok && lane == 0) {
+                mbar_arrive_expect_tx(&bars[LY::BAR_ITEM_FULL + (n & 1)], 16);
+                clc_ask(next_s + 16 * (n & 1), bars_s + 8 * (LY::BAR_ITEM_FULL + (n & 1)));
+            }
+            asked = n + ok;
+        };
+        auto answer = [&]() {
+            const int next = take_item(n + 1);
+            if (next >= 0 && lane == 0) {
+                int head, row;
+                place(next, head, row);
+                const uint32_t bytes = static_cast<uint32_t>((NX - row < BT ? NX - row : BT) * D * 2);
+                const int64_t at = (static_cast<int64_t>(head) * NX + row) * D;
+                prefetch_l2(X1g + at, bytes);
+                prefetch_l2(X2g + at, bytes);
+                if (!LY::DKV) prefetch_l2(Og + at, bytes);
+            }
+            return next;
+        };
+        int item = blockIdx.x;
+        while (item >= 0) {
+            decode(item);
+            if (n > 0) {                                 // the previous item's stationary tiles are read
+                ok = wait_warp(LY::BAR_X_EMPTY, (n - 1) & 1, 0x503);
+                if (ok && LY::X1_TMEM) ok = wait_warp(LY::BAR_X_TMEM, (n - 1) & 1, 0x504);
+                if (!ok) break;
+            }
             if (lane == 0) {
-                prefetch_tensormap(&tmX1); prefetch_tensormap(&tmX2); prefetch_tensormap(&tmY1); prefetch_tensormap(&tmY2);
-                if (LY::X_BYTES > 0) {
-                    mbar_arrive_expect_tx(&bars[LY::BAR_X_FULL], LY::X_BYTES);
+                mbar_arrive_expect_tx(&bars[LY::BAR_X_FULL], LY::X_BYTES);
 #pragma unroll
-                    for (int c = 0; c < D / 64; ++c) {
-                        if (!LY::X1_TMEM) tma_load_3d(X1s + c * BT * 128, &tmX1, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
-                        if (!LY::X2_TMEM) tma_load_3d(X2s + c * BT * 128, &tmX2, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
-                    }
+                for (int c = 0; c < D / 64; ++c) {
+                    tma_load_3d(X1s + c * BT * 128, &tmX1, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
+                    tma_load_3d(X2s + c * BT * 128, &tmX2, &bars[LY::BAR_X_FULL], c * 64, x0, bh);
                 }
             }
-            bool ok = true;
-            int issued = 0;
-            for (int g = 0; g < ncopies && ok; ++g) {
-                const int s1 = g % LY::S1, s2 = g % LY::S2, y = y_begin * BT + g * LY::Y_ROWS;
-                ok = wait_warp(LY::BAR_Y1_EMPTY + s1, ((g / LY::S1) & 1) ^ 1, 0x500);
-                if (!LY::DKV && ok) ok = wait_warp(LY::BAR_Y2_EMPTY + s2, ((g / LY::S2) & 1) ^ 1, 0x501);
+            xs = n + 1;
+            const int copies = LY::PARTS * nsteps, ask_at = copies > LEAD ? copies - LEAD : 0;
+            int next = -3;                               // (not known yet)
+            for (int g = 0; g < copies && ok; ++g) {
+                const int s1 = G % LY::S1, s2 = G % LY::S2, y = y_begin * BT + g * LY::Y_ROWS;
+                if (g == ask_at) ask();
+                if (ok && g == ask_at + 2 * LY::PARTS) next = answer();
+                if (!ok || next == -2) break;
+                ok = wait_warp(LY::BAR_Y1_EMPTY + s1, ((G / LY::S1) & 1) ^ 1, 0x500);
+                if (!LY::DKV && ok) ok = wait_warp(LY::BAR_Y2_EMPTY + s2, ((G / LY::S2) & 1) ^ 1, 0x501);
                 if (!ok) break;
                 if (lane == 0) {
                     mbar_arrive_expect_tx(&bars[LY::BAR_Y_FULL + s1], 2 * LY::Y_BYTES);
@@ -245,15 +345,21 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                         tma_load_3d(Y2s + s2 * LY::Y_BYTES + c * LY::Y_ROWS * 128, &tmY2, &bars[LY::BAR_Y_FULL + s1], c * 64, y, bh);
                     }
                 }
-                issued = g + 1;
+                ++G;
             }
-            if (!ok && lane == 0) {
-                if (LY::X_BYTES > 0) drain_wait(&bars[LY::BAR_X_FULL], 0);
-                for (int g = issued > LY::S1 ? issued - LY::S1 : 0; g < issued; ++g)
-                    drain_wait(&bars[LY::BAR_Y_FULL + g % LY::S1], (g / LY::S1) & 1);
-            }
+            if (ok && copies == 0) ask();
+            if (ok && next == -3) next = answer();
+            if (!ok) break;
+            item = next;
+            ++n;
         }
-    } else if (LY::DKV && warp == EW_WARPS + 3) {
+        if (lane == 0) {                                 // (where everything went well these have all completed)
+            if (xs > 0) drain_wait(&bars[LY::BAR_X_FULL], (xs - 1) & 1);
+            if (!ok || item == -2)
+                for (int g = G > LY::S1 ? G - LY::S1 : 0; g < G; ++g) drain_wait(&bars[LY::BAR_Y_FULL + g % LY::S1], (g / LY::S1) & 1);
+            if (asked > 0) drain_wait(&bars[LY::BAR_ITEM_FULL + ((asked - 1) & 1)], ((asked - 1) >> 1) & 1);
+        }
+      } else if (LY::DKV && warp == EW_WARPS + 3) {
         // ------------------------------------------------------------ the slices that carry lse and delta (MODE_DKV)
         // Four queries per lane and step, fetched a step ahead.  A query that is switched off (no visible key, or past the
         // end) gets a first term so large that 2^(c T1) is 0 whatever its logits are.
@@ -267,35 +373,39 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                 dl[e] = i < Nq ? delta[static_cast<int64_t>(bh) * Nq + i] : 0.f;
             }
         };
-        if (nsteps > 0) fetch(0);
         bool ok = true;
-        for (int j = 0; j < nsteps && ok; ++j) {
-            const int v = j % LY::VSTAGES, g = LY::PARTS * j + LY::PARTS - 1;   // the step's (last) copy
-            float x[4], y[4];
+        int n = 0, gs = 0;
+        for (int item = blockIdx.x; item >= 0 && ok; item = take_item(++n)) {
+            decode(item);
+            if (nsteps > 0) fetch(0);
+            for (int j = 0; j < nsteps && ok; ++j, ++gs) {
+                const int v = gs % LY::VSTAGES, g = LY::PARTS * gs + LY::PARTS - 1;   // the step's (last) copy
+                float x[4], y[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                x[e] = l[e] == -INFINITY ? off : l[e] * inv;
-                x[e] = x[e] > 3e38f ? 3e38f : x[e] < -3e38f ? -3e38f : x[e];
-                y[e] = -dl[e];
-            }
-            if (j + 1 < nsteps) fetch(j + 1);
-            // (slot v was last read by the T MMAs of step j - VSTAGES; that step has released the stage of this step's
-            // (last) copy behind its accumulation, i.e. after them)
-            ok = wait_warp(LY::BAR_Y1_EMPTY + g % LY::S1, ((g / LY::S1) & 1) ^ 1, 0x502);
-            if (!ok) break;
+                for (int e = 0; e < 4; ++e) {
+                    x[e] = l[e] == -INFINITY ? off : l[e] * inv;
+                    x[e] = x[e] > 3e38f ? 3e38f : x[e] < -3e38f ? -3e38f : x[e];
+                    y[e] = -dl[e];
+                }
+                if (j + 1 < nsteps) fetch(j + 1);
+                // (slot v was last read by the T MMAs of step gs - VSTAGES; that step has released the stage of this step's
+                // (last) copy behind its accumulation, i.e. after them)
+                ok = wait_warp(LY::BAR_Y1_EMPTY + g % LY::S1, ((g / LY::S1) & 1) ^ 1, 0x502);
+                if (!ok) break;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                aug_store(aug + (1 + 2 * v) * LY::AUG_BYTES, e * 32 + lane, x[e]);
-                aug_store(aug + (2 + 2 * v) * LY::AUG_BYTES, e * 32 + lane, y[e]);
-            }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&bars[LY::BAR_Y_FULL + g % LY::S1]);
-                if (LY::PARTS == 2) mbar_arrive(&bars[LY::BAR_Y_FULL + (g - 1) % LY::S1]);
+                for (int e = 0; e < 4; ++e) {
+                    aug_store(aug + (1 + 2 * v) * LY::AUG_BYTES, e * 32 + lane, x[e]);
+                    aug_store(aug + (2 + 2 * v) * LY::AUG_BYTES, e * 32 + lane, y[e]);
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&bars[LY::BAR_Y_FULL + g % LY::S1]);
+                    if (LY::PARTS == 2) mbar_arrive(&bars[LY::BAR_Y_FULL + (g - 1) % LY::S1]);
+                }
             }
         }
-    } else if (warp == EW_WARPS + 1 || warp == EW_WARPS + 2) {
+      } else if (warp == EW_WARPS + 1 || warp == EW_WARPS + 2) {
         // ------------------------------------------------------------ MMA issuers
         //   T(j):   T1 = X1 Y1^T and T2 = X2 Y2^T (+ the slices);   ACC(j): acc_a += dS Y1 (and acc_b += P Y2).
         // SEP: warp 17 issues T(j+1) as soon as T(j) is in registers, warp 18 ACC(j) as soon as dS (and P) are written.
@@ -303,276 +413,352 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         // The whole warp walks the loop (uniform control flow) and one elected lane issues: the MMA and
         // commit instructions take their operands from uniform registers, which the compiler can only
         // use when it knows that a single thread runs the code.
-        if (nsteps > 0) {
-            constexpr int YR = LY::Y_ROWS;
-            constexpr uint32_t IDESC_T = make_idesc_bf16(BT, YR, 0, 0), IDESC_ACC = make_idesc_bf16(BT, D, 0, 1);
-            constexpr uint64_t Y16 = LY::Y_BYTES >> 4, AUG16 = LY::AUG_BYTES >> 4;           // descriptor units of 16 bytes
-            bool ok = true;
-            // descriptors of the first feature slice of each operand (the others are constant offsets away)
-            const uint64_t x1d = make_smem_desc_sw128(smem_u32(X1s), 16, 1024);            // K-major
-            const uint64_t x2d = make_smem_desc_sw128(smem_u32(X2s), 16, 1024);
-            const uint64_t y1k = make_smem_desc_sw128(smem_u32(Y1s), 16, 1024), y2k = make_smem_desc_sw128(smem_u32(Y2s), 16, 1024);
-            const uint64_t y1m = make_smem_desc_sw128(smem_u32(Y1s), YR * 128, 1024);      // MN-major
-            const uint64_t y2m = make_smem_desc_sw128(smem_u32(Y2s), YR * 128, 1024);
-            const uint64_t augd = aug_desc(smem_u32(aug));
-            // Consecutive MMAs into ONE accumulator wait for each other, so the slices of independent
-            // products are issued in turn: T1 and T2, and the accumulations acc_a and acc_b.
-            // (feature slice k of a K-major operand: panel k / 4 of 64 features, 32 bytes per slice; a panel
-            // is 128 rows of 128 bytes for the stationary tiles, YR rows for the streamed ones)
-            // g: the copy; half: its column group (0 where a copy is a whole step)
-            auto issue_t = [&](int g, int half) {
-                const uint64_t y1 = y1k + static_cast<uint64_t>(g % LY::S1) * Y16, y2 = y2k + static_cast<uint64_t>(g % LY::S2) * Y16;
-                const uint32_t t1 = tmem + LY::T1_COL + half * HC, t2 = tmem + LY::T2_COL + half * HC;
+        constexpr int YR = LY::Y_ROWS;
+        constexpr uint32_t IDESC_T = make_idesc_bf16(BT, YR, 0, 0), IDESC_ACC = make_idesc_bf16(BT, D, 0, 1);
+        constexpr uint64_t Y16 = LY::Y_BYTES >> 4, AUG16 = LY::AUG_BYTES >> 4;           // descriptor units of 16 bytes
+        // descriptors of the first feature slice of each operand (the others are constant offsets away)
+        const uint64_t x1d = make_smem_desc_sw128(smem_u32(X1s), 16, 1024);            // K-major
+        const uint64_t x2d = make_smem_desc_sw128(smem_u32(X2s), 16, 1024);
+        const uint64_t y1k = make_smem_desc_sw128(smem_u32(Y1s), 16, 1024), y2k = make_smem_desc_sw128(smem_u32(Y2s), 16, 1024);
+        const uint64_t y1m = make_smem_desc_sw128(smem_u32(Y1s), YR * 128, 1024);      // MN-major
+        const uint64_t y2m = make_smem_desc_sw128(smem_u32(Y2s), YR * 128, 1024);
+        const uint64_t augd = aug_desc(smem_u32(aug));
+        // Consecutive MMAs into ONE accumulator wait for each other, so the slices of independent
+        // products are issued in turn: T1 and T2, and the accumulations acc_a and acc_b.
+        // (feature slice k of a K-major operand: panel k / 4 of 64 features, 32 bytes per slice; a panel
+        // is 128 rows of 128 bytes for the stationary tiles, YR rows for the streamed ones)
+        // g: the copy (of all items); where a step is two copies, their halves of the columns
+        auto issue_t = [&](int g) {
+            const int half = LY::PARTS == 2 ? g & 1 : 0;
+            const uint64_t y1 = y1k + static_cast<uint64_t>(g % LY::S1) * Y16, y2 = y2k + static_cast<uint64_t>(g % LY::S2) * Y16;
+            const uint32_t t1 = tmem + LY::T1_COL + half * HC, t2 = tmem + LY::T2_COL + half * HC;
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) {
-                    const uint64_t xoff = static_cast<uint64_t>(((k / 4) * (BT * 128) + (k % 4) * 32) >> 4);
-                    const uint64_t yoff = static_cast<uint64_t>(((k / 4) * (YR * 128) + (k % 4) * 32) >> 4);
-                    if (LY::X1_TMEM) mma_ts(t1, tmem + LY::X1_COL + k * 8, y1 + yoff, IDESC_T, k > 0);
-                    else             mma_ss(t1, x1d + xoff, y1 + yoff, IDESC_T, k > 0);
-                    if (LY::X2_TMEM) mma_ts(t2, tmem + LY::X2_COL + k * 8, y2 + yoff, IDESC_T, k > 0);
-                    else             mma_ss(t2, x2d + xoff, y2 + yoff, IDESC_T, k > 0);
-                }
-                if (LY::DKV) {
-                    const uint64_t av = augd + static_cast<uint64_t>(1 + 2 * ((g / LY::PARTS) % LY::VSTAGES)) * AUG16 + static_cast<uint64_t>((half * HC * 32) >> 4);
-                    mma_ss(t1, augd, av, IDESC_T, 1);
-                    mma_ss(t2, augd, av + AUG16, IDESC_T, 1);
-                }
-                tc_commit(&bars[LY::BAR_T_FULL + half]);
-                if (!LY::DKV) tc_commit(&bars[LY::BAR_Y2_EMPTY + g % LY::S2]);
-            };
-            auto issue_acc = [&](int g, int half) {
-                const uint64_t y1 = y1m + static_cast<uint64_t>(g % LY::S1) * Y16, y2 = y2m + static_cast<uint64_t>(g % LY::S2) * Y16;
+            for (int k = 0; k < D / 16; ++k) {
+                const uint64_t xoff = static_cast<uint64_t>(((k / 4) * (BT * 128) + (k % 4) * 32) >> 4);
+                const uint64_t yoff = static_cast<uint64_t>(((k / 4) * (YR * 128) + (k % 4) * 32) >> 4);
+                if (LY::X1_TMEM) mma_ts(t1, tmem + LY::X1_COL + k * 8, y1 + yoff, IDESC_T, k > 0);
+                else             mma_ss(t1, x1d + xoff, y1 + yoff, IDESC_T, k > 0);
+                if (LY::X2_TMEM) mma_ts(t2, tmem + LY::X2_COL + k * 8, y2 + yoff, IDESC_T, k > 0);
+                else             mma_ss(t2, x2d + xoff, y2 + yoff, IDESC_T, k > 0);
+            }
+            if (LY::DKV) {
+                const uint64_t av = augd + static_cast<uint64_t>(1 + 2 * ((g / LY::PARTS) % LY::VSTAGES)) * AUG16 + static_cast<uint64_t>((half * HC * 32) >> 4);
+                mma_ss(t1, augd, av, IDESC_T, 1);
+                mma_ss(t2, augd, av + AUG16, IDESC_T, 1);
+            }
+            tc_commit(&bars[LY::BAR_T_FULL + half]);
+            if (!LY::DKV) tc_commit(&bars[LY::BAR_Y2_EMPTY + g % LY::S2]);
+        };
+        // first / last: of the item's copies
+        auto issue_acc = [&](int g, bool first, bool last) {
+            const uint32_t pd = tmem + (LY::PARTS == 2 ? (g & 1) * HC : 0);
+            const uint64_t y1 = y1m + static_cast<uint64_t>(g % LY::S1) * Y16, y2 = y2m + static_cast<uint64_t>(g % LY::S2) * Y16;
 #pragma unroll
-                for (int k = 0; k < YR / 16; ++k) {
-                    mma_ts(tmem + LY::ACC_A_COL, tmem + (half == 0 ? LY::ds_slice(k) : LY::ds_slice(4 + k)),
-                           y1 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, (g > 0 || k > 0));
-                    if (LY::DKV)
-                        mma_ts(tmem + LY::ACC_B_COL, tmem + (half == 0 ? LY::p_slice(k) : LY::p_slice(4 + k)),
-                               y2 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, (g > 0 || k > 0));
-                }
-                if (LY::SEP) tc_commit(&bars[LY::BAR_ACC_STEP]);
-                tc_commit(&bars[LY::BAR_Y1_EMPTY + g % LY::S1]);
-                if (g == ncopies - 1) tc_commit(&bars[LY::BAR_ACC_DONE]);
-            };
-            auto y_full = [&](int g, int code) { return wait_warp(LY::BAR_Y_FULL + g % LY::S1, (g / LY::S1) & 1, code); };
+            for (int k = 0; k < YR / 16; ++k) {
+                mma_ts(tmem + LY::ACC_A_COL, pd + LY::ds_slice(k), y1 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, (!first || k > 0));
+                if (LY::DKV)
+                    mma_ts(tmem + LY::ACC_B_COL, pd + LY::p_slice(k), y2 + static_cast<uint64_t>((k * 2048) >> 4), IDESC_ACC, (!first || k > 0));
+            }
+            if (LY::SEP) tc_commit(&bars[LY::BAR_ACC_STEP]);
+            tc_commit(&bars[LY::BAR_Y1_EMPTY + g % LY::S1]);
+            if (last) tc_commit(&bars[LY::BAR_ACC_DONE]);
+        };
+        auto y_full = [&](int g, int code) { return wait_warp(LY::BAR_Y_FULL + g % LY::S1, (g / LY::S1) & 1, code); };
+        auto acc_free = [&](int ne) { return ne == 0 || wait_warp(LY::BAR_ACC_FREE, (ne - 1) & 1, 0x512); };
+        bool ok = true;
+        int n = 0, gs = 0, ne = 0;
+        for (int item = blockIdx.x; item >= 0 && ok; item = take_item(++n)) {
+            decode(item);
             if (warp == EW_WARPS + 1) {
-                if (LY::X_BYTES > 0) ok = wait_warp(LY::BAR_X_FULL, 0, 0x510);
-                if (ok && LY::X1_TMEM) ok = wait_warp(LY::BAR_X_TMEM, 0, 0x511);
+                if (LY::X_SMEM) ok = wait_warp(LY::BAR_X_FULL, n & 1, 0x510);
+                if (ok && LY::X1_TMEM) ok = wait_warp(LY::BAR_X_TMEM, n & 1, 0x511);
+                if (!LY::X_SMEM && ok && lane == 0) mbar_arrive(&bars[LY::BAR_X_EMPTY]);
+                __syncwarp();
             }
             if (LY::SEP && warp == EW_WARPS + 1) {
                 for (int j = 0; j < nsteps && ok; ++j) {
-                    ok = y_full(j, 0x520);
-                    if (ok && j > 0) ok = wait_warp(LY::BAR_T_FREE, (j - 1) & 1, 0x522);
+                    const int g = gs + j;
+                    ok = y_full(g, 0x520);
+                    if (ok && g > 0) ok = wait_warp(LY::BAR_T_FREE, (g & 1) ^ 1, 0x522);
                     if (!ok) break;
                     tc_fence_after();
-                    if (elect_one()) issue_t(j, 0);
+                    if (elect_one()) issue_t(g);
+                    __syncwarp();
+                }
+                if (LY::X_SMEM && ok) {
+                    if (elect_one()) tc_commit(&bars[LY::BAR_X_EMPTY]);
                     __syncwarp();
                 }
             } else if (LY::SEP) {
+                if (nsteps > 0) ok = acc_free(ne);
                 for (int j = 0; j < nsteps && ok; ++j) {
-                    ok = y_full(j, 0x523);
-                    if (ok) ok = wait_warp(LY::BAR_PD_FULL, j & 1, 0x530);
+                    const int g = gs + j;
+                    ok = y_full(g, 0x523);
+                    if (ok) ok = wait_warp(LY::BAR_PD_FULL, g & 1, 0x530);
                     if (!ok) break;
                     tc_fence_after();
-                    if (elect_one()) issue_acc(j, 0);
+                    if (elect_one()) issue_acc(g, j == 0, j == nsteps - 1);
                     __syncwarp();
                 }
             } else if (warp == EW_WARPS + 1) {
-                ok = ok && y_full(0, 0x520) && y_full(1, 0x520);
-                if (ok) {
+                // (copy g of the item: half g & 1 of its columns; -2, -1: only the first T of the halves)
+                const int g0 = 2 * gs, copies = 2 * nsteps;
+                if (copies > 0 && ok) ok = acc_free(ne);
+                for (int g = copies > 0 ? -2 : 0; g < copies && ok; ++g) {
+                    ok = g < 0 ? y_full(g0 + g + 2, 0x520) : wait_warp(LY::BAR_PD_FULL + (g & 1), ((g0 + g) >> 1) & 1, 0x531);
+                    if (!ok) break;
                     tc_fence_after();
-                    if (elect_one()) { issue_t(0, 0); issue_t(1, 1); }
+                    if (elect_one()) {
+                        if (g >= 0) issue_acc(g0 + g, g == 0, g == copies - 1);
+                        if (g + 2 < copies) issue_t(g0 + g + 2);
+                    }
                     __syncwarp();
-                }
-                for (int j = 0; j < nsteps && ok; ++j) {
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        const int g = 2 * j + half;
-                        ok = wait_warp(LY::BAR_PD_FULL + half, j & 1, 0x531);
-                        if (!ok) break;
-                        tc_fence_after();
-                        if (elect_one()) {
-                            issue_acc(g, half);
-                            if (g + 2 < ncopies) issue_t(g + 2, half);
-                        }
+                    if (g + 3 == copies) {               // (behind the last T)
+                        if (elect_one()) tc_commit(&bars[LY::BAR_X_EMPTY]);
                         __syncwarp();
                     }
+                }
+                if (copies == 0 && ok) {
+                    if (elect_one()) tc_commit(&bars[LY::BAR_X_EMPTY]);
+                    __syncwarp();
                 }
             } else {
                 // (the half's next copy: looked at here, so that the issuing warp does not have to; not before the half's
                 // previous phase is over, which this arrival does not belong to)
-                for (int g = 0; g < ncopies && ok; ++g) {
-                    if (g + 2 < ncopies) ok = y_full(g + 2, 0x521);
-                    if (ok && g >= 2) ok = wait_warp(LY::BAR_PD_FULL + (g & 1), ((g >> 1) - 1) & 1, 0x532);
+                const int g0 = 2 * gs, copies = 2 * nsteps;
+                for (int g = 0; g < copies && ok; ++g) {
+                    if (g + 2 < copies) ok = y_full(g0 + g + 2, 0x521);
+                    if (ok && g0 + g >= 2) ok = wait_warp(LY::BAR_PD_FULL + (g & 1), (((g0 + g) >> 1) - 1) & 1, 0x532);
                     if (ok && lane == 0) mbar_arrive(&bars[LY::BAR_PD_FULL + (g & 1)]);
+                    __syncwarp();
                 }
             }
+            gs += nsteps;
+            ne += nsteps > 0;
         }
-    } else if (warp < EW_WARPS) {
+      }
+    } else {
         // ------------------------------------------------------------ element-wise + epilogue (warps 0-15)
         const int q = warp & 3, part = warp >> 2;        // lane quarter, 32 of the step's columns
         const int r = q * 32 + lane;                     // lane of the TMEM = row of the stationary tile
-        const int xr = x0 + r;                           // that row's index (query in MODE_DQ, key in MODE_DKV)
         const uint32_t tl = tmem + (static_cast<uint32_t>(q * 32) << 16);
         const float c2 = exponent_factor(scale);
+        const bool wide = ((reinterpret_cast<uintptr_t>(outA) | (LY::DKV ? reinterpret_cast<uintptr_t>(outB) : 0)) & 31) == 0;
         bool ok = true;
-        // MODE_DQ: the row's quarter (this warp's part of the features) of the stationary operands that live in TMEM (rows
-        // past the end are zeros); lse of the row in base-2 units (+inf switches a row off: no key, or past the end) and
-        // delta = sum_t dO O, each of the row's four warps summing a quarter of the features.
+        // MODE_DQ, per row: lse in base-2 units (+inf switches a row off: no key, or past the end) and delta
         float lse2_r = INFINITY, delta_r = 0.f;
-        if (!LY::DKV) {
-            float sum = 0.f;
-            uint32_t w1[D / 8], w2[D / 8];               // packed pairs of Q and dO
+        // MODE_DQ: brings the item's stationary operands from shared memory to TMEM (a quarter of the features a warp; all T
+        // MMAs of the previous item have completed: their results have been seen here) and computes delta = sum_t dO O:
+        // eight rows a warp, a row's features side by side in its lanes.
+        constexpr int LPR = D / 8, ROWS = 32 / LPR, PASSES = 8 / ROWS;       // lanes a row, rows a pass
+        float sums[PASSES];
+        auto begin_item = [&](int n) {
+            if constexpr (!LY::DKV) {
+                uint4 da[PASSES], db[PASSES];
 #pragma unroll
-            for (int i = 0; i < D / 8; ++i) w1[i] = w2[i] = 0u;
-            if (xr < NX) {
-                const int64_t at_row = (static_cast<int64_t>(bh) * NX + xr) * D + part * (D / 4);
-                const uint4* a = reinterpret_cast<const uint4*>(X1g + at_row);
-                const uint4* b = reinterpret_cast<const uint4*>(X2g + at_row);
-                const uint4* c = reinterpret_cast<const uint4*>(Og + at_row);
-#pragma unroll
-                for (int v = 0; v < D / 32; ++v) {
-                    const uint4 av = a[v], bv = b[v], cv = c[v];
-                    const uint32_t cw[4] = {cv.x, cv.y, cv.z, cv.w};
-                    w1[4 * v] = av.x; w1[4 * v + 1] = av.y; w1[4 * v + 2] = av.z; w1[4 * v + 3] = av.w;
-                    w2[4 * v] = bv.x; w2[4 * v + 1] = bv.y; w2[4 * v + 2] = bv.z; w2[4 * v + 3] = bv.w;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        sum = fmaf(__uint_as_float(w2[4 * v + e] << 16), __uint_as_float(cw[e] << 16), sum);
-                        sum = fmaf(__uint_as_float(w2[4 * v + e] & 0xffff0000u), __uint_as_float(cw[e] & 0xffff0000u), sum);
+                for (int i = 0; i < PASSES; ++i) {
+                    const int row = x0 + warp * 8 + i * ROWS + lane / LPR;
+                    da[i] = db[i] = make_uint4(0u, 0u, 0u, 0u);
+                    if (row < Nq) {
+                        const int64_t at = (static_cast<int64_t>(bh) * Nq + row) * D + (lane % LPR) * 8;
+                        da[i] = *reinterpret_cast<const uint4*>(X2g + at);
+                        db[i] = *reinterpret_cast<const uint4*>(Og + at);
                     }
                 }
-                const float l = lse[static_cast<int64_t>(bh) * Nq + xr];
+                const float l = x0 + r < Nq ? lse[static_cast<int64_t>(bh) * Nq + x0 + r] : -INFINITY;
+                if (!wait_warp(LY::BAR_X_FULL, n & 1, 0x541)) return false;
+                auto to_tmem = [&](const uint8_t* X, uint32_t col) {
+                    uint32_t w[D / 8];                   // packed pairs; (16-byte chunk c of row r is at c ^ (r % 8))
+                    const uint8_t* row = X + (part * (D / 4) / 64) * (BT * 128) + r * 128;
+#pragma unroll
+                    for (int v = 0; v < D / 32; ++v) {
+                        const uint4 x = *reinterpret_cast<const uint4*>(row + ((((part * (D / 4) % 64) / 8 + v) ^ (r & 7)) << 4));
+                        w[4 * v] = x.x; w[4 * v + 1] = x.y; w[4 * v + 2] = x.z; w[4 * v + 3] = x.w;
+                    }
+                    if constexpr (D == 64) tmem_st_x8(tl + col + part * 8, w); else tmem_st_x16(tl + col + part * 16, w);
+                };
+                to_tmem(X1s, LY::X1_COL);
+                if (LY::X2_TMEM) to_tmem(X2s, LY::X2_COL);
+                tc_wait_st();
+                tc_fence_before();
+                fence_proxy_async_smem();                // (read before the next item's copies)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars[LY::BAR_X_TMEM]);
                 lse2_r = l == -INFINITY ? INFINITY : l * LOG2E;
+#pragma unroll
+                for (int i = 0; i < PASSES; ++i) {
+                    const uint32_t a[4] = {da[i].x, da[i].y, da[i].z, da[i].w}, b[4] = {db[i].x, db[i].y, db[i].z, db[i].w};
+                    float sum = 0.f;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        sum = fmaf(__uint_as_float(a[e] << 16), __uint_as_float(b[e] << 16), sum);
+                        sum = fmaf(__uint_as_float(a[e] & 0xffff0000u), __uint_as_float(b[e] & 0xffff0000u), sum);
+                    }
+#pragma unroll
+                    for (int m = LPR / 2; m >= 1; m >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, m);
+                    sums[i] = sum;
+                }
             }
-            // (D / 2 columns hold a row; a quarter is D / 8)
-            if constexpr (D == 64) {
-                tmem_st_x8(tl + LY::X1_COL + part * 8, w1);
-                tmem_st_x8(tl + LY::X2_COL + part * 8, w2);
-            } else {
-                tmem_st_x16(tl + LY::X1_COL + part * 16, w1);
+            return true;
+        };
+        auto finish_delta = [&](int n) {
+            if constexpr (!LY::DKV) {
+                float* d_item = dls + (n & 1) * BT;
+#pragma unroll
+                for (int i = 0; i < PASSES; ++i) {
+                    const int row = warp * 8 + i * ROWS + lane / LPR;
+                    if (lane % LPR == 0) {
+                        d_item[row] = sums[i];
+                        if (x0 + row < Nq) delta[static_cast<int64_t>(bh) * Nq + x0 + row] = sums[i];
+                    }
+                }
+                ew_sync();
+                delta_r = d_item[r];
             }
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars[LY::BAR_X_TMEM]);
-            xch[part * BT + r] = sum;
-            ew_sync();
-            delta_r = (xch[r] + xch[BT + r]) + (xch[2 * BT + r] + xch[3 * BT + r]);
-            if (part == 0 && xr < Nq) delta[static_cast<int64_t>(bh) * Nq + xr] = delta_r;
-        }
-        // keys the row takes part with (MODE_DQ: per query row; MODE_DKV: the row IS a key)
-        const long long rlim = static_cast<long long>(xr) + 1 + coff;
-        const int nrow = rlim < nkeys ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : nkeys;
-        const bool key_live = xr < nkeys;
-        const uint64_t c22 = pack2(c2, c2), nl2 = pack2(-lse2_r, -lse2_r), dl2 = pack2(delta_r, delta_r);
+        };
         const int cq = part * 32;                        // this warp's 32 columns of every step
         const int cgroup = LY::PARTS == 2 ? part >> 1 : 0;
         const uint32_t ds_addr = tl + LY::ds_store(0) + part * (LY::ds_store(1) - LY::ds_store(0));
         const uint32_t p_addr = tl + LY::p_store(0) + part * (LY::p_store(1) - LY::p_store(0));
-        for (int j = 0; j < nsteps && ok; ++j) {
-            ok = wait_warp(LY::BAR_T_FULL + cgroup, j & 1, 0x540 + cgroup);
-            if (!ok) break;
-            tc_fence_after();
-            uint32_t t1[32], t2[32];
-            tmem_ld_x32(tl + LY::T1_COL + cq, t1);
-            tmem_ld_x32(tl + LY::T2_COL + cq, t2);
-            const int y0 = (y_begin + j) * BT + cq;      // index of the first of the columns (key or query)
-            // all 32 x 32 (row, column) pairs of this warp visible?  (then no per-element selection)
-            const bool fast = __all_sync(0xffffffffu, MODE == MODE_DQ ? y0 + 32 <= nrow
-                                                                      : key_live && static_cast<long long>(y0) + coff >= xr);
-            // (own columns for the bf16 tiles: the MMAs that read the previous step's must be done before they are
-            // overwritten.  They mostly are by now; the check here costs nothing, its result is wanted after the exponentials)
-            bool acc_done = true;
-            if (LY::SEP && j > 0) acc_done = mbar_test_wait_s(bars_s + 8 * LY::BAR_ACC_STEP, (j - 1) & 1);
-            tc_wait_ld();
-            if (LY::SEP) {                               // T1, T2 may be overwritten by the next step's
+        int n = 0, gs = 0, ne = 0, item = blockIdx.x;
+        decode(item);
+        ok = begin_item(0);
+        if (ok) finish_delta(0);
+        while (ok) {
+            const int xr = x0 + r;                       // the row's index (query in MODE_DQ, key in MODE_DKV)
+            // keys the row takes part with (MODE_DQ: per query row; MODE_DKV: the row IS a key)
+            const long long rlim = static_cast<long long>(xr) + 1 + coff;
+            const int nrow = rlim < nkeys ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : nkeys;
+            const bool key_live = xr < nkeys;
+            const uint64_t c22 = pack2(c2, c2), nl2 = pack2(-lse2_r, -lse2_r), dl2 = pack2(delta_r, delta_r);
+            for (int j = 0; j < nsteps && ok; ++j) {
+                ok = wait_warp(LY::BAR_T_FULL + cgroup, (gs + j) & 1, 0x540 + cgroup);
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t t1[32], t2[32];
+                tmem_ld_x32(tl + LY::T1_COL + cq, t1);
+                tmem_ld_x32(tl + LY::T2_COL + cq, t2);
+                const int y0 = (y_begin + j) * BT + cq;  // index of the first of the columns (key or query)
+                // all 32 x 32 (row, column) pairs of this warp visible?  (then no per-element selection)
+                const bool fast = __all_sync(0xffffffffu, MODE == MODE_DQ ? y0 + 32 <= nrow
+                                                                          : key_live && static_cast<long long>(y0) + coff >= xr);
+                // (own columns for the bf16 tiles: the MMAs that read the previous step's must be done before they are
+                // overwritten.  They mostly are by now; the check here costs nothing, its result is wanted after the exponentials)
+                bool acc_done = true;
+                if (LY::SEP && j > 0) acc_done = mbar_test_wait_s(bars_s + 8 * LY::BAR_ACC_STEP, (gs + j - 1) & 1);
+                tc_wait_ld();
+                if (LY::SEP) {                           // T1, T2 may be overwritten by the next step's
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_s(bars_s + 8 * LY::BAR_T_FREE);
+                }
+                uint32_t pk[16], dk[16];
+                // MODE_DQ:  p = 2^(c T1 - lse2), ds = p (T2 - delta);  MODE_DKV: p = 2^(c T1), ds = p T2 (lse and delta are in T1
+                // and T2).  On packed pairs: two results per issue slot.
+                if (fast) {
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) {
+                        const uint64_t s2 = pack2(__uint_as_float(t1[i]), __uint_as_float(t1[i + 1]));
+                        float a0, a1;
+                        unpack2(LY::DKV ? mul2(s2, c22) : fma2(s2, c22, nl2), a0, a1);
+                        t1[i] = __float_as_uint(ex2_approx(a0)); t1[i + 1] = __float_as_uint(ex2_approx(a1));
+                    }
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) {
+                        const uint64_t g2 = pack2(__uint_as_float(t2[i]), __uint_as_float(t2[i + 1]));
+                        const float p0 = __uint_as_float(t1[i]), p1 = __uint_as_float(t1[i + 1]);
+                        float d0, d1;
+                        unpack2(mul2(pack2(p0, p1), LY::DKV ? g2 : sub2(g2, dl2)), d0, d1);
+                        if (LY::DKV) pk[i / 2] = pack_bf16x2(p0, p1);
+                        dk[i / 2] = pack_bf16x2(d0, d1);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) {
+                        float p[2], ds[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int col = y0 + i + e;
+                            const bool live = MODE == MODE_DQ ? col < nrow : key_live && static_cast<long long>(col) + coff >= xr;
+                            p[e] = live ? ex2_approx(fmaf(__uint_as_float(t1[i + e]), c2, LY::DKV ? 0.f : -lse2_r)) : 0.f;
+                            ds[e] = p[e] * (__uint_as_float(t2[i + e]) - (LY::DKV ? 0.f : delta_r));
+                        }
+                        if (LY::DKV) pk[i / 2] = pack_bf16x2(p[0], p[1]);
+                        dk[i / 2] = pack_bf16x2(ds[0], ds[1]);
+                    }
+                }
+                if (LY::SEP) {
+                    if (!__all_sync(0xffffffffu, acc_done)) {
+                        ok = wait_warp(LY::BAR_ACC_STEP, static_cast<uint32_t>(gs + j - 1) & 1u, 0x542);
+                        if (!ok) break;
+                    }
+                    tc_fence_after();
+                }
+                if (LY::DKV) tmem_st_x16(p_addr, pk);
+                tmem_st_x16(ds_addr, dk);
+                tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_s(bars_s + 8 * LY::BAR_T_FREE);
+                if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::BAR_PD_FULL + cgroup));
             }
-            uint32_t pk[16], dk[16];
-            // MODE_DQ:  p = 2^(c T1 - lse2), ds = p (T2 - delta);  MODE_DKV: p = 2^(c T1), ds = p T2 (lse and delta are in T1
-            // and T2).  On packed pairs: two results per issue slot.
-            if (fast) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const uint64_t s2 = pack2(__uint_as_float(t1[i]), __uint_as_float(t1[i + 1]));
-                    float a0, a1;
-                    unpack2(LY::DKV ? mul2(s2, c22) : fma2(s2, c22, nl2), a0, a1);
-                    t1[i] = __float_as_uint(ex2_approx(a0)); t1[i + 1] = __float_as_uint(ex2_approx(a1));
-                }
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const uint64_t g2 = pack2(__uint_as_float(t2[i]), __uint_as_float(t2[i + 1]));
-                    const float p0 = __uint_as_float(t1[i]), p1 = __uint_as_float(t1[i + 1]);
-                    float d0, d1;
-                    unpack2(mul2(pack2(p0, p1), LY::DKV ? g2 : sub2(g2, dl2)), d0, d1);
-                    if (LY::DKV) pk[i / 2] = pack_bf16x2(p0, p1);
-                    dk[i / 2] = pack_bf16x2(d0, d1);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    float p[2], ds[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int col = y0 + i + e;
-                        const bool live = MODE == MODE_DQ ? col < nrow : key_live && static_cast<long long>(col) + coff >= xr;
-                        p[e] = live ? ex2_approx(fmaf(__uint_as_float(t1[i + e]), c2, LY::DKV ? 0.f : -lse2_r)) : 0.f;
-                        ds[e] = p[e] * (__uint_as_float(t2[i + e]) - (LY::DKV ? 0.f : delta_r));
-                    }
-                    if (LY::DKV) pk[i / 2] = pack_bf16x2(p[0], p[1]);
-                    dk[i / 2] = pack_bf16x2(ds[0], ds[1]);
-                }
+            if (!ok) break;
+            // The next item's operands first (its T MMAs then run under what follows), then this one's gradients.
+            const int bh_out = bh, xr_out = xr, steps_out = nsteps;
+            item = take_item(n + 1);
+            if (item == -2) break;
+            gs += nsteps;
+            if (item >= 0) {
+                decode(item);
+                ok = begin_item(n + 1);
+                if (!ok) break;
             }
-            if (LY::SEP) {
-                if (!__all_sync(0xffffffffu, acc_done)) {
-                    ok = wait_warp(LY::BAR_ACC_STEP, static_cast<uint32_t>(j - 1) & 1u, 0x542);
-                    if (!ok) break;
-                }
+            if (steps_out > 0) {
+                ok = wait_warp(LY::BAR_ACC_DONE, ne & 1, 0x550);
+                if (!ok) break;
                 tc_fence_after();
+                ++ne;
             }
-            if (LY::DKV) tmem_st_x16(p_addr, pk);
-            tmem_st_x16(ds_addr, dk);
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_s(bars_s + 8 * (LY::BAR_PD_FULL + cgroup));
-        }
-        if (ok && nsteps > 0) ok = __all_sync(0xffffffffu, bounded_wait(&bars[LY::BAR_ACC_DONE], 0, abort_flag, status, 0x550));
-        if (ok) {
-            tc_fence_after();
             // this thread's quarter of the features of its row: acc_a -> outA (dQ, or dK), acc_b -> outB (dV)
+            constexpr int NO = MODE == MODE_DKV ? 2 : 1, NC = D / 64;
 #pragma unroll
-            for (int o = 0; o < (MODE == MODE_DKV ? 2 : 1); ++o) {
-                __nv_bfloat16* out = o == 0 ? outA : outB;
+            for (int o = 0; o < NO; ++o) {
                 const float f = o == 0 ? scale : 1.f;
                 const uint32_t col = (o == 0 ? LY::ACC_A_COL : LY::ACC_B_COL) + part * (D / 4);
-                __nv_bfloat16* orow = out + (static_cast<int64_t>(bh) * NX + xr) * D + part * (D / 4);
+                __nv_bfloat16* orow = (o == 0 ? outA : outB) + (static_cast<int64_t>(bh_out) * NX + xr_out) * D + part * (D / 4);
+                uint32_t a[NC][16];
 #pragma unroll
-                for (int c = 0; c < D / 64; ++c) {
-                    uint32_t a[16];
-                    if (nsteps > 0) {
-                        tmem_ld_x16(tl + col + c * 16, a);
-                        tc_wait_ld();
+                for (int c = 0; c < NC; ++c) {
+                    if (steps_out > 0) {
+                        tmem_ld_x16(tl + col + c * 16, a[c]);
                     } else {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) a[i] = 0u;  // nothing sees this tile: zero gradient
+                        for (int i = 0; i < 16; ++i) a[c][i] = 0u;   // nothing sees this tile: zero gradient
                     }
-                    if (xr < NX) {
+                }
+                tc_wait_ld();
+                if (o == NO - 1 && steps_out > 0) {      // the accumulators may be overwritten by the next item's
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_s(bars_s + 8 * LY::BAR_ACC_FREE);
+                }
+                if (xr_out < NX) {
 #pragma unroll
-                        for (int v = 0; v < 2; ++v) {
-                            uint4 w;
-                            w.x = pack_bf16x2(__uint_as_float(a[8 * v + 0]) * f, __uint_as_float(a[8 * v + 1]) * f);
-                            w.y = pack_bf16x2(__uint_as_float(a[8 * v + 2]) * f, __uint_as_float(a[8 * v + 3]) * f);
-                            w.z = pack_bf16x2(__uint_as_float(a[8 * v + 4]) * f, __uint_as_float(a[8 * v + 5]) * f);
-                            w.w = pack_bf16x2(__uint_as_float(a[8 * v + 6]) * f, __uint_as_float(a[8 * v + 7]) * f);
-                            *reinterpret_cast<uint4*>(orow + c * 16 + v * 8) = w;
+                    for (int c = 0; c < NC; ++c) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            w[i] = pack_bf16x2(__uint_as_float(a[c][2 * i]) * f, __uint_as_float(a[c][2 * i + 1]) * f);
+                        if (wide) {
+                            st_global_32B(orow + c * 16, w);
+                        } else {
+                            *reinterpret_cast<uint4*>(orow + c * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+                            *reinterpret_cast<uint4*>(orow + c * 16 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
                         }
                     }
                 }
             }
+            if (item < 0) break;
+            finish_delta(++n);
         }
     }
     tc_fence_before();
@@ -605,9 +791,9 @@ int launch_bwd_mode(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t
     auto bf = [](const void* x) { return static_cast<const __nv_bfloat16*>(x); };
     const cudaError_t e = cudaLaunchKernelEx(
         &cfg, bwd_tc_kernel<D, MODE>, m[0], m[1], m[2], m[3], bf(MODE == MODE_DQ ? p.Q : p.K), bf(MODE == MODE_DQ ? p.dO : p.V), bf(p.O),
-        p.lse, p.delta, static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? p.dQ : p.dK),
-        static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? nullptr : p.dV), BH, p.H, p.Nq, p.Nk, p.scale, p.k_valid_len,
-        p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status);
+        p.lse, p.delta,
+        static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? p.dQ : p.dK), static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? nullptr : p.dV), BH,
+        p.H, p.Nq, p.Nk, p.scale, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
@@ -615,12 +801,12 @@ template <int D>
 int launch_bwd_d(const BwdProblem& p, cudaStream_t st) {
     // stationary tiles are boxes of 128 rows; streamed ones too, or boxes of 64 rows (the dK dV launch at d = 128)
     constexpr int YR = BL<D, MODE_DKV>::Y_ROWS;
-    CUtensorMap tmK, tmV, tmdO, tmQs, tmdOs;
+    CUtensorMap tmQ, tmK, tmV, tmdO, tmQs, tmdOs;
     const int BH = p.B * p.H;
-    if (!make_map(&tmK, p.K, BH, p.Nk, D, BT) || !make_map(&tmV, p.V, BH, p.Nk, D, BT) || !make_map(&tmdO, p.dO, BH, p.Nq, D, BT) ||
-        !make_map(&tmQs, p.Q, BH, p.Nq, D, YR) || !make_map(&tmdOs, p.dO, BH, p.Nq, D, YR))
+    if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BT) || !make_map(&tmdO, p.dO, BH, p.Nq, D, BT) || !make_map(&tmK, p.K, BH, p.Nk, D, BT) ||
+        !make_map(&tmV, p.V, BH, p.Nk, D, BT) || !make_map(&tmQs, p.Q, BH, p.Nq, D, YR) || !make_map(&tmdOs, p.dO, BH, p.Nq, D, YR))
         return FLAT_ERR_CUDA;
-    const int rc = launch_bwd_mode<D, MODE_DQ>(p, {tmdO, tmdO, tmK, tmV}, st);   // (tmX1: Q goes straight to TMEM, not by TMA)
+    const int rc = launch_bwd_mode<D, MODE_DQ>(p, {tmQ, tmdO, tmK, tmV}, st);
     return rc != FLAT_OK ? rc : launch_bwd_mode<D, MODE_DKV>(p, {tmK, tmV, tmQs, tmdOs}, st);
 }
 

@@ -146,6 +146,33 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const void* tmap, ui
         : "memory");
 }
 
+// Brings `bytes` bytes (a multiple of 16) at `p` (16-byte aligned) to L2.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// ---------------------------------------------------------------- work taken over from CTAs that have not started
+// Asks for the index of a CTA of the grid that has not started yet; that CTA then never starts, its work is the asker's.  The
+// answer, 16 bytes at `answer_addr` (shared, 16-byte aligned), completes 16 bytes on the mbarrier.  Not to be asked again after
+// an answer that there is none.
+__device__ __forceinline__ void clc_ask(uint32_t answer_addr, uint32_t bar_addr) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(answer_addr), "r"(bar_addr) : "memory");
+}
+// The index (x) in an answer, or -1 where there was no CTA left.
+__device__ __forceinline__ int clc_answer(uint32_t answer_addr) {
+    uint32_t got, x;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 a;\n\t.reg .b32 y, z;\n\t"
+        "ld.shared.b128 a, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, y, z, _}, a;\n\t}"
+        : "=r"(got), "=r"(x) : "r"(answer_addr) : "memory");
+    return got ? static_cast<int>(x) : -1;
+}
+
 // ---------------------------------------------------------------- TMEM allocation
 // Warp-collective.  ncols: power of two in [32, 512].  The base address is written to *dst (shared).
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
