@@ -156,27 +156,6 @@ __device__ __forceinline__ float exponent_factor(float scale) {
 
 __device__ __forceinline__ void ew_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
-// Wait by a whole warp, every lane for the barrier that it names.  The warp stays together: its lanes probe and vote as one.
-// (Where each lane loops by itself, the lanes come back one by one after a long wait and what follows starts up to 500
-// cycles late.)
-__device__ __forceinline__ bool warp_wait(uint32_t bar_addr, uint32_t parity, uint32_t abort_addr, int32_t* status, int code) {
-    if (__all_sync(0xffffffffu, mbar_try_wait_s(bar_addr, parity))) return true;
-    const long long t0 = clock64();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 32; ++i)
-            if (__all_sync(0xffffffffu, mbar_try_wait_s(bar_addr, parity))) return true;
-        int aborted;
-        asm volatile("ld.volatile.shared::cta.s32 %0, [%1];" : "=r"(aborted) : "r"(abort_addr) : "memory");
-        if (__any_sync(0xffffffffu, aborted)) return false;
-        if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_CYCLES)) {
-            asm volatile("st.volatile.shared::cta.s32 [%0], %1;" ::"r"(abort_addr), "r"(1) : "memory");
-            if (status) atomicExch(status, code);
-            return false;
-        }
-    }
-}
-
 // X1, X2 / Y1, Y2 by mode:  MODE_DQ: (Q, dO) / (K, V);  MODE_DKV: (K, V) / (Q, dO).
 template <int D, int MODE>
 __global__ void __launch_bounds__(BWD_THREADS, 1)
@@ -200,9 +179,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    // (the shuffles here and below tell the compiler that a value is the same in all lanes: the MMA operands, which come from
-    // uniform registers, are then computed there)
-    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int NX = MODE == MODE_DQ ? Nq : Nk;            // rows of the stationary tensors
     const int tiles = (NX + BT - 1) / BT;
 

@@ -170,7 +170,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     uint64_t* bars = reinterpret_cast<uint64_t*>(base + LY::TILE_BYTES);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
 
     // The CTA's r-th item: (batch, head, slab of 256 rows).
     auto get_item = [&](int r, Item& it) -> bool {
@@ -330,7 +330,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 const uint64_t v_desc = make_smem_desc_sw128(smem_u32(Vs), BN * 128, 1024);
                 bool ok = true;
                 auto wait = [&](int bar, uint32_t parity, int code) {
-                    if (ok) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * bar, parity, abort_s, status, code));
+                    if (ok) ok = warp_wait(bars_s + 8 * bar, parity, abort_s, status, code);
                 };
                 auto issue_s = [&](int j, bool last) {   // S_t(j) = Q_t K_j^T, then release the K stage
                     const uint64_t kd = k_desc + static_cast<uint64_t>(((j % KS) * KV_BYTES) >> 4);
@@ -408,13 +408,13 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         for (int j = 0; j < nsteps; ++j) {
             const int g = J + j;
             const uint32_t s_addr = tl + S_COL(t, g & 1);
-            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 8 * (g & 1), (g >> 1) & 1, abort_s, status, 0xa30 + t));
+            ok = warp_wait(my_bars + 8 * (g & 1), (g >> 1) & 1, abort_s, status, 0xa30 + t);
             if (!ok) break;
             tc_fence_after();
             uint32_t s[BN];
             tmem_ld_x32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
             tmem_ld_x32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-            if (BIAS) ok = __all_sync(0xffffffffu, bounded_wait_s(bars_s + 8 * (LY::B_FULL + (BIAS == 2 ? t : 2 * (g & 1) + t)), (BIAS == 2 ? g : g >> 1) & 1, abort_s, status, 0xa36 + t));
+            if (BIAS) ok = warp_wait(bars_s + 8 * (LY::B_FULL + (BIAS == 2 ? t : 2 * (g & 1) + t)), (BIAS == 2 ? g : g >> 1) & 1, abort_s, status, 0xa36 + t);
             tc_wait_ld();
             if (BIAS) {
                 if (!ok) break;
@@ -448,7 +448,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     const float alpha = m_new == -INFINITY ? 1.f : ex2_approx(m_ref - m_new);   // 0 on the row's first keys
                     l *= alpha;
                     if (j > 0) {
-                        ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_s, status, 0xa32 + t));
+                        ok = warp_wait(my_bars + 64 + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_s, status, 0xa32 + t);
                         if (!ok) break;
                         tc_fence_after();
 #pragma unroll 1                          // (rare; unrolled, its registers made the common path spill: 428 -> 482 us)
@@ -472,7 +472,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (lane == 0) mbar_arrive_s(my_bars + 32 + 8 * (g & 1));
         }
         if (ok && nsteps > 0)
-            ok = __all_sync(0xffffffffu, bounded_wait_s(my_bars + 64 + 8 * ((J + nsteps - 1) & 1), ((J + nsteps - 1) >> 1) & 1, abort_s, status, 0xa34 + t));
+            ok = warp_wait(my_bars + 64 + 8 * ((J + nsteps - 1) & 1), ((J + nsteps - 1) >> 1) & 1, abort_s, status, 0xa34 + t);
         if (MULTI) J += nsteps;
         if (ok) {
             const float inv = l > 0.f ? 1.f / l : 0.f;

@@ -85,7 +85,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __shared__ float2 warp_ml[DEC_WARPS][ROWS];          // (m, l) of every warp's rows
     __shared__ float2 cta_ml[ROWS];
     volatile int* abort_flag = &abort_word;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int warp = warp_index(), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int bh = blockIdx.y;
     const int crank = CS > 1 ? static_cast<int>(cluster_ctarank()) : 0;
 
@@ -166,7 +166,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         const int vrow = warp * LY::WKEYS + (lane & 7) + ((lane >> 3) & 1) * 8, vchunk = (lane >> 4) & 1;
         for (int j = 0; j < ntiles; ++j) {
             const int s = j % STAGES;
-            ok = __all_sync(0xffffffffu, bounded_wait(&full[s], (j / STAGES) & 1, abort_flag, status, 0x910));
+            ok = warp_wait(&full[s], (j / STAGES) & 1, abort_flag, status, 0x910);
             if (!ok) break;
             const uint32_t ks = smem_u32(base + s * 2 * LY::TILE_BYTES), vs = ks + LY::TILE_BYTES;
             float c[NT][4];

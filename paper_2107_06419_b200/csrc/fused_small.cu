@@ -120,7 +120,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int bh = blockIdx.y;
     // (causal: the last rows see the most keys, so they start first)
     const int row0 = static_cast<int>(coff < (1 << 29) ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * BM;
@@ -185,7 +185,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const uint64_t q_desc = small_desc<D>(smem_u32(Qs)), k_desc = small_desc<D>(smem_u32(Ks)), v_desc = small_desc<D>(smem_u32(Vs));
             bool ok = true;
             auto wait = [&](int bar, uint32_t parity, int code) {
-                if (ok) ok = __all_sync(0xffffffffu, bounded_wait(&bars[bar], parity, abort_flag, status, code));
+                if (ok) ok = warp_wait(&bars[bar], parity, abort_flag, status, code);
                 if (ok) tc_fence_after();
             };
             auto issue_s = [&](int j) {
@@ -239,7 +239,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const int nrow = rlim < n ? (rlim < 0 ? 0 : static_cast<int>(rlim)) : n;
         const int nrow_min = __shfl_sync(0xffffffffu, nrow, 0);
         for (int j = 0; j < ntiles; ++j) {
-            ok = __all_sync(0xffffffffu, bounded_wait(&bars[LY::S_FULL], j & 1, abort_flag, status, 0x830));
+            ok = warp_wait(&bars[LY::S_FULL], j & 1, abort_flag, status, 0x830);
             if (!ok) break;
             tc_fence_after();
             uint32_t s[BN];
@@ -261,7 +261,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             bool pv_waited = j == 0;
             auto wait_p_free = [&]() {
                 if (!pv_waited) {
-                    ok = __all_sync(0xffffffffu, bounded_wait(&bars[LY::PV_DONE], (j - 1) & 1, abort_flag, status, 0x831));
+                    ok = warp_wait(&bars[LY::PV_DONE], (j - 1) & 1, abort_flag, status, 0x831);
                     pv_waited = true;
                     tc_fence_after();
                 }
@@ -312,7 +312,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[LY::P_FULL]);
         }
-        if (ok && ntiles > 0) ok = __all_sync(0xffffffffu, bounded_wait(&bars[LY::PV_DONE], (ntiles - 1) & 1, abort_flag, status, 0x832));
+        if (ok && ntiles > 0) ok = warp_wait(&bars[LY::PV_DONE], (ntiles - 1) & 1, abort_flag, status, 0x832);
         if (ok) {
             const float inv = l > 0.f ? 1.f / l : 0.f;
             if (lse && row < Nq)

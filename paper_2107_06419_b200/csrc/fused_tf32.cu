@@ -144,7 +144,11 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const uint32_t sb = smem_u32(base);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = D == 128 ? threadIdx.x >> 5 : warp_index(), lane = threadIdx.x & 31;   // (see there)
+    auto whole_warp_wait = [&](uint64_t* bar, uint32_t parity, int code) {
+        return D == 128 ? __all_sync(0xffffffffu, bounded_wait(bar, parity, abort_flag, status, code))
+                        : warp_wait(bar, parity, abort_flag, status, code);
+    };
     // `group` heads at a time, their tiles side by side, the longest first under the causal mask
     const int slabs = (Nq + BM - 1) / BM, per = group * slabs, first = static_cast<int>(blockIdx.x) / per * group;
     const int heads = BH - first < group ? BH - first : group, at = static_cast<int>(blockIdx.x) % per;
@@ -235,7 +239,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 const uint64_t vl_desc = make_smem_desc_sw128(sb + OFF_VTL, 16, 1024);
                 bool ok = true;
                 auto wait = [&](int bar, uint32_t parity, int code) {
-                    if (ok) ok = __all_sync(0xffffffffu, bounded_wait(&bars[bar], parity, abort_flag, status, code));
+                    if (ok) ok = whole_warp_wait(&bars[bar], parity, code);
                     if (ok) tc_fence_after();
                 };
                 constexpr uint32_t IDESC_S = idesc_tf32(BN), IDESC_PV = idesc_tf32(D);
@@ -303,7 +307,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const int ct = threadIdx.x - 256;
             for (int j = 0; j < ntiles && ok; ++j) {
                 const int s = j % KS;
-                ok = __all_sync(0xffffffffu, bounded_wait(&bars[K_FULL + s], (j / KS) & 1, abort_flag, status, 0x641));
+                ok = whole_warp_wait(&bars[K_FULL + s], (j / KS) & 1, 0x641);
                 if (!ok) break;
                 const uint32_t kh = sb + OFF_KH + s * TILE, kl = sb + OFF_KL + s * TILE;
 #pragma unroll
@@ -324,11 +328,11 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             // 16-byte writes free of bank conflicts under the 128-byte swizzle.
             const int u = lane & 7, tq = lane >> 3;
             if (ntiles > 0)
-                ok = __all_sync(0xffffffffu, bounded_wait(&bars[Q_READY], 0, abort_flag, status, 0x640));   // (Q has left the V^T ring)
+                ok = whole_warp_wait(&bars[Q_READY], 0, 0x640);   // (Q has left the V^T ring)
             for (int j = 0; j < ntiles && ok; ++j) {
                 const int r = j % VR, s = j % VS;
-                ok = __all_sync(0xffffffffu, bounded_wait(&bars[V_FULL + r], (j / VR) & 1, abort_flag, status, 0x642));
-                if (ok) ok = __all_sync(0xffffffffu, bounded_wait(&bars[VT_EMPTY + s], ((j / VS) & 1) ^ 1, abort_flag, status, 0x643));
+                ok = whole_warp_wait(&bars[V_FULL + r], (j / VR) & 1, 0x642);
+                if (ok) ok = whole_warp_wait(&bars[VT_EMPTY + s], ((j / VS) & 1) ^ 1, 0x643);
                 if (!ok) break;
                 // 32 x 32 squares (DB: of the features, KB: of the keys) in turn over the two warps
 #pragma unroll
@@ -380,7 +384,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         if (ntiles > 0) {
             // Q row -> TMEM, scaled by scale * log2(e) and split: the logits arrive in base-2 units
             // (the softmax groups take turns at the 32-feature panels of the tile)
-            ok = __all_sync(0xffffffffu, bounded_wait(&bars[Q_FULL], 0, abort_flag, status, 0x650));
+            ok = whole_warp_wait(&bars[Q_FULL], 0, 0x650);
             if (ok) {
 #pragma unroll
                 for (int pn = g; pn < D / 32; pn += 2) {
@@ -406,7 +410,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
         }
         auto accumulate = [&](int k) {                       // O = alpha_k O + PV(k)  (k: a step of this group)
-            ok = __all_sync(0xffffffffu, bounded_wait(&bars[PV_FULL + g], (k >> 1) & 1, abort_flag, status, 0x660 + g));
+            ok = whole_warp_wait(&bars[PV_FULL + g], (k >> 1) & 1, 0x660 + g);
             if (!ok) return;
             tc_fence_after();
             constexpr int CH = 16;                           // (32 at a time: d = 64 1 % slower, d = 128 spills)
@@ -427,7 +431,7 @@ fused_tf32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             // P V(j) cannot be issued before that buffer is free again)
             if (j >= 2) accumulate(j - 2);
             if (!ok) break;
-            ok = __all_sync(0xffffffffu, bounded_wait(&bars[S_FULL + g], (j >> 1) & 1, abort_flag, status, 0x670 + g));
+            ok = whole_warp_wait(&bars[S_FULL + g], (j >> 1) & 1, 0x670 + g);
             if (!ok) break;
             tc_fence_after();
             uint32_t s[BN];

@@ -62,6 +62,36 @@ __device__ __forceinline__ bool bounded_wait_s(uint32_t bar_addr, uint32_t parit
     }
 }
 
+// The warp's index.  The shuffle tells the compiler that it is the same in all lanes: what follows from it (roles, loops, MMA
+// operands) then stays in uniform registers.  With warp_wait below: backward 3 to 7 % a step, fused_d128 2 to 7 %,
+// fused_tf32 5 % (d = 64), fused_small 4 % (d = 16), proj_gemm and fused_decode 1 %.  Not everywhere: fused_tc3 loses 2 %,
+// fused_tc2 1 % and fused_tf32 at d = 128 11 % (ptxas spills more).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
+
+// bounded_wait by a whole warp.  The warp stays together: its lanes probe and vote as one.  (Where each lane loops by itself,
+// they come back one by one after a long wait and what follows starts up to 500 cycles late.)
+__device__ __forceinline__ bool warp_wait(uint32_t bar_addr, uint32_t parity, uint32_t abort_addr, int32_t* status, int code) {
+    if (__all_sync(0xffffffffu, ptx::mbar_try_wait_s(bar_addr, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 32; ++i)
+            if (__all_sync(0xffffffffu, ptx::mbar_try_wait_s(bar_addr, parity))) return true;
+        int aborted;
+        asm volatile("ld.volatile.shared::cta.s32 %0, [%1];" : "=r"(aborted) : "r"(abort_addr) : "memory");
+        if (__any_sync(0xffffffffu, aborted)) return false;
+        if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_CYCLES)) {
+            asm volatile("st.volatile.shared::cta.s32 [%0], %1;" ::"r"(abort_addr), "r"(1) : "memory");
+            if (status) atomicExch(status, code);
+            return false;
+        }
+    }
+}
+
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code) {
+    return warp_wait(ptx::smem_u32(bar), parity, ptx::smem_u32(const_cast<int*>(abort_flag)), status, code);
+}
+
 // Teardown helper: wait for a copy this thread started, with a time limit and no side effects.
 __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
     const long long t0 = clock64();
