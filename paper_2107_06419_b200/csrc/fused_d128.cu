@@ -23,7 +23,8 @@
 // TMEM columns: S(t, b) 128 t + 64 b (b = step parity), P over the first 32 of them, O_t 256 + 128 t.
 // The softmax takes no row maximum after the first step: any reference gives the exact softmax, and a step whose row sum
 // passes 2^40 is redone with a fresh maximum.  One exponential in four goes through a polynomial on the FMA pipe.
-// MULTI: a CTA walks over items (batch, head, slab of 256 rows); the rings and barriers go on from one to the next.
+// MULTI: a CTA walks over items (batch, head, slab of 256 rows), its own and those it takes over from CTAs that have not started;
+// the rings and barriers go on from one to the next.
 // VL: packed batches (Q, O [total_q, H, d], K, V [total_k, H, d]), an item per (sequence, head, slab of the longest sequence): a
 // CTA each, or (MULTI, sequences of one length) by fixed deal.
 // Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
@@ -58,14 +59,16 @@ __host__ __device__ constexpr uint32_t O_COL(int t) { return 256u + 128u * t; }
 // the others of its tile has its last logits when O += P V of the third last step is done, and would take that one's parity for
 // the last one's.)  B_FULL / B_EMPTY [step parity][tile]: the bias tile / the four softmax warps of the tile have read it.
 // Q_EMPTY / O_FREE [tile], once an item: its logit MMAs are done with the Q tile / its four softmax warps have read the output.
+// ITEM_FULL / ITEM_EMPTY [2]: the next item is known / read by the ten other warps.
 template <int BT> struct Layout {
     static constexpr int KS = BT ? 3 : 5, VS = KS;
     static constexpr int BIAS_BYTES = BT == 2 ? BM * SHIFTED_WIDTH(D) * 2 : BM * BN * 2;   // a bias tile: 128 rows of 64 values (2: of 128)
     static constexpr int TILE_BYTES = 2 * Q_BYTES + (KS + VS) * KV_BYTES + (BT == 2 ? 2 : BT ? 4 : 0) * BIAS_BYTES;
     static constexpr int SMEM_BYTES = TILE_BYTES + 512 + 1024;
     static constexpr int Q_FULL = 0, K_FULL = 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS,
-                         P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, B_FULL = PV_DONE + 4, B_EMPTY = B_FULL + 4, Q_EMPTY = B_EMPTY + 4, O_FREE = Q_EMPTY + 2, NUM_BARS = O_FREE + 2;
-    static_assert(SMEM_BYTES <= 232448 && NUM_BARS * 8 + 8 <= 512, "shared memory");
+                         P_FULL = S_FULL + 4, PV_DONE = P_FULL + 4, B_FULL = PV_DONE + 4, B_EMPTY = B_FULL + 4, Q_EMPTY = B_EMPTY + 4, O_FREE = Q_EMPTY + 2, ITEM_EMPTY = O_FREE + 2,
+                         ITEM_FULL = ITEM_EMPTY + 2, NUM_BARS = ITEM_FULL + 2;
+    static_assert(SMEM_BYTES <= 232448 && 32 + NUM_BARS * 8 + 8 <= 512, "shared memory");
 };
 
 // p_i = 2^(s_i * scale + neg_m) of 64 logits; bf16(p) to 32 TMEM columns at `p_addr`; returns the fp32 sum of the unrounded p.
@@ -167,11 +170,31 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     uint8_t* Ks = Qs + 2 * Q_BYTES;
     uint8_t* Vs = Ks + KS * KV_BYTES;
     uint8_t* Bs = Vs + VS * KV_BYTES;                    // (bias) [step parity][tile]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + LY::TILE_BYTES);
+    uint8_t* next_item = base + LY::TILE_BYTES;          // two answers of 16 bytes
+    uint64_t* bars = reinterpret_cast<uint64_t*>(next_item + 32);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = warp_index(), lane = threadIdx.x & 31;
 
+    // (MULTI, without VL) the r-th item, taken over from a CTA that had not started; -1: there was none, or the wait gave up.
+    // The producer's one lane reads it by itself.
+    auto take_item = [&](int r) {
+        const int slot = (r - 1) & 1, full = smem_u32(&bars[LY::ITEM_FULL + slot]), aborts = smem_u32(const_cast<int*>(abort_flag));
+        const uint32_t parity = ((r - 1) >> 1) & 1, answer = smem_u32(next_item) + 16 * slot;
+        if (warp == 8) {
+            if (!bounded_wait_s(full, parity, aborts, status, 0xa50)) return -1;
+            const int item = clc_answer(answer);
+            fence_proxy_async_smem();
+            return item;
+        }
+        if (!warp_wait(full, parity, aborts, status, 0xa51)) return -1;
+        const int item = __shfl_sync(0xffffffffu, clc_answer(answer), 0);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars[LY::ITEM_EMPTY + slot]);
+        __syncwarp();
+        return item;
+    };
     // The CTA's r-th item: (batch, head, slab of 256 rows).
     auto get_item = [&](int r, Item& it) -> bool {
         if (!MULTI && r > 0) return false;
@@ -196,12 +219,10 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             it.n = kl < 0 || it.q_rows <= 0 ? 0 : kl;
             if (coff < (1 << 29)) it.coff = kl - ql;
         } else {
-            // `group` heads at a time, their slabs side by side, the longest first under the causal mask; CTAs with several
-            // items take them forth and back
-            const unsigned at0 = r * gridDim.x + ((r & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+            // `group` heads at a time, their slabs side by side, the longest first under the causal mask
             const int slabs = (Nq + 2 * BM - 1) / (2 * BM), per = group * slabs;
-            if (at0 >= static_cast<unsigned>(BH * slabs)) return false;
-            const int pos = at0;
+            const int pos = MULTI && r > 0 ? take_item(r) : static_cast<int>(blockIdx.x);
+            if (pos < 0) return false;
             const int first = pos / per * group, heads = BH - first < group ? BH - first : group, at = pos % per;
             it.bh = first + at % heads;
             it.row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * (2 * BM);
@@ -222,7 +243,8 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 
     if (threadIdx.x == 256) {
         for (int i = 0; i < LY::NUM_BARS; ++i)
-            mbar_init(&bars[i], (i >= LY::P_FULL && i < LY::PV_DONE) || (i >= LY::B_EMPTY && i < LY::Q_EMPTY) || i >= LY::O_FREE ? 4
+            mbar_init(&bars[i], i >= LY::ITEM_FULL ? 1 : i >= LY::ITEM_EMPTY ? 10
+                                : (i >= LY::P_FULL && i < LY::PV_DONE) || (i >= LY::B_EMPTY && i < LY::Q_EMPTY) || i >= LY::O_FREE ? 4
                                 : (i >= LY::K_EMPTY && i < LY::V_FULL) || (i >= LY::V_EMPTY && i < LY::S_FULL) ? 2 : 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -294,21 +316,32 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         b_issued = 2 * J + t + 1;
                     }
                 };
+                int asked = 0;
                 for (int r = 0; ok && get_item(r, it); ++r) {
-                    if (it.nsteps == 0) continue;
-                    load_q(0);
-                    load_k(0);
-                    load_q(1);
-                    if (BIAS) load_bias(0);
-                    if (it.nsteps > 1) load_k(1);
-                    if (BIAS == 1 && it.nsteps > 1) load_bias(1);
-                    for (int j = 0; j < it.nsteps && ok; ++j) {
-                        load_v(j);
-                        if (j + 2 < it.nsteps) load_k(j + 2);
-                        if (BIAS && (BIAS == 2 || j > 0) && j + 1 < it.nsteps) load_bias(j + 1);
+                    if (it.nsteps > 0) {
+                        load_q(0);
+                        load_k(0);
+                        load_q(1);
+                        if (BIAS) load_bias(0);
+                        if (it.nsteps > 1) load_k(1);
+                        if (BIAS == 1 && it.nsteps > 1) load_bias(1);
+                        for (int j = 0; j < it.nsteps && ok; ++j) {
+                            load_v(j);
+                            if (j + 2 < it.nsteps) load_k(j + 2);
+                            if (BIAS && (BIAS == 2 || j > 0) && j + 1 < it.nsteps) load_bias(j + 1);
+                        }
+                        if (MULTI) { J0 += it.nsteps; ++q; }
                     }
-                    if (MULTI) { J0 += it.nsteps; ++q; }
+                    if (MULTI && !VL) {                  // all copies of this item are on their way: ask for the next one
+                        if (r >= 2) ok = ok && bounded_wait_s(bars_s + 8 * (LY::ITEM_EMPTY + (r & 1)), ((r >> 1) - 1) & 1, abort_s, status, 0xa52);
+                        if (!ok) break;
+                        mbar_arrive_expect_tx(&bars[LY::ITEM_FULL + (r & 1)], 16);
+                        clc_ask(smem_u32(next_item) + 16 * (r & 1), bars_s + 8 * (LY::ITEM_FULL + (r & 1)));
+                        asked = r + 1;
+                    }
                 }
+                if (asked > 0) drain_wait(&bars[LY::ITEM_FULL + ((asked - 1) & 1)], ((asked - 1) >> 1) & 1);
+                if (*abort_flag) ok = false;             // (a wait for the next item may have given up)
                 if (!ok) {
                     for (int t = 0; t < 2; ++t)
                         if (q_issued[t] > 0) drain_wait(&bars[LY::Q_FULL + t], (q_issued[t] - 1) & 1);
@@ -530,7 +563,7 @@ int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStrea
     const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 4);
     const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(MULTI ? device_sm_count() : slabs * BH);
+    cfg.gridDim = dim3(slabs * BH);
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = st;
@@ -550,15 +583,13 @@ int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStrea
 
 int launch_fused_d128(const Problem& p, const BiasMap& bias, cudaStream_t st) {
     if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias.map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
-    // Short items: one CTA per SM that takes them in turn, so that an item's first loads and logits overlap the last one's output
-    // (us, against a CTA per item: B32 H16 128^2 35 -> 27, 256^2 52 -> 46, 512^2 109 -> 94, 768^2 192 -> 177, B8 H16 1024^2 91 ->
-    // 89).  Its key steps are a few per cent slower (H8 16K^2 955 -> 1,030, B2 H16 2048^2 79 -> 80): up to 1024 keys.  Dealt in
-    // advance, so not for items of unknown length (key counts), and under the causal mask, where the hardware's handing out of
-    // the longest first balances better, only with more items per SM than slabs per head (B16 H16 1024^2, 6.9 items and 4 slabs:
-    // 127 -> 116, B32 H16 2048^2, 28 and 8: 638 -> 613; B8 H16 1024^2, 3.5 and 4: 72 -> 75; B4 H16 4096^2, 6.9 and 16: 269 -> 292).
+    // More items than SMs: a CTA that has issued an item's copies takes over another one (clusterlaunchcontrol), so that its
+    // first loads and logits overlap the last one's output.  us, against a CTA per item: B32 H16 128^2 24.8 -> 19.4, 512^2 96 ->
+    // 88, B8 H16 1024^2 78 -> 74.5, 2048^2 238 -> 233, causal B16 H16 1024^2 111 -> 102, B4 H16 4096^2 256 -> 249.5, key counts
+    // B12 H12 1000^2 73.6 -> 70.3, B6 H12 1024 x 8192 211 -> 209.  With no more items than SMs the last question costs 0.5 to 1 us
+    // for nothing (B4 H8 1000^2 21.2 -> 22.2); from long key sequences on this form's steps make up for it (H4 16K^2 419 -> 408).
     const int sms = device_sm_count(), slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
-    const int64_t items = static_cast<int64_t>(slabs) * p.B * p.H;
-    const bool several = items > sms && !p.k_valid_len && (p.causal ? p.Nk <= 2048 && items > static_cast<int64_t>(slabs) * sms : p.Nk <= 1024);
+    const bool several = static_cast<int64_t>(slabs) * p.B * p.H > sms || p.Nk > 8192;
     const int sr = bias.shifted_rows;
     if (bias.map) {
         const CUtensorMap& tmB = *static_cast<const CUtensorMap*>(bias.map);
