@@ -115,21 +115,21 @@ template <int D, int MODE> struct BL {
     // barriers.  Per item: X_FULL: stationary tiles in shared memory; X_TMEM: in TMEM (one arrival per element-wise warp);
     // X_EMPTY: the T MMAs that read them from shared memory have completed (where none do: warp 17 has seen X_TMEM);
     // ACC_DONE: everything accumulated; ACC_FREE: the accumulators are in registers; ITEM_FULL / ITEM_EMPTY [2]: the next item
-    // is known / read by every warp.
+    // is known / read by every warp; DELTA (MODE_DQ): delta of the item's rows is in shared memory.
     // Y_FULL [S1]: the copy's Y1 and Y2 have landed (and, MODE_DKV, warp 19 has written the step's slices);
     // Y1_EMPTY [S1], Y2_EMPTY [S2] (MODE_DQ): read; ACC_STEP (SEP): the MMAs that read dS, P have completed;
     // per column group: T_FULL: T1, T2 computed; PD_FULL: dS (and P) written; T_FREE (SEP): T1, T2
     // taken into registers.  Without SEP warp 18 arrives on PD_FULL, too, once the half's next copy has landed, so that the
     // issuing warp has one barrier to look at.
     static constexpr int BAR_X_FULL = 0, BAR_X_TMEM = 1, BAR_X_EMPTY = 2, BAR_ACC_FREE = 3, BAR_ITEM_FULL = 4, BAR_ITEM_EMPTY = 6,
-                         BAR_Y_FULL = 8, BAR_Y1_EMPTY = BAR_Y_FULL + S1,
+                         BAR_DELTA = 8, BAR_Y_FULL = 9, BAR_Y1_EMPTY = BAR_Y_FULL + S1,
                          BAR_Y2_EMPTY = BAR_Y1_EMPTY + S1, BAR_ACC_STEP = BAR_Y2_EMPTY + S2, BAR_ACC_DONE = BAR_ACC_STEP + 1,
                          BAR_T_FULL = BAR_ACC_DONE + 1, BAR_T_FREE = BAR_T_FULL + PARTS, BAR_PD_FULL = BAR_T_FREE + 1,
                          NUM_BARS = BAR_PD_FULL + PARTS;
     static constexpr int PD_ARRIVALS = SEP ? EW_WARPS : EW_WARPS / 2 + 1;
     static constexpr int READERS = EW_WARPS + (DKV ? 3 : 2);                 // warps that read an item: all but the producer
     __host__ __device__ static constexpr int arrivals(int i) {
-        return i == BAR_X_TMEM || i == BAR_ACC_FREE || i == BAR_T_FREE ? EW_WARPS
+        return i == BAR_X_TMEM || i == BAR_ACC_FREE || i == BAR_T_FREE || i == BAR_DELTA ? EW_WARPS
                : i == BAR_ITEM_EMPTY || i == BAR_ITEM_EMPTY + 1 ? READERS
                : i >= BAR_Y_FULL && i < BAR_Y1_EMPTY && DKV ? 2 : i >= BAR_PD_FULL ? PD_ARRIVALS : 1;
     }
@@ -153,8 +153,6 @@ __device__ __forceinline__ float exponent_factor(float scale) {
     const float c = scale * LOG2E;
     return fabsf(c) >= 1e-30f ? c : 1e-30f;
 }
-
-__device__ __forceinline__ void ew_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
 // X1, X2 / Y1, Y2 by mode:  MODE_DQ: (Q, dO) / (K, V);  MODE_DKV: (K, V) / (Q, dO).
 template <int D, int MODE>
@@ -528,7 +526,6 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         // MMAs of the previous item have completed: their results have been seen here) and computes delta = sum_t dO O:
         // eight rows a warp, a row's features side by side in its lanes.
         constexpr int LPR = D / 8, ROWS = 32 / LPR, PASSES = 8 / ROWS;       // lanes a row, rows a pass
-        float sums[PASSES];
         auto begin_item = [&](int n) {
             if constexpr (!LY::DKV) {
                 uint4 da[PASSES], db[PASSES];
@@ -573,25 +570,25 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                     }
 #pragma unroll
                     for (int m = LPR / 2; m >= 1; m >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, m);
-                    sums[i] = sum;
+                    const int row = warp * 8 + i * ROWS + lane / LPR;
+                    if (lane % LPR == 0) {
+                        dls[(n & 1) * BT + row] = sum;
+                        if (x0 + row < Nq) delta[static_cast<int64_t>(bh) * Nq + x0 + row] = sum;
+                    }
                 }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars[LY::BAR_DELTA]);
             }
             return true;
         };
+        // Every warp needs what other warps computed.  One that gives up leaves the loop, so they meet at an mbarrier, in a wait
+        // that gives up too: at a named barrier the rest would stand for good.
         auto finish_delta = [&](int n) {
             if constexpr (!LY::DKV) {
-                float* d_item = dls + (n & 1) * BT;
-#pragma unroll
-                for (int i = 0; i < PASSES; ++i) {
-                    const int row = warp * 8 + i * ROWS + lane / LPR;
-                    if (lane % LPR == 0) {
-                        d_item[row] = sums[i];
-                        if (x0 + row < Nq) delta[static_cast<int64_t>(bh) * Nq + x0 + row] = sums[i];
-                    }
-                }
-                ew_sync();
-                delta_r = d_item[r];
+                if (!wait_warp(LY::BAR_DELTA, n & 1, 0x543)) return false;
+                delta_r = dls[(n & 1) * BT + r];
             }
+            return true;
         };
         const int cq = part * 32;                        // this warp's 32 columns of every step
         const int cgroup = LY::PARTS == 2 ? part >> 1 : 0;
@@ -599,8 +596,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         const uint32_t p_addr = tl + LY::p_store(0) + part * (LY::p_store(1) - LY::p_store(0));
         int n = 0, gs = 0, ne = 0, item = blockIdx.x;
         decode(item);
-        ok = begin_item(0);
-        if (ok) finish_delta(0);
+        ok = begin_item(0) && finish_delta(0);
         while (ok) {
             const int xr = x0 + r;                       // the row's index (query in MODE_DQ, key in MODE_DKV)
             // keys the row takes part with (MODE_DQ: per query row; MODE_DKV: the row IS a key)
@@ -735,7 +731,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                 }
             }
             if (item < 0) break;
-            finish_delta(++n);
+            ok = finish_delta(++n);
         }
     }
     tc_fence_before();
