@@ -133,7 +133,7 @@ template <int D, int MODE> struct BL {
                : i == BAR_ITEM_EMPTY || i == BAR_ITEM_EMPTY + 1 ? READERS
                : i >= BAR_Y_FULL && i < BAR_Y1_EMPTY && DKV ? 2 : i >= BAR_PD_FULL ? PD_ARRIVALS : 1;
     }
-    static_assert(NUM_BARS * 8 + 8 + 32 <= 512, "barriers");
+    static_assert(NUM_BARS * 8 + 16 + 32 <= 512, "barriers");
 };
 
 // Shared-memory descriptor of a slice tile: K-major rows of 32 bytes, 32-byte swizzle, eight rows 256 bytes apart.
@@ -176,6 +176,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     uint64_t* bars = reinterpret_cast<uint64_t*>(next_item + 32);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int* first_item = reinterpret_cast<int*>(tmem_slot + 2);
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int NX = MODE == MODE_DQ ? Nq : Nk;            // rows of the stationary tensors
@@ -195,6 +196,21 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         }
         fence_proxy_async_smem();
     }
+    // Item -> (head, tile): `group` heads at a time, their tiles side by side, the longest first under the causal mask
+    // (the last query tiles, the first key tiles); its range of streamed tiles, those with at least one visible (query, key)
+    // pair.  Causal mask (coff = Nk - Nq; 2^30 = none): query i sees key j iff j <= i + coff.
+    int bh, x0, nkeys, y_begin, nsteps;                  // nkeys: keys of this batch that take part at all
+    auto place = [&](int item, int& head, int& row) {
+        const int per = group * tiles, first_head = item / per * group;
+        const int heads = BH - first_head < group ? BH - first_head : group;
+        const int at = item % per;
+        head = first_head + at % heads;
+        row = (MODE == MODE_DQ && coff < (1 << 29) ? tiles - 1 - at / heads : at / heads) * BT;
+    };
+    // (the first item's here, by one thread, under the tail of the previous kernel: behind the wait below, by twenty warps at once,
+    // its divisions take 1,000 cycles)
+    if (threadIdx.x == 0) place(blockIdx.x, first_item[0], first_item[1]);
+
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -208,19 +224,13 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         return warp_wait(bars_s + 8 * bar, parity, abort_s, status, code);
     };
 
-    // Item -> (head, tile): `group` heads at a time, their tiles side by side, the longest first under the causal mask
-    // (the last query tiles, the first key tiles); its range of streamed tiles, those with at least one visible (query, key)
-    // pair.  Causal mask (coff = Nk - Nq; 2^30 = none): query i sees key j iff j <= i + coff.
-    int bh, x0, nkeys, y_begin, nsteps;                  // nkeys: keys of this batch that take part at all
-    auto place = [&](int item, int& head, int& row) {
-        const int per = group * tiles, first_head = item / per * group;
-        const int heads = BH - first_head < group ? BH - first_head : group;
-        const int at = item % per;
-        head = first_head + at % heads;
-        row = (MODE == MODE_DQ && coff < (1 << 29) ? tiles - 1 - at / heads : at / heads) * BT;
-    };
     auto decode = [&](int item) {
-        place(item, bh, x0);
+        if (item == static_cast<int>(blockIdx.x)) {
+            bh = __shfl_sync(0xffffffffu, first_item[0], 0);
+            x0 = __shfl_sync(0xffffffffu, first_item[1], 0);
+        } else {
+            place(item, bh, x0);
+        }
         nkeys = Nk;
         if (valid_len) {
             nkeys = __shfl_sync(0xffffffffu, valid_len[bh / H], 0);
