@@ -178,7 +178,10 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* first_item = reinterpret_cast<int*>(tmem_slot + 2);
 
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    // Roles go by an index that the compiler knows to be the same in all lanes, and so does everything else in MODE_DKV.  Inside
+    // the roles of MODE_DQ it is better not known (with it / without: 128 rows against 16384 keys, d = 64 114 / 104 us, d = 128
+    // 138 / 132; MODE_DKV 16384 rows against 128 keys 124 / 128 and 231 / 249; roles by the other one, too: 107).
+    const int role = warp_index(), warp = MODE == MODE_DQ ? threadIdx.x >> 5 : role, lane = threadIdx.x & 31;
     const int NX = MODE == MODE_DQ ? Nq : Nk;            // rows of the stationary tensors
     const int tiles = (NX + BT - 1) / BT;
 
@@ -264,8 +267,8 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
 
     // Every role walks the same items; n: the item's number, gs: steps before it, ne: items before it that had steps.
     // The rings and the phases of the per-step barriers run on over the items.
-    if (warp >= EW_WARPS) {
-      if (warp == EW_WARPS) {
+    if (role >= EW_WARPS) {
+      if (role == EW_WARPS) {
         // ------------------------------------------------------------ TMA producer (lane 0 issues the copies)
         if (lane == 0) { prefetch_tensormap(&tmX1); prefetch_tensormap(&tmX2); prefetch_tensormap(&tmY1); prefetch_tensormap(&tmY2); }
         // The next item is asked for some steps before the end of this one (six: early enough for what follows, late enough that
