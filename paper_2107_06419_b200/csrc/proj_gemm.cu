@@ -84,7 +84,10 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     uint64_t* bars = reinterpret_cast<uint64_t*>(base + LY::TILE_BYTES + LY::RECV_BYTES);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    // Roles by an index that the compiler knows to be the same in all lanes, the epilogue by one that it does not (all known: forms of
+    // four CTAs spill, M 128 K 768 -> 768 4.86 -> 5.12 us; so: 4.81).  The two forms to head-major tensors that spill even then
+    // (clusters of four; 256 x 256) know it nowhere: M 128 -> 768 5.43 -> 5.12, M 8192 -> 3072 41.2 -> 40.6.
+    const int warp = threadIdx.x >> 5, role = OUT_HEADS && (CS == 4 || TN == 256) ? warp : warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 8 * 32) {
         // (eight epilogue warps free an accumulator; the 8 / CS warps of every other CTA that hold rows of this one send)
@@ -113,7 +116,7 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int ksteps = CS > 1 ? all_steps * (crank + 1) / CS - k_first : all_steps;
     const int tile_first = blockIdx.x / CS, tile_step = gridDim.x / CS;
 
-    if (warp == 8) {
+    if (role == 8) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             prefetch_tensormap(&tmA); prefetch_tensormap(&tmW);
@@ -151,7 +154,7 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 for (int j = issued > STAGES ? issued - STAGES : 0; j < issued; ++j)
                     drain_wait(&bars[LY::FULL + j % STAGES], (j / STAGES) & 1);
         }
-    } else if (warp == 9) {
+    } else if (role == 9) {
         // ------------------------------------------------------------ MMA issuer
         constexpr uint32_t IDESC = make_idesc_bf16(128, TN, 0, 0);
         const uint64_t ad = make_smem_desc_sw128(smem_u32(As), 16, 1024);
