@@ -120,7 +120,10 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    // Roles by an index that the compiler knows to be the same in all lanes, the softmax warps by one that it does not; they wait by
+    // whole warps, the issuer's lanes one by one (us, all known and by whole warps / so: B2 H8 16K^2 d 32 1,598 / 1,535, d 16 1,570 /
+    // 1,519, B16 H8 1000^2 64.6 / 63.0 and 62.9 / 61.7; the softmax warps' waits lane by lane, too: d 16 1,548).
+    const int role = warp_index(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int bh = blockIdx.y;
     // (causal: the last rows see the most keys, so they start first)
     const int row0 = static_cast<int>(coff < (1 << 29) ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * BM;
@@ -147,7 +150,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     }
     const int ntiles = (n + BN - 1) / BN;
 
-    if (warp == 4) {
+    if (role == 4) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0 && ntiles > 0) {
             prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
@@ -177,7 +180,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     drain_wait(&bars[LY::V_FULL + j % STAGES], (j / STAGES) & 1);
             }
         }
-    } else if (warp == 5) {
+    } else if (role == 5) {
         // ------------------------------------------------------------ MMA issuer (whole warp walks, one lane issues)
         if (ntiles > 0) {
             constexpr uint32_t IDESC_S = make_idesc_bf16(BM, BN, 0, 0);
@@ -185,7 +188,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const uint64_t q_desc = small_desc<D>(smem_u32(Qs)), k_desc = small_desc<D>(smem_u32(Ks)), v_desc = small_desc<D>(smem_u32(Vs));
             bool ok = true;
             auto wait = [&](int bar, uint32_t parity, int code) {
-                if (ok) ok = warp_wait(&bars[bar], parity, abort_flag, status, code);
+                if (ok) ok = __all_sync(0xffffffffu, bounded_wait(&bars[bar], parity, abort_flag, status, code));
                 if (ok) tc_fence_after();
             };
             auto issue_s = [&](int j) {
