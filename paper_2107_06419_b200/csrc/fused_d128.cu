@@ -175,14 +175,17 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     uint64_t* bars = reinterpret_cast<uint64_t*>(next_item + 32);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + LY::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    // Roles go by an index that the compiler knows to be the same in all lanes, and so do the softmax warps where a CTA takes several
+    // items (without it 12 % a step).  With one item a CTA it is better not known to them: H2 16K^2 214 -> 208 us, H16 2048^2 32.1 ->
+    // 31.1, H8 4096^2 56.8 -> 55.9.
+    const int role = warp_index(), warp = MULTI ? role : static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
 
     // (MULTI, without VL) the r-th item, taken over from a CTA that had not started; -1: there was none, or the wait gave up.
     // The producer's one lane reads it by itself.
     auto take_item = [&](int r) {
         const int slot = (r - 1) & 1, full = smem_u32(&bars[LY::ITEM_FULL + slot]), aborts = smem_u32(const_cast<int*>(abort_flag));
         const uint32_t parity = ((r - 1) >> 1) & 1, answer = smem_u32(next_item) + 16 * slot;
-        if (warp == 8) {
+        if (role == 8) {
             if (!bounded_wait_s(full, parity, aborts, status, 0xa50)) return -1;
             const int item = clc_answer(answer);
             fence_proxy_async_smem();
@@ -263,9 +266,9 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const uint32_t tmem = *tmem_slot;
     const uint32_t bars_s = smem_u32(bars), abort_s = smem_u32(const_cast<int*>(abort_flag));
 
-    if (warp >= 8) {
+    if (role >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-        if (warp == 8) {
+        if (role == 8) {
             // ------------------------------------------------------------ TMA producer
             if (lane == 0) {
                 prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
@@ -354,9 +357,9 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                             else if (u + 2 >= b_issued) drain_wait(&bars[LY::B_FULL + (u & 1)], (u >> 1) & 1);
                 }
             }
-        } else if (warp <= 10) {
+        } else if (role <= 10) {
             // ------------------------------------------------------------ MMA issuer of tile t (whole warp walks, one lane issues)
-            const int t = warp - 9;
+            const int t = role - 9;
             {
                 constexpr uint32_t IDESC_S = make_idesc_bf16(BM, BN, 0, 0), IDESC_PV = make_idesc_bf16(BM, D, 0, 1);
                 const uint64_t q_desc = make_smem_desc_sw128(smem_u32(Qs) + t * Q_BYTES, 16, 1024);
@@ -587,10 +590,11 @@ int launch_fused_d128(const Problem& p, const BiasMap& bias, cudaStream_t st) {
     // More items than SMs: a CTA that has issued an item's copies takes over another one (clusterlaunchcontrol), so that its
     // first loads and logits overlap the last one's output.  us, against a CTA per item: B32 H16 128^2 24.8 -> 19.4, 512^2 96 ->
     // 88, B8 H16 1024^2 78 -> 74.5, 2048^2 238 -> 233, causal B16 H16 1024^2 111 -> 102, B4 H16 4096^2 256 -> 249.5, key counts
-    // B12 H12 1000^2 73.6 -> 70.3, B6 H12 1024 x 8192 211 -> 209.  With no more items than SMs the last question costs 0.5 to 1 us
-    // for nothing (B4 H8 1000^2 21.2 -> 22.2); from long key sequences on this form's steps make up for it (H4 16K^2 419 -> 408).
+    // B12 H12 1000^2 73.6 -> 70.3, B6 H12 1024 x 8192 211 -> 209.  With no more items than SMs there is nothing to take over: the form
+    // for one item is the faster one at any length (us, taken over / one item: B4 H8 1000^2 20.4 / 19.4, H2 16K^2 213 / 208, H1 32K^2 420 /
+    // 412, H8 4000 x 16K 217 / 211).
     const int sms = device_sm_count(), slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
-    const bool several = static_cast<int64_t>(slabs) * p.B * p.H > sms || p.Nk > 8192;
+    const bool several = static_cast<int64_t>(slabs) * p.B * p.H > sms;
     const int sr = bias.shifted_rows;
     if (bias.map) {
         const CUtensorMap& tmB = *static_cast<const CUtensorMap*>(bias.map);
@@ -611,7 +615,7 @@ int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* 
     const int slabs = (max_seqlen_q + 2 * BM - 1) / (2 * BM), group = causal && slabs <= 65535, sms = device_sm_count();
     const int64_t items = static_cast<int64_t>(slabs) * num_seqs * H;
     // Items that all weigh the same -- sequences of one length, without the causal mask or of one slab -- several per CTA, up to
-    // launch_fused_d128's bound and from three per SM on (us, a CTA each / dealt: 100 of 256 tokens, 16 heads 146 / 129, causal
+    // 1024 tokens and from three per SM on (us, a CTA each / dealt: 100 of 256 tokens, 16 heads 146 / 129, causal
     // 142 / 116; 64 of 128, 8 heads 26.3 / 20.7; 64 of 64, 16 heads 36 / 22; 32 of 1000, 16 heads 281 / 275; with 1.7 and 2.6 per
     // SM, 16 of 512, 8 heads 26.5 / 27.5, 16 of 300, 12 heads 33.1 / 35.4).
     const bool alike = total_q == static_cast<int64_t>(num_seqs) * max_seqlen_q && total_k == total_q && (!causal || slabs == 1);
