@@ -24,15 +24,17 @@
 // TMEM columns: S(t, b) 128 t + 64 b (b = step parity), P over the first 32 of them, O_t 256 + 128 t.
 // The softmax takes no row maximum after the first step: any reference gives the exact softmax, and a step whose row sum
 // passes 2^40 is redone with a fresh maximum.  One exponential in four goes through a polynomial on the FMA pipe.
-// MULTI: a CTA walks over items (batch, head, slab of 256 rows), its own and those it takes over from CTAs that have not started;
-// the rings and barriers go on from one to the next.
+// ITEMS: a CTA has one item (batch, head, slab of 256 rows), several that are dealt in advance, or its own and those it takes over
+// from CTAs that have not started; the rings and barriers go on from one to the next.
 // VL: packed batches (Q, O [total_q, H, d], K, V [total_k, H, d]), an item per (sequence, head, slab of the longest sequence): a
-// CTA each, or (MULTI, sequences of one length) by fixed deal.
+// CTA each, or (sequences of one length) dealt.
 // Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "flat_internal.cuh"
 #include "ptx_sm100.cuh"
@@ -155,7 +157,9 @@ struct Item {
     int head, q_tok0, k_tok0, q_rows;                    // (packed batches)
 };
 
-template <bool VL, int BIAS, bool MULTI>
+enum { ONE_ITEM = 0, DEALT = 1, TAKEN_OVER = 2 };
+
+template <bool VL, int BIAS, int ITEMS>
 __global__ void __launch_bounds__(THREADS, 1)
 fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                   __nv_bfloat16* __restrict__ O, int BH, int H, int Nq, int Nk, float scale_log2e, const int32_t* __restrict__ valid_len,
@@ -163,6 +167,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                   float* __restrict__ lse, const __grid_constant__ CUtensorMap tmBias = CUtensorMap{}, int bias_heads = 0,
                   int bias_batches = 0, const ShiftedBias sb = ShiftedBias{}) {
     using LY = Layout<BIAS>;
+    constexpr bool MULTI = ITEMS != ONE_ITEM;
     constexpr int BIAS_BYTES = LY::BIAS_BYTES;
     constexpr int KS = LY::KS, VS = LY::VS;
     extern __shared__ uint8_t smem_raw[];
@@ -180,7 +185,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // 31.1, H8 4096^2 56.8 -> 55.9.
     const int role = warp_index(), warp = MULTI ? role : static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
 
-    // (MULTI, without VL) the r-th item, taken over from a CTA that had not started; -1: there was none, or the wait gave up.
+    // (TAKEN_OVER) the r-th item, taken over from a CTA that had not started; -1: there was none, or the wait gave up.
     // The producer's one lane reads it by itself.
     auto take_item = [&](int r) {
         const int slot = (r - 1) & 1, full = smem_u32(&bars[LY::ITEM_FULL + slot]), aborts = smem_u32(const_cast<int*>(abort_flag));
@@ -225,8 +230,15 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         } else {
             // `group` heads at a time, their slabs side by side, the longest first under the causal mask
             const int slabs = (Nq + 2 * BM - 1) / (2 * BM), per = group * slabs;
-            const int pos = MULTI && r > 0 ? take_item(r) : static_cast<int>(blockIdx.x);
-            if (pos < 0) return false;
+            int pos = blockIdx.x;
+            if (ITEMS == DEALT) {                        // (forth and back)
+                const unsigned at = r * gridDim.x + ((r & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+                if (at >= static_cast<unsigned>(BH * slabs)) return false;
+                pos = at;
+            } else if (ITEMS == TAKEN_OVER && r > 0) {
+                pos = take_item(r);
+                if (pos < 0) return false;
+            }
             const int first = pos / per * group, heads = BH - first < group ? BH - first : group, at = pos % per;
             it.bh = first + at % heads;
             it.row0 = (coff < (1 << 29) ? slabs - 1 - at / heads : at / heads) * (2 * BM);
@@ -336,7 +348,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         }
                         if (MULTI) { J0 += it.nsteps; ++q; }
                     }
-                    if (MULTI && !VL) {                  // all copies of this item are on their way: ask for the next one
+                    if (ITEMS == TAKEN_OVER) {           // all copies of this item are on their way: ask for the next one
                         if (r >= 2) ok = ok && bounded_wait_s(bars_s + 8 * (LY::ITEM_EMPTY + (r & 1)), ((r >> 1) - 1) & 1, abort_s, status, 0xa52);
                         if (!ok) break;
                         mbar_arrive_expect_tx(&bars[LY::ITEM_FULL + (r & 1)], 16);
@@ -553,7 +565,7 @@ fused_d128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int BIAS, bool MULTI>
+template <int BIAS, int ITEMS>
 int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStream_t st) {
     constexpr int SMEM_BYTES = Layout<BIAS>::SMEM_BYTES;
     CUtensorMap tmQ, tmK, tmV;
@@ -561,13 +573,13 @@ int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStrea
     if (static_cast<int64_t>(slabs) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
     if (!make_map(&tmQ, p.Q, BH, p.Nq, D, BM) || !make_map(&tmK, p.K, BH, p.Nk, D, BN) || !make_map(&tmV, p.V, BH, p.Nk, D, BN))
         return FLAT_ERR_CUDA;
-    if (!ensure_dynamic_smem<fused_d128_kernel<false, BIAS, MULTI>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<fused_d128_kernel<false, BIAS, ITEMS>>(SMEM_BYTES)) return FLAT_ERR_CUDA;
     // without the causal mask the slabs of a head run side by side and share K and V in L2; with it, those of as many heads as
     // fit L2 together (48 MB of K and V) go longest first: what is left at the end are the short ones
     const int64_t fit = (48ll << 20) / (static_cast<int64_t>(p.Nk) * D * 4);
     const int group = !p.causal || fit < 1 ? 1 : fit < BH ? static_cast<int>(fit) : BH;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(slabs * BH);
+    cfg.gridDim = dim3(ITEMS == DEALT ? device_sm_count() : slabs * BH);
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = st;
@@ -576,7 +588,7 @@ int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStrea
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false, BIAS, MULTI>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fused_d128_kernel<false, BIAS, ITEMS>, tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(p.O), BH, p.H, p.Nq, p.Nk,
                                              p.scale * 1.4426950408889634f, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), group, p.status,
                                              static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr), p.lse, tmB, p.bias_sh ? 1 : 0, p.bias_sb ? 1 : 0,
                                              ShiftedBias{static_cast<const uint16_t*>(p.bias), shifted_rows});
@@ -587,21 +599,26 @@ int launch(const Problem& p, const CUtensorMap& tmB, int shifted_rows, cudaStrea
 
 int launch_fused_d128(const Problem& p, const BiasMap& bias, cudaStream_t st) {
     if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias.map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
-    // More items than SMs: a CTA that has issued an item's copies takes over another one (clusterlaunchcontrol), so that its
-    // first loads and logits overlap the last one's output.  us, against a CTA per item: B32 H16 128^2 24.8 -> 19.4, 512^2 96 ->
-    // 88, B8 H16 1024^2 78 -> 74.5, 2048^2 238 -> 233, causal B16 H16 1024^2 111 -> 102, B4 H16 4096^2 256 -> 249.5, key counts
-    // B12 H12 1000^2 73.6 -> 70.3, B6 H12 1024 x 8192 211 -> 209.  With no more items than SMs there is nothing to take over: the form
-    // for one item is the faster one at any length (us, taken over / one item: B4 H8 1000^2 20.4 / 19.4, H2 16K^2 213 / 208, H1 32K^2 420 /
-    // 412, H8 4000 x 16K 217 / 211).
+    // More items than SMs: several items per CTA, so that one's first loads and logits overlap the last one's output.
+    // Items of up to 1024 keys, and no more than three a query, that all weigh the same (no key counts, no causal mask) are dealt in
+    // advance.  Otherwise a CTA that has issued an item's copies takes over another one (clusterlaunchcontrol): long and unequal items
+    // end together, but every role of the CTA has to read the answer before it can go on.  us, taken over / dealt: B32 H8 300^2
+    // 37.0 / 32.7, B81 H8 64^2 16.4 / 15.2, B32 H4 2000 x 500 86.0 / 80.1, B30 H8 600^2 with bias 88.0 / 83.5; B44 H4 100 x 500
+    // 21.3 / 22.5, 200 x 800 32.4 / 34.8, causal B16 H16 512^2 43.9 / 49.6, key counts B12 H12 1000^2 59.9 / 61.0, B4 H16 2048^2
+    // 123.0 / 124.3, H4 16K^2 412 / 424.
+    // With no more items than SMs there is nothing to take over: the form for one item is the faster one at any length (us, taken over
+    // / one item: B4 H8 1000^2 20.4 / 19.4, H2 16K^2 213 / 208, H1 32K^2 420 / 412, H8 4000 x 16K 217 / 211).
     const int sms = device_sm_count(), slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
-    const bool several = static_cast<int64_t>(slabs) * p.B * p.H > sms;
+    const bool alike = !p.k_valid_len && !p.causal && p.Nk <= 1024 && p.Nk <= 3 * static_cast<int64_t>(p.Nq);
+    const int items = static_cast<int64_t>(slabs) * p.B * p.H <= sms ? ONE_ITEM : alike ? DEALT : TAKEN_OVER;
     const int sr = bias.shifted_rows;
-    if (bias.map) {
-        const CUtensorMap& tmB = *static_cast<const CUtensorMap*>(bias.map);
-        if (sr >= 0) return several ? launch<2, true>(p, tmB, sr, st) : launch<2, false>(p, tmB, sr, st);
-        return several ? launch<1, true>(p, tmB, sr, st) : launch<1, false>(p, tmB, sr, st);
-    }
-    return several ? launch<0, true>(p, CUtensorMap{}, sr, st) : launch<0, false>(p, CUtensorMap{}, sr, st);
+    auto run = [&](auto form) {
+        constexpr int BIAS = decltype(form)::value;
+        const CUtensorMap tmB = bias.map ? *static_cast<const CUtensorMap*>(bias.map) : CUtensorMap{};
+        return items == ONE_ITEM ? launch<BIAS, ONE_ITEM>(p, tmB, sr, st) : items == DEALT ? launch<BIAS, DEALT>(p, tmB, sr, st) : launch<BIAS, TAKEN_OVER>(p, tmB, sr, st);
+    };
+    if (!bias.map) return run(std::integral_constant<int, 0>{});
+    return sr >= 0 ? run(std::integral_constant<int, 2>{}) : run(std::integral_constant<int, 1>{});
 }
 
 int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* O, const int32_t* cu_q, const int32_t* cu_k, int num_seqs,
@@ -620,11 +637,11 @@ int launch_fused_d128_varlen(const void* Q, const void* K, const void* V, void* 
     // SM, 16 of 512, 8 heads 26.5 / 27.5, 16 of 300, 12 heads 33.1 / 35.4).
     const bool alike = total_q == static_cast<int64_t>(num_seqs) * max_seqlen_q && total_k == total_q && (!causal || slabs == 1);
     const bool several = alike && items >= 3 * static_cast<int64_t>(sms) && items <= 0x7fffffff && max_seqlen_q <= 1024;
-    if (!(several ? ensure_dynamic_smem<fused_d128_kernel<true, 0, true>>(Layout<0>::SMEM_BYTES)
-                  : ensure_dynamic_smem<fused_d128_kernel<true, 0, false>>(Layout<0>::SMEM_BYTES)))
+    if (!(several ? ensure_dynamic_smem<fused_d128_kernel<true, 0, DEALT>>(Layout<0>::SMEM_BYTES)
+                  : ensure_dynamic_smem<fused_d128_kernel<true, 0, ONE_ITEM>>(Layout<0>::SMEM_BYTES)))
         return FLAT_ERR_CUDA;
     const dim3 grid(several ? sms : group ? num_seqs * H : slabs, several ? 1 : group ? slabs : num_seqs * H);
-    (several ? fused_d128_kernel<true, 0, true> : fused_d128_kernel<true, 0, false>)<<<grid, THREADS, Layout<0>::SMEM_BYTES, st>>>(
+    (several ? fused_d128_kernel<true, 0, DEALT> : fused_d128_kernel<true, 0, ONE_ITEM>)<<<grid, THREADS, Layout<0>::SMEM_BYTES, st>>>(
         tmQ, tmK, tmV, static_cast<__nv_bfloat16*>(O), num_seqs * H, H, max_seqlen_q, 0, scale * 1.4426950408889634f, nullptr,
         causal ? 0 : (1 << 30), group, status, cu_q, cu_k, nullptr, CUtensorMap{}, 0, 0, ShiftedBias{});
     return cudaGetLastError() == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
