@@ -44,3 +44,50 @@ def test_gradients_on_16_byte_boundaries(api, d):  # noqa: F811
         api.flat_attn_bwd_ex(Q, K, V, O, dO, lse, *grads, delta, d ** -0.5)
         got.append(torch.stack(grads).view(torch.int16).cpu())
     assert torch.equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("d", [64, 128])
+def test_many_steps_a_tile(api, d, causal):  # noqa: F811
+    """Tiles of up to twelve steps, so that the next one is asked for in the middle of a tile, more of them than SMs."""
+    B, H, N = 2, 8, 1500
+    rng = np.random.default_rng(d + causal)
+    Qb, Kb, Vb, dOb = (rand_bits(rng, (B, H, N, d)) for _ in range(4))
+    O, lse, dQ, dK, dV = run_fwd_bwd(api, Qb, Kb, Vb, dOb, d ** -0.5, causal=causal)
+    heads = [0, 3, 7, 8, 12, 15]
+    ref = oracle.attention_bwd(Qb, Kb, Vb, dOb, d ** -0.5, causal=causal, heads=heads)
+    for name, got in (("dQ", dQ), ("dK", dK), ("dV", dV)):
+        assert np.all(np.isfinite(got)), name
+        check_grad(got.reshape(B * H, N, d)[heads], ref[name], "%s d=%d causal=%s" % (name, d, causal))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_while_another_stream_holds_sms(api, d):  # noqa: F811
+    """CTAs of a launch start late, and a question may find none while some have not started: the bits of an undisturbed call."""
+    g = torch.Generator(device="cuda").manual_seed(d)
+    B, H, N = 4, 16, 900
+    Q, K, V, dO = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16, generator=g) for _ in range(4))
+    W = torch.randn(4096, 4096, device="cuda", dtype=torch.bfloat16, generator=g)
+    O, lse = torch.empty_like(Q), torch.empty(B, H, N, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    own, other = torch.cuda.Stream(), torch.cuda.Stream()
+    for causal in (False, True):
+        api.flat_attn_fwd_ex(Q, K, V, O, d ** -0.5, lse=lse, causal=causal)
+        calls = []
+        for i in range(7):
+            grads = [torch.full_like(Q, float("nan")) for _ in range(3)]
+            delta = torch.empty_like(lse)
+            own.wait_stream(torch.cuda.current_stream())
+            if i > 0:                                    # (the first one alone)
+                with torch.cuda.stream(other):
+                    for _ in range(2):
+                        torch.matmul(W, W)
+            api.flat_attn_bwd_ex(Q, K, V, O, dO, lse, *grads, delta, d ** -0.5, status=status, causal=causal, stream=own.cuda_stream)
+            if i == 0:
+                torch.cuda.synchronize()
+            calls.append((grads, delta))
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        for grads, delta in calls[1:]:
+            assert torch.equal(delta, calls[0][1])
+            assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(grads, calls[0][0]))
