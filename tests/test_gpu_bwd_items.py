@@ -61,6 +61,20 @@ def test_many_steps_a_tile(api, d, causal):  # noqa: F811
         check_grad(got.reshape(B * H, N, d)[heads], ref[name], "%s d=%d causal=%s" % (name, d, causal))
 
 
+def test_groups_of_heads(api):  # noqa: F811
+    """Under the causal mask the tiles of as many heads as fit L2 go together: 62 heads here, and the other eight."""
+    B, H, N, d = 5, 14, 1500, 128
+    rng = np.random.default_rng(9)
+    Qb, Kb, Vb, dOb = (rand_bits(rng, (B, H, N, d)) for _ in range(4))
+    vl = np.array([1500, 700, 0, 1499, 1300], dtype=np.int32)
+    O, lse, dQ, dK, dV = run_fwd_bwd(api, Qb, Kb, Vb, dOb, d ** -0.5, vl=vl, causal=True)
+    heads = [0, 20, 56, 61, 62, 69]
+    ref = oracle.attention_bwd(Qb, Kb, Vb, dOb, d ** -0.5, causal=True, valid_len=vl, heads=heads)
+    for name, got in (("dQ", dQ), ("dK", dK), ("dV", dV)):
+        assert np.all(np.isfinite(got)) and np.all(got[2] == 0), name
+        check_grad(got.reshape(B * H, N, d)[heads], ref[name], "%s, groups of heads" % name)
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_while_another_stream_holds_sms(api, d):  # noqa: F811
     """CTAs of a launch start late, and a question may find none while some have not started: the bits of an undisturbed call."""
