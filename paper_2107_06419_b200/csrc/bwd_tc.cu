@@ -39,7 +39,7 @@
 //    port per tile (a broadcast read is one wavefront per column and warp); instead they join the contractions: one more
 //    slice of 16 contraction indices, (1, 1, 1, 0 ...) on the stationary side and -lse / scale, or -delta, as the sum of
 //    three bf16 numbers (24 bits) on the streamed side, gives T1 = K Q^T - lse / scale and T2 = V dO^T - delta.
-//  * A CTA that has issued the copies of its tile takes over a tile whose CTA has not started (clusterlaunchcontrol), so that
+//  * With more tiles than SMs a CTA that has issued the copies of its tile takes over a tile whose CTA has not started (clusterlaunchcontrol), so that
 //    no tile pays for launch, allocation, barrier set-up and first loads (3,500 cycles), and the next tile's operands and T are
 //    under way while this one's gradients are stored.  The stationary tiles come by TMA and go to TMEM from shared memory, and
 //    delta's rows are read side by side: a lane per row, 16 bytes an instruction, took 6,600 (d = 64) and 14,300 cycles (128).
@@ -50,7 +50,7 @@
 // Measured (both launches): B4 H16 4096 x 4096 d 64 905 -> 854 us, causal 548 -> 474; B2 H16 3000 d 128 causal 286 -> 239;
 // B8 H8 512 d 64 39.7 -> 35; B4 H8 256 d 128 26.5 -> 22.
 //
-// CTA = 640 threads, an item at a time (a tile of the stationary operands): warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four
+// CTA = 640 threads, an item at a time (a tile of the stationary operands; MULTI: its own and those it takes over): warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four
 // warps per scheduler), warp 16 TMA producer, warp 17 issues the T MMAs and warp 18 the accumulations (where P / dS
 // overlay T, warp 17 issues both), warp 19 writes the slices that carry lse and delta (MODE_DKV).
 // Under the causal mask the tiles of a head differ in length by a factor of their number: the longest tiles of a group of
@@ -181,7 +181,7 @@ __device__ __forceinline__ float exponent_factor(float scale) {
 struct Places { Divisor per, group, rest, H; };
 
 // X1, X2 / Y1, Y2 by mode:  MODE_DQ: (Q, dO) / (K, V);  MODE_DKV: (K, V) / (Q, dO).
-template <int D, int MODE>
+template <int D, int MODE, bool MULTI>
 __global__ void __launch_bounds__(BWD_THREADS, 1)
 bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ CUtensorMap tmX2,
               const __grid_constant__ CUtensorMap tmY1, const __grid_constant__ CUtensorMap tmY2,
@@ -204,10 +204,10 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* first_item = reinterpret_cast<int*>(tmem_slot + 2);
 
-    // Roles go by an index that the compiler knows to be the same in all lanes, and so does everything else in MODE_DKV.  Inside
-    // the roles of MODE_DQ it is better not known (with it / without: 128 rows against 16384 keys, d = 64 114 / 104 us, d = 128
-    // 138 / 132; MODE_DKV 16384 rows against 128 keys 124 / 128 and 231 / 249; roles by the other one, too: 107).
-    const int role = warp_index(), warp = MODE == MODE_DQ ? threadIdx.x >> 5 : role, lane = threadIdx.x & 31;
+    // Roles go by an index that the compiler knows to be the same in all lanes, and so does everything else but for the roles of
+    // MODE_DQ with several tiles (with it / without: 128 rows against 16384 keys, d = 64 114 / 104 us, d = 128 138 / 132; MODE_DKV 16384
+    // rows against 128 keys 124 / 128 and 231 / 249; roles by the other one, too: 107).
+    const int role = warp_index(), warp = MULTI && MODE == MODE_DQ ? threadIdx.x >> 5 : role, lane = threadIdx.x & 31;
     const int NX = MODE == MODE_DQ ? Nq : Nk;            // rows of the stationary tensors
     const int tiles = (NX + BT - 1) / BT;
 
@@ -253,7 +253,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     };
 
     auto decode = [&](int item) {
-        if (item == static_cast<int>(blockIdx.x)) {
+        if (!MULTI || item == static_cast<int>(blockIdx.x)) {
             bh = __shfl_sync(0xffffffffu, first_item[0], 0);
             x0 = __shfl_sync(0xffffffffu, first_item[1], 0);
         } else {
@@ -280,6 +280,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     // The n-th item (n > 0) that this CTA has taken over from one of the grid that had not started; -1: there was none left,
     // -2: gave up.  (The reader's fence orders its read before the next answer, which comes through the asynchronous proxy.)
     auto take_item = [&](int n) {
+        if (!MULTI) return -1;
         const int slot = (n - 1) & 1;
         if (!wait_warp(LY::BAR_ITEM_FULL + slot, ((n - 1) >> 1) & 1, 0x570)) return -2;
         const int item = __shfl_sync(0xffffffffu, clc_answer(next_s + 16 * slot), 0);
@@ -326,7 +327,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         int item = blockIdx.x;
         while (item >= 0) {
             decode(item);
-            if (n > 0) {                                 // the previous item's stationary tiles are read
+            if (MULTI && n > 0) {                        // the previous item's stationary tiles are read
                 ok = wait_warp(LY::BAR_X_EMPTY, (n - 1) & 1, 0x503);
                 if (ok && LY::X1_TMEM) ok = wait_warp(LY::BAR_X_TMEM, (n - 1) & 1, 0x504);
                 if (!ok) break;
@@ -344,8 +345,8 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
             int next = -3;                               // (not known yet)
             for (int g = 0; g < copies && ok; ++g) {
                 const int s1 = G % LY::S1, s2 = G % LY::S2, y = y_begin * BT + g * LY::Y_ROWS;
-                if (g == ask_at) ask();
-                if (ok && g == ask_at + 2 * LY::PARTS) next = answer();
+                if (MULTI && g == ask_at) ask();
+                if (MULTI && ok && g == ask_at + 2 * LY::PARTS) next = answer();
                 if (!ok || next == -2) break;
                 ok = wait_warp(LY::BAR_Y1_EMPTY + s1, ((G / LY::S1) & 1) ^ 1, 0x500);
                 if (!LY::DKV && ok) ok = wait_warp(LY::BAR_Y2_EMPTY + s2, ((G / LY::S2) & 1) ^ 1, 0x501);
@@ -360,8 +361,8 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                 }
                 ++G;
             }
-            if (ok && copies == 0) ask();
-            if (ok && next == -3) next = answer();
+            if (MULTI && ok && copies == 0) ask();
+            if (ok && next == -3) next = MULTI ? answer() : -1;
             if (!ok) break;
             item = next;
             ++n;
@@ -370,7 +371,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
             if (xs > 0) drain_wait(&bars[LY::BAR_X_FULL], (xs - 1) & 1);
             if (!ok || item == -2)
                 for (int g = G > LY::S1 ? G - LY::S1 : 0; g < G; ++g) drain_wait(&bars[LY::BAR_Y_FULL + g % LY::S1], (g / LY::S1) & 1);
-            if (asked > 0) drain_wait(&bars[LY::BAR_ITEM_FULL + ((asked - 1) & 1)], ((asked - 1) >> 1) & 1);
+            if (MULTI && asked > 0) drain_wait(&bars[LY::BAR_ITEM_FULL + ((asked - 1) & 1)], ((asked - 1) >> 1) & 1);
         }
       } else if (LY::DKV && warp == EW_WARPS + 3) {
         // ------------------------------------------------------------ the slices that carry lse and delta (MODE_DKV)
@@ -777,10 +778,10 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     if (warp == 0) tmem_dealloc(tmem, LY::TMEM_COLS);
 }
 
-template <int D, int MODE>
-int launch_bwd_mode(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t st) {
+template <int D, int MODE, bool MULTI>
+int launch_bwd_form(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t st) {
     using LY = BL<D, MODE>;
-    if (!ensure_dynamic_smem<bwd_tc_kernel<D, MODE>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
+    if (!ensure_dynamic_smem<bwd_tc_kernel<D, MODE, MULTI>>(LY::SMEM_BYTES)) return FLAT_ERR_CUDA;
     const int BH = p.B * p.H, tiles = ((MODE == MODE_DQ ? p.Nq : p.Nk) + BT - 1) / BT;
     if (static_cast<int64_t>(tiles) * BH > 0x7fffffff) return FLAT_ERR_SHAPE;
     // Without the causal mask the tiles of a head run side by side and share its streamed tensors in L2.  With it, the
@@ -802,11 +803,20 @@ int launch_bwd_mode(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t
     cfg.numAttrs = 1;
     auto bf = [](const void* x) { return static_cast<const __nv_bfloat16*>(x); };
     const cudaError_t e = cudaLaunchKernelEx(
-        &cfg, bwd_tc_kernel<D, MODE>, m[0], m[1], m[2], m[3], bf(MODE == MODE_DQ ? p.Q : p.K), bf(MODE == MODE_DQ ? p.dO : p.V), bf(p.O),
+        &cfg, bwd_tc_kernel<D, MODE, MULTI>, m[0], m[1], m[2], m[3], bf(MODE == MODE_DQ ? p.Q : p.K), bf(MODE == MODE_DQ ? p.dO : p.V), bf(p.O),
         p.lse, p.delta,
         static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? p.dQ : p.dK), static_cast<__nv_bfloat16*>(MODE == MODE_DQ ? nullptr : p.dV), BH,
         p.Nq, p.Nk, p.scale, p.k_valid_len, p.causal ? p.Nk - p.Nq : (1 << 30), pl, p.status);
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
+}
+
+// With no more tiles than SMs there is nothing to take over: a form without it has 20 KB of instructions less to fetch, and shorter steps
+// (us, the other form / this one: B8 H8 128^2 d 64 11.2 / 9.8, B2 H8 256^2 d 128 16.1 / 15.0, B1 H2 8192^2 117.2 / 115.1 and 187.2 / 183.3; forward and
+// backward B1 H12 512^2 d 64 26.6 / 22.9, B4 H6 629^2 d 128 45.2 / 41.0).
+template <int D, int MODE>
+int launch_bwd_mode(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t st) {
+    const int64_t tiles = ((MODE == MODE_DQ ? p.Nq : p.Nk) + BT - 1) / BT * static_cast<int64_t>(p.B) * p.H;
+    return tiles > device_sm_count() ? launch_bwd_form<D, MODE, true>(p, m, st) : launch_bwd_form<D, MODE, false>(p, m, st);
 }
 
 template <int D>
