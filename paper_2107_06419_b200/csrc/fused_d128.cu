@@ -601,16 +601,20 @@ int launch_fused_d128(const Problem& p, const BiasMap& bias, cudaStream_t st) {
     if (p.dtype != FLAT_DTYPE_BF16 || p.d != D || !p.bias != !bias.map || p.block_mask) return FLAT_ERR_UNSUPPORTED;
     // More items than SMs: several items per CTA, so that one's first loads and logits overlap the last one's output.
     // Items of up to 1024 keys, and no more than three a query, that all weigh the same (no key counts, no causal mask) are dealt in
-    // advance, unless bias rows have to be shifted (B80 H6 201^2 48.4 taken over, 56.6 dealt; B40 H6 323^2 62.6 / 68.4).  Otherwise a CTA that has issued an item's copies takes over another one (clusterlaunchcontrol): long and unequal items
+    // advance.  Otherwise a CTA that has issued an item's copies takes over another one (clusterlaunchcontrol): long and unequal items
     // end together, but every role of the CTA has to read the answer before it can go on.  us, taken over / dealt: B32 H8 300^2
     // 37.0 / 32.7, B81 H8 64^2 16.4 / 15.2, B32 H4 2000 x 500 86.0 / 80.1, B30 H8 600^2 with bias 88.0 / 83.5; B44 H4 100 x 500
     // 21.3 / 22.5, 200 x 800 32.4 / 34.8, causal B16 H16 512^2 43.9 / 49.6, key counts B12 H12 1000^2 59.9 / 61.0, B4 H16 2048^2
     // 123.0 / 124.3, H4 16K^2 412 / 424.
     // With no more items than SMs there is nothing to take over: the form for one item is the faster one at any length (us, taken over
     // / one item: B4 H8 1000^2 20.4 / 19.4, H2 16K^2 213 / 208, H1 32K^2 420 / 412, H8 4000 x 16K 217 / 211).
+    // Nor does it pay where bias rows have to be shifted and an item has more than 256 keys: its steps take twice as long, and the form for one
+    // item has the shorter ones (taken over / one item: B22 H6 323^2 34.6 / 34.4, B40 H6 450^2 79.2 / 78.4, B4 H16 1001^2 69.9 / 65.9, 2001^2 260 / 248,
+    // causal 159 / 157; below, B50 H6 101^2 20.9 / 21.9, B80 H6 201^2 48.3 / 48.6, dealt 56.6).
     const int sms = device_sm_count(), slabs = (p.Nq + 2 * BM - 1) / (2 * BM);
-    const bool alike = !p.k_valid_len && !p.causal && p.Nk <= 1024 && p.Nk <= 3 * static_cast<int64_t>(p.Nq) && bias.shifted_rows < 0;
-    const int items = static_cast<int64_t>(slabs) * p.B * p.H <= sms ? ONE_ITEM : alike ? DEALT : TAKEN_OVER;
+    const bool shifted = bias.shifted_rows >= 0;
+    const bool alike = !p.k_valid_len && !p.causal && p.Nk <= 1024 && p.Nk <= 3 * static_cast<int64_t>(p.Nq) && !shifted;
+    const int items = static_cast<int64_t>(slabs) * p.B * p.H <= sms || (shifted && p.Nk > 256) ? ONE_ITEM : alike ? DEALT : TAKEN_OVER;
     const int sr = bias.shifted_rows;
     auto run = [&](auto form) {
         constexpr int BIAS = decltype(form)::value;

@@ -61,9 +61,11 @@ def test_key_counts_with_bias(B, H, Nq, Nk, causal):
         first = got
 
 
-# Items that weigh the same, on both sides of the lines between dealing them and taking them over (three keys a query; 1024 keys)
+# Items that weigh the same, on both sides of the lines between dealing them, taking them over and one a CTA (three keys a query; 1024
+# keys; bias rows to be shifted, 256 keys)
 @pytest.mark.parametrize("bias", [False, True])
-@pytest.mark.parametrize("B,H,Nq,Nk", [(50, 8, 20, 60), (50, 8, 20, 61), (19, 8, 10, 30), (40, 8, 300, 290), (9, 8, 600, 1024), (9, 8, 600, 1025)])
+@pytest.mark.parametrize("B,H,Nq,Nk", [(50, 8, 20, 60), (50, 8, 20, 61), (19, 8, 10, 30), (40, 8, 300, 290), (9, 8, 600, 1024), (9, 8, 600, 1025),
+                                      (10, 8, 300, 255), (10, 8, 300, 257)])
 def test_equal_items(B, H, Nq, Nk, bias):
     from paper_2107_06419_b200 import api
     rng = np.random.default_rng(Nq + Nk)
