@@ -39,20 +39,23 @@
 //    port per tile (a broadcast read is one wavefront per column and warp); instead they join the contractions: one more
 //    slice of 16 contraction indices, (1, 1, 1, 0 ...) on the stationary side and -lse / scale, or -delta, as the sum of
 //    three bf16 numbers (24 bits) on the streamed side, gives T1 = K Q^T - lse / scale and T2 = V dO^T - delta.
-//  * With more tiles than SMs a CTA that has issued the copies of its tile takes over a tile whose CTA has not started (clusterlaunchcontrol), so that
-//    no tile pays for launch, allocation, barrier set-up and first loads (3,500 cycles), and the next tile's operands and T are
-//    under way while this one's gradients are stored.  The stationary tiles come by TMA and go to TMEM from shared memory, and
-//    delta's rows are read side by side: a lane per row, 16 bytes an instruction, took 6,600 (d = 64) and 14,300 cycles (128).
+//  * With more tiles than SMs a CTA that has issued the copies of its tile takes over a tile whose CTA has not started
+//    (clusterlaunchcontrol), so that no tile pays for launch, allocation, barrier set-up and first loads (3,500 cycles), and the next
+//    tile's operands and T are under way while this one's gradients are stored (MODE_DKV at d = 128: its operands; the warp that
+//    issues T there issues the accumulations, too, and waits until the last ones have been read).  The stationary tiles come by
+//    TMA and go to TMEM from shared memory, and delta's rows are read side by side: a lane per row, 16 bytes an instruction, took
+//    6,600 (d = 64) and 14,300 cycles (128).
 //    Between two tiles are now 3,300 / 3,800 cycles (dQ / dK dV, d = 64) and 5,800 / 7,100 (d = 128) instead of 11,100 / 6,900
 //    and 20,600 / 11,000; a tile of 4096 rows has 48,000 to 98,000 cycles of steps.
-//  * Waits by whole warps and values that the compiler knows to be the same in all lanes (warp_wait, the shuffles): without
-//    them 3 to 7 % a step.
-// Measured (both launches): B4 H16 4096 x 4096 d 64 905 -> 854 us, causal 548 -> 474; B2 H16 3000 d 128 causal 286 -> 239;
-// B8 H8 512 d 64 39.7 -> 35; B4 H8 256 d 128 26.5 -> 22.
+//  * Waits by whole warps (warp_wait); what the compiler knows to be the same in all lanes is chosen per form (at the warp index).
+//  * With no more tiles than SMs a form without any of the taking over: see launch_bwd_mode.
+// Measured (both launches, us, a CTA per tile with waits lane by lane before / now): B4 H16 4096 x 4096 d 64 907 / 825, causal 551 / 458;
+// B2 H16 3000 d 128 causal 287 / 235; B8 H8 512 d 64 35.7 / 27.2, d 128 55 / 39.7; B4 H8 256 d 64 13.2 / 11.5, d 128 21.3 / 15.9.
 //
-// CTA = 640 threads, an item at a time (a tile of the stationary operands; MULTI: its own and those it takes over): warps 0-15 element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four
-// warps per scheduler), warp 16 TMA producer, warp 17 issues the T MMAs and warp 18 the accumulations (where P / dS
-// overlay T, warp 17 issues both), warp 19 writes the slices that carry lse and delta (MODE_DKV).
+// CTA = 640 threads, an item at a time (a tile of the stationary operands; MULTI: its own and those it takes over): warps 0-15
+// element-wise (warp w: TMEM lane quarter w % 4, 32 of a step's 128 columns: w / 4 -- four warps per scheduler), warp 16 TMA
+// producer, warp 17 issues the T MMAs and warp 18 the accumulations (where P / dS overlay T, warp 17 issues both), warp 19 writes
+// the slices that carry lse and delta (MODE_DKV).
 // Under the causal mask the tiles of a head differ in length by a factor of their number: the longest tiles of a group of
 // heads go first (launch_bwd_mode).
 // Every wait is bounded (tc_common.cuh); on expiry the CTA aborts cleanly and reports a code.
@@ -810,9 +813,9 @@ int launch_bwd_form(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t
     return e == cudaSuccess ? FLAT_OK : FLAT_ERR_CUDA;
 }
 
-// With no more tiles than SMs there is nothing to take over: a form without it has 20 KB of instructions less to fetch, and shorter steps
-// (us, the other form / this one: B8 H8 128^2 d 64 11.2 / 9.8, B2 H8 256^2 d 128 16.1 / 15.0, B1 H2 8192^2 117.2 / 115.1 and 187.2 / 183.3; forward and
-// backward B1 H12 512^2 d 64 26.6 / 22.9, B4 H6 629^2 d 128 45.2 / 41.0).
+// With no more tiles than SMs there is nothing to take over: a form without it has 30 KB of instructions less to fetch, and shorter steps
+// (us, the other form / this one: B8 H8 128^2 d 64 11.2 / 9.8, B2 H8 256^2 d 128 16.1 / 15.0, B1 H2 8192^2 117.2 / 115.1 and
+// 187.2 / 183.3; forward and backward B1 H12 512^2 d 64 26.6 / 22.9, B4 H6 629^2 d 128 45.2 / 41.0).
 template <int D, int MODE>
 int launch_bwd_mode(const BwdProblem& p, const CUtensorMap (&m)[4], cudaStream_t st) {
     const int64_t tiles = ((MODE == MODE_DQ ? p.Nq : p.Nk) + BT - 1) / BT * static_cast<int64_t>(p.B) * p.H;

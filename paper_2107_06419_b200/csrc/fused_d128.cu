@@ -14,8 +14,8 @@
 // a port of 128 bytes a cycle): 1280 cycles of the pipe per 64 keys of both tiles, against 1024.
 // Measured, against fused_tc2_kernel on the same GPU in the first 20 ms of launches (us): B4 H16 4096^2 460 -> 428, causal 347 ->
 // 256; H8 64K causal 7,780 -> 6,350 (1,386 TFLOP/s; a cuBLAS GEMM of 8192^3 reaches 1,630 in a burst); B2 H16 3000 causal 120 ->
-// 97; B32 H16 512^2 110 -> 106.  With items taken over and uniform warp indexes 428 -> 418, 257 -> 244, 6,224 -> 6,052, 84 -> 78
-// (with lse), 89 -> 88.  After 20 ms the power cap takes the clock down: in a second of launches H8 64K causal takes 7,160
+// 97; B32 H16 512^2 110 -> 106.  Since then (waits by whole warps and a uniform warp index; items taken over or dealt) 428 -> 418, 257 ->
+// 244, 6,224 -> 6,052, 84 -> 78 (with lse), 90 -> 84.  After 20 ms the power cap takes the clock down: in a second of launches H8 64K causal takes 7,160
 // (1,229 TFLOP/s at 1,462 MHz; cuBLAS sustained 1,376), B4 H16 4096^2 498 at 1,500 MHz.  The causal gain is also the order: the
 // longest slabs first, so that short ones are left at the end.
 //

@@ -63,9 +63,10 @@ __device__ __forceinline__ bool bounded_wait_s(uint32_t bar_addr, uint32_t parit
 }
 
 // The warp's index.  The shuffle tells the compiler that it is the same in all lanes: what follows from it (roles, loops, MMA
-// operands) then stays in uniform registers.  With warp_wait below: backward 3 to 7 % a step, fused_d128 2 to 7 %,
-// fused_tf32 5 % (d = 64), fused_small 4 % (d = 16), proj_gemm and fused_decode 1 %.  Not everywhere: fused_tc3 loses 2 %,
-// fused_tc2 1 % and fused_tf32 at d = 128 11 % (ptxas spills more).
+// operands) then stays in uniform registers.  Whether that helps is a matter of each instantiation (registers, spills, which values
+// the uniform datapath gets), so every kernel says at its index what was measured: with warp_wait below dK dV 3 % a step and dQ 10 %
+// the other way, fused_d128 with several items 12 %, with one 3 % the other way in the softmax warps, fused_tf32 at d = 64 5 %,
+// fused_decode 1 %; fused_tc3 loses 2 %, fused_tc2 1 %, fused_tf32 at d = 128 11 % and the spilling forms of proj_gemm 1 to 6 %.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 
 // bounded_wait by a whole warp.  The warp stays together: its lanes probe and vote as one.  (Where each lane loops by itself,
